@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2) batch_stage_kernel
 template <typename T, int BX, int BY, int NT, bool LEARNED>
 cudaError_t batch_blocks(int* out)
 {
-    using L = TileLayout<BX, BY, false>;
+    using L = TileLayout<BX, BY, false, false, sizeof(T) == 8>;
     constexpr size_t smem = L::template total_bytes<T, NT, LEARNED>();
     static PerDevice<int> blocks;
     return blocks.get(out, [&](int* v) {
@@ -86,7 +86,7 @@ template <typename T, int BX, int BY, int NT, bool LEARNED = false>
 cudaError_t launch_batch_t(const BatchCase* cases, int ncases, int total_tiles, int stage, cudaStream_t s,
                            const SensorDev* sensor = nullptr, bool per_tile = false)
 {
-    using L = TileLayout<BX, BY, false>;
+    using L = TileLayout<BX, BY, false, false, sizeof(T) == 8>;
     constexpr size_t smem = L::template total_bytes<T, NT, LEARNED>();
     int blocks = 0;
     cudaError_t e = batch_blocks<T, BX, BY, NT, LEARNED>(&blocks);

@@ -1,0 +1,427 @@
+// MEG7-prim face states in 64-bit fixed point (the FP64 form's characteristic
+// reconstruction on the integer pipe).
+//
+// GB300 issues one FP64 warp instruction per 19 clocks and SM, where a 64-bit
+// integer add takes one clock and a 64 x 64 -> high 64 product about five, and
+// the two run side by side. Everything between the staged primitives and the
+// face states (gradients, GRB sums, characteristic projection, MP limiter) is
+// linear or a comparison, so it is done here on integers, exactly up to the
+// rounding of the projection products.
+//
+// Measured (four-quadrant problem, FP64 step, 3 stages): 1024^2 6.57 -> 3.66
+// ms, 400^2 1.28 -> 0.73 ms; viscous 1280 x 640 6.06 -> 3.93 ms. FP64
+// gradients, projection, GRB and limiter were half of the FP64 instructions
+// of a stage whose FP64 pipe was saturated; they cost the FP64 pipe nothing
+// now.
+//
+// Scaling. A variable q of one face's stencil (cells j-5 .. j+6) is held as
+// I = q / 2^(e - 1081) with e the largest biased exponent of the stencil, so
+// |I| < 2^kBits: values within 2^6 of the largest are held exactly, smaller
+// ones truncated at 2^-59 of it (an FP64 operation on the largest value
+// rounds at 2^-53 of it). The scale depends on the face's own stencil only:
+// the result does not depend on tiles, slabs or batches.
+//
+// Linear functionals. The left value at j+1/2 and the curvatures of the MP
+// limiter are sums over the even and odd differences about a cell,
+// B_k = q_{+k} + q_{-k} - 2 q_0 and A_k = q_{+k} - q_{-k}; with the
+// sixth-order gradients of Eq. six put into Eq. grb and into d_j,
+//   840 (Phi^L_j - Phi_j) = 169 B1 - 41 B2 + 9 B3 - B4 + 315 A1 - 63 A2 + 7 A3,
+//   120 d_j               = 231 B1 - 44 B2 + 9 B3 - B4,
+// and the right value about cell j+1 takes the odd part with its sign
+// changed. They are formed once per variable and then projected (ten
+// functionals per variable instead of six values and six gradients).
+//
+// The MP test (Eq. mp5Condition) is not taken: where it passes, Phi^L lies
+// between Phi_j and Phi^MP, so inside both intervals of Eq. mp-procedure, and
+// the clamp to [Phi^min, Phi^max] returns it unchanged; on integers this
+// holds exactly. (The test's threshold 1e-40 moves the result by at most
+// 1e-20, below one unit of any FP64 value that such a face state enters.)
+//
+// Overflow. With |I| < 2^59 = M after projection the largest intermediate is
+// the bound UL = Phi_j + 7 (Phi_j - Phi_{j-1}), at most 15 M < 2^63 (LC: 14.7 M).
+#pragma once
+
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define GBR_HD __host__ __device__ __forceinline__
+#else
+#define GBR_HD inline
+#include <string.h>
+#endif
+
+namespace gbr {
+namespace fx {
+
+typedef long long i64;
+typedef unsigned long long u64;
+
+constexpr int kBits = 59;           // |I| < 2^kBits
+constexpr int kExpMin = 128;        // smaller stencils count as zero
+constexpr int kExpMax = 1900;       // larger ones (infinities, NaN included) are refused
+constexpr int kOne = 1022 + kBits;  // I of a stencil with exponent e has units 2^(e - kOne)
+
+GBR_HD u64 bits_of(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (u64)__double_as_longlong(x);
+#else
+    u64 u;
+    memcpy(&u, &x, 8);
+    return u;
+#endif
+}
+GBR_HD double of_bits(u64 u)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((i64)u);
+#else
+    double x;
+    memcpy(&x, &u, 8);
+    return x;
+#endif
+}
+GBR_HD u64 mulhi_u(u64 a, u64 b)
+{
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (u64)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+// floor(x r / 2^64), x signed, r unsigned
+GBR_HD i64 mulhi(i64 x, u64 r) { return (i64)(mulhi_u((u64)x, r) - ((u64)(x >> 63) & r)); }
+
+GBR_HD int exponent(double x) { return (int)(bits_of(x) >> 52) & 0x7ff; }
+// the largest of the magnitudes' high words: exponent in bits 20..30
+GBR_HD unsigned mag(double x) { return (unsigned)(bits_of(x) >> 32) & 0x7fffffffu; }
+
+// x in units of 2^(e - kOne), truncated towards zero; x's exponent is at most
+// e, and e >= kExpMin (a zero or subnormal x is shifted out).
+GBR_HD i64 from_double(double x, int e)
+{
+    const u64 b = bits_of(x);
+    const u64 m = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << (kBits - 53);
+    int s = e - ((int)(b >> 52) & 0x7ff);
+    s = s < 63 ? s : 63;
+    const i64 v = (i64)(m >> s), g = (i64)b >> 63;
+    return (v ^ g) - g;
+}
+
+// x 2^(e - kOne) as a double, rounded to nearest; kExpMin <= e <= kExpMax + 64.
+GBR_HD double to_double(i64 x, int e)
+{
+    const i64 g = x >> 63;
+    const u64 u = (u64)((x ^ g) - g);
+    unsigned h = (unsigned)(u >> 32), l = (unsigned)u;
+    int n = 0;
+    if (h == 0) {
+        h = l;
+        l = 0;
+        n = 32;
+    }
+#ifdef __CUDA_ARCH__
+    const int z = __clz((int)h);
+    h = __funnelshift_l(l, h, z);
+#else
+    const int z = h ? __builtin_clz(h) : 32;
+    h = z == 0 ? h : (z == 32 ? 0u : (h << z) | (l >> (32 - z)));
+#endif
+    l = z == 32 ? 0u : l << z;
+    n += z;
+    const u64 t = ((u64)h << 32) | l;
+    u64 r = ((u64)(unsigned)(e + 63 - kBits - n) << 52) + (t >> 11) + ((t >> 10) & 1u);
+    r |= (u64)g & 0x8000000000000000ull;
+    return of_bits(h == 0 ? 0ull : r);
+}
+
+// Sum of c X over a few X (|X| < 2^62) and small positive integers c, exact.
+struct Acc {
+    i64 hi;
+    u64 lo;
+    GBR_HD Acc() : hi(0), lo(0) {}
+    GBR_HD void add(i64 x, unsigned c)
+    {
+        hi += (i64)(int)(x >> 32) * (int)c;
+        lo += (u64)(unsigned)x * c;
+    }
+    GBR_HD Acc operator+(const Acc& o) const
+    {
+        Acc r;
+        r.hi = hi + o.hi;
+        r.lo = lo + o.lo;
+        return r;
+    }
+    GBR_HD Acc operator-(const Acc& o) const
+    {
+        Acc r;
+        r.hi = hi - o.hi;
+        r.lo = lo - o.lo;  // (signed from here on)
+        return r;
+    }
+    template <int S>
+    GBR_HD i64 shift() const { return hi * (1ll << (32 - S)) + ((i64)lo >> S); }  // floor(sum / 2^S)
+};
+
+// Fixed-point factors: round(num / den 2^64) for num < den.
+constexpr u64 ratio(u64 num, u64 den)
+{
+    u64 q = 0, r = num;
+    for (int i = 0; i < 64; ++i) {
+        r *= 2;
+        q = 2 * q + (r >= den ? 1 : 0);
+        if (r >= den) r -= den;
+    }
+    return q + (2 * r >= den ? 1 : 0);
+}
+
+// The functionals of one variable at one face: its values at cells j-1..j+2,
+// the GRB corrections of the left value (about cell j) and the right one
+// (about j+1), and the curvatures d_{j-1} .. d_{j+2}; corrections and
+// curvatures scaled by kGrb<ORDER> and kCurv.
+struct Functionals {
+    i64 v[4], n[2], d[4];
+};
+constexpr int kGrbShift7 = 10;  // n = 840 delta / 2^10
+constexpr int kGrbShift4 = 13;  // order 4: n = 10080 delta / 2^13
+constexpr int kCurvShift = 7;   // d = 120 d_j / 2^7
+
+template <int ORDER>
+GBR_HD void functionals(const i64 (&q)[12], Functionals& f)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f.v[k] = q[4 + k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c = 4 + k;
+        const i64 c2 = q[c] + q[c];
+        const i64 B1 = q[c + 1] + q[c - 1] - c2, B2 = c2 - q[c + 2] - q[c - 2];  // (B2, B4, A2 with their signs changed)
+        const i64 B3 = q[c + 3] + q[c - 3] - c2, B4 = c2 - q[c + 4] - q[c - 4];
+        Acc d;
+        if (ORDER == 4 || k == 0 || k == 3) {
+            d.add(B1, 231);
+            d.add(B2, 44);
+            d.add(B3, 9);
+            d.add(B4, 1);
+        }
+        if (k == 1 || k == 2) {
+            const i64 A1 = q[c + 1] - q[c - 1], A2 = q[c - 2] - q[c + 2], A3 = q[c + 3] - q[c - 3];
+            Acc even, odd;
+            if (ORDER == 4) {
+                even.add(B1, 1617);
+                even.add(B2, 308);
+                even.add(B3, 63);
+                even.add(B4, 7);
+                odd.add(A1, 3780);
+                odd.add(A2, 756);
+                odd.add(A3, 84);
+            } else {
+                even.add(B1, 169);
+                even.add(B2, 41);
+                even.add(B3, 9);
+                even.add(B4, 1);
+                odd.add(A1, 315);
+                odd.add(A2, 63);
+                odd.add(A3, 7);
+                d = even;
+                d.add(B1, 62);
+                d.add(B2, 3);
+            }
+            const Acc n = k == 1 ? even + odd : even - odd;
+            f.n[k - 1] = n.shift<ORDER == 4 ? kGrbShift4 : kGrbShift7>();
+        }
+        f.d[k] = d.shift<kCurvShift>();
+    }
+}
+
+// f r / 2^64 of every functional.
+GBR_HD void scale(const Functionals& f, u64 r, Functionals& o)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        o.v[k] = mulhi(f.v[k], r);
+        o.d[k] = mulhi(f.d[k], r);
+    }
+    o.n[0] = mulhi(f.n[0], r);
+    o.n[1] = mulhi(f.n[1], r);
+}
+GBR_HD void sum(const Functionals& a, const Functionals& b, Functionals& o)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        o.v[k] = a.v[k] + b.v[k];
+        o.d[k] = a.d[k] + b.d[k];
+    }
+    o.n[0] = a.n[0] + b.n[0];
+    o.n[1] = a.n[1] + b.n[1];
+}
+GBR_HD void difference(const Functionals& a, const Functionals& b, Functionals& o)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        o.v[k] = a.v[k] - b.v[k];
+        o.d[k] = a.d[k] - b.d[k];
+    }
+    o.n[0] = a.n[0] - b.n[0];
+    o.n[1] = a.n[1] - b.n[1];
+}
+
+// Every functional / 2^k: from a finer scale to one k larger.
+GBR_HD void shift_right(Functionals& f, int k)
+{
+    k = k < 63 ? k : 63;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        f.v[i] >>= k;
+        f.d[i] >>= k;
+    }
+    f.n[0] >>= k;
+    f.n[1] >>= k;
+}
+
+// Eq. alpha's minmod.
+GBR_HD i64 minmod(i64 a, i64 b)
+{
+    const bool first = (a < b) != (a < 0);  // same signs: the smaller magnitude
+    const i64 r = first ? a : b;
+    return (a ^ b) < 0 ? 0 : r;
+}
+
+// pl clamped to [Phi^min, Phi^max] of Eq. mp-procedure (min distributes over
+// max: four comparisons a bound instead of five).
+GBR_HD i64 mp_clamp(i64 p2, i64 p3, i64 md, i64 ul, i64 lc, i64 pl)
+{
+    const bool c1 = p3 < md, c2 = ul < lc;
+    const i64 n1 = c1 ? p3 : md, x1 = c1 ? md : p3;
+    const i64 n2 = c2 ? ul : lc, x2 = c2 ? lc : ul;
+    const i64 n3 = n1 > n2 ? n1 : n2, x3 = x1 < x2 ? x1 : x2;
+    const i64 mn = p2 < n3 ? p2 : n3, mx = p2 > x3 ? p2 : x3;
+    const i64 r = pl > mn ? pl : mn;
+    return r < mx ? r : mx;
+}
+
+// n -> delta = Phi^GRB - Phi_j: 2^10 / 840 = 1 + 184/840; 2^13 / 10080.
+template <int ORDER>
+GBR_HD i64 grb_delta(i64 n)
+{
+    return ORDER == 4 ? mulhi(n, ratio(8192, 10080)) : n + mulhi(n, ratio(184, 840));
+}
+
+// The MP-limited left and right values (Eqs. grb, mp-procedure) at the face.
+template <int ORDER>
+GBR_HD void limited(const Functionals& f, i64& vl, i64& vr)
+{
+    const i64 aL = f.v[0] - f.v[1], aR = f.v[3] - f.v[2];
+    const i64 mc = minmod(f.d[1], f.d[2]), mL = minmod(f.d[1], f.d[0]), mR = minmod(f.d[2], f.d[3]);
+    // d = 120 d_j / 128: d_j = d + d 8/120, 4/3 d_j = d + d (512 - 360)/360
+    const i64 md = (f.v[1] + f.v[2] - mc - mulhi(mc, ratio(8, 120))) >> 1;
+    const i64 lcL = f.v[1] - (aL >> 1) + mL + mulhi(mL, ratio(152, 360));
+    const i64 lcR = f.v[2] - (aR >> 1) + mR + mulhi(mR, ratio(152, 360));
+    vl = mp_clamp(f.v[1], f.v[2], md, f.v[1] - 7 * aL, lcL, f.v[1] + grb_delta<ORDER>(f.n[0]));
+    vr = mp_clamp(f.v[2], f.v[1], md, f.v[2] - 7 * aR, lcR, f.v[2] + grb_delta<ORDER>(f.n[1]));
+}
+
+// A stencil's scale.
+GBR_HD int stencil_exponent(const double (&x)[12])
+{
+    unsigned m = (unsigned)kExpMin << 20;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const unsigned h = mag(x[k]);
+        m = h > m ? h : m;
+    }
+    return (int)(m >> 20);
+}
+
+template <int ORDER>
+GBR_HD void variable(const double (&x)[12], int e, Functionals& f)
+{
+    i64 q[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) q[k] = from_double(x[k], e);
+    functionals<ORDER>(q, f);
+}
+
+// A positive factor a applied to a variable of scale e, for a result of scale
+// eo: the r of scale(). The product's own scale is e + exponent(a) - 1022,
+// and eo is at least that.
+GBR_HD u64 factor(double a, int e, int eo)
+{
+    const u64 m = ((bits_of(a) & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;  // a = m 2^(exponent - 1086)
+    int k = eo - (e + exponent(a) - 1022);
+    k = k < 63 ? k : 63;
+    return k < 63 ? m >> k : 0;
+}
+
+// Characteristic face states of one field pair (L, R): sums and differences of
+// the acoustic fields, entropy and shear.
+struct FaceStates {
+    double a03[2], dif[2], s[2], ut[2];  // w1 + w4, w4 - w1, w2, w3 (acoustic fields as p -/+ rho c un)
+    bool ok;                             // false: a stencil value too large, infinite or NaN
+};
+
+// u[m]: primitive planes (rho, un, ut, p) at cell j, su: their stride; rc =
+// rho c and ic2 = 1 / c^2 of the face's mean state.
+template <int ORDER>
+GBR_HD void face_states(const double* const (&u)[4], int su, double rc, double ic2, FaceStates& o)
+{
+    auto load = [&](int m, double (&x)[12]) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) x[k] = u[m][(k - 5) * su];
+    };
+    Functionals P;
+    i64 wl, wr;
+    int ep, es, et, ew;
+    {
+        double x[12];
+        load(3, x);
+        ep = stencil_exponent(x);
+        variable<ORDER>(x, ep, P);
+    }
+    {  // field 2 (entropy): rho - p / c^2
+        double x[12];
+        load(0, x);
+        const int er = stencil_exponent(x), eprod = ep + exponent(ic2) - 1022;
+        es = (er > eprod ? er : eprod) + 1;
+        Functionals R, S;
+        scale(P, factor(ic2, ep, es), S);
+        variable<ORDER>(x, es, R);
+        difference(R, S, R);
+        limited<ORDER>(R, wl, wr);
+        o.s[0] = to_double(wl, es);
+        o.s[1] = to_double(wr, es);
+    }
+    {  // fields 1 and 4 (u -/+ c), carried as p -/+ rho c un
+        double x[12];
+        load(1, x);
+        const int eu = stencil_exponent(x), eprod = eu + exponent(rc) - 1022;
+        ew = (ep > eprod ? ep : eprod) + 1;
+        Functionals U, W;
+        variable<ORDER>(x, eu, U);
+        scale(U, factor(rc, eu, ew), U);
+        shift_right(P, ew - ep);
+        i64 ml, mr;
+        difference(P, U, W);
+        limited<ORDER>(W, ml, mr);
+        sum(P, U, W);
+        limited<ORDER>(W, wl, wr);
+        o.a03[0] = to_double(wl + ml, ew);
+        o.a03[1] = to_double(wr + mr, ew);
+        o.dif[0] = to_double(wl - ml, ew);
+        o.dif[1] = to_double(wr - mr, ew);
+    }
+    {  // field 3 (shear): ut
+        double x[12];
+        load(2, x);
+        et = stencil_exponent(x);
+        Functionals R;
+        variable<ORDER>(x, et, R);
+        limited<ORDER>(R, wl, wr);
+        o.ut[0] = to_double(wl, et);
+        o.ut[1] = to_double(wr, et);
+    }
+    o.ok = ew <= kExpMax && es <= kExpMax && et <= kExpMax;
+}
+
+}  // namespace fx
+}  // namespace gbr

@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fixed_face.cuh"
 #include "fp_convert.cuh"
 #include "gbr_internal.h"
 #include "sensor.cuh"
@@ -72,14 +73,20 @@ struct TileLayout {
     // conservative values; their arrays then come before the gradients, so
     // that the TMA landing area (at the gradients, over the face fluxes) does
     // not overlap them.
+    // GRAD: gradient arrays are kept. FP64 MEG7-prim forms its face states
+    // from the primitives themselves (fixed_face.cuh) and needs gradients for
+    // the viscous flux only.
+    static constexpr bool GRAD = !FLUX0 || CONS || VISC;
     static constexpr int oU = 0;
     static constexpr int oGX = FLUX0 ? oU + 4 * NU + 4 * (NFX + NFY) : oU + 4 * NU;
-    static constexpr int oGY = oGX + 4 * NGX;
+    static constexpr int oGY = oGX + (GRAD ? 4 * NGX : 0);
     static constexpr int oFX = FLUX0 ? oU + 4 * NU : oGY + 4 * NGY;
     static constexpr int oFY = oFX + 4 * NFX;
-    static constexpr int oHX = FLUX0 ? oGY + 4 * NGY : oFY + 4 * NFY;
+    static constexpr int oHX = FLUX0 ? oGY + (GRAD ? 4 * NGY : 0) : oFY + 4 * NFY;
     static constexpr int oHY = oHX + 4 * NHX;
-    static constexpr int oQc = oHY + 4 * NHY;         // conservative values (MEG7-cons)
+    static constexpr int oH1 = oHY + 4 * NHY;
+    // (without gradients the staging's landing area outgrows the face fluxes)
+    static constexpr int oQc = !GRAD && oH1 < oGX + 4 * NU ? oGX + 4 * NU : oH1;  // conservative values (MEG7-cons)
     static constexpr int oEnd = oQc + (CONS ? 4 * NU : 0);
 
     // learned sensor: per-cell decisions on the bounding box of both
@@ -603,8 +610,21 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
     const T ic2 = icb * icb;         // 1 / c^2
     const T be = T(0.5) * ic2;       // 1 / (2 c^2)
 
+    // FP64 MEG7-prim: the characteristic face states on the integer pipe
+    constexpr bool FIXED = sizeof(T) == 8 && !CONS;
     T wL[4], wR[4];
-    if constexpr (!CONS) {
+    if constexpr (FIXED) {
+        fx::FaceStates st;
+        fx::face_states<ORDER>(in.u, su, rb * cb, ic2, st);
+        wL[0] = st.a03[0];
+        wR[0] = st.a03[1];
+        wL[3] = st.dif[0];
+        wR[3] = st.dif[1];
+        wL[1] = st.ok ? st.s[0] : T(-1);  // (a refused stencil takes the positivity fallback below)
+        wR[1] = st.ok ? st.s[1] : T(-1);
+        wL[2] = st.ut[0];
+        wR[2] = st.ut[1];
+    } else if constexpr (!CONS) {
         {  // fields 1 and 4 (u - c and u + c) share un and p. They are
            // carried scaled by 2 c^2, as p -/+ rho c un: GRB, the limiter's
            // bounds and its clamp are linear and scale-free, and the MP
@@ -671,13 +691,13 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         // a = w1 + w4, rho = a / (2 c^2) + w2, p = a / 2 and
         // un = (w4 - w1) / (2 rho c)
         const T hrc = T(0.5) * y;  // 1 / (2 rho c): rho c = gamma p rho y = 1 / y
-        const T aL03 = wL[0] + wL[3], aR03 = wR[0] + wR[3];
+        const T aL03 = FIXED ? wL[0] : wL[0] + wL[3], aR03 = FIXED ? wR[0] : wR[0] + wR[3];
         rL = rfma(be, aL03, wL[1]);
-        unL = hrc * (wL[3] - wL[0]);
+        unL = hrc * (FIXED ? wL[3] : wL[3] - wL[0]);
         utL = wL[2];
         pL = T(0.5) * aL03;
         rR = rfma(be, aR03, wR[1]);
-        unR = hrc * (wR[3] - wR[0]);
+        unR = hrc * (FIXED ? wR[3] : wR[3] - wR[0]);
         utR = wR[2];
         pR = T(0.5) * aR03;
         // positivity fallback: a face state with rho <= 0 or p <= 0 takes the
@@ -1414,13 +1434,13 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
 
     // Phase 1: per-cell quantities, each computed once per tile.
     const T* const sV = CONS ? sQc : sU;  // the reconstructed variables
-    for (int idx = tid; idx < L::NGX; idx += NT) {  // x-gradients (Eq. six)
+    for (int idx = tid; idx < (L::GRAD ? L::NGX : 0); idx += NT) {  // x-gradients (Eq. six)
         const int a = idx / L::GXW, b = idx - a * L::GXW;
         const T* s = sV + (a + 6 - V) * RW + (b + 3);
 #pragma unroll
         for (int m = 0; m < 4; ++m) sGX[m * L::NGX + idx] = grad6(s + m * NU, 1);
     }
-    for (int idx = tid; idx < L::NGY; idx += NT) {  // y-gradients
+    for (int idx = tid; idx < (L::GRAD ? L::NGY : 0); idx += NT) {  // y-gradients
         const int a = idx / L::GYW, b = idx - a * L::GYW;
         const T* s = sV + (a + 3) * RW + (b + 6 - V);
 #pragma unroll

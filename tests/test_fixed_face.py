@@ -1,0 +1,137 @@
+"""The fixed-point face states (csrc/fixed_face.cuh, the FP64 form's
+characteristic reconstruction) compiled for the host and compared with the
+MEG7 procedure written out in long double (64 mantissa bits or more): the
+reconstruction is exact on integers up to the projection's truncations (about
+ten units of at most 2^-56 of the stencil's largest value) and the rounding of
+each result to FP64, hence the tolerance 2^-53 |value| + 2^-52 scale."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2305_00762_gb300", "csrc")
+
+SRC = r"""
+#include <cmath>
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+#include "fixed_face.cuh"
+using namespace gbr;
+typedef long double R;
+static R mm(R a, R b) { return (a < 0) != (b < 0) ? 0 : (fabsl(a) < fabsl(b) ? a : b); }
+static R meg(const R* w, const R* e, int order)
+{
+    const R d0 = w[0] - w[2], d1 = w[1] - w[2], d2 = w[3] - w[2], d3 = w[4] - w[2];
+    const R pl = order == 4 ? w[2] + e[2] / 2 + (e[1] - e[3]) / 24 + (d1 + d2) / 6
+                            : w[2] + (420 * e[2] + 60 * (e[1] - e[3]) + 178 * (d1 + d2) + 3 * (d0 + d3)) / 840;
+    const R mp = w[2] + mm(d2, -7 * d1);
+    if ((pl - w[2]) * (pl - mp) <= 1e-40L) return pl;
+    const R cm = 2 * (w[2] - 2 * w[1] + w[0]) - (e[2] - e[0]) / 2, c0 = 2 * (w[3] - 2 * w[2] + w[1]) - (e[3] - e[1]) / 2;
+    const R cp = 2 * (w[4] - 2 * w[3] + w[2]) - (e[4] - e[2]) / 2;
+    const R md = (w[2] + w[3]) / 2 - mm(c0, cp) / 2, ul = w[2] - 7 * d1, lc = (3 * w[2] - w[1]) / 2 + mm(c0, cm) * 4 / 3;
+    const R lo = fmaxl(fminl(fminl(w[2], w[3]), md), fminl(fminl(w[2], ul), lc));
+    const R hi = fminl(fmaxl(fmaxl(w[2], w[3]), md), fmaxl(fmaxl(w[2], ul), lc));
+    return pl < lo ? lo : (pl > hi ? hi : pl);
+}
+template <int ORDER>
+static int run(int mode, int stride)
+{
+    std::mt19937_64 g(7 + mode);
+    std::uniform_real_distribution<double> U(-1, 1);
+    double worst = 0;
+    for (int it = 0; it < 20000; ++it) {
+        double v[4][12 * 3];
+        const double sc = mode == 2 ? std::pow(10.0, 6 * U(g)) : 1;
+        for (int m = 0; m < 4; ++m) {
+            const bool pos = m == 0 || m == 3;
+            const double base = pos ? 1.5 + U(g) : (mode == 3 ? 30 * U(g) : U(g)), amp = std::pow(10.0, -8 * std::fabs(U(g)));
+            const double jump = mode == 0 ? 0 : (pos ? std::fabs(U(g)) * 100 : U(g));
+            const int at = (int)(g() % 13);
+            for (int k = 0; k < 12; ++k) {
+                double x = base + amp * (std::sin(0.7 * k + base) + 0.1 * U(g)) + (k < at ? jump : 0);
+                if (mode == 4) x = pos ? 1.25 : (k % 2 ? 0.0 : -0.0);
+                v[m][k * stride] = sc * (pos ? std::fabs(x) + 1e-3 : x);
+            }
+        }
+        const double* u[4] = {v[0] + 5 * stride, v[1] + 5 * stride, v[2] + 5 * stride, v[3] + 5 * stride};
+        const double rb = 0.5 * (u[0][0] + u[0][stride]), pb = 0.5 * (u[3][0] + u[3][stride]);
+        const double c = std::sqrt(1.4 * pb / rb), rc = rb * c, ic2 = 1 / (c * c);
+        fx::FaceStates o;
+        fx::face_states<ORDER>(u, stride, rc, ic2, o);
+        if (!o.ok) return std::printf("refused\n"), 1;
+        R wl[4], wr[4], big[3] = {0, 0, 0};
+        for (int f = 0; f < 4; ++f) {
+            R q[12], e[12], a[5], b[5];
+            for (int k = 0; k < 12; ++k) {
+                const R r = v[0][k * stride], n = v[1][k * stride], t = v[2][k * stride], p = v[3][k * stride];
+                q[k] = f == 0 ? p - (R)rc * n : f == 3 ? p + (R)rc * n : f == 1 ? r - (R)ic2 * p : t;
+                const R s = f == 1 ? r + (R)ic2 * p : f == 2 ? fabsl(t) : p + (R)rc * fabsl(n);
+                R& B = big[f == 1 ? 1 : f == 2 ? 2 : 0];
+                B = fmaxl(B, s);
+            }
+            for (int k = 3; k < 9; ++k) e[k] = (45 * (q[k + 1] - q[k - 1]) - 9 * (q[k + 2] - q[k - 2]) + (q[k + 3] - q[k - 3])) / 60;
+            for (int k = 0; k < 5; ++k) a[k] = q[3 + k], b[k] = e[3 + k];
+            wl[f] = meg(a, b, ORDER);
+            for (int k = 0; k < 5; ++k) a[k] = q[8 - k], b[k] = -e[8 - k];
+            wr[f] = meg(a, b, ORDER);
+        }
+        const R ref[8] = {wl[0] + wl[3], wr[0] + wr[3], wl[3] - wl[0], wr[3] - wr[0], wl[1], wr[1], wl[2], wr[2]};
+        const double got[8] = {o.a03[0], o.a03[1], o.dif[0], o.dif[1], o.s[0], o.s[1], o.ut[0], o.ut[1]};
+        for (int k = 0; k < 8; ++k) {
+            const R tol = ldexpl(fabsl(ref[k]), -53) + ldexpl(big[k < 4 ? 0 : k < 6 ? 1 : 2], -52);
+            const R d = fabsl(ref[k] - (R)got[k]);
+            if (!(d <= tol)) return std::printf("order %d mode %d value %d: %g off, %g allowed\n", ORDER, mode, k, (double)d, (double)tol), 1;
+            if (tol > 0 && (double)(d / tol) > worst) worst = (double)(d / tol);
+        }
+    }
+    std::printf("order %d mode %d: at most %.2f of the tolerance\n", ORDER, mode, worst);
+    return 0;
+}
+static int limits()
+{
+    // integers round to double and back; infinities, NaN and overflowing scales are refused
+    std::mt19937_64 g(1);
+    for (int i = 0; i < 1000000; ++i) {
+        const long long x = (long long)(g() >> (2 + g() % 62)) * (g() & 1 ? 1 : -1);
+        const double d = fx::to_double(x, fx::kOne);
+        if (std::fabs((double)((R)d - (R)x)) > std::ldexp(std::fabs((double)x), -53)) return std::printf("%lld -> %.17g\n", x, d), 1;
+        if (std::fabs((double)x) < 9e15 && fx::from_double(d, 1081) != x * 1) return std::printf("back %lld\n", x), 1;
+    }
+    if (fx::to_double(0, 700) != 0.0 || fx::from_double(0.0, fx::kExpMin) != 0 || fx::from_double(-5e-324, 900) != 0) return 1;
+    for (double bad : {(double)INFINITY, (double)NAN, 1e300, -(double)INFINITY}) {
+        double v[12];
+        for (int m = 0; m < 4; ++m) {
+            double w[4][12];
+            for (int i = 0; i < 4; ++i)
+                for (int k = 0; k < 12; ++k) w[i][k] = 1.0;
+            w[m][3] = bad;
+            const double* u[4] = {w[0] + 5, w[1] + 5, w[2] + 5, w[3] + 5};
+            fx::FaceStates o;
+            fx::face_states<7>(u, 1, 1.2, 0.7, o);
+            if (o.ok) return std::printf("%g accepted in plane %d\n", bad, m), 1;
+        }
+        (void)v;
+    }
+    return 0;
+}
+int main()
+{
+    int bad = limits();
+    for (int mode = 0; mode < 5; ++mode) bad |= run<7>(mode, 1 + mode % 3) | run<4>(mode, 1 + mode % 3);
+    return bad;
+}
+"""
+
+
+def test_fixed_point_face_states(tmp_path):
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no host compiler")
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text(SRC)
+    subprocess.run([cxx, "-O2", "-std=c++17", "-Wno-unknown-pragmas", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
