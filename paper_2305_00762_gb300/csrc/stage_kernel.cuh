@@ -18,6 +18,7 @@
 #include <stdint.h>
 
 #include "fixed_face.cuh"
+#include "fixed_math.cuh"
 #include "fp_convert.cuh"
 #include "gbr_internal.h"
 #include "sensor.cuh"
@@ -121,10 +122,13 @@ __device__ __forceinline__ T tmax(T a, T b) { return a > b ? a : b; }
 // FP32: one min / max instruction (the same value for operands that are not NaN)
 __device__ __forceinline__ float tmin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ float tmax(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double tsqrt(double x) { return sqrt(x); }
+// FP64 roots and reciprocals come from the integer pipe (fixed_math.cuh).
+__device__ __forceinline__ double tsqrt(double x) { return __double_as_longlong(x) == 0 ? x : x * fx::rsqrt(x); }
 __device__ __forceinline__ float tsqrt(float x) { return sqrtf(x); }
-__device__ __forceinline__ double trsqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ double trsqrt(double x) { return fx::rsqrt(x); }
 __device__ __forceinline__ float trsqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double trcp(double x) { return fx::rcp(x); }
+__device__ __forceinline__ float trcp(float x) { return 1.f / x; }
 __device__ __forceinline__ double tsinpi(double x) { return sinpi(x); }
 __device__ __forceinline__ float tsinpi(float x) { return sinpif(x); }
 __device__ __forceinline__ double tabs(double x) { return fabs(x); }
@@ -237,7 +241,7 @@ template <typename T>
 __device__ __forceinline__ void prims_of(double q0, double q1, double q2, double q3, T gm1, T& r, T& u, T& v, T& p)
 {
     r = from_f64<T>(q0);
-    const T ir = T(1) / r;
+    const T ir = trcp(r);
     u = from_f64<T>(q1) * ir;
     v = from_f64<T>(q2) * ir;
     p = gm1 * rfma(-rmul(T(0.5), r), sumsq(u, v), from_f64<T>(q3));
@@ -253,7 +257,7 @@ __device__ __forceinline__ T cell_wavespeed_t(double q0, double q1, double q2, d
 {
     T r, u, v, p;
     prims_of(q0, q1, q2, q3, gm1, r, u, v, p);
-    const T ir = T(1) / r;
+    const T ir = trcp(r);
     const T cs = tsqrt(gamma * p * ir);
     T l = tmax((tabs(u) + cs) * inv_dx, (tabs(v) + cs) * inv_dy);
     if (mu > T(0)) {
@@ -743,7 +747,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         rL = QL[0];
         EL = QL[3];
         {
-            const T ir = T(1) / rL;
+            const T ir = trcp(rL);
             unL = QL[1] * ir;
             utL = QL[2] * ir;
             pL = P.gm1 * (EL - T(0.5) * rL * (unL * unL + utL * utL));
@@ -751,7 +755,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         rR = QR[0];
         ER = QR[3];
         {
-            const T ir = T(1) / rR;
+            const T ir = trcp(rR);
             unR = QR[1] * ir;
             utR = QR[2] * ir;
             pR = P.gm1 * (ER - T(0.5) * rR * (unR * unR + utR * utR));
@@ -811,7 +815,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         // Roe averages (a_L + q a_R) / (1 + q), q = sqrt(rho_R / rho_L)
         const T xq = rR * irL;
         const T q = xq * trsqrt(xq);
-        const T oL = T(1) / (T(1) + q);
+        const T oL = trcp(T(1) + q);
         const T ut = oL * rfma(q, unR, unL);
         const T vt = oL * rfma(q, utR, utL);
         const T Ht = oL * rfma(q, HR, HL);
@@ -826,7 +830,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         const T num = pR - pL + mL * unL - mR * unR, den = mL - mR;
         const T nL = SL * den - num, nR = SR * den - num;
         const T nLR = nL * nR;
-        const T z = T(1) / (den * nLR);
+        const T z = trcp(den * nLR);
         const T Ss = num * nLR * z;
         const T d2z = den * den * z;
         const T iL = nR * d2z, iR = nL * d2z;  // 1/(S_L - S*), 1/(S_R - S*)
@@ -872,7 +876,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         T dn0 = in.g[1][0], dn1 = in.g[1][sg];
         T dt0 = in.g[2][0], dt1 = in.g[2][sg];
         T dp0 = in.g[3][0], dp1 = in.g[3][sg];
-        const T ir0 = T(1) / r0, ir1 = T(1) / r1;
+        const T ir0 = trcp(r0), ir1 = trcp(r1);
         if constexpr (CONS) {  // primitive gradients from the conservative ones (chain rule)
             const T k0 = T(0.5) * (n0 * n0 + t0 * t0), k1 = T(0.5) * (n1 * n1 + t1 * t1);
             const T e0 = dp0, e1 = dp1;  // dE
