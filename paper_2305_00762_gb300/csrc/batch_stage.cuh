@@ -6,7 +6,7 @@
 // whose dt is zero (stopped at their end time) are skipped.
 #pragma once
 
-#include "stage_kernel.cuh"
+#include "fixed_stage.cuh"
 
 namespace gbr {
 
@@ -19,6 +19,14 @@ __device__ __forceinline__ int batch_case_of(const BatchCase* cases, int ncases,
         else hi = mid - 1;
     }
     return lo;
+}
+
+// Dynamic shared memory of one tile.
+template <typename T, int BX, int BY, int NT, bool LEARNED>
+constexpr size_t batch_smem()
+{
+    if constexpr (sizeof(T) == 8) return FixedLayout<BX, BY, false>::bytes;
+    else return TileLayout<BX, BY, false>::template total_bytes<T, NT, LEARNED>();
 }
 
 // Register budgets for the CTAs per SM that shared memory allows: three in
@@ -55,7 +63,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2) batch_stage_kernel
         P.dec = C.dec;
         P.stall_bytes = 0;
         P.stall_mma = 0;
-        stage_tile<T, BX, BY, NT, false, LEARNED>(P, tx * BX, ty * BY, smem_raw);
+        if constexpr (sizeof(T) == 8) fixed_tile<BX, BY, NT, false, 7, false>(P, tx * BX, ty * BY, smem_raw);
+        else stage_tile<T, BX, BY, NT, false, LEARNED>(P, tx * BX, ty * BY, smem_raw);
     }
 }
 
@@ -65,8 +74,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2) batch_stage_kernel
 template <typename T, int BX, int BY, int NT, bool LEARNED>
 cudaError_t batch_blocks(int* out)
 {
-    using L = TileLayout<BX, BY, false, false, sizeof(T) == 8>;
-    constexpr size_t smem = L::template total_bytes<T, NT, LEARNED>();
+    constexpr size_t smem = batch_smem<T, BX, BY, NT, LEARNED>();
     static PerDevice<int> blocks;
     return blocks.get(out, [&](int* v) {
         auto kern = batch_stage_kernel<T, BX, BY, NT, LEARNED>;
@@ -86,8 +94,7 @@ template <typename T, int BX, int BY, int NT, bool LEARNED = false>
 cudaError_t launch_batch_t(const BatchCase* cases, int ncases, int total_tiles, int stage, cudaStream_t s,
                            const SensorDev* sensor = nullptr, bool per_tile = false)
 {
-    using L = TileLayout<BX, BY, false, false, sizeof(T) == 8>;
-    constexpr size_t smem = L::template total_bytes<T, NT, LEARNED>();
+    constexpr size_t smem = batch_smem<T, BX, BY, NT, LEARNED>();
     int blocks = 0;
     cudaError_t e = batch_blocks<T, BX, BY, NT, LEARNED>(&blocks);
     if (e != cudaSuccess || total_tiles <= 0) return e;

@@ -17,7 +17,7 @@
 // Scaling. A variable q of one face's stencil (cells j-5 .. j+6) is held as
 // I = q / 2^(e - 1081) with e the largest biased exponent of the stencil, so
 // |I| < 2^kBits: values within 2^6 of the largest are held exactly, smaller
-// ones truncated at 2^-59 of it (an FP64 operation on the largest value
+// ones rounded down at 2^-59 of it (an FP64 operation on the largest value
 // rounds at 2^-53 of it). The scale depends on the face's own stencil only:
 // the result does not depend on tiles, slabs or batches.
 //
@@ -93,19 +93,29 @@ GBR_HD u64 mulhi_u(u64 a, u64 b)
 GBR_HD i64 mulhi(i64 x, u64 r) { return (i64)(mulhi_u((u64)x, r) - ((u64)(x >> 63) & r)); }
 
 GBR_HD int exponent(double x) { return (int)(bits_of(x) >> 52) & 0x7ff; }
-// the largest of the magnitudes' high words: exponent in bits 20..30
-GBR_HD unsigned mag(double x) { return (unsigned)(bits_of(x) >> 32) & 0x7fffffffu; }
 
-// x in units of 2^(e - kOne), truncated towards zero; x's exponent is at most
-// e, and e >= kExpMin (a zero or subnormal x is shifted out).
-GBR_HD i64 from_double(double x, int e)
+// A double taken apart once, where it is produced, so that each of the many
+// stencils that read it only shifts: x = m 2^(e - kOne), |m| < 2^kBits, e the
+// biased exponent (zeros and subnormals: m = 0, e = 1).
+GBR_HD void split(double x, i64& m, unsigned short& e)
 {
     const u64 b = bits_of(x);
-    const u64 m = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << (kBits - 53);
-    int s = e - ((int)(b >> 52) & 0x7ff);
-    s = s < 63 ? s : 63;
-    const i64 v = (i64)(m >> s), g = (i64)b >> 63;
-    return (v ^ g) - g;
+    const int ex = (int)(b >> 52) & 0x7ff;
+    const i64 v = (i64)(((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << (kBits - 53)), g = (i64)b >> 63;
+    m = ex == 0 ? 0 : (v ^ g) - g;
+    e = (unsigned short)(ex == 0 ? 1 : ex);
+}
+GBR_HD double unsplit(i64 m, int e)  // exact
+{
+    const i64 g = m >> 63;
+    const u64 a = (u64)((m ^ g) - g) >> (kBits - 53);
+    return of_bits((((u64)(unsigned)(e - 1) << 52) + a) | ((u64)g & 0x8000000000000000ull));
+}
+// The split value m, ex in units 2^(e - kOne), ex <= e, rounded down.
+GBR_HD i64 aligned(i64 m, int ex, int e)
+{
+    const int s = e - ex;
+    return m >> (s < 63 ? s : 63);
 }
 
 // x 2^(e - kOne) as a double, rounded to nearest; kExpMin <= e <= kExpMax + 64.
@@ -321,24 +331,25 @@ GBR_HD void limited(const Functionals& f, i64& vl, i64& vr)
     vr = mp_clamp(f.v[2], f.v[1], md, f.v[2] - 7 * aR, lcR, f.v[2] + grb_delta<ORDER>(f.n[1]));
 }
 
-// A stencil's scale.
-GBR_HD int stencil_exponent(const double (&x)[12])
+// Twelve split values of one variable, cells j-5 .. j+6, and their scale.
+struct Stencil {
+    i64 m[12];
+    int e[12];
+};
+GBR_HD int stencil_exponent(const Stencil& x)
 {
-    unsigned m = (unsigned)kExpMin << 20;
+    int e = kExpMin;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const unsigned h = mag(x[k]);
-        m = h > m ? h : m;
-    }
-    return (int)(m >> 20);
+    for (int k = 0; k < 12; ++k) e = x.e[k] > e ? x.e[k] : e;
+    return e;
 }
 
 template <int ORDER>
-GBR_HD void variable(const double (&x)[12], int e, Functionals& f)
+GBR_HD void variable(const Stencil& x, int e, Functionals& f)
 {
     i64 q[12];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) q[k] = from_double(x[k], e);
+    for (int k = 0; k < 12; ++k) q[k] = aligned(x.m[k], x.e[k], e);
     functionals<ORDER>(q, f);
 }
 
@@ -360,26 +371,22 @@ struct FaceStates {
     bool ok;                             // false: a stencil value too large, infinite or NaN
 };
 
-// u[m]: primitive planes (rho, un, ut, p) at cell j, su: their stride; rc =
-// rho c and ic2 = 1 / c^2 of the face's mean state.
-template <int ORDER>
-GBR_HD void face_states(const double* const (&u)[4], int su, double rc, double ic2, FaceStates& o)
+// load(m, x): the stencil of variable m (0 rho, 1 un, 2 ut, 3 p); rc = rho c
+// and ic2 = 1 / c^2 of the face's mean state.
+template <int ORDER, typename F>
+GBR_HD void face_states(F load, double rc, double ic2, FaceStates& o)
 {
-    auto load = [&](int m, double (&x)[12]) {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) x[k] = u[m][(k - 5) * su];
-    };
     Functionals P;
     i64 wl, wr;
     int ep, es, et, ew;
     {
-        double x[12];
+        Stencil x;
         load(3, x);
         ep = stencil_exponent(x);
         variable<ORDER>(x, ep, P);
     }
     {  // field 2 (entropy): rho - p / c^2
-        double x[12];
+        Stencil x;
         load(0, x);
         const int er = stencil_exponent(x), eprod = ep + exponent(ic2) - 1022;
         es = (er > eprod ? er : eprod) + 1;
@@ -392,7 +399,7 @@ GBR_HD void face_states(const double* const (&u)[4], int su, double rc, double i
         o.s[1] = to_double(wr, es);
     }
     {  // fields 1 and 4 (u -/+ c), carried as p -/+ rho c un
-        double x[12];
+        Stencil x;
         load(1, x);
         const int eu = stencil_exponent(x), eprod = eu + exponent(rc) - 1022;
         ew = (ep > eprod ? ep : eprod) + 1;
@@ -411,7 +418,7 @@ GBR_HD void face_states(const double* const (&u)[4], int su, double rc, double i
         o.dif[1] = to_double(wr - mr, ew);
     }
     {  // field 3 (shear): ut
-        double x[12];
+        Stencil x;
         load(2, x);
         et = stencil_exponent(x);
         Functionals R;
@@ -421,6 +428,52 @@ GBR_HD void face_states(const double* const (&u)[4], int su, double rc, double i
         o.ut[1] = to_double(wr, et);
     }
     o.ok = ew <= kExpMax && es <= kExpMax && et <= kExpMax;
+}
+
+// 1/2 (F(f_L) + F(f_R)) at the face after cell j of one flux component, the
+// symmetric 10-point stencil of Eq. flux-full and its mirror over split values
+// at cells j-4 .. j+5 (weights / 1680; order 4: Eq. fourth, / 2880), exact up to
+// the alignment of the values (2^-58 of the largest) and the final rounding.
+template <int ORDER>
+GBR_HD double recon_mean(const i64 (&m)[10], const int (&ex)[10])
+{
+    int e = kExpMin;
+#pragma unroll
+    for (int k = 0; k < 10; ++k) e = ex[k] > e ? ex[k] : e;
+    i64 q[10];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) q[k] = aligned(m[k], ex[k], e);
+    Acc a;
+    a.add(q[4] + q[5], ORDER == 4 ? 1821 : 1052);
+    a.add(-q[3] - q[6], ORDER == 4 ? 461 : 250);
+    a.add(q[2] + q[7], ORDER == 4 ? 85 : 38);
+    if (ORDER == 4) {
+        a.add(-q[1] - q[8], 4);
+        a.add(-q[0] - q[9], 1);
+    } else {
+        a.add(q[1] + q[8] - q[0] - q[9], 1);
+    }
+    const i64 n = a.shift<ORDER == 4 ? 12 : 11>();  // 2^12 / 2880 = 1 + 1216/2880, 2^11 / 1680 = 1 + 368/1680
+    const double f = to_double(n + mulhi(n, ORDER == 4 ? ratio(1216, 2880) : ratio(368, 1680)), e);
+    return e <= kExpMax ? f : of_bits(0x7ff8000000000000ull);
+}
+
+// 60 Phi' of Eq. six at a cell from the split values of cells j-3 .. j+3 (the
+// centre is not used): 45 A1 - 9 A2 + A3 in units of 2^8.
+GBR_HD double grad60(const i64 (&m)[7], const int (&ex)[7])
+{
+    int e = kExpMin;
+#pragma unroll
+    for (int k = 0; k < 7; ++k) e = k != 3 && ex[k] > e ? ex[k] : e;
+    i64 q[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) q[k] = aligned(m[k], ex[k], e);
+    Acc a;
+    a.add(q[4] - q[2], 45);
+    a.add(q[1] - q[5], 9);
+    a.add(q[6] - q[0], 1);
+    const double g = to_double(a.shift<8>(), e + 8);
+    return e <= kExpMax ? g : of_bits(0x7ff8000000000000ull);
 }
 
 }  // namespace fx

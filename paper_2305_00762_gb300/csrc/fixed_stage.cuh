@@ -1,0 +1,337 @@
+// The FP64 MEG7-prim tile: the phases of stage_tile (stage_kernel.cuh) with
+// everything linear on the integer pipe. Primitives and cell fluxes are kept
+// in shared memory taken apart (fx::split: 64-bit integer and exponent), so a
+// face's stencils are aligned to their own scale by a shift each; face states
+// (fixed_face.cuh), flux reconstruction and the viscous gradients are integer
+// sums. FP64 arithmetic remains for the primitives, the cell fluxes, the
+// Riemann solver, the viscous flux and the stage update.
+#pragma once
+
+#include "stage_kernel.cuh"
+
+namespace gbr {
+
+template <int BX, int BY, bool VISC>
+struct FixedLayout {
+    using G = TileLayout<BX, BY, VISC>;  // index ranges
+    typedef long long i64;
+    static constexpr int NU = G::NU, NFX = G::NFX, NFY = G::NFY;
+    static constexpr size_t up(size_t b) { return (b + 127) / 128 * 128; }
+    static constexpr size_t oM = 0;                                          // primitives: integers [4][NU]
+    static constexpr size_t oFX = oM + sizeof(i64) * 4 * NU;                 // x fluxes [4][NFX]
+    static constexpr size_t oFY = oFX + sizeof(i64) * 4 * NFX;               // y fluxes [4][NFY]
+    // The FP64 tile + halo lands here; viscous gradients and face fluxes, all
+    // written after phase 0, take its place.
+    static constexpr size_t oRaw = up(oFY + sizeof(i64) * 4 * NFY);
+    static constexpr size_t oGX = oRaw, oGY = oGX + (VISC ? sizeof(double) * 4 * G::NGX : 0);
+    static constexpr size_t oHX = oGY + (VISC ? sizeof(double) * 4 * G::NGY : 0);
+    static constexpr size_t oHY = oHX + sizeof(double) * 4 * G::NHX;
+    static constexpr size_t oH1 = oHY + sizeof(double) * 4 * G::NHY, oR1 = oRaw + sizeof(double) * 4 * NU;
+    static constexpr size_t oR = oH1 > oR1 ? oH1 : oR1;                      // densities in FP32 [NU]
+    static constexpr size_t oE = oR + sizeof(float) * NU;                    // exponents of the integers above
+    static constexpr size_t oEX = oE + sizeof(short) * 4 * NU;
+    static constexpr size_t oEY = oEX + sizeof(short) * 4 * NFX;
+    static constexpr size_t oPX = oEY + sizeof(short) * 4 * NFY;             // detector flags
+    static constexpr size_t oPY = oPX + G::NPX;
+    static constexpr size_t bytes = (oPY + G::NPY + 15) / 16 * 16;
+};
+
+// Eq. detector's test (trouble_cell) at FP32 cost: the comparison is taken on
+// the densities rounded to FP32 wherever the rounding cannot change its sign
+// (all but a few cells in a thousand), else on the FP64 values as trouble_cell
+// takes it (`exact`). With |r| <= R each density is off by at most 2^-24 R, a
+// and b (sums of two differences, three roundings) by at most d = 24 2^-24 R,
+// and t = (a^2 + b^2 + eps) - 2 (2ab + eps) by at most 8 d (a + b) + 6 d^2 plus
+// the roundings of t itself, below 2^-21 of its terms.
+template <typename F>
+__device__ __forceinline__ bool trouble_filtered(const float* r, int st, F exact)
+{
+    const float eps = float(0.9 * 0.5 / (1.0 - 0.9 * 0.5) * 1e-6);
+    const float c = r[0], m1 = r[-st], m2 = r[-2 * st], p1 = r[st], p2 = r[2 * st];
+    const float a = fabsf(c - m1) + fabsf(fmaf(-2.f, m1, c) + m2);
+    const float b = fabsf(c - p1) + fabsf(fmaf(-2.f, p1, c) + p2);
+    const float R = fmaxf(fmaxf(fmaxf(fabsf(c), fabsf(m1)), fmaxf(fabsf(m2), fabsf(p1))), fabsf(p2));
+    const float d = 24.f / 16777216.f * R, ab = a * b, sq = fmaf(a, a, b * b);
+    const float t = (sq + eps) - 2.f * fmaf(2.f, ab, eps);
+    const float off = fmaf(8.f * d, a + b, 6.f * d * d) + (sq + 4.f * ab + 3.f * eps) * (1.f / 2097152.f);
+    if (t > off) return true;
+    if (t < -off) return false;
+    return exact();  // (also where a density overflows FP32)
+}
+
+template <int BX, int BY, int NT, bool VISC, int ORDER, bool TMA>
+__device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, const int ty0, unsigned char* smem,
+                                           const CUtensorMap* tmap = nullptr)
+{
+    typedef long long i64;
+    typedef unsigned short u16;
+    using F = FixedLayout<BX, BY, VISC>;
+    using L = typename F::G;
+    using X = typename L::template Cross<0>;  // the staged cells
+    constexpr int RW = L::RW, NU = L::NU, V = L::V;
+    i64* const sM = reinterpret_cast<i64*>(smem + F::oM);
+    i64* const sFX = reinterpret_cast<i64*>(smem + F::oFX);
+    i64* const sFY = reinterpret_cast<i64*>(smem + F::oFY);
+    double* const sGX = reinterpret_cast<double*>(smem + F::oGX);
+    double* const sGY = reinterpret_cast<double*>(smem + F::oGY);
+    double* const sHX = reinterpret_cast<double*>(smem + F::oHX);
+    double* const sHY = reinterpret_cast<double*>(smem + F::oHY);
+    float* const sR = reinterpret_cast<float*>(smem + F::oR);
+    u16* const sE = reinterpret_cast<u16*>(smem + F::oE);
+    u16* const sEX = reinterpret_cast<u16*>(smem + F::oEX);
+    u16* const sEY = reinterpret_cast<u16*>(smem + F::oEY);
+    unsigned char* const sPX = smem + F::oPX;
+    unsigned char* const sPY = smem + F::oPY;
+    const int nx = P.g.nx, ny = P.g.ny, tid = threadIdx.x;
+
+    PhysT<double> ph;
+    ph.gamma = P.ph.gamma;
+    ph.gm1 = P.ph.gm1;
+    ph.igm1 = P.ph.igm1;
+    ph.mu = P.ph.mu;
+    ph.kq = P.ph.kq;
+    ph.lm = P.ph.riemann;
+    const double inv_dx = P.ph.inv_dx, inv_dy = P.ph.inv_dy;
+
+    // Phase 0: primitives (Eq. pressure) and cell fluxes F^c = (rho u, rho u u
+    // + p, rho u v, u (E + p)), G^c (Sec. 1; rho u, rho v, E from the state).
+    const bool staged = stage_region<BX, BY, NT, X, TMA>(
+        P, tx0, ty0, reinterpret_cast<double*>(smem + F::oRaw), tmap,
+        [&](int idx, double q0, double q1, double q2, double q3) {
+            double w[4];
+            prims_of(q0, q1, q2, q3, ph.gm1, w[0], w[1], w[2], w[3]);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) fx::split(w[m], sM[m * NU + idx], sE[m * NU + idx]);
+            sR[idx] = f64_to_f32_rn(w[0]);
+            const int ry = idx / RW, rx = idx - ry * RW;
+            if (ry >= 6 && ry < 6 + BY && rx >= 1 && rx < BX + 11) {
+                const int f = (ry - 6) * L::FXW + (rx - 1);
+                const double h[4] = {q1, rfma(q1, w[1], w[3]), rmul(q1, w[2]), rmul(w[1], q3 + w[3])};
+#pragma unroll
+                for (int m = 0; m < 4; ++m) fx::split(h[m], sFX[m * L::NFX + f], sEX[m * L::NFX + f]);
+            }
+            if (ry >= 1 && ry < BY + 11 && rx >= 6 && rx < BX + 6) {
+                const int f = (ry - 1) * BX + (rx - 6);
+                const double h[4] = {q2, rmul(q2, w[1]), rfma(q2, w[2], w[3]), rmul(w[2], q3 + w[3])};
+#pragma unroll
+                for (int m = 0; m < 4; ++m) fx::split(h[m], sFY[m * L::NFY + f], sEY[m * L::NFY + f]);
+            }
+        });
+    if (!staged) return;
+    __syncthreads();
+
+    // Phase 1: detector flags, and the gradients the viscous flux takes.
+    auto flag = [&](int c, int st) {
+        return trouble_filtered(sR + c, st, [&] {
+            double r[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) r[k] = fx::unsplit(sM[c + (k - 2) * st], sE[c + (k - 2) * st]);
+            return trouble_cell(r + 2, 1);
+        }) ? 1 : 0;
+    };
+    for (int idx = tid; idx < L::NPX; idx += NT) {
+        const int a = idx / L::PXW, b = idx - a * L::PXW;
+        sPX[idx] = flag((a + 6) * RW + (b + 3), 1);
+    }
+    for (int idx = tid; idx < L::NPY; idx += NT) {
+        const int a = idx / BX, b = idx - a * BX;
+        sPY[idx] = flag((a + 3) * RW + (b + 6), RW);
+    }
+    if constexpr (VISC) {
+        auto gradient = [&](int m, int c, int st) {
+            i64 q[7];
+            int e[7];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                q[k] = sM[m * NU + c + (k - 3) * st];
+                e[k] = sE[m * NU + c + (k - 3) * st];
+            }
+            return fx::grad60(q, e);
+        };
+        for (int idx = tid; idx < L::NGX; idx += NT) {
+            const int a = idx / L::GXW, b = idx - a * L::GXW;
+            for (int m = 0; m < 4; ++m) sGX[m * L::NGX + idx] = gradient(m, (a + 6 - V) * RW + (b + 3), 1);
+        }
+        for (int idx = tid; idx < L::NGY; idx += NT) {
+            const int a = idx / L::GYW, b = idx - a * L::GYW;
+            for (int m = 0; m < 4; ++m) sGY[m * L::NGY + idx] = gradient(m, (a + 3) * RW + (b + 6 - V), RW);
+        }
+    }
+    __syncthreads();
+
+    // Phase 2: every x face and y face of the tile, once (one thread per face).
+    for (int w = tid; w < L::NF; w += NT) {
+        const bool xf = w < L::NHX;
+        const int w2 = xf ? w : w - L::NHX;
+        const int fw = xf ? L::HXW : BX;
+        const int fr = w2 / fw, fc = w2 - fr * fw;                // x faces: row, face; y faces: face, column
+        const int c = (fr + (xf ? 6 : 5)) * RW + fc + (xf ? 5 : 6);  // the cell before the face
+        const int su = xf ? 1 : RW;
+        const int pn = xf ? 1 : 2;  // plane of the normal velocity
+        // Eq. buffer: sigma = 0 if psi_k < psi_c for any k in j-2..j+3.
+        const unsigned char* tr = xf ? sPX + fr * L::PXW + fc + 2 : sPY + (fr + 2) * BX + fc;
+        const int st = xf ? 1 : BX;
+        bool trouble = false;
+#pragma unroll
+        for (int k = -2; k <= 3; ++k) trouble |= tr[k * st] != 0;
+
+        // Primitives (rho, un, ut, p) of the face's two cells
+        double u0[4], u1[4];
+        auto cell = [&](int m, int o) {
+            const int at = (m == 1 ? pn : m == 2 ? 3 - pn : m) * NU + c + o;
+            return fx::unsplit(sM[at], sE[at]);
+        };
+        u0[0] = cell(0, 0);
+        u1[0] = cell(0, su);
+        u0[3] = cell(3, 0);
+        u1[3] = cell(3, su);
+        // Characteristic projection at the arithmetic-mean state, every
+        // factor from one reciprocal square root y = 1/sqrt(gamma p rho).
+        const double rb = 0.5 * (u0[0] + u1[0]), gp = ph.gamma * (0.5 * (u0[3] + u1[3]));
+        const double y = fx::rsqrt(gp * rb);
+        const double icb = rb * y, cb = gp * y;  // 1 / c, c
+        const double ic2 = icb * icb;
+        fx::FaceStates s;
+        fx::face_states<ORDER>(
+            [&](int m, fx::Stencil& x) {
+                const int at = (m == 1 ? pn : m == 2 ? 3 - pn : m) * NU + c;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {
+                    x.m[k] = sM[at + (k - 5) * su];
+                    x.e[k] = sE[at + (k - 5) * su];
+                }
+            },
+            rb * cb, ic2, s);
+        // Back to primitives: the acoustic fields are p -/+ rho c un, so with
+        // a = w1 + w4, rho = a / (2 c^2) + w2, p = a / 2, un = (w4 - w1) / (2 rho c).
+        const double hrc = 0.5 * y, be = 0.5 * ic2;
+        double rL = rfma(be, s.a03[0], s.s[0]), unL = hrc * s.dif[0], utL = s.ut[0], pL = 0.5 * s.a03[0];
+        double rR = rfma(be, s.a03[1], s.s[1]), unR = hrc * s.dif[1], utR = s.ut[1], pR = 0.5 * s.a03[1];
+        // positivity fallback: a face state with rho <= 0 or p <= 0 (or from a
+        // refused stencil) takes the adjacent cell's state
+        if (!(s.ok && tpositive(rL) && tpositive(pL))) {
+            rL = u0[0];
+            unL = cell(1, 0);
+            utL = cell(2, 0);
+            pL = u0[3];
+        }
+        if (!(s.ok && tpositive(rR) && tpositive(pR))) {
+            rR = u1[0];
+            unR = cell(1, su);
+            utR = cell(2, su);
+            pR = u1[3];
+        }
+        // E = p / (gamma - 1) + (rho un un + rho ut ut) / 2, from the momenta
+        double QL[4], QR[4];
+        QL[0] = rL;
+        QL[1] = rL * unL;
+        QL[2] = rL * utL;
+        QL[3] = rfma(0.5, rfma(QL[1], unL, rmul(QL[2], utL)), rmul(pL, ph.igm1));
+        QR[0] = rR;
+        QR[1] = rR * unR;
+        QR[2] = rR * utR;
+        QR[3] = rfma(0.5, rfma(QR[1], unR, rmul(QR[2], utR)), rmul(pR, ph.igm1));
+
+        // Central part 1/2 (F_L + F_R) of the hybrid face fluxes (Sec. 2.4).
+        double Fc[4];
+        if (!trouble) {
+            const int at = xf ? fr * L::FXW + fc + 4 : (fr + 4) * BX + fc, sf = xf ? 1 : BX;
+            const int nf = xf ? L::NFX : L::NFY;
+            const i64* fm = (xf ? sFX : sFY) + at;
+            const u16* fe = (xf ? sEX : sEY) + at;
+#pragma unroll 1
+            for (int m = 0; m < 4; ++m) {
+                const int pl = (m == 1 ? pn : m == 2 ? 3 - pn : m) * nf;
+                i64 q[10];
+                int e[10];
+#pragma unroll
+                for (int k = 0; k < 10; ++k) {
+                    q[k] = fm[pl + (k - 4) * sf];
+                    e[k] = fe[pl + (k - 4) * sf];
+                }
+                const double f = fx::recon_mean<ORDER>(q, e);
+                if (m == 0) Fc[0] = f;
+                if (m == 1) Fc[1] = f;
+                if (m == 2) Fc[2] = f;
+                if (m == 3) Fc[3] = f;
+            }
+        } else {
+            Fc[0] = 0.5 * (QL[1] + QR[1]);
+            Fc[1] = 0.5 * ((QL[1] * unL + pL) + (QR[1] * unR + pR));
+            Fc[2] = 0.5 * (QL[1] * utL + QR[1] * utR);
+            Fc[3] = 0.5 * (unL * (QL[3] + pL) + unR * (QR[3] + pR));
+        }
+        double out[4];
+        hllc_flux(ph, Fc, QL, QR, rL, unL, utL, pL, QL[3], rR, unR, utR, pR, QR[3], out);
+        if constexpr (VISC) {
+            u0[1] = cell(1, 0);
+            u1[1] = cell(1, su);
+            u0[2] = cell(2, 0);
+            u1[2] = cell(2, su);
+            FaceIn<double> in;
+            // gradients along the face normal at the cell before the face, and
+            // the tangential derivatives of un and ut
+            const double* gn = xf ? sGX + (fr + V) * L::GXW + fc + 2 : sGY + (fr + 2) * L::GYW + fc + V;
+            const double* gt = xf ? sGY + (fr + 3) * L::GYW + fc + V - 1 : sGX + (fr - 1 + V) * L::GXW + fc + 3;
+            const int nn = xf ? L::NGX : L::NGY, nt = xf ? L::NGY : L::NGX;
+            in.g[0] = gn;
+            in.g[1] = gn + pn * nn;
+            in.g[2] = gn + (3 - pn) * nn;
+            in.g[3] = gn + 3 * nn;
+            in.sg = xf ? 1 : L::GYW;
+            in.tun = gt + pn * nt;
+            in.tut = gt + (3 - pn) * nt;
+            in.stq = xf ? 1 : L::GXW;
+            viscous_flux<double, false>(in, u0, u1, ph, xf ? inv_dx : inv_dy, xf ? inv_dy : inv_dx, out);
+        }
+        if (xf) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) sHX[m * L::NHX + w] = out[m];
+            if (P.sigx) {
+                const int i = ty0 + fr, jf = tx0 + fc;
+                if (i < ny && jf <= nx) P.sigx[(long long)i * (nx + 1) + jf] = trouble ? 0 : 1;
+            }
+        } else {
+            sHY[w2] = out[0];
+            sHY[L::NHY + w2] = out[2];
+            sHY[2 * L::NHY + w2] = out[1];
+            sHY[3 * L::NHY + w2] = out[3];
+            if (P.sigy) {
+                const int j = tx0 + fc, iface = ty0 + fr;
+                if (j < nx && iface <= ny) P.sigy[(long long)iface * nx + j] = trouble ? 0 : 1;
+            }
+        }
+    }
+    __syncthreads();
+    finish_tile<double, BX, BY, NT>(P, ph, inv_dx, inv_dy, tx0, ty0, sHX, sHY);
+}
+
+// One CTA per tile, two CTAs per SM.
+template <int BX, int BY, int NT, bool VISC, int ORDER>
+__global__ void __launch_bounds__(NT, 2) fixed_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    fixed_tile<BX, BY, NT, VISC, ORDER, true>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
+}
+
+template <int BX, int BY, int NT, bool VISC, int ORDER>
+cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
+{
+    using F = FixedLayout<BX, BY, VISC>;
+    static PerDevice<int> configured;  // the shared-memory limit is raised once per device
+    auto kern = fixed_kernel<BX, BY, NT, VISC, ORDER>;
+    int ok = 0;
+    cudaError_t e = configured.get(&ok, [&](int* v) {
+        *v = 1;
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::bytes);
+    });
+    if (e != cudaSuccess) return e;
+    CUtensorMap map;
+    e = encode_state_map(p.g, p.q, F::G::RW, F::G::RH, &map);
+    if (e != cudaSuccess) return e;
+    dim3 grid((p.g.nx + BX - 1) / BX, (p.g.ny + BY - 1) / BY);
+    kern<<<grid, NT, F::bytes, s>>>(p, map);
+    return cudaGetLastError();
+}
+
+}  // namespace gbr

@@ -74,20 +74,14 @@ struct TileLayout {
     // conservative values; their arrays then come before the gradients, so
     // that the TMA landing area (at the gradients, over the face fluxes) does
     // not overlap them.
-    // GRAD: gradient arrays are kept. FP64 MEG7-prim forms its face states
-    // from the primitives themselves (fixed_face.cuh) and needs gradients for
-    // the viscous flux only.
-    static constexpr bool GRAD = !FLUX0 || CONS || VISC;
     static constexpr int oU = 0;
     static constexpr int oGX = FLUX0 ? oU + 4 * NU + 4 * (NFX + NFY) : oU + 4 * NU;
-    static constexpr int oGY = oGX + (GRAD ? 4 * NGX : 0);
+    static constexpr int oGY = oGX + 4 * NGX;
     static constexpr int oFX = FLUX0 ? oU + 4 * NU : oGY + 4 * NGY;
     static constexpr int oFY = oFX + 4 * NFX;
-    static constexpr int oHX = FLUX0 ? oGY + (GRAD ? 4 * NGY : 0) : oFY + 4 * NFY;
+    static constexpr int oHX = FLUX0 ? oGY + 4 * NGY : oFY + 4 * NFY;
     static constexpr int oHY = oHX + 4 * NHX;
-    static constexpr int oH1 = oHY + 4 * NHY;
-    // (without gradients the staging's landing area outgrows the face fluxes)
-    static constexpr int oQc = !GRAD && oH1 < oGX + 4 * NU ? oGX + 4 * NU : oH1;  // conservative values (MEG7-cons)
+    static constexpr int oQc = oHY + 4 * NHY;         // conservative values (MEG7-cons)
     static constexpr int oEnd = oQc + (CONS ? 4 * NU : 0);
 
     // learned sensor: per-cell decisions on the bounding box of both
@@ -570,6 +564,130 @@ struct PhysT {
     int lm;                      // 1: shock-stable HLLC-LM dissipation
 };
 
+// HLLC in the form 1/2 (F_L + F_R) - 1/2 |A| (Q_R - Q_L), Eq. Riemann_revisit,
+// with Toro's star states; k (E/rho + (S*-u)(S* + p/(rho (S-u)))) is
+// expanded so that the only divisions are 1/((S_L - S*)(S_R - S*)), S* and
+// the Roe weight.
+template <typename T>
+__device__ __forceinline__ void hllc_flux(const PhysT<T>& P, const T (&Fc)[4], const T (&QL)[4], const T (&QR)[4], T rL,
+                                          T unL, T utL, T pL, T EL, T rR, T unR, T utR, T pR, T ER, T (&out)[4])
+{
+    // Per side one reciprocal square root y = 1/sqrt(gamma p rho):
+    // c = gamma p y, 1/c = rho y, 1/rho = c y.
+    const T gpL = P.gamma * pL, gpR = P.gamma * pR;
+    const T yL = trsqrt(gpL * rL), yR = trsqrt(gpR * rR);
+    const T cL = gpL * yL, cR = gpR * yR;
+    const T icL = rL * yL, icR = rR * yR;
+    const T irL = cL * yL, irR = cR * yR;
+    const T eL = EL * irL, eR = ER * irR;  // E / rho
+    const T HL = rfma(pL, irL, eL), HR = rfma(pR, irR, eR);
+    // Roe averages (a_L + q a_R) / (1 + q), q = sqrt(rho_R / rho_L)
+    const T xq = rR * irL;
+    const T q = xq * trsqrt(xq);
+    const T oL = trcp(T(1) + q);
+    const T ut = oL * rfma(q, unR, unL);
+    const T vt = oL * rfma(q, utR, utL);
+    const T Ht = oL * rfma(q, HR, HL);
+    const T c2t = P.gm1 * (Ht - T(0.5) * (ut * ut + vt * vt));
+    const T ct = c2t * trsqrt(c2t);
+    const T SL = tmin(unL - cL, ut - ct);
+    const T SR = tmax(unR + cR, ut + ct);
+    const T mL = rL * (SL - unL), mR = rR * (SR - unR);
+    // S* = num / den and 1/(S_L - S*), 1/(S_R - S*) from one division:
+    // with nL = S_L den - num, nR = S_R den - num and z = 1/(den nL nR),
+    // S* = num nL nR z, 1/(S_L - S*) = den^2 nR z, 1/(S_R - S*) = den^2 nL z
+    const T num = pR - pL + mL * unL - mR * unR, den = mL - mR;
+    const T nL = SL * den - num, nR = SR * den - num;
+    const T nLR = nL * nR;
+    const T z = trcp(den * nLR);
+    const T Ss = num * nLR * z;
+    const T d2z = den * den * z;
+    const T iL = nR * d2z, iR = nL * d2z;  // 1/(S_L - S*), 1/(S_R - S*)
+    T aL = tabs(SL), aR = tabs(SR);
+    const T aS = tabs(Ss);
+    if (P.lm) {
+        // Shock-stable HLLC-LM (Fleischmann, Adami and Adams 2020, used by
+        // Examples 7 and 8): the acoustic dissipation scaled by
+        // phi = sin(pi/2 min(1, Ma / 0.1)), Ma the larger face-normal Mach
+        // number of the two face states; phi = 1 leaves HLLC unchanged.
+        const T z = tmax(tabs(unL) * icL, tabs(unR) * icR) * T(10);
+        if (z < T(1)) {
+            const T phi = tsinpi(T(0.5) * z);
+            aL *= phi;
+            aR *= phi;
+        }
+    }
+    // 1/2 |A| dQ = 1/2 (aL (QsL - QL) + aS (QsR - QsL) + aR (QR - QsR)),
+    // regrouped by state: hL QsL + hS QsR - hQL QL + hQR QR. The star
+    // states are Q*_K = k_K (1, S*, ut_K, E_K / rho_K + (S* - un_K) S*)
+    // + (0, 0, 0, (S* - un_K) p_K / (S_K - S*)), k_K = m_K / (S_K - S*):
+    // the factors h / (S_K - S*) and h k are formed once and the star
+    // states never built.
+    const T hL = T(0.5) * (aL - aS), hS = T(0.5) * (aS - aR), hQL = T(0.5) * aL, hQR = T(0.5) * aR;
+    const T giL = hL * iL, giR = hS * iR;
+    const T fL = giL * mL, fR = giR * mR;
+    const T tL = Ss - unL, tR = Ss - unR;
+    out[0] = Fc[0] - fL - fR + hQL * QL[0] - hQR * QR[0];
+    out[1] = Fc[1] - (fL + fR) * Ss + hQL * QL[1] - hQR * QR[1];
+    out[2] = Fc[2] - fL * utL - fR * utR + hQL * QL[2] - hQR * QR[2];
+    out[3] = Fc[3] - fL * (eL + tL * Ss) - giL * (tL * pL) - fR * (eR + tR * Ss) - giR * (tR * pR) +
+             hQL * QL[3] - hQR * QR[3];
+}
+
+// The viscous part of the face flux, subtracted from out: u0, u1 the primitives
+// (rho, un, ut, p) of the face's two cells, gradients through `in`.
+template <typename T, bool CONS>
+__device__ __forceinline__ void viscous_flux(const FaceIn<T>& in, const T (&u0)[4], const T (&u1)[4], const PhysT<T>& P,
+                                             T inv_dn, T inv_dt, T (&out)[4])
+{
+    // Sec. 2.1: alpha-damping (Eq. alphad, alpha_v = 4) on the shared
+    // gradients; T = gamma p / rho with T' by the chain rule.
+    const T r0 = u0[0], r1 = u1[0];
+    const T n0 = u0[1], n1 = u1[1];
+    const T t0 = u0[2], t1 = u1[2];
+    const T p0 = u0[3], p1 = u1[3];
+    T dr0 = in.g[0][0], dr1 = in.g[0][in.sg];
+    T dn0 = in.g[1][0], dn1 = in.g[1][in.sg];
+    T dt0 = in.g[2][0], dt1 = in.g[2][in.sg];
+    T dp0 = in.g[3][0], dp1 = in.g[3][in.sg];
+    const T ir0 = trcp(r0), ir1 = trcp(r1);
+    if constexpr (CONS) {  // primitive gradients from the conservative ones (chain rule)
+        const T k0 = T(0.5) * (n0 * n0 + t0 * t0), k1 = T(0.5) * (n1 * n1 + t1 * t1);
+        const T e0 = dp0, e1 = dp1;  // dE
+        dp0 = P.gm1 * (e0 - n0 * dn0 - t0 * dt0 + k0 * dr0);
+        dp1 = P.gm1 * (e1 - n1 * dn1 - t1 * dt1 + k1 * dr1);
+        dn0 = (dn0 - n0 * dr0) * ir0;
+        dn1 = (dn1 - n1 * dr1) * ir1;
+        dt0 = (dt0 - t0 * dr0) * ir0;
+        dt1 = (dt1 - t1 * dr1) * ir1;
+    }
+    const T T0 = P.gamma * p0 * ir0, T1 = P.gamma * p1 * ir1;
+    const T dT0 = P.gamma * (dp0 * ir0 - p0 * dr0 * ir0 * ir0);
+    const T dT1 = P.gamma * (dp1 * ir1 - p1 * dr1 * ir1 * ir1);
+    // (the gradients, and so T', at their carried scale kGrad)
+    const T hg = T(0.5 / kGrad);
+    const T un_n = (hg * (dn0 + dn1) + T(2) * (n1 - hg * dn1 - n0 - hg * dn0)) * inv_dn;
+    const T ut_n = (hg * (dt0 + dt1) + T(2) * (t1 - hg * dt1 - t0 - hg * dt0)) * inv_dn;
+    const T T_n = (hg * (dT0 + dT1) + T(2) * (T1 - hg * dT1 - T0 - hg * dT0)) * inv_dn;
+    T gn0 = in.tun[0], gn1 = in.tun[in.stq], gt0 = in.tut[0], gt1 = in.tut[in.stq];
+    if constexpr (CONS) {  // tangential derivatives of un, ut from those of rho un, rho ut, rho
+        const T ra0 = in.tr0[0], ra1 = in.tr0[in.stq];
+        gn0 = (gn0 - n0 * ra0) * ir0;
+        gn1 = (gn1 - n1 * ra1) * ir1;
+        gt0 = (gt0 - t0 * ra0) * ir0;
+        gt1 = (gt1 - t1 * ra1) * ir1;
+    }
+    const T un_t = hg * (gn0 + gn1) * inv_dt;
+    const T ut_t = hg * (gt0 + gt1) * inv_dt;
+    const T unf = T(0.5) * (n0 + n1), utf = T(0.5) * (t0 + t1);
+    const T tau_nn = T(2.0 / 3.0) * P.mu * (T(2) * un_n - ut_t);
+    const T tau_nt = P.mu * (un_t + ut_n);
+    const T q_n = -P.kq * T_n;
+    out[1] -= tau_nn;
+    out[2] -= tau_nt;
+    out[3] += -(tau_nn * unf + tau_nt * utf) + q_n;
+}
+
 // The whole interface procedure of Secs. 2.1-2.4 at face j+1/2. Returns the
 // total flux in face-normal order and the detector flag sigma.
 // Projection of a conservative vector q = (rho, rho un, rho ut, E) onto the
@@ -590,7 +708,7 @@ __device__ __forceinline__ void cons_project(T q0, T q1, T q2, T q3, T ub, T vb,
 }
 
 template <typename T, bool VISC, int ORDER, bool CONS = false>
-__device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P, T inv_dn, T inv_dt, T out[4],
+__device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P, T inv_dn, T inv_dt, T (&out)[4],
                                           bool& smooth)
 {
     const GrbCoef<T> coef = grb_coef<T>(ORDER);  // compile-time constants
@@ -614,21 +732,8 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
     const T ic2 = icb * icb;         // 1 / c^2
     const T be = T(0.5) * ic2;       // 1 / (2 c^2)
 
-    // FP64 MEG7-prim: the characteristic face states on the integer pipe
-    constexpr bool FIXED = sizeof(T) == 8 && !CONS;
     T wL[4], wR[4];
-    if constexpr (FIXED) {
-        fx::FaceStates st;
-        fx::face_states<ORDER>(in.u, su, rb * cb, ic2, st);
-        wL[0] = st.a03[0];
-        wR[0] = st.a03[1];
-        wL[3] = st.dif[0];
-        wR[3] = st.dif[1];
-        wL[1] = st.ok ? st.s[0] : T(-1);  // (a refused stencil takes the positivity fallback below)
-        wR[1] = st.ok ? st.s[1] : T(-1);
-        wL[2] = st.ut[0];
-        wR[2] = st.ut[1];
-    } else if constexpr (!CONS) {
+    if constexpr (!CONS) {
         {  // fields 1 and 4 (u - c and u + c) share un and p. They are
            // carried scaled by 2 c^2, as p -/+ rho c un: GRB, the limiter's
            // bounds and its clamp are linear and scale-free, and the MP
@@ -695,13 +800,13 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         // a = w1 + w4, rho = a / (2 c^2) + w2, p = a / 2 and
         // un = (w4 - w1) / (2 rho c)
         const T hrc = T(0.5) * y;  // 1 / (2 rho c): rho c = gamma p rho y = 1 / y
-        const T aL03 = FIXED ? wL[0] : wL[0] + wL[3], aR03 = FIXED ? wR[0] : wR[0] + wR[3];
+        const T aL03 = wL[0] + wL[3], aR03 = wR[0] + wR[3];
         rL = rfma(be, aL03, wL[1]);
-        unL = hrc * (FIXED ? wL[3] : wL[3] - wL[0]);
+        unL = hrc * (wL[3] - wL[0]);
         utL = wL[2];
         pL = T(0.5) * aL03;
         rR = rfma(be, aR03, wR[1]);
-        unR = hrc * (FIXED ? wR[3] : wR[3] - wR[0]);
+        unR = hrc * (wR[3] - wR[0]);
         utR = wR[2];
         pR = T(0.5) * aR03;
         // positivity fallback: a face state with rho <= 0 or p <= 0 takes the
@@ -798,120 +903,15 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
         Fc[3] = T(0.5) * (unL * (EL + pL) + unR * (ER + pR));
     }
 
-    // HLLC in the form 1/2 (F_L + F_R) - 1/2 |A| (Q_R - Q_L), Eq. Riemann_revisit,
-    // with Toro's star states; k (E/rho + (S*-u)(S* + p/(rho (S-u)))) is
-    // expanded so that the only divisions are 1/((S_L - S*)(S_R - S*)), S* and
-    // the Roe weight.
-    {
-        // Per side one reciprocal square root y = 1/sqrt(gamma p rho):
-        // c = gamma p y, 1/c = rho y, 1/rho = c y.
-        const T gpL = P.gamma * pL, gpR = P.gamma * pR;
-        const T yL = trsqrt(gpL * rL), yR = trsqrt(gpR * rR);
-        const T cL = gpL * yL, cR = gpR * yR;
-        const T icL = rL * yL, icR = rR * yR;
-        const T irL = cL * yL, irR = cR * yR;
-        const T eL = EL * irL, eR = ER * irR;  // E / rho
-        const T HL = rfma(pL, irL, eL), HR = rfma(pR, irR, eR);
-        // Roe averages (a_L + q a_R) / (1 + q), q = sqrt(rho_R / rho_L)
-        const T xq = rR * irL;
-        const T q = xq * trsqrt(xq);
-        const T oL = trcp(T(1) + q);
-        const T ut = oL * rfma(q, unR, unL);
-        const T vt = oL * rfma(q, utR, utL);
-        const T Ht = oL * rfma(q, HR, HL);
-        const T c2t = P.gm1 * (Ht - T(0.5) * (ut * ut + vt * vt));
-        const T ct = c2t * trsqrt(c2t);
-        const T SL = tmin(unL - cL, ut - ct);
-        const T SR = tmax(unR + cR, ut + ct);
-        const T mL = rL * (SL - unL), mR = rR * (SR - unR);
-        // S* = num / den and 1/(S_L - S*), 1/(S_R - S*) from one division:
-        // with nL = S_L den - num, nR = S_R den - num and z = 1/(den nL nR),
-        // S* = num nL nR z, 1/(S_L - S*) = den^2 nR z, 1/(S_R - S*) = den^2 nL z
-        const T num = pR - pL + mL * unL - mR * unR, den = mL - mR;
-        const T nL = SL * den - num, nR = SR * den - num;
-        const T nLR = nL * nR;
-        const T z = trcp(den * nLR);
-        const T Ss = num * nLR * z;
-        const T d2z = den * den * z;
-        const T iL = nR * d2z, iR = nL * d2z;  // 1/(S_L - S*), 1/(S_R - S*)
-        T aL = tabs(SL), aR = tabs(SR);
-        const T aS = tabs(Ss);
-        if (P.lm) {
-            // Shock-stable HLLC-LM (Fleischmann, Adami and Adams 2020, used by
-            // Examples 7 and 8): the acoustic dissipation scaled by
-            // phi = sin(pi/2 min(1, Ma / 0.1)), Ma the larger face-normal Mach
-            // number of the two face states; phi = 1 leaves HLLC unchanged.
-            const T z = tmax(tabs(unL) * icL, tabs(unR) * icR) * T(10);
-            if (z < T(1)) {
-                const T phi = tsinpi(T(0.5) * z);
-                aL *= phi;
-                aR *= phi;
-            }
-        }
-        // 1/2 |A| dQ = 1/2 (aL (QsL - QL) + aS (QsR - QsL) + aR (QR - QsR)),
-        // regrouped by state: hL QsL + hS QsR - hQL QL + hQR QR. The star
-        // states are Q*_K = k_K (1, S*, ut_K, E_K / rho_K + (S* - un_K) S*)
-        // + (0, 0, 0, (S* - un_K) p_K / (S_K - S*)), k_K = m_K / (S_K - S*):
-        // the factors h / (S_K - S*) and h k are formed once and the star
-        // states never built.
-        const T hL = T(0.5) * (aL - aS), hS = T(0.5) * (aS - aR), hQL = T(0.5) * aL, hQR = T(0.5) * aR;
-        const T giL = hL * iL, giR = hS * iR;
-        const T fL = giL * mL, fR = giR * mR;
-        const T tL = Ss - unL, tR = Ss - unR;
-        out[0] = Fc[0] - fL - fR + hQL * QL[0] - hQR * QR[0];
-        out[1] = Fc[1] - (fL + fR) * Ss + hQL * QL[1] - hQR * QR[1];
-        out[2] = Fc[2] - fL * utL - fR * utR + hQL * QL[2] - hQR * QR[2];
-        out[3] = Fc[3] - fL * (eL + tL * Ss) - giL * (tL * pL) - fR * (eR + tR * Ss) - giR * (tR * pR) +
-                 hQL * QL[3] - hQR * QR[3];
-    }
-
+    hllc_flux(P, Fc, QL, QR, rL, unL, utL, pL, EL, rR, unR, utR, pR, ER, out);
     if constexpr (VISC) {
-        // Sec. 2.1: alpha-damping (Eq. alphad, alpha_v = 4) on the shared
-        // gradients; T = gamma p / rho with T' by the chain rule.
-        const T r0 = in.u[0][0], r1 = in.u[0][su];
-        const T n0 = in.u[1][0], n1 = in.u[1][su];
-        const T t0 = in.u[2][0], t1 = in.u[2][su];
-        const T p0 = in.u[3][0], p1 = in.u[3][su];
-        T dr0 = in.g[0][0], dr1 = in.g[0][sg];
-        T dn0 = in.g[1][0], dn1 = in.g[1][sg];
-        T dt0 = in.g[2][0], dt1 = in.g[2][sg];
-        T dp0 = in.g[3][0], dp1 = in.g[3][sg];
-        const T ir0 = trcp(r0), ir1 = trcp(r1);
-        if constexpr (CONS) {  // primitive gradients from the conservative ones (chain rule)
-            const T k0 = T(0.5) * (n0 * n0 + t0 * t0), k1 = T(0.5) * (n1 * n1 + t1 * t1);
-            const T e0 = dp0, e1 = dp1;  // dE
-            dp0 = P.gm1 * (e0 - n0 * dn0 - t0 * dt0 + k0 * dr0);
-            dp1 = P.gm1 * (e1 - n1 * dn1 - t1 * dt1 + k1 * dr1);
-            dn0 = (dn0 - n0 * dr0) * ir0;
-            dn1 = (dn1 - n1 * dr1) * ir1;
-            dt0 = (dt0 - t0 * dr0) * ir0;
-            dt1 = (dt1 - t1 * dr1) * ir1;
+        T u0[4], u1[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            u0[m] = in.u[m][0];
+            u1[m] = in.u[m][su];
         }
-        const T T0 = P.gamma * p0 * ir0, T1 = P.gamma * p1 * ir1;
-        const T dT0 = P.gamma * (dp0 * ir0 - p0 * dr0 * ir0 * ir0);
-        const T dT1 = P.gamma * (dp1 * ir1 - p1 * dr1 * ir1 * ir1);
-        // (the gradients, and so T', at their carried scale kGrad)
-        const T hg = T(0.5 / kGrad);
-        const T un_n = (hg * (dn0 + dn1) + T(2) * (n1 - hg * dn1 - n0 - hg * dn0)) * inv_dn;
-        const T ut_n = (hg * (dt0 + dt1) + T(2) * (t1 - hg * dt1 - t0 - hg * dt0)) * inv_dn;
-        const T T_n = (hg * (dT0 + dT1) + T(2) * (T1 - hg * dT1 - T0 - hg * dT0)) * inv_dn;
-        T gn0 = in.tun[0], gn1 = in.tun[in.stq], gt0 = in.tut[0], gt1 = in.tut[in.stq];
-        if constexpr (CONS) {  // tangential derivatives of un, ut from those of rho un, rho ut, rho
-            const T ra0 = in.tr0[0], ra1 = in.tr0[in.stq];
-            gn0 = (gn0 - n0 * ra0) * ir0;
-            gn1 = (gn1 - n1 * ra1) * ir1;
-            gt0 = (gt0 - t0 * ra0) * ir0;
-            gt1 = (gt1 - t1 * ra1) * ir1;
-        }
-        const T un_t = hg * (gn0 + gn1) * inv_dt;
-        const T ut_t = hg * (gt0 + gt1) * inv_dt;
-        const T unf = T(0.5) * (n0 + n1), utf = T(0.5) * (t0 + t1);
-        const T tau_nn = T(2.0 / 3.0) * P.mu * (T(2) * un_n - ut_t);
-        const T tau_nt = P.mu * (un_t + ut_n);
-        const T q_n = -P.kq * T_n;
-        out[1] -= tau_nn;
-        out[2] -= tau_nt;
-        out[3] += -(tau_nn * unf + tau_nt * utf) + q_n;
+        viscous_flux<T, CONS>(in, u0, u1, P, inv_dn, inv_dt, out);
     }
 }
 
@@ -1276,6 +1276,138 @@ __device__ bool fused_sensor_decisions(const StageParams& P, const float* sU, un
     return ok;
 }
 
+// Phase 0 of a tile: stage_cell(region cell, q0..q3) for every cell of X (the
+// region cells later phases read) of the tile whose first region cell is padded
+// cell (tx0, ty0). With TMA the whole region arrives in one tensor copy at raw
+// (128-byte aligned; else plain loads); cells beyond the padded extent (ragged
+// last tiles) read as zero there, as the clamped cell otherwise, and only feed
+// results that are never stored. False: the copy's bounded wait gave up
+// (uniform over the CTA; the error word is set).
+template <int BX, int BY, int NT, typename X, bool TMA, typename F>
+__device__ __forceinline__ bool stage_region(const StageParams& P, int tx0, int ty0, double* raw,
+                                             const CUtensorMap* tmap, F stage_cell)
+{
+    constexpr int RW = BX + 12, RH = BY + 12, NU = RW * RH;
+    const int tid = threadIdx.x;
+    if constexpr (TMA) {
+        static_assert(BX % 2 == 0 && RW % 2 == 0, "TMA x offsets and rows must be 16-byte multiples");
+        static_assert(RW <= 256 && RH <= 256, "TMA box too large");
+        __shared__ __align__(8) unsigned long long tma_bar;  // never reused for anything else
+        unsigned long long* bar = &tma_bar;
+        if ((smem_addr(raw) & 127u) == 0) {  // uniform: the copy needs a 128-byte aligned destination
+            if (tid == 0) {
+                mbar_init(bar, 1);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
+            __syncthreads();
+            if (tid == 0) {
+                mbar_arrive_expect_tx(bar, (unsigned)(sizeof(double) * 4 * NU) + P.stall_bytes);
+                tma_load_3d(raw, tmap, tx0, ty0, 0, bar);
+            }
+            const bool ok = mbar_wait_bounded(bar);
+            if (__syncthreads_or(!ok)) {
+                // Give the copy one more bounded wait before the CTA leaves.
+                // Leaving is safe only once the copy's bytes have landed: a
+                // copy still in flight after this second wait would write
+                // into shared memory the SM may have handed to another CTA.
+                // The timeout bit set here makes the next synchronising call
+                // fail and stays set until gbr_set_state, so no result
+                // computed after such an event is reported as valid.
+                mbar_wait_bounded(bar);
+                if (tid == 0) atomicOr(P.err, kErrTimeout);
+                return false;
+            }
+            for (int e = tid; e < X::N; e += NT) {
+                const int idx = X::cell(e);
+                stage_cell(idx, raw[idx], raw[NU + idx], raw[2 * NU + idx], raw[3 * NU + idx]);
+            }
+            return true;
+        }
+    }
+    // Plain loads, clamped to the padded extent.
+    const int pitch = P.g.pitch;
+    const long long plane = P.g.plane;
+    for (int e = tid; e < X::N; e += NT) {
+        const int idx = X::cell(e);
+        const int ry = idx / RW, rx = idx - ry * RW;
+        const int gx = min(tx0 + rx, P.g.nx + 2 * kGhost - 1);
+        const int gy = min(ty0 + ry, P.g.ny + 2 * kGhost - 1);
+        const long long o = (long long)gy * pitch + gx;
+        stage_cell(idx, P.q[o], P.q[o + plane], P.q[o + 2 * plane], P.q[o + 3 * plane]);
+    }
+    return true;
+}
+
+// Phase 3 of a tile, from its face fluxes (x faces [4][BY][BX + 1], y faces
+// [4][BY + 1][BX] in shared memory, written before the caller's barrier); ends
+// with all threads synchronised.
+template <typename T, int BX, int BY, int NT>
+__device__ __forceinline__ void finish_tile(const StageParams& P, const PhysT<T>& ph, T inv_dx, T inv_dy, int tx0, int ty0,
+                                            const T* sHX, const T* sHY)
+{
+    constexpr int NHX = (BX + 1) * BY, NHY = BX * (BY + 1);
+    const int nx = P.g.nx, ny = P.g.ny, pitch = P.g.pitch;
+    const long long plane = P.g.plane;
+    const int tid = threadIdx.x;
+    // Phase 3: residual (Eq. deriv) and the FP64 stage update (Eq. rk).
+    const double dt = P.dt_ptr ? *P.dt_ptr : P.dt;
+    const double cdt = P.cc * dt;
+    T lam = T(0);  // max in T, widened once (the same value as widening each cell's)
+    bool bad = false;
+    for (int idx = tid; idx < BX * BY; idx += NT) {
+        const int r = idx / BX, c = idx - r * BX;
+        const int j = tx0 + c, i = ty0 + r;
+        if (j >= nx || i >= ny) continue;
+        double res[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const T dF = sHX[m * NHX + r * (BX + 1) + c + 1] - sHX[m * NHX + r * (BX + 1) + c];
+            const T dG = sHY[m * NHY + (r + 1) * BX + c] - sHY[m * NHY + r * BX + c];
+            res[m] = to_f64(-(rmul(dF, inv_dx) + rmul(dG, inv_dy)));
+        }
+        if (P.res) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) P.res[(long long)m * nx * ny + (long long)i * nx + j] = res[m];
+        }
+        if (P.qout) {
+            const long long o = (long long)(i + kGhost) * pitch + (j + kGhost);
+            double qv[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                double v = P.cb * P.q[o + m * plane] + cdt * res[m];
+                if (P.ca != 0.0) v += P.ca * P.qn[o + m * plane];
+                qv[m] = v;
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m) P.qout[o + m * plane] = qv[m];
+            // Positivity in FP64: rho > 0 and p > 0 <=> 2 rho E > |rho u|^2
+            // (the comparisons on the bits, off the FP64 pipe).
+            const double e2 = 2.0 * qv[0] * qv[3] - (qv[1] * qv[1] + qv[2] * qv[2]);
+            const bool ok = finite_bits(qv[0]) && finite_bits(qv[1]) && finite_bits(qv[2]) && finite_bits(qv[3]) &&
+                            positive_bits(qv[0]) && positive_bits(e2);
+            bad |= !ok;
+            if (P.lam_out)  // Sec. 2.5 wavespeed of the new state
+                lam = tmax_nan(lam, cell_wavespeed_t<T>(qv[0], qv[1], qv[2], qv[3], ph.gamma, ph.gm1, ph.mu,
+                                                        inv_dx, inv_dy));
+        }
+    }
+    if (P.qout) {
+        if (__syncthreads_or(bad) && tid == 0) atomicOr(P.err, kErrNonPhysical);
+    }
+    if (P.lam_out) {
+        __shared__ double red[NT / 32];
+        const double lmax = warp_max(to_f64(lam));
+        if ((tid & 31) == 0) red[tid >> 5] = lmax;
+        __syncthreads();
+        if (tid < 32) {
+            double v = (tid < NT / 32) ? red[tid] : 0.0;
+            v = warp_max(v);
+            if (tid == 0) atomicMax(P.lam_out, (unsigned long long)__double_as_longlong(v));
+        }
+    }
+    __syncthreads();
+}
+
 // LEARNED: 0 = the density detector; 1 = the learned sensor's decisions
 // read from the decision pass (P.dec); 2 = the learned sensor's inference
 // fused into the stage (FP32 only).
@@ -1350,60 +1482,11 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
             sQc[3 * NU + idx] = from_f64<T>(q3);
         }
     };
-    bool staged = false;
-    if constexpr (TMA) {
-        // The whole region in one tensor copy; cells beyond the padded extent
-        // (ragged last tiles) read as zero and only feed results that are
-        // never stored.
-        static_assert(BX % 2 == 0 && L::RW % 2 == 0, "TMA x offsets and rows must be 16-byte multiples");
-        static_assert(L::RW <= 256 && L::RH <= 256, "TMA box too large");
-        static_assert(L::template raw_offset<T>() + L::kRawBytes <= L::template raw_limit<T>(),
-                      "TMA landing area overlaps live shared memory");
-        double* raw = reinterpret_cast<double*>(smem_raw + L::template raw_offset<T>());
-        __shared__ __align__(8) unsigned long long tma_bar;  // never reused for anything else
-        unsigned long long* bar = &tma_bar;
-        if ((smem_addr(raw) & 127u) == 0) {  // uniform: the copy needs a 128-byte aligned destination
-            if (tid == 0) {
-                mbar_init(bar, 1);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            }
-            __syncthreads();
-            if (tid == 0) {
-                mbar_arrive_expect_tx(bar, (unsigned)L::kRawBytes + P.stall_bytes);
-                tma_load_3d(raw, tmap, tx0, ty0, 0, bar);
-            }
-            const bool ok = mbar_wait_bounded(bar);
-            if (__syncthreads_or(!ok)) {
-                // Give the copy one more bounded wait before the CTA leaves.
-                // Leaving is safe only once the copy's bytes have landed: a
-                // copy still in flight after this second wait would write
-                // into shared memory the SM may have handed to another CTA.
-                // The timeout bit set here makes the next synchronising call
-                // fail and stays set until gbr_set_state, so no result
-                // computed after such an event is reported as valid.
-                mbar_wait_bounded(bar);
-                if (tid == 0) atomicOr(P.err, kErrTimeout);
-                return;
-            }
-            for (int e = tid; e < X::N; e += NT) {
-                const int idx = X::cell(e);
-                stage_cell(idx, raw[idx], raw[NU + idx], raw[2 * NU + idx], raw[3 * NU + idx]);
-            }
-            staged = true;
-        }
-    }
-    if (!staged) {
-        // Plain loads, clamped to the padded extent (the clamped cells only
-        // feed results that are never stored).
-        for (int e = tid; e < X::N; e += NT) {
-            const int idx = X::cell(e);
-            const int ry = idx / RW, rx = idx - ry * RW;
-            const int gx = min(tx0 + rx, nx + 2 * kGhost - 1);
-            const int gy = min(ty0 + ry, ny + 2 * kGhost - 1);
-            const long long o = (long long)gy * pitch + gx;
-            stage_cell(idx, P.q[o], P.q[o + plane], P.q[o + 2 * plane], P.q[o + 3 * plane]);
-        }
-    }
+    static_assert(!TMA || L::template raw_offset<T>() + L::kRawBytes <= L::template raw_limit<T>(),
+                  "TMA landing area overlaps live shared memory");
+    if (!stage_region<BX, BY, NT, X, TMA>(P, tx0, ty0, reinterpret_cast<double*>(smem_raw + L::template raw_offset<T>()), tmap,
+                                          stage_cell))
+        return;
     if constexpr (LEARNED == 1) {
         // The learned sensor's per-cell decisions (1 = trouble, 0 = smooth,
         // 2 = unsure: the plain detector decides below) of the detector's
@@ -1438,13 +1521,13 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
 
     // Phase 1: per-cell quantities, each computed once per tile.
     const T* const sV = CONS ? sQc : sU;  // the reconstructed variables
-    for (int idx = tid; idx < (L::GRAD ? L::NGX : 0); idx += NT) {  // x-gradients (Eq. six)
+    for (int idx = tid; idx < L::NGX; idx += NT) {  // x-gradients (Eq. six)
         const int a = idx / L::GXW, b = idx - a * L::GXW;
         const T* s = sV + (a + 6 - V) * RW + (b + 3);
 #pragma unroll
         for (int m = 0; m < 4; ++m) sGX[m * L::NGX + idx] = grad6(s + m * NU, 1);
     }
-    for (int idx = tid; idx < (L::GRAD ? L::NGY : 0); idx += NT) {  // y-gradients
+    for (int idx = tid; idx < L::NGY; idx += NT) {  // y-gradients
         const int a = idx / L::GYW, b = idx - a * L::GYW;
         const T* s = sV + (a + 3) * RW + (b + 6 - V);
 #pragma unroll
@@ -1633,63 +1716,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     }
     __syncthreads();
 
-    // Phase 3: residual (Eq. deriv) and the FP64 stage update (Eq. rk).
-    const double dt = P.dt_ptr ? *P.dt_ptr : P.dt;
-    const double cdt = P.cc * dt;
-    T lam = T(0);  // max in T, widened once (the same value as widening each cell's)
-    bool bad = false;
-    for (int idx = tid; idx < BX * BY; idx += NT) {
-        const int r = idx / BX, c = idx - r * BX;
-        const int j = tx0 + c, i = ty0 + r;
-        if (j >= nx || i >= ny) continue;
-        double res[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const T dF = sHX[m * L::NHX + r * L::HXW + c + 1] - sHX[m * L::NHX + r * L::HXW + c];
-            const T dG = sHY[m * L::NHY + (r + 1) * BX + c] - sHY[m * L::NHY + r * BX + c];
-            res[m] = to_f64(-(rmul(dF, inv_dx) + rmul(dG, inv_dy)));
-        }
-        if (P.res) {
-#pragma unroll
-            for (int m = 0; m < 4; ++m) P.res[(long long)m * nx * ny + (long long)i * nx + j] = res[m];
-        }
-        if (P.qout) {
-            const long long o = (long long)(i + kGhost) * pitch + (j + kGhost);
-            double qv[4];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                double v = P.cb * P.q[o + m * plane] + cdt * res[m];
-                if (P.ca != 0.0) v += P.ca * P.qn[o + m * plane];
-                qv[m] = v;
-            }
-#pragma unroll
-            for (int m = 0; m < 4; ++m) P.qout[o + m * plane] = qv[m];
-            // Positivity in FP64: rho > 0 and p > 0 <=> 2 rho E > |rho u|^2
-            // (the comparisons on the bits, off the FP64 pipe).
-            const double e2 = 2.0 * qv[0] * qv[3] - (qv[1] * qv[1] + qv[2] * qv[2]);
-            const bool ok = finite_bits(qv[0]) && finite_bits(qv[1]) && finite_bits(qv[2]) && finite_bits(qv[3]) &&
-                            positive_bits(qv[0]) && positive_bits(e2);
-            bad |= !ok;
-            if (P.lam_out)  // Sec. 2.5 wavespeed of the new state
-                lam = tmax_nan(lam, cell_wavespeed_t<T>(qv[0], qv[1], qv[2], qv[3], ph.gamma, ph.gm1, ph.mu,
-                                                        inv_dx, inv_dy));
-        }
-    }
-    if (P.qout) {
-        if (__syncthreads_or(bad) && tid == 0) atomicOr(P.err, kErrNonPhysical);
-    }
-    if (P.lam_out) {
-        __shared__ double red[NT / 32];
-        const double lmax = warp_max(to_f64(lam));
-        if ((tid & 31) == 0) red[tid >> 5] = lmax;
-        __syncthreads();
-        if (tid < 32) {
-            double v = (tid < NT / 32) ? red[tid] : 0.0;
-            v = warp_max(v);
-            if (tid == 0) atomicMax(P.lam_out, (unsigned long long)__double_as_longlong(v));
-        }
-    }
-    __syncthreads();
+    finish_tile<T, BX, BY, NT>(P, ph, inv_dx, inv_dy, tx0, ty0, sHX, sHY);
 }
 
 // One CTA per tile; the tile + halo is staged by a tensor copy described by

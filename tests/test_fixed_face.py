@@ -36,6 +36,18 @@ static R meg(const R* w, const R* e, int order)
     const R hi = fminl(fmaxl(fmaxl(w[2], w[3]), md), fmaxl(fmaxl(w[2], ul), lc));
     return pl < lo ? lo : (pl > hi ? hi : pl);
 }
+struct Planes {  // the kernel's split planes of one face
+    const double* const* u;
+    int su;
+    void operator()(int m, fx::Stencil& x) const
+    {
+        for (int k = 0; k < 12; ++k) {
+            unsigned short e;
+            fx::split(u[m][(k - 5) * su], x.m[k], e);
+            x.e[k] = e;
+        }
+    }
+};
 template <int ORDER>
 static int run(int mode, int stride)
 {
@@ -60,7 +72,7 @@ static int run(int mode, int stride)
         const double rb = 0.5 * (u[0][0] + u[0][stride]), pb = 0.5 * (u[3][0] + u[3][stride]);
         const double c = std::sqrt(1.4 * pb / rb), rc = rb * c, ic2 = 1 / (c * c);
         fx::FaceStates o;
-        fx::face_states<ORDER>(u, stride, rc, ic2, o);
+        fx::face_states<ORDER>(Planes{u, stride}, rc, ic2, o);
         if (!o.ok) return std::printf("refused\n"), 1;
         R wl[4], wr[4], big[3] = {0, 0, 0};
         for (int f = 0; f < 4; ++f) {
@@ -98,9 +110,19 @@ static int limits()
         const long long x = (long long)(g() >> (2 + g() % 62)) * (g() & 1 ? 1 : -1);
         const double d = fx::to_double(x, fx::kOne);
         if (std::fabs((double)((R)d - (R)x)) > std::ldexp(std::fabs((double)x), -53)) return std::printf("%lld -> %.17g\n", x, d), 1;
-        if (std::fabs((double)x) < 9e15 && fx::from_double(d, 1081) != x * 1) return std::printf("back %lld\n", x), 1;
+        long long m;
+        unsigned short e;
+        fx::split(d, m, e);
+        if (fx::unsplit(m, e) != d) return std::printf("split %.17g\n", d), 1;
+        if (std::fabs((double)x) < 9e15 && fx::aligned(m, e, fx::kOne) != x) return std::printf("back %lld\n", x), 1;
     }
-    if (fx::to_double(0, 700) != 0.0 || fx::from_double(0.0, fx::kExpMin) != 0 || fx::from_double(-5e-324, 900) != 0) return 1;
+    for (double d : {0.0, 1.0, -1.0, 2.2250738585072014e-308, -1.7976931348623157e308, (double)INFINITY}) {
+        long long m;
+        unsigned short e;
+        fx::split(d, m, e);
+        if (fx::unsplit(m, e) != d) return std::printf("split %.17g\n", d), 1;
+    }
+    if (fx::to_double(0, 700) != 0.0) return 1;
     for (double bad : {(double)INFINITY, (double)NAN, 1e300, -(double)INFINITY}) {
         double v[12];
         for (int m = 0; m < 4; ++m) {
@@ -110,16 +132,52 @@ static int limits()
             w[m][3] = bad;
             const double* u[4] = {w[0] + 5, w[1] + 5, w[2] + 5, w[3] + 5};
             fx::FaceStates o;
-            fx::face_states<7>(u, 1, 1.2, 0.7, o);
+            fx::face_states<7>(Planes{u, 1}, 1.2, 0.7, o);
             if (o.ok) return std::printf("%g accepted in plane %d\n", bad, m), 1;
         }
         (void)v;
     }
     return 0;
 }
+// The flux mean and the gradient against long double: exact but for the
+// alignment (one unit of 2^-58 of the largest value each, times the weights'
+// absolute sum over the divisor, at most 1.7 and 110) and the final rounding.
+template <int ORDER>
+static int sums(int mode)
+{
+    std::mt19937_64 g(11 + mode);
+    std::uniform_real_distribution<double> U(-1, 1);
+    const int w7[5] = {1052, -250, 38, 1, -1}, w4[5] = {1821, -461, 85, -4, -1};
+    for (int it = 0; it < 50000; ++it) {
+        double f[10];
+        long long m[10];
+        int ex[10];
+        R big = 0, mean = 0, big7 = 0;
+        for (int k = 0; k < 10; ++k) {
+            f[k] = mode == 2 && k % 3 == 0 ? 0.0 : U(g) * std::pow(10.0, mode ? 8 * U(g) : 0.0);
+            unsigned short e;
+            fx::split(f[k], m[k], e);
+            ex[k] = e;
+            big = fmaxl(big, fabsl((R)f[k]));
+            if (k < 7 && k != 3) big7 = fmaxl(big7, fabsl((R)f[k]));
+        }
+        for (int k = 0; k < 5; ++k) mean += (R)(ORDER == 4 ? w4 : w7)[k] * ((R)f[4 - k] + (R)f[5 + k]);
+        mean /= ORDER == 4 ? 2880 : 1680;
+        const double got = fx::recon_mean<ORDER>(m, ex);
+        if (!(fabsl(got - mean) <= ldexpl(fabsl(mean), -53) + 4 * ldexpl(big, -57))) return std::printf("mean: %g %g\n", got, (double)mean), 1;
+        long long m7[7];
+        int e7[7];
+        for (int k = 0; k < 7; ++k) m7[k] = m[k], e7[k] = ex[k];
+        const R grad = 45 * ((R)f[4] - f[2]) - 9 * ((R)f[5] - f[1]) + ((R)f[6] - f[0]);
+        const double gg = fx::grad60(m7, e7);
+        if (!(fabsl(gg - grad) <= ldexpl(fabsl(grad), -53) + 400 * ldexpl(big7, -57))) return std::printf("gradient: %g %g\n", gg, (double)grad), 1;
+    }
+    return 0;
+}
 int main()
 {
     int bad = limits();
+    for (int mode = 0; mode < 3; ++mode) bad |= sums<7>(mode) | sums<4>(mode);
     for (int mode = 0; mode < 5; ++mode) bad |= run<7>(mode, 1 + mode % 3) | run<4>(mode, 1 + mode % 3);
     return bad;
 }
