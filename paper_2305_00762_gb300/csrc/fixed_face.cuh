@@ -364,20 +364,21 @@ GBR_HD u64 factor(double a, int e, int eo)
     return k < 63 ? m >> k : 0;
 }
 
-// Characteristic face states of one field pair (L, R): sums and differences of
-// the acoustic fields, entropy and shear.
+// The face states (L, R) back in primitives.
 struct FaceStates {
-    double a03[2], dif[2], s[2], ut[2];  // w1 + w4, w4 - w1, w2, w3 (acoustic fields as p -/+ rho c un)
-    bool ok;                             // false: a stencil value too large, infinite or NaN
+    double r[2], un[2], ut[2], p[2];
+    bool ok;  // false: a stencil value too large, infinite or NaN
 };
 
-// load(m, x): the stencil of variable m (0 rho, 1 un, 2 ut, 3 p); rc = rho c
-// and ic2 = 1 / c^2 of the face's mean state.
+// load(m, x): the stencil of variable m (0 rho, 1 un, 2 ut, 3 p); of the face's
+// mean state, y = 1 / (2 rho c), rc2 = 2 rho c and ic2 = 1 / c^2. Fields: entropy
+// w2 = rho - p / c^2; w1, w4 = p -/+ rho c un; shear w3 = ut. Back: p =
+// (w1 + w4) / 2, un = (w4 - w1) y, rho = w2 + p / c^2.
 template <int ORDER, typename F>
-GBR_HD void face_states(F load, double rc, double ic2, FaceStates& o)
+GBR_HD void face_states(F load, double y, double rc2, double ic2, FaceStates& o)
 {
     Functionals P;
-    i64 wl, wr;
+    i64 sl, sr;
     int ep, es, et, ew;
     {
         Stencil x;
@@ -394,28 +395,36 @@ GBR_HD void face_states(F load, double rc, double ic2, FaceStates& o)
         scale(P, factor(ic2, ep, es), S);
         variable<ORDER>(x, es, R);
         difference(R, S, R);
-        limited<ORDER>(R, wl, wr);
-        o.s[0] = to_double(wl, es);
-        o.s[1] = to_double(wr, es);
+        limited<ORDER>(R, sl, sr);
     }
     {  // fields 1 and 4 (u -/+ c), carried as p -/+ rho c un
         Stencil x;
         load(1, x);
-        const int eu = stencil_exponent(x), eprod = eu + exponent(rc) - 1022;
+        const int eu = stencil_exponent(x), eprod = eu - 1 + exponent(rc2) - 1022;  // (half of rc2)
         ew = (ep > eprod ? ep : eprod) + 1;
         Functionals U, W;
         variable<ORDER>(x, eu, U);
-        scale(U, factor(rc, eu, ew), U);
+        scale(U, factor(rc2, eu - 1, ew), U);
         shift_right(P, ew - ep);
-        i64 ml, mr;
+        i64 ml, mr, pl, pr;
         difference(P, U, W);
         limited<ORDER>(W, ml, mr);
         sum(P, U, W);
-        limited<ORDER>(W, wl, wr);
-        o.a03[0] = to_double(wl + ml, ew);
-        o.a03[1] = to_double(wr + mr, ew);
-        o.dif[0] = to_double(wl - ml, ew);
-        o.dif[1] = to_double(wr - mr, ew);
+        limited<ORDER>(W, pl, pr);
+        const u64 fy = factor(y, 0, exponent(y) - 1022);  // (the whole mantissa)
+        const int ev = ew + exponent(y) - 1022;
+        const bool some = ev >= kExpMin;  // smaller velocities count as zero
+        o.un[0] = to_double(some ? mulhi(pl - ml, fy) : 0, some ? ev : kExpMin);
+        o.un[1] = to_double(some ? mulhi(pr - mr, fy) : 0, some ? ev : kExpMin);
+        pl += ml;  // 2 p: p in units one exponent lower
+        pr += mr;
+        o.p[0] = to_double(pl, ew - 1);
+        o.p[1] = to_double(pr, ew - 1);
+        const int eprod2 = ew - 1 + exponent(ic2) - 1022, er = (es > eprod2 ? es : eprod2) + 1;
+        const u64 fi = factor(ic2, ew - 1, er);
+        o.r[0] = to_double(aligned(sl, es, er) + mulhi(pl, fi), er);
+        o.r[1] = to_double(aligned(sr, es, er) + mulhi(pr, fi), er);
+        o.ok = er <= kExpMax && ev <= kExpMax;
     }
     {  // field 3 (shear): ut
         Stencil x;
@@ -423,11 +432,12 @@ GBR_HD void face_states(F load, double rc, double ic2, FaceStates& o)
         et = stencil_exponent(x);
         Functionals R;
         variable<ORDER>(x, et, R);
-        limited<ORDER>(R, wl, wr);
-        o.ut[0] = to_double(wl, et);
-        o.ut[1] = to_double(wr, et);
+        i64 tl, tr;
+        limited<ORDER>(R, tl, tr);
+        o.ut[0] = to_double(tl, et);
+        o.ut[1] = to_double(tr, et);
     }
-    o.ok = ew <= kExpMax && es <= kExpMax && et <= kExpMax;
+    o.ok = o.ok && ew <= kExpMax && es <= kExpMax && et <= kExpMax;
 }
 
 // 1/2 (F(f_L) + F(f_R)) at the face after cell j of one flux component, the

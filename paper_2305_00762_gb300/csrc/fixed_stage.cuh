@@ -104,15 +104,16 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             for (int m = 0; m < 4; ++m) fx::split(w[m], sM[m * NU + idx], sE[m * NU + idx]);
             sR[idx] = f64_to_f32_rn(w[0]);
             const int ry = idx / RW, rx = idx - ry * RW;
+            const double ep = q3 + w[3];
             if (ry >= 6 && ry < 6 + BY && rx >= 1 && rx < BX + 11) {
                 const int f = (ry - 6) * L::FXW + (rx - 1);
-                const double h[4] = {q1, rfma(q1, w[1], w[3]), rmul(q1, w[2]), rmul(w[1], q3 + w[3])};
+                const double h[4] = {q1, rfma(q1, w[1], w[3]), rmul(q1, w[2]), rmul(w[1], ep)};
 #pragma unroll
                 for (int m = 0; m < 4; ++m) fx::split(h[m], sFX[m * L::NFX + f], sEX[m * L::NFX + f]);
             }
             if (ry >= 1 && ry < BY + 11 && rx >= 6 && rx < BX + 6) {
                 const int f = (ry - 1) * BX + (rx - 6);
-                const double h[4] = {q2, rmul(q2, w[1]), rfma(q2, w[2], w[3]), rmul(w[2], q3 + w[3])};
+                const double h[4] = {q2, rmul(q2, w[1]), rfma(q2, w[2], w[3]), rmul(w[2], ep)};
 #pragma unroll
                 for (int m = 0; m < 4; ++m) fx::split(h[m], sFY[m * L::NFY + f], sEY[m * L::NFY + f]);
             }
@@ -187,10 +188,11 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         u1[3] = cell(3, su);
         // Characteristic projection at the arithmetic-mean state, every
         // factor from one reciprocal square root y = 1/sqrt(gamma p rho).
-        const double rb = 0.5 * (u0[0] + u1[0]), gp = ph.gamma * (0.5 * (u0[3] + u1[3]));
-        const double y = fx::rsqrt(gp * rb);
-        const double icb = rb * y, cb = gp * y;  // 1 / c, c
-        const double ic2 = icb * icb;
+        // (Twice the means: X = (2 rho)(2 gamma p), y = 1/sqrt(X) = 1/(2 rho c),
+        // 1/c = 2 rho y, 2 rho c = X y.)
+        const double rb = u0[0] + u1[0], gp = ph.gamma * (u0[3] + u1[3]), xx = rmul(gp, rb);
+        const double y = fx::rsqrt(xx);
+        const double icb = rmul(rb, y), ic2 = rmul(icb, icb);
         fx::FaceStates s;
         fx::face_states<ORDER>(
             [&](int m, fx::Stencil& x) {
@@ -201,12 +203,9 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                     x.e[k] = sE[at + (k - 5) * su];
                 }
             },
-            rb * cb, ic2, s);
-        // Back to primitives: the acoustic fields are p -/+ rho c un, so with
-        // a = w1 + w4, rho = a / (2 c^2) + w2, p = a / 2, un = (w4 - w1) / (2 rho c).
-        const double hrc = 0.5 * y, be = 0.5 * ic2;
-        double rL = rfma(be, s.a03[0], s.s[0]), unL = hrc * s.dif[0], utL = s.ut[0], pL = 0.5 * s.a03[0];
-        double rR = rfma(be, s.a03[1], s.s[1]), unR = hrc * s.dif[1], utR = s.ut[1], pR = 0.5 * s.a03[1];
+            y, rmul(xx, y), ic2, s);
+        double rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
+        double rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
         // positivity fallback: a face state with rho <= 0 or p <= 0 (or from a
         // refused stencil) takes the adjacent cell's state
         if (!(s.ok && tpositive(rL) && tpositive(pL))) {
@@ -221,19 +220,8 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             utR = cell(2, su);
             pR = u1[3];
         }
-        // E = p / (gamma - 1) + (rho un un + rho ut ut) / 2, from the momenta
-        double QL[4], QR[4];
-        QL[0] = rL;
-        QL[1] = rL * unL;
-        QL[2] = rL * utL;
-        QL[3] = rfma(0.5, rfma(QL[1], unL, rmul(QL[2], utL)), rmul(pL, ph.igm1));
-        QR[0] = rR;
-        QR[1] = rR * unR;
-        QR[2] = rR * utR;
-        QR[3] = rfma(0.5, rfma(QR[1], unR, rmul(QR[2], utR)), rmul(pR, ph.igm1));
-
-        // Central part 1/2 (F_L + F_R) of the hybrid face fluxes (Sec. 2.4).
-        double Fc[4];
+        // Flux reconstruction of the central part where sigma = 1 (Sec. 2.4).
+        double Fs[4];
         if (!trouble) {
             const int at = xf ? fr * L::FXW + fc + 4 : (fr + 4) * BX + fc, sf = xf ? 1 : BX;
             const int nf = xf ? L::NFX : L::NFY;
@@ -250,19 +238,14 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                     e[k] = fe[pl + (k - 4) * sf];
                 }
                 const double f = fx::recon_mean<ORDER>(q, e);
-                if (m == 0) Fc[0] = f;
-                if (m == 1) Fc[1] = f;
-                if (m == 2) Fc[2] = f;
-                if (m == 3) Fc[3] = f;
+                if (m == 0) Fs[0] = f;
+                if (m == 1) Fs[1] = f;
+                if (m == 2) Fs[2] = f;
+                if (m == 3) Fs[3] = f;
             }
-        } else {
-            Fc[0] = 0.5 * (QL[1] + QR[1]);
-            Fc[1] = 0.5 * ((QL[1] * unL + pL) + (QR[1] * unR + pR));
-            Fc[2] = 0.5 * (QL[1] * utL + QR[1] * utR);
-            Fc[3] = 0.5 * (unL * (QL[3] + pL) + unR * (QR[3] + pR));
         }
         double out[4];
-        hllc_flux(ph, Fc, QL, QR, rL, unL, utL, pL, QL[3], rR, unR, utR, pR, QR[3], out);
+        hllc_flux(ph, !trouble, Fs, rL, unL, utL, pL, rR, unR, utR, pR, out);
         if constexpr (VISC) {
             u0[1] = cell(1, 0);
             u1[1] = cell(1, su);

@@ -126,6 +126,12 @@ __device__ __forceinline__ float trcp(float x) { return 1.f / x; }
 __device__ __forceinline__ double tsinpi(double x) { return sinpi(x); }
 __device__ __forceinline__ float tsinpi(float x) { return sinpif(x); }
 __device__ __forceinline__ double tabs(double x) { return fabs(x); }
+// |x| / 2 by the exponent, off the FP64 pipe; subnormal results are zero
+__device__ __forceinline__ double thalfabs(double x)
+{
+    const int h = __double2hiint(x) & 0x7fffffff;
+    return h >= 0x00200000 ? (h >= 0x7ff00000 ? fabs(x) : __hiloint2double(h - 0x00100000, __double2loint(x))) : 0.0;
+}
 __device__ __forceinline__ float tabs(float x) { return fabsf(x); }
 
 // FP64 comparisons on the integer pipe. GB300 runs every FP64 instruction,
@@ -238,7 +244,10 @@ __device__ __forceinline__ void prims_of(double q0, double q1, double q2, double
     const T ir = trcp(r);
     u = from_f64<T>(q1) * ir;
     v = from_f64<T>(q2) * ir;
-    p = gm1 * rfma(-rmul(T(0.5), r), sumsq(u, v), from_f64<T>(q3));
+    if constexpr (sizeof(T) == 8)  // (rho u^2 from the momentum: one product fewer, exact state)
+        p = rmul(gm1, rfma(T(-0.5), rmul(q1, u) + rmul(q2, v), q3));
+    else
+        p = gm1 * rfma(-rmul(T(0.5), r), sumsq(u, v), from_f64<T>(q3));
 }
 
 // Sec. 2.5: CFL wavespeed of one cell state, max((|u| + c)/dx, (|v| + c)/dy)
@@ -565,6 +574,79 @@ struct PhysT {
 };
 
 // HLLC in the form 1/2 (F_L + F_R) - 1/2 |A| (Q_R - Q_L), Eq. Riemann_revisit,
+// from the face states (rho, un, ut, p). The central part is Fs (flux
+// reconstruction) where `smooth`, else F(Q_L), F(Q_R) of the states
+// (Sec. 2.4). Toro's star states Q*_K = k_K (1, S*, ut_K, e_K + t_K S*) +
+// (0, 0, 0, t_K p_K / (S_K - S*)) with e = E / rho, t_K = S* - un_K, k_K = m_K /
+// (S_K - S*), m_K = rho_K (S_K - un_K) are never built: with a = |S| / 2 and
+// 1/2 |A| dQ = (aL - aS) Q*_L + (aS - aR) Q*_R - aL Q_L + aR Q_R, the factors
+// gi_K of 1/(S_K - S*), f_K of k_K and g_L = aL rho_L - f_L, g_R = aR rho_R + f_R
+// leave two to four products per component.
+// FP64: roots and reciprocals cost the FP64 pipe nothing (fixed_math.cuh).
+__device__ __forceinline__ void hllc_flux(const PhysT<double>& P, bool smooth, const double (&Fs)[4], double rL, double unL,
+                                          double utL, double pL, double rR, double unR, double utR, double pR,
+                                          double (&out)[4])
+{
+    typedef double T;
+    const T irL = trcp(rL), irR = trcp(rR);
+    const T vL = rmul(pL, irL), vR = rmul(pR, irR);  // p / rho
+    const T c2L = rmul(P.gamma, vL), c2R = rmul(P.gamma, vR);
+    const T cL = rmul(c2L, trsqrt(c2L)), cR = rmul(c2R, trsqrt(c2R));
+    const T eL = rfma(T(0.5), rfma(utL, utL, rmul(unL, unL)), rmul(vL, P.igm1));
+    const T eR = rfma(T(0.5), rfma(utR, utR, rmul(unR, unR)), rmul(vR, P.igm1));
+    const T HL = eL + vL, HR = eR + vR;
+    T Fc[4];
+    if (smooth) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) Fc[m] = Fs[m];
+    } else {
+        const T jL = rmul(rL, unL), jR = rmul(rR, unR);
+        Fc[0] = T(0.5) * (jL + jR);
+        Fc[1] = T(0.5) * (rfma(jL, unL, pL) + rfma(jR, unR, pR));
+        Fc[2] = T(0.5) * rfma(jL, utL, rmul(jR, utR));
+        Fc[3] = T(0.5) * rfma(jL, HL, rmul(jR, HR));
+    }
+    // Roe averages (a_L + q a_R) / (1 + q), q = sqrt(rho_R / rho_L)
+    const T xq = rmul(rR, irL);
+    const T q = rmul(xq, trsqrt(xq));
+    const T oL = trcp(T(1) + q);
+    const T ut = rmul(oL, rfma(q, unR, unL));
+    const T vt = rmul(oL, rfma(q, utR, utL));
+    const T Ht = rmul(oL, rfma(q, HR, HL));
+    const T c2t = rmul(P.gm1, rfma(T(-0.5), rfma(vt, vt, rmul(ut, ut)), Ht));
+    const T ct = rmul(c2t, trsqrt(c2t));
+    const T SL = tmin(unL - cL, ut - ct);
+    const T SR = tmax(unR + cR, ut + ct);
+    const T mL = rmul(rL, SL - unL), mR = rmul(rR, SR - unR);
+    const T num = rfma(-mR, unR, rfma(mL, unL, pR - pL)), den = mL - mR;  // S* = num / den
+    const T Ss = rmul(num, trcp(den)), iL = trcp(SL - Ss), iR = trcp(SR - Ss);
+    T aL = thalfabs(SL), aR = thalfabs(SR);
+    const T aS = thalfabs(Ss);
+    if (P.lm) {
+        // Shock-stable HLLC-LM (Fleischmann, Adami and Adams 2020, used by
+        // Examples 7 and 8): the acoustic dissipation scaled by
+        // phi = sin(pi/2 min(1, Ma / 0.1)), Ma the larger face-normal Mach
+        // number of the two face states; phi = 1 leaves HLLC unchanged.
+        const T z = tmax(tabs(unL) * trcp(cL), tabs(unR) * trcp(cR)) * T(10);
+        if (z < T(1)) {
+            const T phi = tsinpi(T(0.5) * z);
+            aL *= phi;
+            aR *= phi;
+        }
+    }
+    const T giL = rmul(aL - aS, iL), giR = rmul(aS - aR, iR);
+    const T fL = rmul(giL, mL), fR = rmul(giR, mR);
+    const T tL = Ss - unL, tR = Ss - unR;
+    const T gL = rfma(aL, rL, -fL), gR = rfma(aR, rR, fR);
+    out[0] = (Fc[0] + gL) - gR;
+    out[1] = rfma(-fR, tR, rfma(-fL, tL, rfma(-gR, unR, rfma(gL, unL, Fc[1]))));
+    out[2] = rfma(-gR, utR, rfma(gL, utL, Fc[2]));
+    out[3] = rfma(-tR, rfma(giR, pR, rmul(fR, Ss)),
+                  rfma(-tL, rfma(giL, pL, rmul(fL, Ss)), rfma(-gR, eR, rfma(gL, eL, Fc[3]))));
+}
+
+// The same flux for the FP32 form, from the conservative states as well, whose
+// divisions are not free: HLLC in the form 1/2 (F_L + F_R) - 1/2 |A| (Q_R - Q_L),
 // with Toro's star states; k (E/rho + (S*-u)(S* + p/(rho (S-u)))) is
 // expanded so that the only divisions are 1/((S_L - S*)(S_R - S*)), S* and
 // the Roe weight.
@@ -896,14 +978,15 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
     if (smooth) {
 #pragma unroll
         for (int m = 0; m < 4; ++m) Fc[m] = recon_mean(in.f[m], in.sf, coef);
-    } else {
+    } else if constexpr (sizeof(T) == 4) {
         Fc[0] = T(0.5) * (QL[1] + QR[1]);
         Fc[1] = T(0.5) * ((QL[1] * unL + pL) + (QR[1] * unR + pR));
         Fc[2] = T(0.5) * (QL[1] * utL + QR[1] * utR);
         Fc[3] = T(0.5) * (unL * (EL + pL) + unR * (ER + pR));
     }
 
-    hllc_flux(P, Fc, QL, QR, rL, unL, utL, pL, EL, rR, unR, utR, pR, ER, out);
+    if constexpr (sizeof(T) == 8) hllc_flux(P, smooth, Fc, rL, unL, utL, pL, rR, unR, utR, pR, out);
+    else hllc_flux(P, Fc, QL, QR, rL, unL, utL, pL, EL, rR, unR, utR, pR, ER, out);
     if constexpr (VISC) {
         T u0[4], u1[4];
 #pragma unroll
@@ -1352,37 +1435,41 @@ __device__ __forceinline__ void finish_tile(const StageParams& P, const PhysT<T>
     // Phase 3: residual (Eq. deriv) and the FP64 stage update (Eq. rk).
     const double dt = P.dt_ptr ? *P.dt_ptr : P.dt;
     const double cdt = P.cc * dt;
+    constexpr bool kScaled = sizeof(T) == 8;
+    const T sx = kScaled && P.qout ? T(cdt) * inv_dx : inv_dx, sy = kScaled && P.qout ? T(cdt) * inv_dy : inv_dy;
     T lam = T(0);  // max in T, widened once (the same value as widening each cell's)
     bool bad = false;
     for (int idx = tid; idx < BX * BY; idx += NT) {
         const int r = idx / BX, c = idx - r * BX;
         const int j = tx0 + c, i = ty0 + r;
         if (j >= nx || i >= ny) continue;
-        double res[4];
+        double res[4];  // FP64: -dt Res when there is a stage update (cdt within sx, sy)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             const T dF = sHX[m * NHX + r * (BX + 1) + c + 1] - sHX[m * NHX + r * (BX + 1) + c];
             const T dG = sHY[m * NHY + (r + 1) * BX + c] - sHY[m * NHY + r * BX + c];
-            res[m] = to_f64(-(rmul(dF, inv_dx) + rmul(dG, inv_dy)));
+            // (square cells in FP64: one product)
+            const T sum = kScaled && sx == sy ? rmul(dF + dG, sx) : rmul(dF, sx) + rmul(dG, sy);
+            res[m] = to_f64(kScaled ? sum : -sum);
         }
         if (P.res) {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) P.res[(long long)m * nx * ny + (long long)i * nx + j] = res[m];
+            for (int m = 0; m < 4; ++m) P.res[(long long)m * nx * ny + (long long)i * nx + j] = kScaled ? -res[m] : res[m];
         }
         if (P.qout) {
             const long long o = (long long)(i + kGhost) * pitch + (j + kGhost);
             double qv[4];
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                double v = P.cb * P.q[o + m * plane] + cdt * res[m];
-                if (P.ca != 0.0) v += P.ca * P.qn[o + m * plane];
+                double v = kScaled ? rfma(P.cb, P.q[o + m * plane], -res[m]) : P.cb * P.q[o + m * plane] + cdt * res[m];
+                if (P.ca != 0.0) v = rfma(P.ca, P.qn[o + m * plane], v);
                 qv[m] = v;
             }
 #pragma unroll
             for (int m = 0; m < 4; ++m) P.qout[o + m * plane] = qv[m];
             // Positivity in FP64: rho > 0 and p > 0 <=> 2 rho E > |rho u|^2
             // (the comparisons on the bits, off the FP64 pipe).
-            const double e2 = 2.0 * qv[0] * qv[3] - (qv[1] * qv[1] + qv[2] * qv[2]);
+            const double e2 = rfma(qv[0] + qv[0], qv[3], -rfma(qv[1], qv[1], rmul(qv[2], qv[2])));
             const bool ok = finite_bits(qv[0]) && finite_bits(qv[1]) && finite_bits(qv[2]) && finite_bits(qv[3]) &&
                             positive_bits(qv[0]) && positive_bits(e2);
             bad |= !ok;

@@ -72,7 +72,7 @@ static int run(int mode, int stride)
         const double rb = 0.5 * (u[0][0] + u[0][stride]), pb = 0.5 * (u[3][0] + u[3][stride]);
         const double c = std::sqrt(1.4 * pb / rb), rc = rb * c, ic2 = 1 / (c * c);
         fx::FaceStates o;
-        fx::face_states<ORDER>(Planes{u, stride}, rc, ic2, o);
+        fx::face_states<ORDER>(Planes{u, stride}, 0.5 / rc, 2 * rc, ic2, o);
         if (!o.ok) return std::printf("refused\n"), 1;
         R wl[4], wr[4], big[3] = {0, 0, 0};
         for (int f = 0; f < 4; ++f) {
@@ -90,10 +90,12 @@ static int run(int mode, int stride)
             for (int k = 0; k < 5; ++k) a[k] = q[8 - k], b[k] = -e[8 - k];
             wr[f] = meg(a, b, ORDER);
         }
-        const R ref[8] = {wl[0] + wl[3], wr[0] + wr[3], wl[3] - wl[0], wr[3] - wr[0], wl[1], wr[1], wl[2], wr[2]};
-        const double got[8] = {o.a03[0], o.a03[1], o.dif[0], o.dif[1], o.s[0], o.s[1], o.ut[0], o.ut[1]};
+        const R y = 0.5 / rc, pl = (wl[0] + wl[3]) / 2, pr = (wr[0] + wr[3]) / 2;
+        const R ref[8] = {pl, pr, (wl[3] - wl[0]) * y, (wr[3] - wr[0]) * y, wl[1] + pl * ic2, wr[1] + pr * ic2, wl[2], wr[2]};
+        const R scale[4] = {big[0], big[0] * y * 2, big[1] + big[0] * ic2, big[2]};
+        const double got[8] = {o.p[0], o.p[1], o.un[0], o.un[1], o.r[0], o.r[1], o.ut[0], o.ut[1]};
         for (int k = 0; k < 8; ++k) {
-            const R tol = ldexpl(fabsl(ref[k]), -53) + ldexpl(big[k < 4 ? 0 : k < 6 ? 1 : 2], -52);
+            const R tol = ldexpl(fabsl(ref[k]), -53) + ldexpl(scale[k / 2], -52);
             const R d = fabsl(ref[k] - (R)got[k]);
             if (!(d <= tol)) return std::printf("order %d mode %d value %d: %g off, %g allowed\n", ORDER, mode, k, (double)d, (double)tol), 1;
             if (tol > 0 && (double)(d / tol) > worst) worst = (double)(d / tol);
@@ -132,7 +134,7 @@ static int limits()
             w[m][3] = bad;
             const double* u[4] = {w[0] + 5, w[1] + 5, w[2] + 5, w[3] + 5};
             fx::FaceStates o;
-            fx::face_states<7>(Planes{u, 1}, 1.2, 0.7, o);
+            fx::face_states<7>(Planes{u, 1}, 1 / 1.2, 1.2, 0.7, o);
             if (o.ok) return std::printf("%g accepted in plane %d\n", bad, m), 1;
         }
         (void)v;
