@@ -440,6 +440,103 @@ GBR_HD void face_states(F load, double y, double rc2, double ic2, FaceStates& o)
     o.ok = o.ok && ew <= kExpMax && es <= kExpMax && et <= kExpMax;
 }
 
+// MEG7-cons: the reconstructed variables are rho, rho un, rho ut, E, projected
+// with the left eigenvectors of the conservative flux Jacobian at the mean
+// state. With A = b2 q0 - b1 (u q1 + v q2 - q3), b1 = (gamma - 1) / c^2, b2 =
+// b1 (u^2 + v^2) / 2 and t = (u q0 - q1) / c the fields are w1 = (A + t) / 2,
+// w2 = q0 - A, w3 = q2 - v q0, w4 = (A - t) / 2. The face state is returned as
+// sums: rho = w1 + w2 + w4, s = w1 + w4, d = w4 - w1, w3.
+struct ConsCoefs {
+    double b1, b1u, b1v, b2, uc, ic, v;  // b1, b1 u, b1 v, b2, u / c, 1 / c, v
+};
+struct ConsStates {
+    double r[2], s[2], d[2], w3[2];
+    bool ok;  // false: a stencil value too large, infinite or NaN
+};
+
+// acc += a f (acc -= with `minus`), a of any sign, r the factor() of |a|.
+GBR_HD void accumulate(Functionals& acc, const Functionals& f, double a, u64 r, bool minus)
+{
+    const i64 g = (bits_of(a) >> 63) != (minus ? 1u : 0u) ? -1 : 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        acc.v[k] += (mulhi(f.v[k], r) ^ g) - g;
+        acc.d[k] += (mulhi(f.d[k], r) ^ g) - g;
+    }
+    acc.n[0] += (mulhi(f.n[0], r) ^ g) - g;
+    acc.n[1] += (mulhi(f.n[1], r) ^ g) - g;
+}
+GBR_HD int larger(int a, int b) { return a > b ? a : b; }
+
+// load(m, x): the stencil of variable m; scale(m): its stencil's exponent.
+template <int ORDER, typename F, typename E>
+GBR_HD void cons_states(F load, E scale_of, const ConsCoefs& C, ConsStates& o)
+{
+    int e[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) e[m] = scale_of(m);
+    auto product = [](int es, double a) { return es + exponent(a) - 1022; };
+    // A and t are sums of four and two terms, 2 w1 = A + t of six: three bits
+    int ea = larger(larger(product(e[0], C.b2), product(e[1], C.b1u)), larger(product(e[2], C.b1v), product(e[3], C.b1)));
+    ea = larger(ea, larger(product(e[0], C.uc), product(e[1], C.ic))) + 3;
+    ea = larger(ea, kExpMin);
+    const int es = larger(e[2], product(e[0], C.v)) + 1, er = larger(e[0], ea) + 1;
+    Functionals Q0, A, T, W;
+    i64 tl, tr;
+    {
+        Stencil x;
+        load(0, x);
+        variable<ORDER>(x, e[0], Q0);
+        scale(Q0, factor(C.b2, e[0], ea), A);
+        const i64 g = (i64)bits_of(C.uc) >> 63;
+        scale(Q0, factor(C.uc, e[0], ea), T);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            T.v[k] = (T.v[k] ^ g) - g;
+            T.d[k] = (T.d[k] ^ g) - g;
+        }
+        T.n[0] = (T.n[0] ^ g) - g;
+        T.n[1] = (T.n[1] ^ g) - g;
+    }
+    {
+        Stencil x;
+        Functionals Q;
+        load(1, x);
+        variable<ORDER>(x, e[1], Q);
+        accumulate(A, Q, C.b1u, factor(C.b1u, e[1], ea), true);
+        accumulate(T, Q, C.ic, factor(C.ic, e[1], ea), true);
+        load(3, x);
+        variable<ORDER>(x, e[3], Q);
+        accumulate(A, Q, C.b1, factor(C.b1, e[3], ea), false);
+        load(2, x);
+        variable<ORDER>(x, e[2], Q);
+        accumulate(A, Q, C.b1v, factor(C.b1v, e[2], ea), true);
+        W = Q;
+        shift_right(W, es - e[2]);
+        accumulate(W, Q0, C.v, factor(C.v, e[0], es), true);
+        limited<ORDER>(W, tl, tr);
+    }
+    i64 al, ar, bl, br, cl, cr;  // 2 w1, 2 w4, w2
+    sum(A, T, W);
+    limited<ORDER>(W, al, ar);
+    difference(A, T, W);
+    limited<ORDER>(W, bl, br);
+    shift_right(Q0, er - e[0]);
+    shift_right(A, er - ea);
+    difference(Q0, A, W);
+    limited<ORDER>(W, cl, cr);
+    o.s[0] = to_double(al + bl, ea - 1);
+    o.s[1] = to_double(ar + br, ea - 1);
+    o.d[0] = to_double(bl - al, ea - 1);
+    o.d[1] = to_double(br - ar, ea - 1);
+    o.w3[0] = to_double(tl, es);
+    o.w3[1] = to_double(tr, es);
+    const int k = er + 1 - ea < 63 ? er + 1 - ea : 63;  // (al + bl is twice w1 + w4: one exponent lower)
+    o.r[0] = to_double(cl + ((al + bl) >> k), er);
+    o.r[1] = to_double(cr + ((ar + br) >> k), er);
+    o.ok = ea <= kExpMax && es <= kExpMax && er <= kExpMax && e[3] <= kExpMax;
+}
+
 // 1/2 (F(f_L) + F(f_R)) at the face after cell j of one flux component, the
 // symmetric 10-point stencil of Eq. flux-full and its mirror over split values
 // at cells j-4 .. j+5 (weights / 1680; order 4: Eq. fourth, / 2880), exact up to

@@ -1,23 +1,25 @@
-// The FP64 MEG7-prim tile: the phases of stage_tile (stage_kernel.cuh) with
+// The FP64 tile: the phases of stage_tile (stage_kernel.cuh) with
 // everything linear on the integer pipe. Primitives and cell fluxes are kept
 // in shared memory taken apart (fx::split: 64-bit integer and exponent), so a
 // face's stencils are aligned to their own scale by a shift each; face states
 // (fixed_face.cuh), flux reconstruction and the viscous gradients are integer
 // sums. FP64 arithmetic remains for the primitives, the cell fluxes, the
-// Riemann solver, the viscous flux and the stage update.
+// Riemann solver, the viscous flux and the stage update. With CONS (MEG7-cons)
+// the planes taken apart are the conservative variables, and the primitives of
+// the cells beside faces are kept as they are.
 #pragma once
 
 #include "stage_kernel.cuh"
 
 namespace gbr {
 
-template <int BX, int BY, bool VISC>
+template <int BX, int BY, bool VISC, bool CONS = false>
 struct FixedLayout {
     using G = TileLayout<BX, BY, VISC>;  // index ranges
     typedef long long i64;
     static constexpr int NU = G::NU, NFX = G::NFX, NFY = G::NFY;
     static constexpr size_t up(size_t b) { return (b + 127) / 128 * 128; }
-    static constexpr size_t oM = 0;                                          // primitives: integers [4][NU]
+    static constexpr size_t oM = 0;                                          // reconstructed variables: integers [4][NU]
     static constexpr size_t oFX = oM + sizeof(i64) * 4 * NU;                 // x fluxes [4][NFX]
     static constexpr size_t oFY = oFX + sizeof(i64) * 4 * NFX;               // y fluxes [4][NFY]
     // The FP64 tile + halo lands here; viscous gradients and face fluxes, all
@@ -27,7 +29,9 @@ struct FixedLayout {
     static constexpr size_t oHX = oGY + (VISC ? sizeof(double) * 4 * G::NGY : 0);
     static constexpr size_t oHY = oHX + sizeof(double) * 4 * G::NHX;
     static constexpr size_t oH1 = oHY + sizeof(double) * 4 * G::NHY, oR1 = oRaw + sizeof(double) * 4 * NU;
-    static constexpr size_t oR = oH1 > oR1 ? oH1 : oR1;                      // densities in FP32 [NU]
+    static constexpr size_t oW = oH1 > oR1 ? oH1 : oR1;                      // CONS: u, v, p of cells [5, B + 7) [3][NW]
+    static constexpr int WW = BX + 2, NW = WW * (BY + 2);
+    static constexpr size_t oR = oW + (CONS ? sizeof(double) * 3 * NW : 0);  // densities in FP32 [NU]
     static constexpr size_t oE = oR + sizeof(float) * NU;                    // exponents of the integers above
     static constexpr size_t oEX = oE + sizeof(short) * 4 * NU;
     static constexpr size_t oEY = oEX + sizeof(short) * 4 * NFX;
@@ -59,13 +63,13 @@ __device__ __forceinline__ bool trouble_filtered(const float* r, int st, F exact
     return exact();  // (also where a density overflows FP32)
 }
 
-template <int BX, int BY, int NT, bool VISC, int ORDER, bool TMA>
+template <int BX, int BY, int NT, bool VISC, int ORDER, bool TMA, bool CONS = false>
 __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, const int ty0, unsigned char* smem,
                                            const CUtensorMap* tmap = nullptr)
 {
     typedef long long i64;
     typedef unsigned short u16;
-    using F = FixedLayout<BX, BY, VISC>;
+    using F = FixedLayout<BX, BY, VISC, CONS>;
     using L = typename F::G;
     using X = typename L::template Cross<0>;  // the staged cells
     constexpr int RW = L::RW, NU = L::NU, V = L::V;
@@ -76,6 +80,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     double* const sGY = reinterpret_cast<double*>(smem + F::oGY);
     double* const sHX = reinterpret_cast<double*>(smem + F::oHX);
     double* const sHY = reinterpret_cast<double*>(smem + F::oHY);
+    double* const sW = reinterpret_cast<double*>(smem + F::oW);
     float* const sR = reinterpret_cast<float*>(smem + F::oR);
     u16* const sE = reinterpret_cast<u16*>(smem + F::oE);
     u16* const sEX = reinterpret_cast<u16*>(smem + F::oEX);
@@ -100,10 +105,21 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         [&](int idx, double q0, double q1, double q2, double q3) {
             double w[4];
             prims_of(q0, q1, q2, q3, ph.gm1, w[0], w[1], w[2], w[3]);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) fx::split(w[m], sM[m * NU + idx], sE[m * NU + idx]);
-            sR[idx] = f64_to_f32_rn(w[0]);
             const int ry = idx / RW, rx = idx - ry * RW;
+            if constexpr (CONS) {
+                const double q[4] = {q0, q1, q2, q3};
+#pragma unroll
+                for (int m = 0; m < 4; ++m) fx::split(q[m], sM[m * NU + idx], sE[m * NU + idx]);
+                if (ry >= 5 && ry < BY + 7 && rx >= 5 && rx < BX + 7) {
+                    const int c = (ry - 5) * F::WW + rx - 5;
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) sW[m * F::NW + c] = w[m + 1];
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) fx::split(w[m], sM[m * NU + idx], sE[m * NU + idx]);
+            }
+            sR[idx] = f64_to_f32_rn(w[0]);
             const double ep = q3 + w[3];
             if (ry >= 6 && ry < 6 + BY && rx >= 1 && rx < BX + 11) {
                 const int f = (ry - 6) * L::FXW + (rx - 1);
@@ -178,9 +194,20 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
 
         // Primitives (rho, un, ut, p) of the face's two cells
         double u0[4], u1[4];
-        auto cell = [&](int m, int o) {
-            const int at = (m == 1 ? pn : m == 2 ? 3 - pn : m) * NU + c + o;
+        auto plane = [&](int m) { return m == 1 ? pn : m == 2 ? 3 - pn : m; };
+        const int cw = (fr + (xf ? 1 : 0)) * F::WW + fc + (xf ? 0 : 1), sw = xf ? 1 : F::WW;
+        auto cell = [&](int m, int o) {  // variable m of the cell before (o = 0) or after (su) the face
+            if (CONS && m > 0) return sW[(plane(m) - 1) * F::NW + cw + (o ? sw : 0)];
+            const int at = plane(m) * NU + c + o;
             return fx::unsplit(sM[at], sE[at]);
+        };
+        auto load = [&](int m, fx::Stencil& x) {
+            const int at = plane(m) * NU + c;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                x.m[k] = sM[at + (k - 5) * su];
+                x.e[k] = sE[at + (k - 5) * su];
+            }
         };
         u0[0] = cell(0, 0);
         u1[0] = cell(0, su);
@@ -193,28 +220,64 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         const double rb = u0[0] + u1[0], gp = ph.gamma * (u0[3] + u1[3]), xx = rmul(gp, rb);
         const double y = fx::rsqrt(xx);
         const double icb = rmul(rb, y), ic2 = rmul(icb, icb);
-        fx::FaceStates s;
-        fx::face_states<ORDER>(
-            [&](int m, fx::Stencil& x) {
-                const int at = (m == 1 ? pn : m == 2 ? 3 - pn : m) * NU + c;
+        double rL, unL, utL, pL, rR, unR, utR, pR;
+        bool ok;
+        if constexpr (!CONS) {
+            fx::FaceStates s;
+            fx::face_states<ORDER>(load, y, rmul(xx, y), ic2, s);
+            rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
+            rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
+            ok = s.ok;
+        } else {
+            u0[1] = cell(1, 0);
+            u1[1] = cell(1, su);
+            u0[2] = cell(2, 0);
+            u1[2] = cell(2, su);
+            const double ub = 0.5 * (u0[1] + u1[1]), vb = 0.5 * (u0[2] + u1[2]), cb = rmul(gp, y);
+            fx::ConsCoefs C;
+            C.b1 = rmul(ph.gm1, ic2);
+            C.b1u = rmul(C.b1, ub);
+            C.b1v = rmul(C.b1, vb);
+            C.b2 = rmul(0.5, rfma(C.b1u, ub, rmul(C.b1v, vb)));
+            C.uc = rmul(ub, icb);
+            C.ic = icb;
+            C.v = vb;
+            fx::ConsStates s;
+            fx::cons_states<ORDER>(
+                load,
+                [&](int m) {
+                    const int at = plane(m) * NU + c;
+                    int e = fx::kExpMin;
 #pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    x.m[k] = sM[at + (k - 5) * su];
-                    x.e[k] = sE[at + (k - 5) * su];
-                }
-            },
-            y, rmul(xx, y), ic2, s);
-        double rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
-        double rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
+                    for (int k = -5; k <= 6; ++k) e = max(e, (int)sE[at + k * su]);
+                    return e;
+                },
+                C, s);
+            ok = s.ok;
+            // Back with the right eigenvectors, to primitives: rho un = u rho
+            // + c d, rho ut = v rho + w3, so un = u + a, ut = v + b with a =
+            // c d / rho, b = w3 / rho, and E - rho (un^2 + ut^2) / 2 =
+            // c^2 s / (gamma - 1) - (c d a + w3 b) / 2.
+            const double c2 = rmul(cb, cb), hg = -0.5 * ph.gm1;
+            auto back = [&](int k, double& r, double& un, double& ut, double& p) {
+                r = s.r[k];
+                const double ir = fx::rcp(r), cd = rmul(cb, s.d[k]), a = rmul(cd, ir), b = rmul(s.w3[k], ir);
+                un = ub + a;
+                ut = vb + b;
+                p = rfma(hg, rfma(cd, a, rmul(s.w3[k], b)), rmul(c2, s.s[k]));
+            };
+            back(0, rL, unL, utL, pL);
+            back(1, rR, unR, utR, pR);
+        }
         // positivity fallback: a face state with rho <= 0 or p <= 0 (or from a
         // refused stencil) takes the adjacent cell's state
-        if (!(s.ok && tpositive(rL) && tpositive(pL))) {
+        if (!(ok && tpositive(rL) && tpositive(pL))) {
             rL = u0[0];
             unL = cell(1, 0);
             utL = cell(2, 0);
             pL = u0[3];
         }
-        if (!(s.ok && tpositive(rR) && tpositive(pR))) {
+        if (!(ok && tpositive(rR) && tpositive(pR))) {
             rR = u1[0];
             unR = cell(1, su);
             utR = cell(2, su);
@@ -247,10 +310,12 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         double out[4];
         hllc_flux(ph, !trouble, Fs, rL, unL, utL, pL, rR, unR, utR, pR, out);
         if constexpr (VISC) {
-            u0[1] = cell(1, 0);
-            u1[1] = cell(1, su);
-            u0[2] = cell(2, 0);
-            u1[2] = cell(2, su);
+            if constexpr (!CONS) {
+                u0[1] = cell(1, 0);
+                u1[1] = cell(1, su);
+                u0[2] = cell(2, 0);
+                u1[2] = cell(2, su);
+            }
             FaceIn<double> in;
             // gradients along the face normal at the cell before the face, and
             // the tangential derivatives of un and ut
@@ -265,7 +330,8 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             in.tun = gt + pn * nt;
             in.tut = gt + (3 - pn) * nt;
             in.stq = xf ? 1 : L::GXW;
-            viscous_flux<double, false>(in, u0, u1, ph, xf ? inv_dx : inv_dy, xf ? inv_dy : inv_dx, out);
+            in.tr0 = gt;
+            viscous_flux<double, CONS>(in, u0, u1, ph, xf ? inv_dx : inv_dy, xf ? inv_dy : inv_dx, out);
         }
         if (xf) {
 #pragma unroll
@@ -289,20 +355,20 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     finish_tile<double, BX, BY, NT>(P, ph, inv_dx, inv_dy, tx0, ty0, sHX, sHY);
 }
 
-// One CTA per tile, two CTAs per SM.
-template <int BX, int BY, int NT, bool VISC, int ORDER>
-__global__ void __launch_bounds__(NT, 2) fixed_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
+// One CTA per tile, two CTAs per SM (viscous MEG7-cons: one, by shared memory).
+template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS>
+__global__ void __launch_bounds__(NT, CONS && VISC ? 1 : 2) fixed_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    fixed_tile<BX, BY, NT, VISC, ORDER, true>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
+    fixed_tile<BX, BY, NT, VISC, ORDER, true, CONS>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
 }
 
-template <int BX, int BY, int NT, bool VISC, int ORDER>
+template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS = false>
 cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
 {
-    using F = FixedLayout<BX, BY, VISC>;
+    using F = FixedLayout<BX, BY, VISC, CONS>;
     static PerDevice<int> configured;  // the shared-memory limit is raised once per device
-    auto kern = fixed_kernel<BX, BY, NT, VISC, ORDER>;
+    auto kern = fixed_kernel<BX, BY, NT, VISC, ORDER, CONS>;
     int ok = 0;
     cudaError_t e = configured.get(&ok, [&](int* v) {
         *v = 1;

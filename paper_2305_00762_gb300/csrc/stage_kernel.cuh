@@ -8,9 +8,11 @@
 // flux), differences the face fluxes into the residual and applies the stage
 // update in FP64. References are to arXiv:2305.00762.
 //
-// T is the arithmetic type of the stencil, reconstruction and flux work
-// (double, or float for the FP32 form); the state, the stage combination and
-// the positivity check are always FP64.
+// T is the arithmetic type of the stencil, reconstruction and flux work: float
+// here (the FP32 form); the FP64 form runs the same phases on the integer pipe
+// (fixed_stage.cuh) and shares the staging, the Riemann solver's frame, the
+// viscous flux and the stage update. The state, the stage combination and the
+// positivity check are always FP64.
 #pragma once
 
 #include <cuda.h>
@@ -25,7 +27,7 @@
 
 namespace gbr {
 
-template <int BX, int BY, bool VISC, bool CONS = false, bool FLUX0 = false>
+template <int BX, int BY, bool VISC, bool CONS = false>
 struct TileLayout {
     static constexpr int V = VISC ? 1 : 0;
     static constexpr int RW = BX + 12, RH = BY + 12;  // staged region (tile + halo)
@@ -70,16 +72,12 @@ struct TileLayout {
 
     static constexpr int NF = NHX + NHY;  // faces of the tile
 
-    // FLUX0: the cell fluxes are written in phase 0, from the staged
-    // conservative values; their arrays then come before the gradients, so
-    // that the TMA landing area (at the gradients, over the face fluxes) does
-    // not overlap them.
     static constexpr int oU = 0;
-    static constexpr int oGX = FLUX0 ? oU + 4 * NU + 4 * (NFX + NFY) : oU + 4 * NU;
+    static constexpr int oGX = oU + 4 * NU;
     static constexpr int oGY = oGX + 4 * NGX;
-    static constexpr int oFX = FLUX0 ? oU + 4 * NU : oGY + 4 * NGY;
+    static constexpr int oFX = oGY + 4 * NGY;
     static constexpr int oFY = oFX + 4 * NFX;
-    static constexpr int oHX = FLUX0 ? oGY + 4 * NGY : oFY + 4 * NFY;
+    static constexpr int oHX = oFY + 4 * NFY;
     static constexpr int oHY = oHX + 4 * NHX;
     static constexpr int oQc = oHY + 4 * NHY;         // conservative values (MEG7-cons)
     static constexpr int oEnd = oQc + (CONS ? 4 * NU : 0);
@@ -99,9 +97,9 @@ struct TileLayout {
     }
 
     // TMA staging: the FP64 conservative tile + halo lands as [4][RH][RW]
-    // doubles on top of the gradient, face-flux and (without FLUX0)
-    // cell-flux arrays, all first written after phase 0, and below the
-    // MEG7-cons copy that phase 0 fills.
+    // doubles on top of the gradient, face-flux and cell-flux arrays, all
+    // first written after phase 0, and below the MEG7-cons copy that phase 0
+    // fills.
     static constexpr size_t kRawBytes = sizeof(double) * 4 * (size_t)NU;
     template <typename T>
     static constexpr size_t raw_offset() { return sizeof(T) * (size_t)oGX; }
@@ -135,14 +133,13 @@ __device__ __forceinline__ double thalfabs(double x)
 __device__ __forceinline__ float tabs(float x) { return fabsf(x); }
 
 // FP64 comparisons on the integer pipe. GB300 runs every FP64 instruction,
-// compares and min/max included, on a unit that retires 2 thread-operations
-// per SM per clock, against 64 for the 32-bit integer pipe; the MP limiter is
-// mostly comparisons. For doubles that are not NaN, the signed 64-bit order of
-// ordkey(x) is the order of x (with -0 just below +0), ordkey is its own
-// inverse, and |x| orders as the bit pattern of x with the sign cleared.
-// Values chosen this way equal those of the floating-point comparisons; only
-// the sign of a zero result may differ, which no later sum or product turns
-// into a different non-zero value.
+// compares and min/max included, at one warp instruction per 19 clocks and SM,
+// against two per clock for 32-bit integers. For doubles that are not NaN, the
+// signed 64-bit order of ordkey(x) is the order of x (with -0 just below +0),
+// and |x| orders as the bit pattern of x with the sign cleared. Values chosen
+// this way equal those of the floating-point comparisons; only the sign of a
+// zero result may differ, which no later sum or product turns into a different
+// non-zero value.
 __device__ __forceinline__ long long ordkey(double x)
 {
     const long long b = __double_as_longlong(x);
@@ -152,29 +149,18 @@ __device__ __forceinline__ double tmin(double a, double b) { return ordkey(a) < 
 __device__ __forceinline__ double tmax(double a, double b) { return ordkey(a) > ordkey(b) ? a : b; }
 
 // Eq. alpha: minmod(a, b) = 1/2 (sign a + sign b) min(|a|, |b|): the operand
-// of smaller magnitude when the signs agree, else 0. FP32: that is the
-// median of a, b and 0, four min / max instructions; FP64: the sign test on
-// the bits and the magnitudes compared as integers. Only the sign of a zero
-// result may differ from the formula's.
+// of smaller magnitude when the signs agree, else 0: the median of a, b and
+// 0, four min / max instructions. Only the sign of a zero result may differ
+// from the formula's.
 __device__ __forceinline__ float minmod(float a, float b)
 {
     return fmaxf(fminf(a, b), fminf(fmaxf(a, b), 0.f));
 }
-__device__ __forceinline__ double minmod(double a, double b)
-{
-    const long long ba = __double_as_longlong(a), bb = __double_as_longlong(b);
-    const unsigned long long ma = (unsigned long long)ba & 0x7FFFFFFFFFFFFFFFULL;
-    const unsigned long long mb = (unsigned long long)bb & 0x7FFFFFFFFFFFFFFFULL;
-    const double r = ma <= mb ? a : b;  // the smaller magnitude
-    return (ba ^ bb) < 0 ? 0.0 : r;     // opposite signs
-}
-
 // The MP test's comparison x <= thr (Eq. mp5Condition: 1e-40 for a field in
 // the paper's scaling, 1e-40 s^2 for one carried scaled by s; grb_mp tests
 // a multiple of the product and scales thr alike).
 template <typename T>
 __device__ __forceinline__ bool mp_accept(T x, T thr) { return x <= thr; }
-__device__ __forceinline__ bool mp_accept(double x, double thr) { return ordkey(x) <= ordkey(thr); }
 
 // The last step of Eq. mp-procedure from Phi_j, Phi_{j+1}, Phi^MD, Phi^UL,
 // Phi^LC and the GRB value pl. Phi^min = max(min(Phi_j, Phi_{j+1}, MD),
@@ -212,15 +198,6 @@ __device__ __forceinline__ float mp_clamp(float p2, float p3, float md, float ul
     const float pmax = fminf(fmax3(p2, p3, md), fmax3(p2, ul, lc));
     return fminf(fmaxf(pl, pmin), pmax);
 }
-__device__ __forceinline__ double mp_clamp(double p2, double p3, double md, double ul, double lc, double pl)
-{
-    const long long k2 = ordkey(p2), k3 = ordkey(p3), km = ordkey(md), ku = ordkey(ul), kl = ordkey(lc);
-    const long long kmin = min(k2, max(min(k3, km), min(ku, kl)));
-    const long long kmax = max(k2, min(max(k3, km), max(ku, kl)));
-    const long long k = min(max(ordkey(pl), kmin), kmax);
-    return __longlong_as_double(k ^ ((k >> 63) & 0x7FFFFFFFFFFFFFFFLL));
-}
-
 // Explicitly rounded products and fused multiply-adds. Per-cell work that is
 // done once along x and once along y sits at two call sites, where the
 // compiler could contract a*b + c into an FMA at one and not at the other.
@@ -401,41 +378,17 @@ __device__ __forceinline__ T grb_mp(T pj, T Dm1, T Dp1s, T s1, T S2, T dj, T dd,
     return rfma(T(1.0 / kGrbD), D, pj);
 }
 
-// Eq. mp-procedure: the MP-limited value given the GRB value pl. The
-// curvature d_j = 2 (Phi_{j-1} - 2 Phi_j + Phi_{j+1}) - (Phi'_{j+1} -
-// Phi'_{j-1})/2 can come from the sums the GRB value was formed with: s1 =
-// Dm1 + Dp1 and dd = Phi'_{j-1} - Phi'_{j+1}.
-// Its products are explicitly rounded: the packed path of meg7_pair inlines
-// it and the per-lane path runs the same arithmetic in mp_limit_pair, and
-// the two must round alike.
-// The curvature d_{j+1} is the other side's d_j (the right value at the same
-// face is centred on cell j+1, mirrored, and the curvature is unchanged by
-// the mirror): it comes from that side's sums s1o, ddo.
-// The curvatures are carried as 2 kGrad d (one operation fewer each, with
-// the gradients at their carried scale; minmod(s a, s b) = s minmod(a, b)
+// Eq. mp-procedure for both values of one face and field (w = Phi_{j-2..j+3}, e
+// their gradients; aL, aR, s1L, s1R, ddL, ddR as formed for the GRB values):
+// the MP-limited values given the GRB values vl, vr. The curvature d_j =
+// 2 (Phi_{j-1} - 2 Phi_j + Phi_{j+1}) - (Phi'_{j+1} - Phi'_{j-1})/2 comes from
+// the sums the GRB value was formed with, s1 = Dm1 + Dp1 and dd = Phi'_{j-1} -
+// Phi'_{j+1}; curvatures are carried as 2 kGrad d (one operation fewer each,
+// with the gradients at their carried scale; minmod(s a, s b) = s minmod(a, b)
 // for s > 0), so Phi^MD and Phi^LC take the factors 1/(2 kGrad) and
-// 2/(3 kGrad).
-template <typename T>
-__device__ __forceinline__ T mp_limit(const T* p, const T* d, T pl, T s1, T dd, T s1o, T ddo)
-{
-    const T dm1 = rfma(T(4 * kGrad), rfma(T(-2), p[1], p[2]) + p[0], d[0] - d[2]);
-    // (d_j and d_{j+1} from the sums: one FMA each)
-    const T dj = rfma(T(4 * kGrad), s1, dd);
-    const T dp1 = rfma(T(4 * kGrad), s1o, ddo);
-    const T md = rmul(T(0.5), rfma(T(-0.5 / kGrad), minmod(dj, dp1), p[2] + p[3]));
-    const T Dm1 = p[1] - p[2];
-    const T ul = rfma(T(-7), Dm1, p[2]);
-    const T lc = rfma(T(2.0 / (3.0 * kGrad)), minmod(dj, dm1), rfma(T(-0.5), Dm1, p[2]));
-    return mp_clamp(p[2], p[3], md, ul, lc, pl);
-}
-
-// mp_limit for both values of one face and field, where a lane limits its
-// own left and right values (w = Phi_{j-2..j+3}, e their gradients; aL, aR,
-// s1L, s1R, ddL, ddR as formed for the GRB values). The two sides share
-// Phi^MD: the right value's stencil is the left's mirrored about the face,
-// so Phi_j + Phi_{j+1} and minmod(d_j, d_{j+1}) are the same for both (the
-// sum and minmod are symmetric in their operands), and each side's d_{j+1}
-// is the other side's d_j. Every value is bitwise that of mp_limit.
+// 2/(3 kGrad). The two sides share Phi^MD: the right value's stencil is the
+// left's mirrored about the face, so Phi_j + Phi_{j+1} and minmod(d_j, d_{j+1})
+// are the same for both, and each side's d_{j+1} is the other side's d_j.
 template <typename T>
 __device__ __forceinline__ void mp_limit_pair(const T (&w)[6], const T (&e)[6], T aL, T aR, T s1L, T s1R, T ddL,
                                               T ddR, T& vl, T& vr, bool needL, bool needR)
@@ -451,35 +404,13 @@ __device__ __forceinline__ void mp_limit_pair(const T (&w)[6], const T (&e)[6], 
     if (needR) vr = mp_clamp(w[3], w[2], md, ulR, lcR, vr);
 }
 
-// Position of the n-th (0-based) set bit of m; m has more than n set bits.
-__device__ __forceinline__ int nth_set_bit(unsigned m, int n)
-{
-    int pos = 0;
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
-        const int c = __popc(m & ((1u << s) - 1u));
-        if (n >= c) {
-            n -= c;
-            m >>= s;
-            pos += s;
-        }
-    }
-    return pos;
-}
-
 // MEG7 left and right values at face j+1/2 of one characteristic field, from
 // its values w[0..5] and gradients e[0..5] at cells j-2..j+3: the left value
 // from cells j-2..j+2, the right one from the stencil mirrored about the face
 // (cell j+1-k in the place of cell j+k, gradients with their sign changed).
 //
 // Where the MP test fails (a third of the values or more in developed flow),
-// the limiter runs; with one face per lane nearly every warp has such a lane,
-// so per lane the limiter would cost the whole warp every time. In FP64, on a
-// warp whose left and right failures together number at most 32, the failing
-// values are packed onto the warp's lanes instead (each lane fetches one
-// stencil by shuffle), limited in one pass and returned by shuffle. Every
-// lane of the warp must call this together. The arithmetic of each value is
-// unchanged, so the result is the same.
+// the limiter runs.
 template <typename T>
 __device__ __forceinline__ void meg7_pair(const GrbCoef<T>& C, const T (&w)[6], const T (&e)[6], T& vl, T& vr,
                                           T thr = T(1e-40 * kMP))
@@ -494,42 +425,6 @@ __device__ __forceinline__ void meg7_pair(const GrbCoef<T>& C, const T (&w)[6], 
     const T bs = T(kGrbD) * b;
     vl = grb_mp(w[2], aL, bs, s1L, rfma(T(-2), w[2], w[0] + w[4]), e[2], ddL, needL, C, thr);
     vr = grb_mp(w[3], aR, -bs, s1R, rfma(T(-2), w[3], w[5] + w[1]), -e[3], ddR, needR, C, thr);
-    if constexpr (sizeof(T) == 8) {
-        const unsigned mL = __ballot_sync(0xffffffffu, needL), mR = __ballot_sync(0xffffffffu, needR);
-        const int nL = __popc(mL), nR = __popc(mR);
-        if (nL + nR <= 32) {  // warp-uniform
-            const int lane = threadIdx.x & 31;
-            const bool isR = lane >= nL;
-            const bool act = lane < nL + nR;
-            const int src = !act ? lane : (isR ? nth_set_bit(mR, lane - nL) : nth_set_bit(mL, lane));
-            T W[6], E[6];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                W[k] = __shfl_sync(0xffffffffu, w[k], src);
-                E[k] = __shfl_sync(0xffffffffu, e[k], src);
-            }
-            // (the source lane's left and right values both travel; the
-            // receiving lane picks the side it limits)
-            const T gl = __shfl_sync(0xffffffffu, vl, src), gr = __shfl_sync(0xffffffffu, vr, src);
-            const T sl = __shfl_sync(0xffffffffu, s1L, src), sr = __shfl_sync(0xffffffffu, s1R, src);
-            const T dl = __shfl_sync(0xffffffffu, ddL, src), dr = __shfl_sync(0xffffffffu, ddR, src);
-            const T g = isR ? gr : gl, s1 = isR ? sr : sl, dd = isR ? dr : dl;
-            const T s1o = isR ? sl : sr, ddo = isR ? dl : dr;
-            T p[5], d[5];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                p[k] = isR ? W[5 - k] : W[k];
-                d[k] = isR ? -E[5 - k] : E[k];
-            }
-            const T lim = mp_limit(p, d, g, s1, dd, s1o, ddo);
-            const unsigned below = (1u << lane) - 1u;
-            const T rl = __shfl_sync(0xffffffffu, lim, __popc(mL & below));
-            const T rr = __shfl_sync(0xffffffffu, lim, (nL + __popc(mR & below)) & 31);
-            if (needL) vl = rl;
-            if (needR) vr = rr;
-            return;
-        }
-    }
     if (needL || needR) mp_limit_pair(w, e, aL, aR, s1L, s1R, ddL, ddR, vl, vr, needL, needR);
 }
 
@@ -978,15 +873,14 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
     if (smooth) {
 #pragma unroll
         for (int m = 0; m < 4; ++m) Fc[m] = recon_mean(in.f[m], in.sf, coef);
-    } else if constexpr (sizeof(T) == 4) {
+    } else {
         Fc[0] = T(0.5) * (QL[1] + QR[1]);
         Fc[1] = T(0.5) * ((QL[1] * unL + pL) + (QR[1] * unR + pR));
         Fc[2] = T(0.5) * (QL[1] * utL + QR[1] * utR);
         Fc[3] = T(0.5) * (unL * (EL + pL) + unR * (ER + pR));
     }
 
-    if constexpr (sizeof(T) == 8) hllc_flux(P, smooth, Fc, rL, unL, utL, pL, rR, unR, utR, pR, out);
-    else hllc_flux(P, Fc, QL, QR, rL, unL, utL, pL, EL, rR, unR, utR, pR, ER, out);
+    hllc_flux(P, Fc, QL, QR, rL, unL, utL, pL, EL, rR, unR, utR, pR, ER, out);
     if constexpr (VISC) {
         T u0[4], u1[4];
 #pragma unroll
@@ -1503,10 +1397,7 @@ template <typename T, int BX, int BY, int NT, bool VISC, int LEARNED = 0, int OR
 __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, const int ty0,
                                            unsigned char* smem_raw, const CUtensorMap* tmap = nullptr)
 {
-    // FP64: the cell fluxes come from the staged conservative values in
-    // phase 0 (FLUX0)
-    constexpr bool FLUX0 = sizeof(T) == 8;
-    using L = TileLayout<BX, BY, VISC, CONS, FLUX0>;
+    using L = TileLayout<BX, BY, VISC, CONS>;
     using X = typename L::template Cross<LEARNED>;  // the staged cells
     T* const sm = reinterpret_cast<T*>(smem_raw);
     T* const sU = sm + L::oU;
@@ -1543,25 +1434,6 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
         sU[NU + idx] = u;
         sU[2 * NU + idx] = v;
         sU[3 * NU + idx] = p;
-        if constexpr (FLUX0) {
-            // cell fluxes F^c = (rho u, rho u u + p, rho u v, u (E + p)) and
-            // G^c (Sec. 1) with rho u, rho v and E taken from the state
-            const int ry = idx / RW, rx = idx - ry * RW;
-            if (ry >= 6 && ry < 6 + BY && rx >= 1 && rx < BX + 11) {
-                const int f = (ry - 6) * L::FXW + (rx - 1);
-                sFX[f] = q1;
-                sFX[L::NFX + f] = rfma(T(q1), u, p);
-                sFX[2 * L::NFX + f] = T(q1) * v;
-                sFX[3 * L::NFX + f] = u * (T(q3) + p);
-            }
-            if (ry >= 1 && ry < BY + 11 && rx >= 6 && rx < BX + 6) {
-                const int f = (ry - 1) * BX + (rx - 6);
-                sFY[f] = q2;
-                sFY[L::NFY + f] = T(q2) * u;
-                sFY[2 * L::NFY + f] = rfma(T(q2), v, p);
-                sFY[3 * L::NFY + f] = v * (T(q3) + p);
-            }
-        }
         if constexpr (CONS) {
             sQc[idx] = r;
             sQc[NU + idx] = from_f64<T>(q1);
@@ -1630,7 +1502,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
             sPY[idx] = trouble_cell(sU + (a + 3) * RW + (b + 6), RW) ? 1 : 0;
         }
     }
-    for (int idx = tid; idx < (FLUX0 ? 0 : L::NFX); idx += NT) {  // cell x-fluxes F^c (Sec. 1)
+    for (int idx = tid; idx < L::NFX; idx += NT) {  // cell x-fluxes F^c (Sec. 1)
         const int a = idx / L::FXW, b = idx - a * L::FXW;
         const int c = (a + 6) * RW + (b + 1);
         const T r = sU[c], u = sU[NU + c], v = sU[2 * NU + c], p = sU[3 * NU + c];
@@ -1641,7 +1513,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
         sFX[2 * L::NFX + idx] = ru * v;
         sFX[3 * L::NFX + idx] = u * (E + p);
     }
-    for (int idx = tid; idx < (FLUX0 ? 0 : L::NFY); idx += NT) {  // cell y-fluxes G^c
+    for (int idx = tid; idx < L::NFY; idx += NT) {  // cell y-fluxes G^c
         const int a = idx / BX, b = idx - a * BX;
         const int c = (a + 1) * RW + (b + 6);
         const T r = sU[c], u = sU[NU + c], v = sU[2 * NU + c], p = sU[3 * NU + c];
@@ -1829,7 +1701,7 @@ __global__ void __launch_bounds__(NT, stage_min_blocks<T, VISC, CONS, LEARNED>()
 template <typename T, int BX, int BY, int NT, bool VISC, int LEARNED = 0, int ORDER = 7, bool CONS = false>
 cudaError_t launch_stage_t(const StageParams& p, cudaStream_t s)
 {
-    using L = TileLayout<BX, BY, VISC, CONS, sizeof(T) == 8>;
+    using L = TileLayout<BX, BY, VISC, CONS>;
     constexpr size_t smem = L::template total_bytes<T, NT, LEARNED != 0>();
     static PerDevice<int> configured;  // the shared-memory limit is raised once per device
     auto kern = stage_kernel<T, BX, BY, NT, VISC, LEARNED, ORDER, CONS>;

@@ -104,6 +104,62 @@ static int run(int mode, int stride)
     std::printf("order %d mode %d: at most %.2f of the tolerance\n", ORDER, mode, worst);
     return 0;
 }
+// MEG7-cons: each functional of A and t carries at most seven truncations
+// (alignment and six products) of one unit, 2^-59 of a scale at most 2^5 times
+// the largest term; the limiter's bounds amplify them to at most 25 units and
+// a returned sum takes two fields, hence 2^-53 |value| + 2^-48 of the largest
+// term (the fields of one product more than cover theirs).
+static int cons(int mode, int stride)
+{
+    std::mt19937_64 g(29 + mode);
+    std::uniform_real_distribution<double> U(-1, 1);
+    for (int it = 0; it < 20000; ++it) {
+        double v[4][12 * 3];
+        const double sc = mode == 2 ? std::pow(10.0, 5 * U(g)) : 1, mach = mode == 3 ? 20 : 1;
+        const double r0 = 1.5 + U(g), p0 = 1.5 + U(g), u0 = mach * U(g), t0 = mach * U(g), amp = std::pow(10.0, -8 * std::fabs(U(g)));
+        const double jump = mode ? 5 * std::fabs(U(g)) : 0;
+        const int at = (int)(g() % 13);
+        for (int k = 0; k < 12; ++k) {
+            const double J = k < at ? jump : 0, r = r0 + J + amp * std::sin(k + r0), p = p0 + 3 * J + 0.3 * amp * U(g);
+            const double n = mode == 4 ? 0 : u0 + 0.2 * J + amp * U(g), t = mode == 4 ? 0 : t0 + amp * U(g);
+            v[0][k * stride] = sc * r, v[1][k * stride] = sc * r * n, v[2][k * stride] = sc * r * t;
+            v[3][k * stride] = sc * (p / 0.4 + 0.5 * r * (n * n + t * t));
+        }
+        const double* u[4] = {v[0] + 5 * stride, v[1] + 5 * stride, v[2] + 5 * stride, v[3] + 5 * stride};
+        const double c2 = 1.4 * p0 / r0, c = std::sqrt(c2);
+        fx::ConsCoefs C;
+        C.b1 = 0.4 / c2, C.b1u = C.b1 * u0, C.b1v = C.b1 * t0, C.b2 = 0.5 * C.b1 * (u0 * u0 + t0 * t0);
+        C.uc = u0 / c, C.ic = 1 / c, C.v = t0;
+        const Planes load{u, stride};
+        fx::ConsStates o;
+        fx::cons_states<7>(load, [&](int m) { fx::Stencil x; load(m, x); return fx::stencil_exponent(x); }, C, o);
+        if (!o.ok) return std::printf("refused\n"), 1;
+        R wl[4], wr[4], big = 0, big2 = 0;  // 2 w1, 2 w4, w2, w3
+        for (int f = 0; f < 4; ++f) {
+            R q[12], e[12], a[5], b[5];
+            for (int k = 0; k < 12; ++k) {
+                const R x0 = v[0][k * stride], x1 = v[1][k * stride], x2 = v[2][k * stride], x3 = v[3][k * stride];
+                const R A = C.b2 * x0 - C.b1u * x1 - C.b1v * x2 + C.b1 * x3, t = C.uc * x0 - C.ic * x1;
+                q[k] = f == 0 ? A + t : f == 1 ? A - t : f == 2 ? x0 - A : x2 - C.v * x0;
+                for (R y : {C.b2 * x0, C.b1u * x1, C.b1v * x2, C.b1 * x3, C.uc * x0, C.ic * x1, x0}) big = fmaxl(big, fabsl(y));
+                big2 = fmaxl(big2, fmaxl(fabsl(x2), fabsl(C.v * x0)));
+            }
+            for (int k = 3; k < 9; ++k) e[k] = (45 * (q[k + 1] - q[k - 1]) - 9 * (q[k + 2] - q[k - 2]) + (q[k + 3] - q[k - 3])) / 60;
+            for (int k = 0; k < 5; ++k) a[k] = q[3 + k], b[k] = e[3 + k];
+            wl[f] = meg(a, b, 7);
+            for (int k = 0; k < 5; ++k) a[k] = q[8 - k], b[k] = -e[8 - k];
+            wr[f] = meg(a, b, 7);
+        }
+        const R ref[8] = {(wl[0] + wl[1]) / 2 + wl[2], (wr[0] + wr[1]) / 2 + wr[2], (wl[0] + wl[1]) / 2, (wr[0] + wr[1]) / 2,
+                          (wl[1] - wl[0]) / 2, (wr[1] - wr[0]) / 2, wl[3], wr[3]};
+        const double got[8] = {o.r[0], o.r[1], o.s[0], o.s[1], o.d[0], o.d[1], o.w3[0], o.w3[1]};
+        for (int k = 0; k < 8; ++k) {
+            const R tol = ldexpl(fabsl(ref[k]), -53) + ldexpl(k < 6 ? big : big2, -48), d = fabsl(ref[k] - (R)got[k]);
+            if (!(d <= tol)) return std::printf("cons mode %d value %d: %g off, %g allowed\n", mode, k, (double)d, (double)tol), 1;
+        }
+    }
+    return 0;
+}
 static int limits()
 {
     // integers round to double and back; infinities, NaN and overflowing scales are refused
@@ -179,6 +235,7 @@ static int sums(int mode)
 int main()
 {
     int bad = limits();
+    for (int mode = 0; mode < 5; ++mode) bad |= cons(mode, 1 + mode % 3);
     for (int mode = 0; mode < 3; ++mode) bad |= sums<7>(mode) | sums<4>(mode);
     for (int mode = 0; mode < 5; ++mode) bad |= run<7>(mode, 1 + mode % 3) | run<4>(mode, 1 + mode % 3);
     return bad;
