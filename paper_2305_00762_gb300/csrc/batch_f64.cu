@@ -4,7 +4,7 @@
 
 namespace gbr {
 
-static const TileShape kShapesF64[] = {{32, 8}, {16, 16}, {64, 4}};
+static const TileShape kShapesF64[] = {{16, 15}, {16, 8}, {32, 8}};
 
 int batch_tile_shapes_f64(const TileShape** shapes)
 {
@@ -16,9 +16,9 @@ cudaError_t launch_batch_stage_f64(int shape, const BatchCase* cases, int ncases
                                    cudaStream_t s, bool per_tile)
 {
     switch (shape) {
-    case 0: return launch_batch_t<double, 32, 8, 256>(cases, ncases, total_tiles, stage, s, nullptr, per_tile);
-    case 1: return launch_batch_t<double, 16, 16, 256>(cases, ncases, total_tiles, stage, s, nullptr, per_tile);
-    default: return launch_batch_t<double, 64, 4, 256>(cases, ncases, total_tiles, stage, s, nullptr, per_tile);
+    case 0: return launch_batch_t<double, 16, 15, 256>(cases, ncases, total_tiles, stage, s, nullptr, per_tile);
+    case 1: return launch_batch_t<double, 16, 8, 288>(cases, ncases, total_tiles, stage, s, nullptr, per_tile);
+    default: return launch_batch_t<double, 32, 8, 288>(cases, ncases, total_tiles, stage, s, nullptr, per_tile);
     }
 }
 

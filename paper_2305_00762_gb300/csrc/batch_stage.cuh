@@ -25,7 +25,7 @@ __device__ __forceinline__ int batch_case_of(const BatchCase* cases, int ncases,
 template <typename T, int BX, int BY, int NT, bool LEARNED>
 constexpr size_t batch_smem()
 {
-    if constexpr (sizeof(T) == 8) return FixedLayout<BX, BY, false>::bytes;
+    if constexpr (sizeof(T) == 8) return FixedLayout<BX, BY, false, false, false>::bytes;
     else return TileLayout<BX, BY, false>::template total_bytes<T, NT, LEARNED>();
 }
 

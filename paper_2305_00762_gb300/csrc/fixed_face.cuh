@@ -8,11 +8,13 @@
 // linear or a comparison, so it is done here on integers, exactly up to the
 // rounding of the projection products.
 //
-// Measured (four-quadrant problem, FP64 step, 3 stages): 1024^2 6.57 -> 3.66
-// ms, 400^2 1.28 -> 0.73 ms; viscous 1280 x 640 6.06 -> 3.93 ms. FP64
-// gradients, projection, GRB and limiter were half of the FP64 instructions
-// of a stage whose FP64 pipe was saturated; they cost the FP64 pipe nothing
-// now.
+// Measured, FP64 step of three stages: with FP64 arithmetic throughout (the FP64
+// pipe saturated) 1024^2 6.57 ms, 400^2 1.28 ms, viscous 1280 x 640 6.06 ms;
+// with the face states here 3.66 / 0.73 / 3.93 ms; with the roots and
+// reciprocals, the primitives, the cell fluxes and their reconstruction on
+// integers too (fixed_math.cuh, fixed_stage.cuh) 1.94 / 0.37 / 2.13 ms. The
+// stage is then bound by the integer pipe and FP64 about alike (54% and 58% of
+// what each can issue), at 16 warps an SM.
 //
 // Scaling. A variable q of one face's stencil (cells j-5 .. j+6) is held as
 // I = q / 2^(e - 1081) with e the largest biased exponent of the stencil, so
@@ -89,14 +91,21 @@ GBR_HD u64 mulhi_u(u64 a, u64 b)
     return (u64)(((unsigned __int128)a * b) >> 64);
 #endif
 }
-// floor(x r / 2^64), x signed, r unsigned
-GBR_HD i64 mulhi(i64 x, u64 r) { return (i64)(mulhi_u((u64)x, r) - ((u64)(x >> 63) & r)); }
+// x r / 2^64, x signed, r < 2^63, less at most four units: three 32 x 32 -> 64
+// products (the low halves' product and the lowest bits of r's halves are
+// dropped) instead of four and the sign's correction.
+GBR_HD i64 mulhi(i64 x, u64 r)
+{
+    const int xh = (int)(x >> 32), rh = (int)(r >> 32);
+    const i64 mid = (i64)xh * (int)((unsigned)r >> 1) + (i64)((u64)(unsigned)x * ((unsigned)rh >> 1));
+    return (i64)xh * rh + (mid >> 31);
+}
 
 GBR_HD int exponent(double x) { return (int)(bits_of(x) >> 52) & 0x7ff; }
 
-// A double taken apart once, where it is produced, so that each of the many
-// stencils that read it only shifts: x = m 2^(e - kOne), |m| < 2^kBits, e the
-// biased exponent (zeros and subnormals: m = 0, e = 1).
+// A value taken apart once, where it is produced, so that each of the many
+// stencils that read it only shifts: x = m 2^(e - kOne), |m| < 2^kBits. For a
+// double, e is its biased exponent (zeros and subnormals: m = 0, e = 1).
 GBR_HD void split(double x, i64& m, unsigned short& e)
 {
     const u64 b = bits_of(x);
@@ -105,17 +114,17 @@ GBR_HD void split(double x, i64& m, unsigned short& e)
     m = ex == 0 ? 0 : (v ^ g) - g;
     e = (unsigned short)(ex == 0 ? 1 : ex);
 }
-GBR_HD double unsplit(i64 m, int e)  // exact
-{
-    const i64 g = m >> 63;
-    const u64 a = (u64)((m ^ g) - g) >> (kBits - 53);
-    return of_bits((((u64)(unsigned)(e - 1) << 52) + a) | ((u64)g & 0x8000000000000000ull));
-}
 // The split value m, ex in units 2^(e - kOne), ex <= e, rounded down.
 GBR_HD i64 aligned(i64 m, int ex, int e)
 {
+#ifdef __CUDA_ARCH__
+    i64 r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(e - ex));  // (a shift past the width counts as the width)
+    return r;
+#else
     const int s = e - ex;
     return m >> (s < 63 ? s : 63);
+#endif
 }
 
 // x 2^(e - kOne) as a double, rounded to nearest; kExpMin <= e <= kExpMax + 64.
@@ -143,6 +152,13 @@ GBR_HD double to_double(i64 x, int e)
     u64 r = ((u64)(unsigned)(e + 63 - kBits - n) << 52) + (t >> 11) + ((t >> 10) & 1u);
     r |= (u64)g & 0x8000000000000000ull;
     return of_bits(h == 0 ? 0ull : r);
+}
+
+// The double nearest to a split value.
+GBR_HD double unsplit(i64 m, int e)
+{
+    const double x = to_double(m, e < kExpMin ? kExpMin : e);
+    return e < kExpMin ? 0.0 : e <= kExpMax ? x : of_bits(0x7ff8000000000000ull);
 }
 
 // Sum of c X over a few X (|X| < 2^62) and small positive integers c, exact.
@@ -310,11 +326,11 @@ GBR_HD i64 mp_clamp(i64 p2, i64 p3, i64 md, i64 ul, i64 lc, i64 pl)
     return r < mx ? r : mx;
 }
 
-// n -> delta = Phi^GRB - Phi_j: 2^10 / 840 = 1 + 184/840; 2^13 / 10080.
+// n -> delta = Phi^GRB - Phi_j: 2^10 / 840 = 1 + 184/840; 2^13 / 10080 = 1 - 1888/10080.
 template <int ORDER>
 GBR_HD i64 grb_delta(i64 n)
 {
-    return ORDER == 4 ? mulhi(n, ratio(8192, 10080)) : n + mulhi(n, ratio(184, 840));
+    return ORDER == 4 ? n - mulhi(n, ratio(1888, 10080)) : n + mulhi(n, ratio(184, 840));
 }
 
 // The MP-limited left and right values (Eqs. grb, mp-procedure) at the face.
@@ -353,15 +369,27 @@ GBR_HD void variable(const Stencil& x, int e, Functionals& f)
     functionals<ORDER>(q, f);
 }
 
-// A positive factor a applied to a variable of scale e, for a result of scale
-// eo: the r of scale(). The product's own scale is e + exponent(a) - 1022,
-// and eo is at least that.
-GBR_HD u64 factor(double a, int e, int eo)
+// A positive number m / 2^63 2^(e - 1023), 2^63 <= m < 2^64, e a biased exponent
+// that may run outside a double's range. Products are rounded down in the last
+// of 63 bits.
+struct Pos {
+    u64 m;
+    int e;
+};
+
+// A factor a applied to a variable of scale e, for a result of scale eo: the r
+// of scale(). The product's own scale is e + a.e - 1022, and eo is at least that.
+GBR_HD u64 factor(const Pos& a, int e, int eo)
 {
-    const u64 m = ((bits_of(a) & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;  // a = m 2^(exponent - 1086)
-    int k = eo - (e + exponent(a) - 1022);
-    k = k < 63 ? k : 63;
-    return k < 63 ? m >> k : 0;
+    const int k = eo - (e + a.e - 1022);
+    return k < 63 ? a.m >> k : 0;
+}
+GBR_HD u64 factor(double a, int e, int eo)  // of |a|
+{
+    Pos p;
+    p.m = (bits_of(a) << 11) | 0x8000000000000000ull;
+    p.e = exponent(a);
+    return factor(p, e, eo);
 }
 
 // The face states (L, R) back in primitives.
@@ -375,7 +403,7 @@ struct FaceStates {
 // w2 = rho - p / c^2; w1, w4 = p -/+ rho c un; shear w3 = ut. Back: p =
 // (w1 + w4) / 2, un = (w4 - w1) y, rho = w2 + p / c^2.
 template <int ORDER, typename F>
-GBR_HD void face_states(F load, double y, double rc2, double ic2, FaceStates& o)
+GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, FaceStates& o)
 {
     Functionals P;
     i64 sl, sr;
@@ -389,7 +417,7 @@ GBR_HD void face_states(F load, double y, double rc2, double ic2, FaceStates& o)
     {  // field 2 (entropy): rho - p / c^2
         Stencil x;
         load(0, x);
-        const int er = stencil_exponent(x), eprod = ep + exponent(ic2) - 1022;
+        const int er = stencil_exponent(x), eprod = ep + ic2.e - 1022;
         es = (er > eprod ? er : eprod) + 1;
         Functionals R, S;
         scale(P, factor(ic2, ep, es), S);
@@ -400,7 +428,7 @@ GBR_HD void face_states(F load, double y, double rc2, double ic2, FaceStates& o)
     {  // fields 1 and 4 (u -/+ c), carried as p -/+ rho c un
         Stencil x;
         load(1, x);
-        const int eu = stencil_exponent(x), eprod = eu - 1 + exponent(rc2) - 1022;  // (half of rc2)
+        const int eu = stencil_exponent(x), eprod = eu - 1 + rc2.e - 1022;  // (half of rc2)
         ew = (ep > eprod ? ep : eprod) + 1;
         Functionals U, W;
         variable<ORDER>(x, eu, U);
@@ -411,16 +439,15 @@ GBR_HD void face_states(F load, double y, double rc2, double ic2, FaceStates& o)
         limited<ORDER>(W, ml, mr);
         sum(P, U, W);
         limited<ORDER>(W, pl, pr);
-        const u64 fy = factor(y, 0, exponent(y) - 1022);  // (the whole mantissa)
-        const int ev = ew + exponent(y) - 1022;
+        const int ev = ew + y.e - 1021;  // (half the mantissa: a bit to spare)
         const bool some = ev >= kExpMin;  // smaller velocities count as zero
-        o.un[0] = to_double(some ? mulhi(pl - ml, fy) : 0, some ? ev : kExpMin);
-        o.un[1] = to_double(some ? mulhi(pr - mr, fy) : 0, some ? ev : kExpMin);
+        o.un[0] = to_double(some ? mulhi(pl - ml, y.m >> 1) : 0, some ? ev : kExpMin);
+        o.un[1] = to_double(some ? mulhi(pr - mr, y.m >> 1) : 0, some ? ev : kExpMin);
         pl += ml;  // 2 p: p in units one exponent lower
         pr += mr;
         o.p[0] = to_double(pl, ew - 1);
         o.p[1] = to_double(pr, ew - 1);
-        const int eprod2 = ew - 1 + exponent(ic2) - 1022, er = (es > eprod2 ? es : eprod2) + 1;
+        const int eprod2 = ew - 1 + ic2.e - 1022, er = (es > eprod2 ? es : eprod2) + 1;
         const u64 fi = factor(ic2, ew - 1, er);
         o.r[0] = to_double(aligned(sl, es, er) + mulhi(pl, fi), er);
         o.r[1] = to_double(aligned(sr, es, er) + mulhi(pr, fi), er);

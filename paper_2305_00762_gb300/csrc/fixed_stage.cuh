@@ -3,8 +3,9 @@
 // in shared memory taken apart (fx::split: 64-bit integer and exponent), so a
 // face's stencils are aligned to their own scale by a shift each; face states
 // (fixed_face.cuh), flux reconstruction and the viscous gradients are integer
-// sums. FP64 arithmetic remains for the primitives, the cell fluxes, the
-// Riemann solver, the viscous flux and the stage update. With CONS (MEG7-cons)
+// sums, and so are the primitives and the cell fluxes (fixed_math.cuh). FP64
+// arithmetic remains for the Riemann solver, the viscous flux and the stage
+// update. With CONS (MEG7-cons)
 // the planes taken apart are the conservative variables, and the primitives of
 // the cells beside faces are kept as they are.
 #pragma once
@@ -13,7 +14,7 @@
 
 namespace gbr {
 
-template <int BX, int BY, bool VISC, bool CONS = false>
+template <int BX, int BY, bool VISC, bool CONS = false, bool TMA = true>
 struct FixedLayout {
     using G = TileLayout<BX, BY, VISC>;  // index ranges
     typedef long long i64;
@@ -28,11 +29,12 @@ struct FixedLayout {
     static constexpr size_t oGX = oRaw, oGY = oGX + (VISC ? sizeof(double) * 4 * G::NGX : 0);
     static constexpr size_t oHX = oGY + (VISC ? sizeof(double) * 4 * G::NGY : 0);
     static constexpr size_t oHY = oHX + sizeof(double) * 4 * G::NHX;
-    static constexpr size_t oH1 = oHY + sizeof(double) * 4 * G::NHY, oR1 = oRaw + sizeof(double) * 4 * NU;
+    static constexpr size_t oH1 = oHY + sizeof(double) * 4 * G::NHY, oR1 = oRaw + (TMA ? sizeof(double) * 4 : sizeof(float)) * NU;
     static constexpr size_t oW = oH1 > oR1 ? oH1 : oR1;                      // CONS: u, v, p of cells [5, B + 7) [3][NW]
     static constexpr int WW = BX + 2, NW = WW * (BY + 2);
-    static constexpr size_t oR = oW + (CONS ? sizeof(double) * 3 * NW : 0);  // densities in FP32 [NU]
-    static constexpr size_t oE = oR + sizeof(float) * NU;                    // exponents of the integers above
+    // densities in FP32 [NU], read before the face fluxes are written
+    static constexpr size_t oR = TMA || VISC ? oW + (CONS ? sizeof(double) * 3 * NW : 0) : oRaw;
+    static constexpr size_t oE = TMA || VISC ? oR + sizeof(float) * NU : oW + (CONS ? sizeof(double) * 3 * NW : 0);  // exponents of the integers above
     static constexpr size_t oEX = oE + sizeof(short) * 4 * NU;
     static constexpr size_t oEY = oEX + sizeof(short) * 4 * NFX;
     static constexpr size_t oPX = oEY + sizeof(short) * 4 * NFY;             // detector flags
@@ -69,7 +71,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
 {
     typedef long long i64;
     typedef unsigned short u16;
-    using F = FixedLayout<BX, BY, VISC, CONS>;
+    using F = FixedLayout<BX, BY, VISC, CONS, TMA>;
     using L = typename F::G;
     using X = typename L::template Cross<0>;  // the staged cells
     constexpr int RW = L::RW, NU = L::NU, V = L::V;
@@ -97,41 +99,49 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     ph.kq = P.ph.kq;
     ph.lm = P.ph.riemann;
     const double inv_dx = P.ph.inv_dx, inv_dy = P.ph.inv_dy;
+    const fx::Pos gamma = fx::pos(ph.gamma), gm1 = fx::pos(ph.gm1);
 
     // Phase 0: primitives (Eq. pressure) and cell fluxes F^c = (rho u, rho u u
     // + p, rho u v, u (E + p)), G^c (Sec. 1; rho u, rho v, E from the state).
     const bool staged = stage_region<BX, BY, NT, X, TMA>(
         P, tx0, ty0, reinterpret_cast<double*>(smem + F::oRaw), tmap,
         [&](int idx, double q0, double q1, double q2, double q3) {
-            double w[4];
-            prims_of(q0, q1, q2, q3, ph.gm1, w[0], w[1], w[2], w[3]);
+            fx::Cell w;
+            fx::cell_of(q0, q1, q2, q3, gm1, w);
             const int ry = idx / RW, rx = idx - ry * RW;
+            auto put = [&](int m, const fx::Split& x) { fx::store(x, sM[m * NU + idx], sE[m * NU + idx]); };
+            put(0, w.r);
             if constexpr (CONS) {
-                const double q[4] = {q0, q1, q2, q3};
-#pragma unroll
-                for (int m = 0; m < 4; ++m) fx::split(q[m], sM[m * NU + idx], sE[m * NU + idx]);
+                put(1, w.ru);
+                put(2, w.rv);
+                put(3, fx::split(q3));
                 if (ry >= 5 && ry < BY + 7 && rx >= 5 && rx < BX + 7) {
                     const int c = (ry - 5) * F::WW + rx - 5;
-#pragma unroll
-                    for (int m = 0; m < 3; ++m) sW[m * F::NW + c] = w[m + 1];
+                    sW[c] = fx::unsplit(w.u.m, w.u.e);
+                    sW[F::NW + c] = fx::unsplit(w.v.m, w.v.e);
+                    sW[2 * F::NW + c] = fx::unsplit(w.p.m, w.p.e);
                 }
             } else {
-#pragma unroll
-                for (int m = 0; m < 4; ++m) fx::split(w[m], sM[m * NU + idx], sE[m * NU + idx]);
+                put(1, w.u);
+                put(2, w.v);
+                put(3, w.p);
             }
-            sR[idx] = f64_to_f32_rn(w[0]);
-            const double ep = q3 + w[3];
+            sR[idx] = f64_to_f32_rn(q0);
             if (ry >= 6 && ry < 6 + BY && rx >= 1 && rx < BX + 11) {
                 const int f = (ry - 6) * L::FXW + (rx - 1);
-                const double h[4] = {q1, rfma(q1, w[1], w[3]), rmul(q1, w[2]), rmul(w[1], ep)};
-#pragma unroll
-                for (int m = 0; m < 4; ++m) fx::split(h[m], sFX[m * L::NFX + f], sEX[m * L::NFX + f]);
+                auto flux = [&](int m, const fx::Split& x) { fx::store(x, sFX[m * L::NFX + f], sEX[m * L::NFX + f]); };
+                flux(0, w.ru);
+                flux(1, fx::sum(w.ruu, w.p));
+                flux(2, fx::product(w.ru, w.v));
+                flux(3, fx::product(w.u, w.h));
             }
             if (ry >= 1 && ry < BY + 11 && rx >= 6 && rx < BX + 6) {
                 const int f = (ry - 1) * BX + (rx - 6);
-                const double h[4] = {q2, rmul(q2, w[1]), rfma(q2, w[2], w[3]), rmul(w[2], ep)};
-#pragma unroll
-                for (int m = 0; m < 4; ++m) fx::split(h[m], sFY[m * L::NFY + f], sEY[m * L::NFY + f]);
+                auto flux = [&](int m, const fx::Split& x) { fx::store(x, sFY[m * L::NFY + f], sEY[m * L::NFY + f]); };
+                flux(0, w.rv);
+                flux(1, fx::product(w.rv, w.u));
+                flux(2, fx::sum(w.rvv, w.p));
+                flux(3, fx::product(w.v, w.h));
             }
         });
     if (!staged) return;
@@ -142,7 +152,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         return trouble_filtered(sR + c, st, [&] {
             double r[5];
 #pragma unroll
-            for (int k = 0; k < 5; ++k) r[k] = fx::unsplit(sM[c + (k - 2) * st], sE[c + (k - 2) * st]);
+            for (int k = 0; k < 5; ++k) r[k] = fx::unsplit(sM[c + (k - 2) * st], sE[c + (k - 2) * st]);  // (exact: rho is the state's)
             return trouble_cell(r + 2, 1);
         }) ? 1 : 0;
     };
@@ -192,14 +202,19 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
 #pragma unroll
         for (int k = -2; k <= 3; ++k) trouble |= tr[k * st] != 0;
 
-        // Primitives (rho, un, ut, p) of the face's two cells
-        double u0[4], u1[4];
         auto plane = [&](int m) { return m == 1 ? pn : m == 2 ? 3 - pn : m; };
         const int cw = (fr + (xf ? 1 : 0)) * F::WW + fc + (xf ? 0 : 1), sw = xf ? 1 : F::WW;
         auto cell = [&](int m, int o) {  // variable m of the cell before (o = 0) or after (su) the face
             if (CONS && m > 0) return sW[(plane(m) - 1) * F::NW + cw + (o ? sw : 0)];
             const int at = plane(m) * NU + c + o;
             return fx::unsplit(sM[at], sE[at]);
+        };
+        auto value = [&](int m, int o) {
+            const int at = plane(m) * NU + c + o;
+            fx::Split x;
+            x.m = sM[at];
+            x.e = sE[at];
+            return x;
         };
         auto load = [&](int m, fx::Stencil& x) {
             const int at = plane(m) * NU + c;
@@ -209,38 +224,35 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                 x.e[k] = sE[at + (k - 5) * su];
             }
         };
-        u0[0] = cell(0, 0);
-        u1[0] = cell(0, su);
-        u0[3] = cell(3, 0);
-        u1[3] = cell(3, su);
         // Characteristic projection at the arithmetic-mean state, every
         // factor from one reciprocal square root y = 1/sqrt(gamma p rho).
         // (Twice the means: X = (2 rho)(2 gamma p), y = 1/sqrt(X) = 1/(2 rho c),
         // 1/c = 2 rho y, 2 rho c = X y.)
-        const double rb = u0[0] + u1[0], gp = ph.gamma * (u0[3] + u1[3]), xx = rmul(gp, rb);
-        const double y = fx::rsqrt(xx);
-        const double icb = rmul(rb, y), ic2 = rmul(icb, icb);
+        const fx::Split rs = fx::sum(value(0, 0), value(0, su));
+        fx::Split ps;
+        if constexpr (!CONS) ps = fx::sum(value(3, 0), value(3, su));
+        else ps = fx::split(cell(3, 0) + cell(3, su));
+        const bool positive = rs.m > 0 && ps.m > 0;  // (else the fallback below)
+        const fx::Pos rb = fx::pos(positive ? rs.m : 1, rs.e), gp = gamma * fx::pos(positive ? ps.m : 1, ps.e);
+        const fx::Pos xx = gp * rb, y = fx::rsqrt(xx), icb = rb * y, ic2 = icb * icb;
         double rL, unL, utL, pL, rR, unR, utR, pR;
         bool ok;
         if constexpr (!CONS) {
             fx::FaceStates s;
-            fx::face_states<ORDER>(load, y, rmul(xx, y), ic2, s);
+            fx::face_states<ORDER>(load, y, xx * y, ic2, s);
             rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
             rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
             ok = s.ok;
         } else {
-            u0[1] = cell(1, 0);
-            u1[1] = cell(1, su);
-            u0[2] = cell(2, 0);
-            u1[2] = cell(2, su);
-            const double ub = 0.5 * (u0[1] + u1[1]), vb = 0.5 * (u0[2] + u1[2]), cb = rmul(gp, y);
+            const double ub = rmul(0.5, cell(1, 0) + cell(1, su)), vb = rmul(0.5, cell(2, 0) + cell(2, su));
+            const double cb = fx::to_double(gp * y), ic = fx::to_double(icb);
             fx::ConsCoefs C;
-            C.b1 = rmul(ph.gm1, ic2);
+            C.b1 = fx::to_double(gm1 * ic2);
             C.b1u = rmul(C.b1, ub);
             C.b1v = rmul(C.b1, vb);
             C.b2 = rmul(0.5, rfma(C.b1u, ub, rmul(C.b1v, vb)));
-            C.uc = rmul(ub, icb);
-            C.ic = icb;
+            C.uc = rmul(ub, ic);
+            C.ic = ic;
             C.v = vb;
             fx::ConsStates s;
             fx::cons_states<ORDER>(
@@ -271,17 +283,18 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         }
         // positivity fallback: a face state with rho <= 0 or p <= 0 (or from a
         // refused stencil) takes the adjacent cell's state
+        ok = ok && positive;
         if (!(ok && tpositive(rL) && tpositive(pL))) {
-            rL = u0[0];
+            rL = cell(0, 0);
             unL = cell(1, 0);
             utL = cell(2, 0);
-            pL = u0[3];
+            pL = cell(3, 0);
         }
         if (!(ok && tpositive(rR) && tpositive(pR))) {
-            rR = u1[0];
+            rR = cell(0, su);
             unR = cell(1, su);
             utR = cell(2, su);
-            pR = u1[3];
+            pR = cell(3, su);
         }
         // Flux reconstruction of the central part where sigma = 1 (Sec. 2.4).
         double Fs[4];
@@ -310,11 +323,12 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         double out[4];
         hllc_flux(ph, !trouble, Fs, rL, unL, utL, pL, rR, unR, utR, pR, out);
         if constexpr (VISC) {
-            if constexpr (!CONS) {
-                u0[1] = cell(1, 0);
-                u1[1] = cell(1, su);
-                u0[2] = cell(2, 0);
-                u1[2] = cell(2, su);
+            // Primitives (rho, un, ut, p) of the face's two cells
+            double u0[4], u1[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                u0[m] = cell(m, 0);
+                u1[m] = cell(m, su);
             }
             FaceIn<double> in;
             // gradients along the face normal at the cell before the face, and
@@ -357,14 +371,15 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
 
 // One CTA per tile, two CTAs per SM (viscous MEG7-cons: one, by shared memory).
 template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS>
-__global__ void __launch_bounds__(NT, CONS && VISC ? 1 : 2) fixed_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
+__global__ void __launch_bounds__(NT, CONS && VISC ? 1 : 2)
+    fixed_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     fixed_tile<BX, BY, NT, VISC, ORDER, true, CONS>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
 }
 
-template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS = false>
-cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
+template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS>
+cudaError_t launch_fixed_tiles(const StageParams& p, cudaStream_t s)
 {
     using F = FixedLayout<BX, BY, VISC, CONS>;
     static PerDevice<int> configured;  // the shared-memory limit is raised once per device
@@ -381,6 +396,40 @@ cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
     dim3 grid((p.g.nx + BX - 1) / BX, (p.g.ny + BY - 1) / BY);
     kern<<<grid, NT, F::bytes, s>>>(p, map);
     return cudaGetLastError();
+}
+
+// Tile shapes. The faces of 16 x 15 (511) are two rounds of 256 threads without
+// spills at 128 registers, the fastest per cell where there are tiles enough
+// (1024^2 step 1.94 ms; 16 x 16 with 288 threads 2.03, 20 x 12 1.97, 28 x 8
+// 2.05). A grid of few tiles is bound by the tiles the busiest SM gets, so a
+// smaller tile that divides the work further wins: 16 x 8 with its 280 faces in
+// one round, 8 x 4 where even that leaves SMs idle. A step's time is close to
+// 50 us + c k with k the tiles of the busiest SM and c = 63, 36.5 and 15.5 us
+// (measured at 32^2 .. 1024^2: 64^2 70 us with 8 x 4, 125 us with 16 x 15;
+// 200^2 167 us with 16 x 8, 181 / 182 us with the others; 256^2 181 us with
+// 16 x 15, 205 / 267 us with the others); the smallest c k is taken, k rounded
+// up while it is small and the last wave counts. The result does not depend on
+// the shape.
+template <bool VISC, int ORDER, bool CONS = false>
+cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
+{
+    static PerDevice<int> sm_count;
+    int sms = 0;
+    cudaError_t e = sm_count.get(&sms, [](int* v) {
+        int dev = 0;
+        const cudaError_t r = cudaGetDevice(&dev);
+        return r != cudaSuccess ? r : cudaDeviceGetAttribute(v, cudaDevAttrMultiProcessorCount, dev);
+    });
+    if (e != cudaSuccess) return e;
+    auto cost = [&](int bx, int by, double c) {
+        const double k = (double)((p.g.nx + bx - 1) / bx) * ((p.g.ny + by - 1) / by) / sms;
+        const double up = (double)(long long)k;
+        return c * (k <= 16.0 ? (k > up ? up + 1.0 : up) : k + 0.5);
+    };
+    const double big = cost(16, 15, 63.0), mid = cost(16, 8, 36.5), tiny = cost(8, 4, 15.5);
+    if (tiny < mid && tiny < big) return launch_fixed_tiles<8, 4, 96, VISC, ORDER, CONS>(p, s);
+    if (mid < big) return launch_fixed_tiles<16, 8, 288, VISC, ORDER, CONS>(p, s);
+    return launch_fixed_tiles<16, 15, 256, VISC, ORDER, CONS>(p, s);
 }
 
 }  // namespace gbr

@@ -200,6 +200,8 @@ cudaError_t launch_wavespeed(const Grid& g, const Physics& ph, const double* q, 
                              int precision, cudaStream_t s);
 cudaError_t launch_stage_f64(const StageParams& p, cudaStream_t s);
 cudaError_t launch_stage_f32(const StageParams& p, cudaStream_t s);
+cudaError_t launch_stage_viscous_f64(const StageParams& p, cudaStream_t s);
+cudaError_t launch_stage_order4_f64(const StageParams& p, cudaStream_t s);
 cudaError_t launch_stage_cons_f64(const StageParams& p, cudaStream_t s);
 cudaError_t launch_stage_cons_f32(const StageParams& p, cudaStream_t s);
 
