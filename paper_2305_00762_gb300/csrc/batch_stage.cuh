@@ -38,31 +38,34 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2) batch_stage_kernel
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const double ca = stage == 0 ? 0.0 : (stage == 1 ? 0.75 : 1.0 / 3.0);
     const double cbc = stage == 0 ? 1.0 : (stage == 1 ? 0.25 : 2.0 / 3.0);
+    __shared__ StageParams P;  // (per thread it would take the registers the tile needs)
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
         const BatchCase& C = cases[batch_case_of(cases, ncases, tile)];
         if (C.ds->dt == 0.0) continue;  // uniform over the CTA
         const int local = tile - C.tile_begin;
         const int ty = local / C.tiles_x, tx = local - ty * C.tiles_x;
-        StageParams P;
-        P.g = C.g;
-        P.ph = C.ph;
-        P.q = C.q[stage];
-        P.qn = C.q[0];
-        P.qout = C.q[(stage + 1) % 3];
-        P.res = nullptr;
-        P.sigx = nullptr;
-        P.sigy = nullptr;
-        P.lam_out = stage == 2 ? &C.ds->lam[0] : nullptr;
-        P.err = &C.ds->err;
-        P.dt_ptr = &C.ds->dt;
-        P.dt = 0.0;
-        P.ca = ca;
-        P.cb = cbc;
-        P.cc = cbc;
-        P.sensor = sensor;
-        P.dec = C.dec;
-        P.stall_bytes = 0;
-        P.stall_mma = 0;
+        if (threadIdx.x == 0) {  // (the previous tile ended with all threads synchronised)
+            P.g = C.g;
+            P.ph = C.ph;
+            P.q = C.q[stage];
+            P.qn = C.q[0];
+            P.qout = C.q[(stage + 1) % 3];
+            P.res = nullptr;
+            P.sigx = nullptr;
+            P.sigy = nullptr;
+            P.lam_out = stage == 2 ? &C.ds->lam[0] : nullptr;
+            P.err = &C.ds->err;
+            P.dt_ptr = &C.ds->dt;
+            P.dt = 0.0;
+            P.ca = ca;
+            P.cb = cbc;
+            P.cc = cbc;
+            P.sensor = sensor;
+            P.dec = C.dec;
+            P.stall_bytes = 0;
+            P.stall_mma = 0;
+        }
+        __syncthreads();
         if constexpr (sizeof(T) == 8) fixed_tile<BX, BY, NT, false, 7, false>(P, tx * BX, ty * BY, smem_raw);
         else stage_tile<T, BX, BY, NT, false, LEARNED>(P, tx * BX, ty * BY, smem_raw);
     }

@@ -73,6 +73,11 @@ struct Physics {
     // spends FP64 divisions on them: gamma - 1, 1/(gamma - 1), the heat
     // conduction coefficient mu / (Pr (gamma - 1)), 1/dx, 1/dy.
     double gm1, igm1, kq, inv_dx, inv_dy;
+    // The same rounded to FP32, for the FP32 form (a conversion issues on the
+    // FP64 pipe, and every thread would do seven).
+    struct {
+        float gamma, gm1, igm1, mu, kq, inv_dx, inv_dy;
+    } f32;
 };
 
 // Fill the derived members of ph from gamma, mu, Pr, dx, dy.
@@ -83,6 +88,13 @@ inline void derive_physics(Physics& ph)
     ph.kq = ph.mu / (ph.Pr * (ph.gamma - 1.0));
     ph.inv_dx = 1.0 / ph.dx;
     ph.inv_dy = 1.0 / ph.dy;
+    ph.f32.gamma = (float)ph.gamma;
+    ph.f32.gm1 = (float)ph.gm1;
+    ph.f32.igm1 = (float)ph.igm1;
+    ph.f32.mu = (float)ph.mu;
+    ph.f32.kq = (float)ph.kq;
+    ph.f32.inv_dx = (float)ph.inv_dx;
+    ph.f32.inv_dy = (float)ph.inv_dy;
 }
 
 struct SensorDev;

@@ -428,29 +428,32 @@ __device__ __forceinline__ void meg7_pair(const GrbCoef<T>& C, const T (&w)[6], 
     if (needL || needR) mp_limit_pair(w, e, aL, aR, s1L, s1R, ddL, ddR, vl, vr, needL, needR);
 }
 
-// 1/2 (F(f_L) + F(f_R)) at the face after cell f[0]: the sum of Eq.
-// flux-full and its mirror Eq. flux-right is the symmetric 10-point stencil
-// (-1, 1, 38, -250, 1052 | 1052, -250, 38, 1, -1) / 840 over f_{j-4..j+5}.
+// 1/2 (F(f_L) + F(f_R)) at the face after cell f[0], all four components: the
+// sum of Eq. flux-full and its mirror Eq. flux-right is the symmetric 10-point
+// stencil (-1, 1, 38, -250, 1052 | 1052, -250, 38, 1, -1) / 840 over f_{j-4..j+5}.
 template <typename T>
-__device__ __forceinline__ T recon_mean(const T* f, int s, const GrbCoef<T>& C)
+__device__ __forceinline__ void recon_mean(const float4* f, int s, const GrbCoef<T>& C, T (&F)[4])
 {
     // the weights divided by den (compile-time products): one product, four FMAs
-    T acc = rmul(C.c1 * C.inv_den, f[0] + f[s]);
-    acc = rfma(C.c2 * C.inv_den, f[-s] + f[2 * s], acc);
-    acc = rfma(C.c3 * C.inv_den, f[-2 * s] + f[3 * s], acc);
-    acc = rfma(C.c4 * C.inv_den, f[-3 * s] + f[4 * s], acc);
-    return rfma(C.c5 * C.inv_den, f[-4 * s] + f[5 * s], acc);
+    const T c[5] = {C.c1 * C.inv_den, C.c2 * C.inv_den, C.c3 * C.inv_den, C.c4 * C.inv_den, C.c5 * C.inv_den};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const float4 a = f[-k * s], b = f[(k + 1) * s];
+        const T v[4] = {a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w};
+#pragma unroll
+        for (int m = 0; m < 4; ++m) F[m] = k == 0 ? rmul(c[0], v[m]) : rfma(c[k], v[m], F[m]);
+    }
 }
 
 template <typename T>
 struct FaceIn {
     const T* u[4];  // primitive planes in face-normal order (rho, un, ut, p) at cell j
     int su;
-    const T* g[4];  // dx-scaled normal gradients, same order, at cell j
+    const T* g[4];  // dx-scaled normal gradients, same order, at cell j (FP32: one array of float4, sg in floats)
     int sg;
     const unsigned char* tr;  // detector trouble flags at cell j
     int st;
-    const T* f[4];  // cell convective fluxes in face-normal order at cell j
+    const float4* f;  // FP32: cell convective fluxes in face-normal order at cell j
     int sf;
     const T* tun;  // tangential derivative (dx-scaled) of un at cell j
     const T* tut;  // ... of ut
@@ -710,6 +713,9 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
     const T be = T(0.5) * ic2;       // 1 / (2 c^2)
 
     T wL[4], wR[4];
+    float4 G[6];  // gradients (rho, un, ut, p; MEG7-cons rho, rho un, rho ut, E) of cells j-2 .. j+3
+#pragma unroll
+    for (int k = 0; k < 6; ++k) G[k] = reinterpret_cast<const float4*>(in.g[0])[(k - 2) * (sg / 4)];
     if constexpr (!CONS) {
         {  // fields 1 and 4 (u - c and u + c) share un and p. They are
            // carried scaled by 2 c^2, as p -/+ rho c un: GRB, the limiter's
@@ -724,7 +730,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
                 const T un = in.u[1][o * su], p = in.u[3][o * su];
                 w0[k] = rfma(-rc, un, p);
                 w3[k] = rfma(rc, un, p);
-                const T gu = in.g[1][o * sg], gp = in.g[3][o * sg];
+                const T gu = G[k].y, gp = G[k].w;
                 e0[k] = rfma(-rc, gu, gp);
                 e3[k] = rfma(rc, gu, gp);
             }
@@ -737,7 +743,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
             for (int k = 0; k < 6; ++k) {
                 const int o = (k - 2);
                 w[k] = rfma(-ic2, in.u[3][o * su], in.u[0][o * su]);
-                e[k] = rfma(-ic2, in.g[3][o * sg], in.g[0][o * sg]);
+                e[k] = rfma(-ic2, G[k].w, G[k].x);
             }
             meg7_pair(coef, w, e, wL[1], wR[1]);
         }
@@ -747,7 +753,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
             for (int k = 0; k < 6; ++k) {
                 const int o = (k - 2);
                 w[k] = in.u[2][o * su];
-                e[k] = in.g[2][o * sg];
+                e[k] = G[k].z;
             }
             meg7_pair(coef, w, e, wL[2], wR[2]);
         }
@@ -760,7 +766,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
             const int o = (k - 2);
             cons_project(in.q[0][o * su], in.q[1][o * su], in.q[2][o * su], in.q[3][o * su], ub, vb, icb, b1, b2,
                          w[0][k], w[1][k], w[2][k], w[3][k]);
-            cons_project(in.g[0][o * sg], in.g[1][o * sg], in.g[2][o * sg], in.g[3][o * sg], ub, vb, icb, b1, b2,
+            cons_project(G[k].x, G[k].y, G[k].z, G[k].w, ub, vb, icb, b1, b2,
                          e[0][k], e[1][k], e[2][k], e[3][k]);
         }
 #pragma unroll
@@ -871,8 +877,7 @@ __device__ __forceinline__ void face_flux(const FaceIn<T>& in, const PhysT<T>& P
     // flux reconstruction where sigma = 1, F(Q_L), F(Q_R) where sigma = 0.
     T Fc[4];
     if (smooth) {
-#pragma unroll
-        for (int m = 0; m < 4; ++m) Fc[m] = recon_mean(in.f[m], in.sf, coef);
+        recon_mean(in.f, in.sf, coef, Fc);
     } else {
         Fc[0] = T(0.5) * (QL[1] + QR[1]);
         Fc[1] = T(0.5) * ((QL[1] * unL + pL) + (QR[1] * unR + pR));
@@ -1315,8 +1320,23 @@ __device__ __forceinline__ bool stage_region(const StageParams& P, int tx0, int 
     return true;
 }
 
-// Phase 3 of a tile, from its face fluxes (x faces [4][BY][BX + 1], y faces
-// [4][BY + 1][BX] in shared memory, written before the caller's barrier); ends
+// The four components of face e: planes of n values in FP64, float4 in FP32.
+__device__ __forceinline__ void load_face(const double* h, int n, int e, double (&v)[4])
+{
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = h[m * n + e];
+}
+__device__ __forceinline__ void load_face(const float* h, int, int e, float (&v)[4])
+{
+    const float4 f = reinterpret_cast<const float4*>(h)[e];
+    v[0] = f.x;
+    v[1] = f.y;
+    v[2] = f.z;
+    v[3] = f.w;
+}
+
+// Phase 3 of a tile, from its face fluxes (x faces [BY][BX + 1], y faces
+// [BY + 1][BX] in shared memory, written before the caller's barrier); ends
 // with all threads synchronised.
 template <typename T, int BX, int BY, int NT>
 __device__ __forceinline__ void finish_tile(const StageParams& P, const PhysT<T>& ph, T inv_dx, T inv_dy, int tx0, int ty0,
@@ -1338,10 +1358,14 @@ __device__ __forceinline__ void finish_tile(const StageParams& P, const PhysT<T>
         const int j = tx0 + c, i = ty0 + r;
         if (j >= nx || i >= ny) continue;
         double res[4];  // FP64: -dt Res when there is a stage update (cdt within sx, sy)
+        T hw[4], he[4], hs[4], hn[4];
+        load_face(sHX, NHX, r * (BX + 1) + c, hw);
+        load_face(sHX, NHX, r * (BX + 1) + c + 1, he);
+        load_face(sHY, NHY, r * BX + c, hs);
+        load_face(sHY, NHY, (r + 1) * BX + c, hn);
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            const T dF = sHX[m * NHX + r * (BX + 1) + c + 1] - sHX[m * NHX + r * (BX + 1) + c];
-            const T dG = sHY[m * NHY + (r + 1) * BX + c] - sHY[m * NHY + r * BX + c];
+            const T dF = he[m] - hw[m], dG = hn[m] - hs[m];
             // (square cells in FP64: one product)
             const T sum = kScaled && sx == sy ? rmul(dF + dG, sx) : rmul(dF, sx) + rmul(dG, sy);
             res[m] = to_f64(kScaled ? sum : -sum);
@@ -1401,12 +1425,20 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     using X = typename L::template Cross<LEARNED>;  // the staged cells
     T* const sm = reinterpret_cast<T*>(smem_raw);
     T* const sU = sm + L::oU;
-    T* const sGX = sm + L::oGX;
-    T* const sGY = sm + L::oGY;
-    T* const sFX = sm + L::oFX;
-    T* const sFY = sm + L::oFY;
-    T* const sHX = sm + L::oHX;
-    T* const sHY = sm + L::oHY;
+    // Four components at a time: gradients and cell fluxes in the face-normal
+    // order of their direction, face fluxes in the state's order. One 16-byte
+    // access replaces four, and its conflicts are counted over eight lanes, so
+    // a warp whose faces span two tile rows rarely has one.
+    static_assert(sizeof(T) == 4, "the FP64 form has a tile of its own (fixed_stage.cuh)");
+    float4* const sGX4 = reinterpret_cast<float4*>(sm + L::oGX);
+    float4* const sGY4 = reinterpret_cast<float4*>(sm + L::oGY);
+    float4* const sFX4 = reinterpret_cast<float4*>(sm + L::oFX);
+    float4* const sFY4 = reinterpret_cast<float4*>(sm + L::oFY);
+    float4* const sHX4 = reinterpret_cast<float4*>(sm + L::oHX);
+    float4* const sHY4 = reinterpret_cast<float4*>(sm + L::oHY);
+    static_assert(L::oGX % 4 == 0 && L::oGY % 4 == 0 && L::oFX % 4 == 0 && L::oFY % 4 == 0 && L::oHX % 4 == 0 &&
+                      L::oHY % 4 == 0,
+                  "16-byte arrays");
     T* const sQc = sm + L::oQc;  // MEG7-cons only
     unsigned char* const sPX = reinterpret_cast<unsigned char*>(sm + L::template nT<T, NT>());
     unsigned char* const sPY = sPX + L::NPX;
@@ -1417,13 +1449,13 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     const int tid = threadIdx.x;
 
     PhysT<T> ph;
-    ph.gamma = T(P.ph.gamma);
-    ph.gm1 = T(P.ph.gm1);
-    ph.igm1 = T(P.ph.igm1);
-    ph.mu = T(P.ph.mu);
-    ph.kq = T(P.ph.kq);
+    ph.gamma = P.ph.f32.gamma;
+    ph.gm1 = P.ph.f32.gm1;
+    ph.igm1 = P.ph.f32.igm1;
+    ph.mu = P.ph.f32.mu;
+    ph.kq = P.ph.f32.kq;
     ph.lm = P.ph.riemann;
-    const T inv_dx = T(P.ph.inv_dx), inv_dy = T(P.ph.inv_dy);
+    const T inv_dx = P.ph.f32.inv_dx, inv_dy = P.ph.f32.inv_dy;
 
     // Phase 0: stage the tile + halo as primitive variables (Eq. pressure).
     // Region cell (rx, ry) is padded cell (tx0 + rx, ty0 + ry).
@@ -1483,14 +1515,12 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     for (int idx = tid; idx < L::NGX; idx += NT) {  // x-gradients (Eq. six)
         const int a = idx / L::GXW, b = idx - a * L::GXW;
         const T* s = sV + (a + 6 - V) * RW + (b + 3);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) sGX[m * L::NGX + idx] = grad6(s + m * NU, 1);
+        sGX4[idx] = make_float4(grad6(s, 1), grad6(s + NU, 1), grad6(s + 2 * NU, 1), grad6(s + 3 * NU, 1));
     }
     for (int idx = tid; idx < L::NGY; idx += NT) {  // y-gradients
         const int a = idx / L::GYW, b = idx - a * L::GYW;
         const T* s = sV + (a + 3) * RW + (b + 6 - V);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) sGY[m * L::NGY + idx] = grad6(s + m * NU, RW);
+        sGY4[idx] = make_float4(grad6(s, RW), grad6(s + 2 * NU, RW), grad6(s + NU, RW), grad6(s + 3 * NU, RW));
     }
     if constexpr (!LEARNED) {
         for (int idx = tid; idx < L::NPX; idx += NT) {  // x detector (Eq. detector)
@@ -1508,10 +1538,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
         const T r = sU[c], u = sU[NU + c], v = sU[2 * NU + c], p = sU[3 * NU + c];
         const T E = rfma(p, ph.igm1, rmul(T(0.5) * r, sumsq(u, v)));
         const T ru = r * u;
-        sFX[idx] = ru;
-        sFX[L::NFX + idx] = rfma(ru, u, p);
-        sFX[2 * L::NFX + idx] = ru * v;
-        sFX[3 * L::NFX + idx] = u * (E + p);
+        sFX4[idx] = make_float4(ru, rfma(ru, u, p), ru * v, u * (E + p));
     }
     for (int idx = tid; idx < L::NFY; idx += NT) {  // cell y-fluxes G^c
         const int a = idx / BX, b = idx - a * BX;
@@ -1519,10 +1546,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
         const T r = sU[c], u = sU[NU + c], v = sU[2 * NU + c], p = sU[3 * NU + c];
         const T E = rfma(p, ph.igm1, rmul(T(0.5) * r, sumsq(u, v)));
         const T rv = r * v;
-        sFY[idx] = rv;
-        sFY[L::NFY + idx] = rv * u;
-        sFY[2 * L::NFY + idx] = rfma(rv, v, p);
-        sFY[3 * L::NFY + idx] = v * (E + p);
+        sFY4[idx] = make_float4(rv, rfma(rv, v, p), rv * u, v * (E + p));
     }
     __syncthreads();
     if constexpr (LEARNED) {
@@ -1581,24 +1605,20 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
                 in.u[2] = u + 2 * NU;
                 in.u[3] = u + 3 * NU;
                 in.su = 1;
-                const T* gx = sGX + (r + V) * L::GXW + (rx - 3);
+                const T* gx = reinterpret_cast<const T*>(sGX4 + (r + V) * L::GXW + (rx - 3));
                 in.g[0] = gx;
-                in.g[1] = gx + L::NGX;
-                in.g[2] = gx + 2 * L::NGX;
-                in.g[3] = gx + 3 * L::NGX;
-                in.sg = 1;
+                in.g[1] = gx + 1;
+                in.g[2] = gx + 2;
+                in.g[3] = gx + 3;
+                in.sg = 4;
                 in.tr = sPX + r * L::PXW + (rx - 3);
                 in.st = 1;
-                const T* fx = sFX + r * L::FXW + (rx - 1);
-                in.f[0] = fx;
-                in.f[1] = fx + L::NFX;
-                in.f[2] = fx + 2 * L::NFX;
-                in.f[3] = fx + 3 * L::NFX;
+                in.f = sFX4 + r * L::FXW + (rx - 1);
                 in.sf = 1;
-                const T* ty = sGY + (ry - 3) * L::GYW + (rx - 6 + V);
-                in.tun = ty + L::NGY;      // d u / d y (cons: d rho u / d y)
-                in.tut = ty + 2 * L::NGY;  // d v / d y (cons: d rho v / d y)
-                in.stq = 1;
+                const T* ty = reinterpret_cast<const T*>(sGY4 + (ry - 3) * L::GYW + (rx - 6 + V));
+                in.tun = ty + 2;  // d u / d y (cons: d rho u / d y)
+                in.tut = ty + 1;  // d v / d y (cons: d rho v / d y)
+                in.stq = 4;
                 if constexpr (CONS) {
                     const T* qc = sQc + ry * RW + rx;
                     in.q[0] = qc;
@@ -1620,24 +1640,20 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
                 in.u[2] = u + NU;      // tangential velocity u
                 in.u[3] = u + 3 * NU;
                 in.su = RW;
-                const T* gy = sGY + (ry - 3) * L::GYW + (rx - 6 + V);
+                const T* gy = reinterpret_cast<const T*>(sGY4 + (ry - 3) * L::GYW + (rx - 6 + V));
                 in.g[0] = gy;
-                in.g[1] = gy + 2 * L::NGY;
-                in.g[2] = gy + L::NGY;
-                in.g[3] = gy + 3 * L::NGY;
-                in.sg = L::GYW;
+                in.g[1] = gy + 1;
+                in.g[2] = gy + 2;
+                in.g[3] = gy + 3;
+                in.sg = 4 * L::GYW;
                 in.tr = sPY + (ry - 3) * BX + c;
                 in.st = BX;
-                const T* fy = sFY + (ry - 1) * BX + c;
-                in.f[0] = fy;
-                in.f[1] = fy + 2 * L::NFY;  // rho v^2 + p
-                in.f[2] = fy + L::NFY;      // rho u v
-                in.f[3] = fy + 3 * L::NFY;
+                in.f = sFY4 + (ry - 1) * BX + c;
                 in.sf = BX;
-                const T* tx = sGX + (ry - 6 + V) * L::GXW + (rx - 3);
-                in.tun = tx + 2 * L::NGX;  // d v / d x (cons: d rho v / d x)
-                in.tut = tx + L::NGX;      // d u / d x (cons: d rho u / d x)
-                in.stq = L::GXW;
+                const T* tx = reinterpret_cast<const T*>(sGX4 + (ry - 6 + V) * L::GXW + (rx - 3));
+                in.tun = tx + 2;  // d v / d x (cons: d rho v / d x)
+                in.tut = tx + 1;  // d u / d x (cons: d rho u / d x)
+                in.stq = 4 * L::GXW;
                 if constexpr (CONS) {
                     const T* qc = sQc + ry * RW + rx;
                     in.q[0] = qc;
@@ -1654,17 +1670,13 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
             face_flux<T, VISC, ORDER, CONS>(in, ph, inv_n, inv_t, out, smooth);
             if (valid) {
                 if (xf) {
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) sHX[m * L::NHX + w] = out[m];
+                    sHX4[w] = make_float4(out[0], out[1], out[2], out[3]);
                     if (P.sigx) {
                         const int i = ty0 + r, jf = tx0 + f;
                         if (i < ny && jf <= nx) P.sigx[(long long)i * (nx + 1) + jf] = smooth ? 1 : 0;
                     }
                 } else {
-                    sHY[w2] = out[0];
-                    sHY[L::NHY + w2] = out[2];
-                    sHY[2 * L::NHY + w2] = out[1];
-                    sHY[3 * L::NHY + w2] = out[3];
+                    sHY4[w2] = make_float4(out[0], out[2], out[1], out[3]);
                     if (P.sigy) {
                         const int j = tx0 + c, iface = ty0 + f;
                         if (j < nx && iface <= ny) P.sigy[(long long)iface * nx + j] = smooth ? 1 : 0;
@@ -1675,7 +1687,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     }
     __syncthreads();
 
-    finish_tile<T, BX, BY, NT>(P, ph, inv_dx, inv_dy, tx0, ty0, sHX, sHY);
+    finish_tile<T, BX, BY, NT>(P, ph, inv_dx, inv_dy, tx0, ty0, sm + L::oHX, sm + L::oHY);
 }
 
 // One CTA per tile; the tile + halo is staged by a tensor copy described by
