@@ -12,6 +12,7 @@ namespace gbr {
 // the per-step scalar bookkeeping of GhostParams::mode.
 __global__ void ghost_kernel(const GhostParams P)
 {
+    dependent_start();
     const long long total = ghost_count(P.g);
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id == 0 && P.mode != 0) {
@@ -53,8 +54,7 @@ cudaError_t launch_ghosts(const GhostParams& p, cudaStream_t s)
     const long long total = ghost_count(p.g);
     const int nt = 256;
     const unsigned nb = (unsigned)((total + nt - 1) / nt);
-    ghost_kernel<<<nb, nt, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(ghost_kernel, dim3(nb), nt, 0, s, p);
 }
 
 // Ghost cells of buffer `buf` of every grid of a batch (one thread per ghost
@@ -65,6 +65,7 @@ cudaError_t launch_ghosts(const GhostParams& p, cudaStream_t s)
 __global__ void batch_ghost_kernel(const BatchCase* __restrict__ cases, int ncases, long long total, int buf,
                                    int mode, double cfl, const double* __restrict__ dts)
 {
+    dependent_start();
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (mode == 2 && id < ncases) {
         DevScalars* d = cases[id].ds;
@@ -100,9 +101,8 @@ cudaError_t launch_batch_ghosts(const BatchCase* cases, int ncases, long long to
 {
     long long n = total_ghosts > ncases ? total_ghosts : ncases;
     const int nt = 256;
-    batch_ghost_kernel<<<(unsigned)((n + nt - 1) / nt), nt, 0, s>>>(cases, ncases, total_ghosts, buf, mode, cfl,
-                                                                     dts);
-    return cudaGetLastError();
+    return launch_dependent(batch_ghost_kernel, dim3((unsigned)((n + nt - 1) / nt)), nt, 0, s, cases, ncases, total_ghosts,
+                            buf, mode, cfl, dts);
 }
 
 __device__ __forceinline__ double warp_max_d(double v)

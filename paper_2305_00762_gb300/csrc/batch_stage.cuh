@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2) batch_stage_kernel
                                                          int total_tiles, int stage, const SensorDev* sensor)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    dependent_start();
     const double ca = stage == 0 ? 0.0 : (stage == 1 ? 0.75 : 1.0 / 3.0);
     const double cbc = stage == 0 ? 1.0 : (stage == 1 ? 0.25 : 2.0 / 3.0);
     __shared__ StageParams P;  // (per thread it would take the registers the tile needs)
@@ -102,8 +103,8 @@ cudaError_t launch_batch_t(const BatchCase* cases, int ncases, int total_tiles, 
     cudaError_t e = batch_blocks<T, BX, BY, NT, LEARNED>(&blocks);
     if (e != cudaSuccess || total_tiles <= 0) return e;
     const int grid = (per_tile || total_tiles < blocks) ? total_tiles : blocks;
-    batch_stage_kernel<T, BX, BY, NT, LEARNED><<<grid, NT, smem, s>>>(cases, ncases, total_tiles, stage, sensor);
-    return cudaGetLastError();
+    return launch_dependent(batch_stage_kernel<T, BX, BY, NT, LEARNED>, dim3(grid), NT, smem, s, cases, ncases, total_tiles,
+                            stage, sensor);
 }
 
 }  // namespace gbr

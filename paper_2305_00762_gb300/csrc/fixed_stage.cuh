@@ -375,6 +375,7 @@ __global__ void __launch_bounds__(NT, CONS && VISC ? 1 : 2)
     fixed_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    dependent_start();
     fixed_tile<BX, BY, NT, VISC, ORDER, true, CONS>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
 }
 
@@ -394,8 +395,7 @@ cudaError_t launch_fixed_tiles(const StageParams& p, cudaStream_t s)
     e = encode_state_map(p.g, p.q, F::G::RW, F::G::RH, &map);
     if (e != cudaSuccess) return e;
     dim3 grid((p.g.nx + BX - 1) / BX, (p.g.ny + BY - 1) / BY);
-    kern<<<grid, NT, F::bytes, s>>>(p, map);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, NT, F::bytes, s, p, map);
 }
 
 // Tile shapes. The faces of 16 x 15 (511) are two rounds of 256 threads without

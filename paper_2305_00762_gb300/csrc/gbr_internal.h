@@ -36,6 +36,36 @@ struct PerDevice {
     }
 };
 
+// Launches of one step follow each other on one stream, each reading what the
+// one before wrote. With programmatic serialisation the next kernel's blocks
+// may start while the last ones of the kernel before still run; they wait in
+// dependent_start() until that grid has ended and its writes are visible, so
+// only the launch latency overlaps. (A kernel whose predecessor on the stream
+// is anything else waits as usual.)
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A&&... a)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, static_cast<A&&>(a)...);
+}
+#ifdef __CUDACC__
+// The first statement of a kernel launched so.
+__device__ __forceinline__ void dependent_start()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 constexpr int kGhost = 6;  // ghost layers per side (Sec. 2.3, LC bound reach)
 
 // Device-resident scalars of one solver context.

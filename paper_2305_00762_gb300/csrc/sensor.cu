@@ -396,6 +396,7 @@ __global__ void __launch_bounds__(128 * G, 8 / G)
     sensor_tc_kernel(const SensorTileParams P, unsigned* err, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(1024) unsigned char tc_raw[];
+    dependent_start();  // (before the tensor memory is allocated: no two grids hold columns at a time)
     TcSmem& S = *reinterpret_cast<TcSmem*>(tc_raw);
     const int tid = threadIdx.x;
     const int tx0 = blockIdx.x * kTX, ty0 = blockIdx.y * kTY;
@@ -459,6 +460,7 @@ __global__ void __launch_bounds__(128 * G, 8 / G)
     batch_sensor_tc_kernel(const BatchCase* __restrict__ cases, int ncases, int buf, const SensorDev* w)
 {
     extern __shared__ __align__(1024) unsigned char tc_raw[];
+    dependent_start();
     TcSmem& S = *reinterpret_cast<TcSmem*>(tc_raw);
     const int tile = blockIdx.x;
     int lo = 0, hi = ncases - 1;
@@ -504,8 +506,7 @@ static cudaError_t launch_sensor_tc(const SensorTileParams& P, dim3 grid, unsign
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     if ((e = encode_state_map(P.g, P.q, kRawW, kRH, &map)) != cudaSuccess) return e;
-    sensor_tc_kernel<kTcGroups><<<grid, 128 * kTcGroups, smem, s>>>(P, err, map);
-    return cudaGetLastError();
+    return launch_dependent(sensor_tc_kernel<kTcGroups>, grid, 128 * kTcGroups, smem, s, P, err, map);
 }
 
 cudaError_t launch_sensor_tile(const Grid& g, double gamma, const double* q, const SensorDev* w, float* prob,
@@ -572,8 +573,7 @@ cudaError_t launch_batch_sensor_decide(const BatchCase* cases, int ncases, int t
     });
     if (e != cudaSuccess) return e;
     if (total_tiles <= 0) return cudaSuccess;  // prepare only (or nothing to do)
-    kern<<<total_tiles, 128 * kTcGroups, smem, s>>>(cases, ncases, buf, w);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(total_tiles), 128 * kTcGroups, smem, s, cases, ncases, buf, w);
 }
 
 // ---------------------------------------------------------------------------

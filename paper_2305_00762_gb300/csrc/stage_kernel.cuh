@@ -1445,7 +1445,6 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     constexpr int RW = L::RW, NU = L::NU, V = L::V;
 
     const int nx = P.g.nx, ny = P.g.ny, pitch = P.g.pitch;
-    const long long plane = P.g.plane;
     const int tid = threadIdx.x;
 
     PhysT<T> ph;
@@ -1706,6 +1705,7 @@ template <typename T, int BX, int BY, int NT, bool VISC, int LEARNED, int ORDER,
 __global__ void __launch_bounds__(NT, stage_min_blocks<T, VISC, CONS, LEARNED>()) stage_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    dependent_start();
     stage_tile<T, BX, BY, NT, VISC, LEARNED, ORDER, CONS, true>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw,
                                                                  &tmap);
 }
@@ -1727,8 +1727,7 @@ cudaError_t launch_stage_t(const StageParams& p, cudaStream_t s)
     e = encode_state_map(p.g, p.q, L::RW, L::RH, &map);
     if (e != cudaSuccess) return e;
     dim3 grid((p.g.nx + BX - 1) / BX, (p.g.ny + BY - 1) / BY);
-    kern<<<grid, NT, smem, s>>>(p, map);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, NT, smem, s, p, map);
 }
 
 }  // namespace gbr
