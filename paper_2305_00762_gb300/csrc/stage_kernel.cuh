@@ -264,6 +264,25 @@ __device__ __forceinline__ bool positive_bits(double x)
     const long long b = __double_as_longlong(x);
     return b > 0 && b <= 0x7ff0000000000000LL;
 }
+// The leading 21 bits of x as FP32 (relative error below 2^-20; zero below
+// 2^-62). `in` is cleared from 2^62 on, for infinities and for NaN.
+__device__ __forceinline__ float leading_bits(double x, bool& in)
+{
+    const unsigned h = (unsigned)__double2hiint(x), m = h & 0x7fffffffu;
+    in = in && m < ((1023u + 62u) << 20);
+    return m < ((1023u - 62u) << 20) ? 0.f : __uint_as_float((h & 0x80000000u) | ((m - (896u << 20)) << 3));
+}
+// A conservative state whose positivity (rho > 0 and 2 rho E > |rho u|^2, all
+// finite) the leading bits decide: the difference is off by less than 2^-18 of
+// its terms, and by 2^-60 where a term counted as zero. Only the few states near
+// a vanishing pressure still take the four FP64 operations.
+__device__ __forceinline__ bool surely_physical(double q0, double q1, double q2, double q3)
+{
+    bool in = true;
+    const float r = leading_bits(q0, in), u = leading_bits(q1, in), v = leading_bits(q2, in), e = leading_bits(q3, in);
+    const float k = fmaf(u, u, v * v), re = 2.f * r * e;
+    return in && r > 0.f && re - k > fmaf(re + k, 1.f / 65536.f, 1e-15f);
+}
 // 0 < x in T: the comparison itself in FP32, the bit test in FP64 (off the
 // FP64 pipe; the same answer for every value, NaN included).
 __device__ __forceinline__ bool tpositive(float x) { return x > 0.0f; }
@@ -941,13 +960,21 @@ __device__ __forceinline__ bool mbar_test(unsigned long long* bar, unsigned pari
     return done != 0;
 }
 
-// Wait for phase 0 of the mbarrier with an iteration limit (about a second);
-// false if it gave up.
+// Wait for phase 0 of the mbarrier: each try suspends the thread for at most
+// about a microsecond (waking when the phase completes, where polling would
+// sleep past it), with an iteration limit of about a second; false if it gave up.
 __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar)
 {
-    for (int it = 0; it < (1 << 24); ++it) {
-        if (mbar_test(bar, 0)) return true;
-        __nanosleep(64);
+    for (int it = 0; it < (1 << 20); ++it) {
+        unsigned done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0, 1000;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(smem_addr(bar))
+            : "memory");
+        if (done) return true;
     }
     return false;
 }
@@ -1387,10 +1414,11 @@ __device__ __forceinline__ void finish_tile(const StageParams& P, const PhysT<T>
             for (int m = 0; m < 4; ++m) P.qout[o + m * plane] = qv[m];
             // Positivity in FP64: rho > 0 and p > 0 <=> 2 rho E > |rho u|^2
             // (the comparisons on the bits, off the FP64 pipe).
-            const double e2 = rfma(qv[0] + qv[0], qv[3], -rfma(qv[1], qv[1], rmul(qv[2], qv[2])));
-            const bool ok = finite_bits(qv[0]) && finite_bits(qv[1]) && finite_bits(qv[2]) && finite_bits(qv[3]) &&
-                            positive_bits(qv[0]) && positive_bits(e2);
-            bad |= !ok;
+            if (!surely_physical(qv[0], qv[1], qv[2], qv[3])) {
+                const double e2 = rfma(qv[0] + qv[0], qv[3], -rfma(qv[1], qv[1], rmul(qv[2], qv[2])));
+                bad |= !(finite_bits(qv[0]) && finite_bits(qv[1]) && finite_bits(qv[2]) && finite_bits(qv[3]) &&
+                         positive_bits(qv[0]) && positive_bits(e2));
+            }
             if (P.lam_out)  // Sec. 2.5 wavespeed of the new state
                 lam = tmax_nan(lam, cell_wavespeed_t<T>(qv[0], qv[1], qv[2], qv[3], ph.gamma, ph.gm1, ph.mu,
                                                         inv_dx, inv_dy));
