@@ -26,8 +26,9 @@ void pack_sensor(const float* w, SensorDev* out)
     const float b3 = w3[kSensorH];
     for (int n = 0; n < kSensorH; ++n) {
         for (int k = 0; k < kSensorK; ++k)
-            out->w1t[n * kW1Pitch + k] = __float2bfloat16_rn(k < kSensorIn ? W1[k * kSensorH + n] : 0.f);
-        for (int k = 0; k < kSensorH; ++k) out->w2t[n * kW2Pitch + k] = __float2bfloat16_rn(W2[k * kSensorH + n]);
+            out->w1c[core_index(n, k, kSensorK / 8)] = __float2bfloat16_rn(k < kSensorIn ? W1[k * kSensorH + n] : 0.f);
+        for (int k = 0; k < kSensorH; ++k)
+            out->w2c[core_index(n, k, kSensorH / 8)] = __float2bfloat16_rn(W2[k * kSensorH + n]);
         out->b1[n] = b1[n];
         out->b2[n] = b2[n];
         out->w3[n] = w3[n];
@@ -60,9 +61,9 @@ struct SensorTileParams {
 
 // The staged region of one tile and the per-cell normalisation scales.
 struct SensorRegion {
-    float sr[kRH * kRW], sp[kRH * kRW];  // staged rho, p (tile + 2-cell halo)
-    float hr[2 * kRH * kTX], hp[2 * kRH * kTX];  // max, then min, over 5 columns
-    float scr[kTY * kTX], scp[kTY * kTX];  // per-cell normalisation scales
+    float2 q[kRH * kRW];   // staged rho, p (tile + 2-cell halo)
+    float4 h[kRH * kTX];   // over 5 columns: max and min of rho, max and min of p
+    float2 sc[kTY * kTX];  // per-cell normalisation scales of rho, p
 };
 
 // Stage the tile's region as FP32 rho, p exactly as the FP32 stage kernel
@@ -83,8 +84,7 @@ __device__ void sensor_stage(const SensorTileParams& P, const int tx0, const int
         const long long o = (long long)gy * P.g.pitch + gx;
         float r, u, v, pr;
         prims_of(P.q[o], P.q[o + P.g.plane], P.q[o + 2 * P.g.plane], P.q[o + 3 * P.g.plane], gm1, r, u, v, pr);
-        S.sr[idx] = r;
-        S.sp[idx] = pr;
+        S.q[idx] = make_float2(r, pr);
     }
     __syncthreads();
     if (scales) sensor_scales(S);
@@ -99,37 +99,27 @@ __device__ void sensor_scales(SensorRegion& S)
     // for bit.
     for (int idx = threadIdx.x; idx < kRH * kTX; idx += blockDim.x) {
         const int ry = idx / kTX, cx = idx - ry * kTX;
-        const float* r = S.sr + ry * kRW + cx;
-        const float* p = S.sp + ry * kRW + cx;
-        float rmx = r[0], rmn = r[0], pmx = p[0], pmn = p[0];
+        const float2* q = S.q + ry * kRW + cx;
+        float4 m = make_float4(q[0].x, q[0].x, q[0].y, q[0].y);
 #pragma unroll
         for (int d = 1; d < 5; ++d) {
-            rmx = fmaxf(rmx, r[d]);
-            rmn = fminf(rmn, r[d]);
-            pmx = fmaxf(pmx, p[d]);
-            pmn = fminf(pmn, p[d]);
+            const float2 v = q[d];
+            m = make_float4(fmaxf(m.x, v.x), fminf(m.y, v.x), fmaxf(m.z, v.y), fminf(m.w, v.y));
         }
-        S.hr[idx] = rmx;
-        S.hr[kRH * kTX + idx] = rmn;
-        S.hp[idx] = pmx;
-        S.hp[kRH * kTX + idx] = pmn;
+        S.h[idx] = m;
     }
     __syncthreads();
     for (int c = threadIdx.x; c < kTY * kTX; c += blockDim.x) {
         const int cy = c / kTX, cx = c - cy * kTX;
-        float rmx = S.hr[c], rmn = S.hr[kRH * kTX + c], pmx = S.hp[c], pmn = S.hp[kRH * kTX + c];
+        float4 m = S.h[c];
 #pragma unroll
         for (int d = 1; d < 5; ++d) {
-            const int o = c + d * kTX;
-            rmx = fmaxf(rmx, S.hr[o]);
-            rmn = fminf(rmn, S.hr[kRH * kTX + o]);
-            pmx = fmaxf(pmx, S.hp[o]);
-            pmn = fminf(pmn, S.hp[kRH * kTX + o]);
+            const float4 v = S.h[c + d * kTX];
+            m = make_float4(fmaxf(m.x, v.x), fminf(m.y, v.y), fmaxf(m.z, v.z), fminf(m.w, v.w));
         }
-        const float rc = S.sr[(cy + kH) * kRW + cx + kH], pc = S.sp[(cy + kH) * kRW + cx + kH];
-        const float mr = fmaxf(0.f, fmaxf(rmx - rc, rc - rmn)), mp = fmaxf(0.f, fmaxf(pmx - pc, pc - pmn));
-        S.scr[c] = 1.f / (mr + kSensorFloor);
-        S.scp[c] = 1.f / (mp + kSensorFloor);
+        const float2 q = S.q[(cy + kH) * kRW + cx + kH];
+        const float mr = fmaxf(0.f, fmaxf(m.x - q.x, q.x - m.y)), mp = fmaxf(0.f, fmaxf(m.z - q.y, q.y - m.w));
+        S.sc[c] = make_float2(1.f / (mr + kSensorFloor), 1.f / (mp + kSensorFloor));
     }
     __syncthreads();
 }
@@ -145,12 +135,12 @@ __device__ void sensor_dataset_tile(const SensorTileParams& P, const int tx0, co
         for (int c = threadIdx.x; c < kTX * kTY; c += blockDim.x) {
             const int cy = c / kTX, cx = c - cy * kTX, i = ty0 + cy, j = tx0 + cx;
             if (i >= ny || j >= nx) continue;
-            const float* r = S.sr + (cy + kH) * kRW + (cx + kH);
-            const float* p = S.sp + (cy + kH) * kRW + (cx + kH);
-            const float s1 = S.scr[c], s2 = S.scp[c];
+            const float* r = &S.q[(cy + kH) * kRW + (cx + kH)].x;
+            const float2 s = S.sc[c];
             uint32_t* out = reinterpret_cast<uint32_t*>(P.feat + ((long long)i * nx + j) * kSensorK);
             for (int k = 0; k < kSensorK; k += 2)
-                out[k / 2] = pack_bf16(sensor_feature(r, p, kRW, s1, s2, k), sensor_feature(r, p, kRW, s1, s2, k + 1));
+                out[k / 2] = pack_bf16(sensor_feature<2>(r, r + 1, kRW, s.x, s.y, k),
+                                       sensor_feature<2>(r, r + 1, kRW, s.x, s.y, k + 1));
         }
     }
     if (P.label || P.target) {  // plain detector in FP64 on the density (Eq. detector)
@@ -207,7 +197,7 @@ constexpr size_t tc_smem_bytes() { return G == 4 ? 80 * 1024 : (G == 2 ? 56 * 10
 // rounded down to even (16-byte aligned), 2 columns wider than the region.
 constexpr int kRawW = kRW + 2;
 constexpr size_t kRawBytes = sizeof(double) * 4 * kRawW * kRH;
-constexpr size_t kRegionScratch = sizeof(SensorRegion) - sizeof(float) * 2 * kRH * kRW;  // hr .. scp
+constexpr size_t kRegionScratch = sizeof(SensorRegion) - sizeof(float2) * kRH * kRW;  // h, sc
 
 struct TcSmem {
     // W1^T [32 n][64 k] and W2^T [32 n][32 k], BF16, K-major in 8 x 8 core
@@ -215,10 +205,13 @@ struct TcSmem {
     // (n/8, k/8) at ((n/8) * KG + k/8) * 128 bytes, KG = k-groups per row.
     alignas(128) __nv_bfloat16 w1c[kSensorH * kSensorK];
     alignas(128) __nv_bfloat16 w2c[kSensorH * kSensorH];
-    float b1[kSensorH], b2[kSensorH], w3[kSensorH], b3;
+    alignas(16) float b1[kSensorH];
+    alignas(16) float b2[kSensorH];
+    alignas(16) float w3[kSensorH];
+    float b3;
     alignas(8) unsigned long long mbar, tma_bar;
     unsigned taddr;
-    // the tensor copy lands on R.hr .. R.scp and the tail after them (free
+    // the tensor copy lands on R.h, R.sc and the tail after them (free
     // until the window maxima are formed, after the conversion)
     alignas(128) SensorRegion R;
     unsigned char raw_tail[kRawBytes > kRegionScratch ? kRawBytes - kRegionScratch : 1];
@@ -245,14 +238,7 @@ __device__ uint32_t tc_setup(const SensorDev* w, TcSmem& S)
 {
     constexpr int kThreads = 128 * G;
     const int tid = threadIdx.x;
-    for (int i = tid; i < kSensorH * kSensorK; i += kThreads) {
-        const int n = i / kSensorK, k = i - n * kSensorK;
-        S.w1c[core_index(n, k, kSensorK / 8)] = w->w1t[n * kW1Pitch + k];
-    }
-    for (int i = tid; i < kSensorH * kSensorH; i += kThreads) {
-        const int n = i / kSensorH, k = i - n * kSensorH;
-        S.w2c[core_index(n, k, kSensorH / 8)] = w->w2t[n * kW2Pitch + k];
-    }
+    copy_weights(w, S.w1c, S.w2c);
     if (tid < kSensorH) {
         S.b1[tid] = w->b1[tid];
         S.b2[tid] = w->b2[tid];
@@ -305,18 +291,29 @@ __device__ bool tc_tile(const SensorTileParams& P, const int tx0, const int ty0,
     const uint64_t d2 = tc_smem_desc(S.w2c, 128, 128 * (kSensorH / 8));
     for (int round = 0; round < kTX * kTY / kThreads; ++round) {
         const int c = round * kThreads + tid, cy = c / kTX, cx = c - cy * kTX;
-        const float* r = S.R.sr + (cy + kH) * kRW + (cx + kH);
-        const float* p = S.R.sp + (cy + kH) * kRW + (cx + kH);
-        const float sr = S.R.scr[c], sp = S.R.scp[c];
+        const float2* q = S.R.q + (cy + kH) * kRW + (cx + kH);
+        const float2 sc = S.R.sc[c], qc = q[0];
+        {
+            // rho and p features of a neighbour side by side (one 8-byte load,
+            // packed arithmetic; the values are sensor_feature's), BF16 pairs
+            // along each field: rho 0 .. 23, (rho 24, p 0), p 1 .. 24, zeros
+            uint32_t a[2][16];
+            float2 prev = make_float2(0.f, 0.f);
+            float p0 = 0.f;
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {  // features 32 half .. 32 half + 31
-            uint32_t a[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int k = 32 * half + 2 * j;
-                a[j] = pack_bf16(sensor_feature(r, p, kRW, sr, sp, k), sensor_feature(r, p, kRW, sr, sp, k + 1));
+            for (int k = 0; k < 25; ++k) {
+                const float2 v = q[(k / 5 - 2) * kRW + k % 5 - 2];
+                const float2 f = __fmul2_rn(__ffma2_rn(make_float2(-1.f, -1.f), qc, v), sc);
+                if (k == 0) p0 = f.y;
+                if (k == 24) a[0][12] = pack_bf16(f.x, p0);
+                if (k & 1) a[0][k / 2] = pack_bf16(prev.x, f.x);
+                else if (k > 0) a[(25 + k) / 2 / 16][(25 + k) / 2 % 16] = pack_bf16(prev.y, f.y);
+                prev = f;
             }
-            tc_st16(tm + lanes + kColA + 16 * half, a);
+#pragma unroll
+            for (int j = 25; j < 32; ++j) a[1][j - 16] = 0u;
+            tc_st16(tm + lanes + kColA, a[0]);
+            tc_st16(tm + lanes + kColA + 16, a[1]);
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         tc_fence_before();
@@ -341,10 +338,12 @@ __device__ bool tc_tile(const SensorTileParams& P, const int tx0, const int ty0,
             tc_ld16(tm + lanes + kColD + 16 * half, d);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int n = 16 * half + 2 * j;
-                h[8 * half + j] = pack_bf16(fmaxf(__uint_as_float(d[2 * j]) + S.b1[n], 0.f),
-                                            fmaxf(__uint_as_float(d[2 * j + 1]) + S.b1[n + 1], 0.f));
+            for (int j = 0; j < 4; ++j) {
+                const float4 b = reinterpret_cast<const float4*>(S.b1)[4 * half + j];
+                h[8 * half + 2 * j] = pack_bf16(fmaxf(__uint_as_float(d[4 * j]) + b.x, 0.f),
+                                                fmaxf(__uint_as_float(d[4 * j + 1]) + b.y, 0.f));
+                h[8 * half + 2 * j + 1] = pack_bf16(fmaxf(__uint_as_float(d[4 * j + 2]) + b.z, 0.f),
+                                                    fmaxf(__uint_as_float(d[4 * j + 3]) + b.w, 0.f));
             }
         }
         tc_st16(tm + lanes + kColA, h);
@@ -371,9 +370,13 @@ __device__ bool tc_tile(const SensorTileParams& P, const int tx0, const int ty0,
             tc_ld16(tm + lanes + kColD + 16 * half, d);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int n = 16 * half + j;
-                z += fmaxf(__uint_as_float(d[j]) + S.b2[n], 0.f) * S.w3[n];
+            for (int j = 0; j < 4; ++j) {
+                const float4 b = reinterpret_cast<const float4*>(S.b2)[4 * half + j];
+                const float4 v = reinterpret_cast<const float4*>(S.w3)[4 * half + j];
+                z += fmaxf(__uint_as_float(d[4 * j]) + b.x, 0.f) * v.x;
+                z += fmaxf(__uint_as_float(d[4 * j + 1]) + b.y, 0.f) * v.y;
+                z += fmaxf(__uint_as_float(d[4 * j + 2]) + b.z, 0.f) * v.z;
+                z += fmaxf(__uint_as_float(d[4 * j + 3]) + b.w, 0.f) * v.w;
             }
         }
         const float pv = 1.f / (1.f + expf(-(z + S.b3)));
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__(128 * G, 8 / G)
     const int org = P.dec ? kDecOrigin : kGhost;
     const int gx0 = tx0 + org - kH, gy0 = ty0 + org - kH;  // padded coordinates of region cell (0, 0)
     const int xa = gx0 & ~1, ox = gx0 - xa;                // 16-byte aligned copy origin
-    double* raw = reinterpret_cast<double*>(S.R.hr);
+    double* raw = reinterpret_cast<double*>(S.R.h);
     const bool tma = (smem_addr(raw) & 127u) == 0;         // uniform: the copy needs 128-byte alignment
     if (tid == 0) {
         mbar_init(&S.mbar, 1);
@@ -436,8 +439,7 @@ __global__ void __launch_bounds__(128 * G, 8 / G)
                 const int o = ry * kRawW + rx + ox;
                 float r, u, v, pr;
                 prims_of(raw[o], raw[plane + o], raw[2 * plane + o], raw[3 * plane + o], gm1, r, u, v, pr);
-                S.R.sr[idx] = r;
-                S.R.sp[idx] = pr;
+                S.R.q[idx] = make_float2(r, pr);
             }
             __syncthreads();
             sensor_scales(S.R);

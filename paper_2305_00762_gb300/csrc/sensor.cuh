@@ -22,8 +22,13 @@ constexpr int kSensorK = 64;      // padded input width
 constexpr int kSensorH = 32;      // hidden width
 // Row pitches of the transposed weights in the device copy (the kernels
 // re-order them into the tensor cores' core-matrix layout in shared memory).
-constexpr int kW1Pitch = kSensorK + 8;
-constexpr int kW2Pitch = kSensorH + 8;
+// Position of element (n, k) of a K-major operand in 8 x 8 core matrices (8
+// rows of 16 bytes each) with kgroups of them along k: the tensor cores'
+// shared-memory layout without swizzle.
+__host__ __device__ constexpr int core_index(int n, int k, int kgroups)
+{
+    return ((n >> 3) * kgroups + (k >> 3)) * 64 + (n & 7) * 8 + (k & 7);
+}
 constexpr float kSensorFloor = 1e-3f;
 constexpr float kSensorLo = 0.3f;  // p < lo: smooth
 constexpr float kSensorHi = 0.7f;  // p > hi: discontinuity; otherwise the plain detector decides
@@ -35,13 +40,22 @@ constexpr double kSensorTau = 0.02;
 // Host weight vector: W1[50][32], b1[32], W2[32][32], b2[32], w3[32], b3.
 constexpr int kSensorParams = kSensorIn * kSensorH + kSensorH + kSensorH * kSensorH + kSensorH + kSensorH + 1;
 
-// Device copy used by the kernels: W1 and W2 transposed (n-major, k
-// contiguous) and rounded to BF16; biases and the output layer in FP32.
-struct SensorDev {
-    __nv_bfloat16 w1t[kSensorH * kW1Pitch];  // [n][k], k >= 50 zero
-    __nv_bfloat16 w2t[kSensorH * kW2Pitch];  // [n][k]
+// Device copy used by the kernels: W1^T [n][k] (k >= 50 zero) and W2^T [n][k]
+// rounded to BF16, already in core-matrix order so that a CTA copies them as
+// they are; biases and the output layer in FP32.
+struct alignas(16) SensorDev {
+    __nv_bfloat16 w1c[kSensorH * kSensorK];
+    __nv_bfloat16 w2c[kSensorH * kSensorH];
     float b1[kSensorH], b2[kSensorH], w3[kSensorH], b3, pad[3];
 };
+// The weights into shared memory (16-byte aligned), by the whole block.
+__device__ __forceinline__ void copy_weights(const SensorDev* w, __nv_bfloat16* w1c, __nv_bfloat16* w2c)
+{
+    constexpr int n1 = kSensorH * kSensorK / 8, n2 = kSensorH * kSensorH / 8;
+    const uint4* a = reinterpret_cast<const uint4*>(w->w1c);  // w2c follows w1c
+    for (int i = threadIdx.x; i < n1 + n2; i += blockDim.x)
+        (i < n1 ? reinterpret_cast<uint4*>(w1c)[i] : reinterpret_cast<uint4*>(w2c)[i - n1]) = a[i];
+}
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 {
@@ -49,16 +63,18 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// Feature k of a cell (0 <= k < 64) given its scales.
+// Feature k of a cell (0 <= k < 64) given its scales; ES: the values' distance
+// in floats along a row, rows st cells apart.
+template <int ES = 1>
 __device__ __forceinline__ float sensor_feature(const float* r, const float* p, int st, float sr, float sp, int k)
 {
     if (k < 25) {
         const int dy = k / 5 - 2, dx = k % 5 - 2;
-        return (r[dy * st + dx] - r[0]) * sr;
+        return (r[(dy * st + dx) * ES] - r[0]) * sr;
     }
     if (k < 50) {
         const int kk = k - 25, dy = kk / 5 - 2, dx = kk % 5 - 2;
-        return (p[dy * st + dx] - p[0]) * sp;
+        return (p[(dy * st + dx) * ES] - p[0]) * sp;
     }
     return 0.f;
 }

@@ -1000,11 +1000,6 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
 // accumulators of both layers in turn).
 constexpr unsigned kColA = 0, kColD = 32, kColsPerGroup = 64;
 
-__host__ __device__ constexpr int core_index(int n, int k, int kgroups)
-{
-    return ((n >> 3) * kgroups + (k >> 3)) * 64 + (n & 7) * 8 + (k & 7);
-}
-
 // Shared-memory matrix descriptor (no swizzle, K-major core matrices):
 // start address, leading byte offset (between core matrices adjacent in K),
 // stride byte offset (between adjacent 8-row groups), descriptor version 1.
@@ -1114,14 +1109,7 @@ __device__ bool fused_sensor_decisions(const StageParams& P, const float* sU, un
     __shared__ __align__(8) unsigned long long mma_bar;  // never reused for anything else
     __shared__ unsigned tmem_base;
     const SensorDev* w = P.sensor;
-    for (int i = tid; i < kSensorH * kSensorK; i += NT) {
-        const int n = i / kSensorK, k = i - n * kSensorK;
-        w1c[core_index(n, k, kSensorK / 8)] = w->w1t[n * kW1Pitch + k];
-    }
-    for (int i = tid; i < kSensorH * kSensorH; i += NT) {
-        const int n = i / kSensorH, k = i - n * kSensorH;
-        w2c[core_index(n, k, kSensorH / 8)] = w->w2t[n * kW2Pitch + k];
-    }
+    copy_weights(w, w1c, w2c);
     if (tid < kSensorH) {
         b1[tid] = w->b1[tid];
         b2[tid] = w->b2[tid];
