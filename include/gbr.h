@@ -165,7 +165,8 @@ typedef enum {
 /* Kernel classes reported by gbr_get_timing. */
 typedef enum {
     GBR_KERNEL_STAGE = 0, /* fused residual + stage update (or residual only) */
-    GBR_KERNEL_GHOST = 1, /* ghost-cell fill (+ per-step scalars) */
+    GBR_KERNEL_GHOST = 1, /* ghost-cell fill (+ per-step scalars); none on small FP64 grids, whose
+                           * stages read ghost cells through the boundary rules */
     GBR_KERNEL_WAVESPEED = 2, /* standalone CFL wavespeed reduction */
     GBR_KERNEL_CLASSES = 3
 } gbr_kernel_class;

@@ -15,24 +15,9 @@ __global__ void ghost_kernel(const GhostParams P)
     dependent_start();
     const long long total = ghost_count(P.g);
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id == 0 && P.mode != 0) {
-        DevScalars* d = P.ds;
-        double dt = P.dt;
-        if (P.mode == 2) {
-            const double lam = __longlong_as_double((long long)d->lam[P.cur]);
-            dt = fmin(P.cfl / lam, P.dt_max);
-        }
-        d->dt = dt;
-        d->t += dt;
-        d->ts[P.next] = d->ts[P.cur] + dt;
-        d->lam[P.next] = 0ull;
-    }
+    if (id == 0 && P.mode != 0) begin_step(P);
     if (id >= total) return;
-    // Boundary time of this stage: the step's start time ts[cur] (not written
-    // by this launch) plus c_stage dt (dt was written by an earlier launch
-    // whenever c_stage != 0).
-    const double t = P.ds->ts[P.cur] + (P.c_stage != 0.0 ? P.c_stage * P.ds->dt : 0.0);
-    fill_ghost(P.g, P.q, P.bc, id, P.side, P.dx, P.dy, t);
+    fill_ghost(P.g, P.q, P.bc, id, P.side, P.dx, P.dy, boundary_time(P));
 }
 
 // Simulated time of the current state: the reported time and the step start

@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2) batch_stage_kernel
             P.dec = C.dec;
             P.stall_bytes = 0;
             P.stall_mma = 0;
+            P.map = 0;
         }
         __syncthreads();
         if constexpr (sizeof(T) == 8) fixed_tile<BX, BY, NT, false, 7, false>(P, tx * BX, ty * BY, smem_raw);

@@ -65,7 +65,7 @@ __device__ __forceinline__ bool trouble_filtered(const float* r, int st, F exact
     return exact();  // (also where a density overflows FP32)
 }
 
-template <int BX, int BY, int NT, bool VISC, int ORDER, bool TMA, bool CONS = false>
+template <int BX, int BY, int NT, bool VISC, int ORDER, bool TMA, bool CONS = false, bool MAP = false>
 __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, const int ty0, unsigned char* smem,
                                            const CUtensorMap* tmap = nullptr)
 {
@@ -100,10 +100,12 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     ph.lm = P.ph.riemann;
     const double inv_dx = P.ph.inv_dx, inv_dy = P.ph.inv_dy;
     const fx::Pos gamma = fx::pos(ph.gamma), gm1 = fx::pos(ph.gm1);
+    __shared__ double step_dt;
+    stage_scalars<MAP>(P, &step_dt);
 
     // Phase 0: primitives (Eq. pressure) and cell fluxes F^c = (rho u, rho u u
     // + p, rho u v, u (E + p)), G^c (Sec. 1; rho u, rho v, E from the state).
-    const bool staged = stage_region<BX, BY, NT, X, TMA>(
+    const bool staged = stage_region<BX, BY, NT, X, TMA, MAP>(
         P, tx0, ty0, reinterpret_cast<double*>(smem + F::oRaw), tmap,
         [&](int idx, double q0, double q1, double q2, double q3) {
             fx::Cell w;
@@ -366,8 +368,14 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         }
     }
     __syncthreads();
-    finish_tile<double, BX, BY, NT>(P, ph, inv_dx, inv_dy, tx0, ty0, sHX, sHY);
+    finish_tile<double, BX, BY, NT>(P, step_dt, ph, inv_dx, inv_dy, tx0, ty0, sHX, sHY);
 }
+
+// The instances of the smallest tile read ghost cells through the boundary
+// rules: on the grids that take it a ghost fill before every stage is a
+// quarter of the step (64^2: 57 -> 49 us without), where in the larger tiles the
+// code for it costs registers that they need (1024^2 2.0% slower with it).
+constexpr bool fixed_maps_ghosts(int bx) { return bx == 8; }
 
 // One CTA per tile, two CTAs per SM (viscous MEG7-cons: one, by shared memory).
 template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS>
@@ -376,7 +384,7 @@ __global__ void __launch_bounds__(NT, CONS && VISC ? 1 : 2)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     dependent_start();
-    fixed_tile<BX, BY, NT, VISC, ORDER, true, CONS>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
+    fixed_tile<BX, BY, NT, VISC, ORDER, true, CONS, fixed_maps_ghosts(BX)>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
 }
 
 template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS>
@@ -410,8 +418,7 @@ cudaError_t launch_fixed_tiles(const StageParams& p, cudaStream_t s)
 // 16 x 15, 205 / 267 us with the others); the smallest c k is taken, k rounded
 // up while it is small and the last wave counts. The result does not depend on
 // the shape.
-template <bool VISC, int ORDER, bool CONS = false>
-cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
+inline cudaError_t fixed_tile_shape(const Grid& g, TileShape* t)
 {
     static PerDevice<int> sm_count;
     int sms = 0;
@@ -422,13 +429,23 @@ cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
     });
     if (e != cudaSuccess) return e;
     auto cost = [&](int bx, int by, double c) {
-        const double k = (double)((p.g.nx + bx - 1) / bx) * ((p.g.ny + by - 1) / by) / sms;
+        const double k = (double)((g.nx + bx - 1) / bx) * ((g.ny + by - 1) / by) / sms;
         const double up = (double)(long long)k;
         return c * (k <= 16.0 ? (k > up ? up + 1.0 : up) : k + 0.5);
     };
     const double big = cost(16, 15, 63.0), mid = cost(16, 8, 36.5), tiny = cost(8, 4, 15.5);
-    if (tiny < mid && tiny < big) return launch_fixed_tiles<8, 4, 96, VISC, ORDER, CONS>(p, s);
-    if (mid < big) return launch_fixed_tiles<16, 8, 288, VISC, ORDER, CONS>(p, s);
+    *t = tiny < mid && tiny < big ? TileShape{8, 4} : mid < big ? TileShape{16, 8} : TileShape{16, 15};
+    return cudaSuccess;
+}
+
+template <bool VISC, int ORDER, bool CONS = false>
+cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
+{
+    TileShape t;
+    const cudaError_t e = fixed_tile_shape(p.g, &t);
+    if (e != cudaSuccess) return e;
+    if (t.bx == 8) return launch_fixed_tiles<8, 4, 96, VISC, ORDER, CONS>(p, s);
+    if (t.by == 8) return launch_fixed_tiles<16, 8, 288, VISC, ORDER, CONS>(p, s);
     return launch_fixed_tiles<16, 15, 256, VISC, ORDER, CONS>(p, s);
 }
 

@@ -158,9 +158,8 @@ struct Timed {
     }
 };
 
-int ghosts(gbr_ctx* c, double* q, int mode, double dt, double cfl, double dt_max, double c_stage = 0.0)
+GhostParams ghost_params(gbr_ctx* c, double* q, int mode, double dt, double cfl, double dt_max, double c_stage)
 {
-    Timed tm(c, GBR_KERNEL_GHOST);
     GhostParams p;
     memset(&p, 0, sizeof(p));
     p.g = c->g;
@@ -177,7 +176,25 @@ int ghosts(gbr_ctx* c, double* q, int mode, double dt, double cfl, double dt_max
     p.dt = dt;
     p.cfl = cfl;
     p.dt_max = dt_max;
-    return cuda_status(launch_ghosts(p, c->stream));
+    return p;
+}
+
+int ghosts(gbr_ctx* c, double* q, int mode, double dt, double cfl, double dt_max, double c_stage = 0.0)
+{
+    Timed tm(c, GBR_KERNEL_GHOST);
+    return cuda_status(launch_ghosts(ghost_params(c, q, mode, dt, cfl, dt_max, c_stage), c->stream));
+}
+
+// Before a stage reads the state q: its ghost cells are filled, or, on small
+// FP64 grids, left to the stage to read through the boundary rules (p.map).
+int stage_ghosts(gbr_ctx* c, StageParams& p, double* q, int mode, double dt, double cfl, double dt_max, double c_stage)
+{
+    bool maps = false;
+    if (c->precision == 64) GBR_TRY(stage_f64_maps_ghosts(c->g, &maps));
+    if (!maps) return ghosts(c, q, mode, dt, cfl, dt_max, c_stage);
+    p.map = 1;
+    p.gh = ghost_params(c, q, mode, dt, cfl, dt_max, c_stage);
+    return GBR_OK;
 }
 
 StageParams stage_params(gbr_ctx* c, const double* q)
@@ -232,8 +249,8 @@ int rk3_stage(gbr_ctx* c, int k, int mode, double dt, double cfl, double dt_max)
     static const double c_stage[3] = {0.0, 1.0, 0.5};
     int rc;
     double* in = stage_input(c, k);
-    if ((rc = ghosts(c, in, k == 0 ? mode : 0, dt, cfl, dt_max, c_stage[k])) != GBR_OK) return rc;
     StageParams p = stage_params(c, in);
+    if ((rc = stage_ghosts(c, p, in, k == 0 ? mode : 0, dt, cfl, dt_max, c_stage[k])) != GBR_OK) return rc;
     p.qout = k == 2 ? c->Qn : stage_input(c, k + 1);  // stage 3: each cell reads its own Q^n before writing it
     p.dt = dt;
     p.dt_ptr = (mode == 2) ? &c->ds->dt : nullptr;
@@ -395,9 +412,9 @@ int gbr_residual(gbr_ctx* c, double* res, int on_device)
     Range r("gbr residual");
     if (!c->have_state) return GBR_ERR_STATE;
     DeviceGuard dg(c->device);
-    int rc = ghosts(c, c->Qn, 0, 0, 0, 0);
-    if (rc != GBR_OK) return rc;
     StageParams p = stage_params(c, c->Qn);
+    int rc = stage_ghosts(c, p, c->Qn, 0, 0, 0, 0, 0.0);
+    if (rc != GBR_OK) return rc;
     p.res = on_device ? res : c->R;
     if ((rc = stage(c, p)) != GBR_OK) return rc;
     if (on_device) return GBR_OK;

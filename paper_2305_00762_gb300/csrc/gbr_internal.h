@@ -129,6 +129,22 @@ inline void derive_physics(Physics& ph)
 
 struct SensorDev;
 
+// Ghost fill of one padded state, plus the per-step scalar bookkeeping done
+// by its first thread (mode 1: add dt to t and clear lam[next]; mode 2: form
+// dt = min(cfl / lam[cur], dt_max) on the device first).
+struct GhostParams {
+    Grid g;
+    double* q;
+    int bc[4];  // west, east, south, north
+    DevScalars* ds;
+    int mode;
+    int cur, next;
+    double dt, cfl, dt_max;
+    SideBC side[4];     // GBR_BC_CUSTOM sides
+    double dx, dy;      // cell sizes (positions along custom sides)
+    double c_stage;     // stage abscissa: the boundary time is ts[cur] + c_stage dt
+};
+
 // One fused residual (+ stage update) pass, Secs. 2.1-2.5.
 struct StageParams {
     Grid g;
@@ -148,22 +164,13 @@ struct StageParams {
     const unsigned char* dec;  // learned-sensor decisions of padded cells [3, n+9) (pitch g.pitch), with sensor
     unsigned stall_bytes;    // failure-detection test hook: extra bytes the tile staging waits for (0)
     unsigned stall_mma;      // failure-detection test hook: the fused sensor withholds its first MMA batch (0)
-};
-
-// Ghost fill of one padded state, plus the per-step scalar bookkeeping done
-// by its first thread (mode 1: add dt to t and clear lam[next]; mode 2: form
-// dt = min(cfl / lam[cur], dt_max) on the device first).
-struct GhostParams {
-    Grid g;
-    double* q;
-    int bc[4];  // west, east, south, north
-    DevScalars* ds;
-    int mode;
-    int cur, next;
-    double dt, cfl, dt_max;
-    SideBC side[4];     // GBR_BC_CUSTOM sides
-    double dx, dy;      // cell sizes (positions along custom sides)
-    double c_stage;     // stage abscissa: the boundary time is ts[cur] + c_stage dt
+    // 1 (small FP64 grids, see stage_f64_maps_ghosts): the ghost cells of q are
+    // not in memory; the stage reads each one a tile needs through the boundary
+    // rules of gh (a halo side's rows excepted), takes a mode-2 step's dt from the
+    // wavespeed and does the step's scalars, as the ghost kernel does. 0: a
+    // ghost fill came before.
+    int map;
+    GhostParams gh;
 };
 
 // One grid of a batch, as the device sees it. tiles_x / tile_begin describe
@@ -241,6 +248,9 @@ cudaError_t launch_sensor_train(const void* X_bf16, const unsigned char* y, long
 cudaError_t launch_wavespeed(const Grid& g, const Physics& ph, const double* q, unsigned long long* lam,
                              int precision, cudaStream_t s);
 cudaError_t launch_stage_f64(const StageParams& p, cudaStream_t s);
+// Whether the FP64 stage of this grid can read ghost cells through the boundary
+// rules (StageParams::map).
+cudaError_t stage_f64_maps_ghosts(const Grid& g, bool* maps);
 cudaError_t launch_stage_f32(const StageParams& p, cudaStream_t s);
 cudaError_t launch_stage_viscous_f64(const StageParams& p, cudaStream_t s);
 cudaError_t launch_stage_order4_f64(const StageParams& p, cudaStream_t s);

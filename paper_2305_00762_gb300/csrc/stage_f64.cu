@@ -4,6 +4,14 @@
 
 namespace gbr {
 
+cudaError_t stage_f64_maps_ghosts(const Grid& g, bool* maps)
+{
+    TileShape t;
+    const cudaError_t e = fixed_tile_shape(g, &t);
+    if (e == cudaSuccess) *maps = fixed_maps_ghosts(t.bx);
+    return e;
+}
+
 cudaError_t launch_stage_f64(const StageParams& p, cudaStream_t s)
 {
     if (p.ph.cons) return launch_stage_cons_f64(p, s);

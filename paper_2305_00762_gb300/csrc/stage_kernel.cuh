@@ -23,6 +23,7 @@
 #include "fixed_math.cuh"
 #include "fp_convert.cuh"
 #include "gbr_internal.h"
+#include "ghost.cuh"
 #include "sensor.cuh"
 
 namespace gbr {
@@ -1279,13 +1280,24 @@ __device__ bool fused_sensor_decisions(const StageParams& P, const float* sU, un
 // (128-byte aligned; else plain loads); cells beyond the padded extent (ragged
 // last tiles) read as zero there, as the clamped cell otherwise, and only feed
 // results that are never stored. False: the copy's bounded wait gave up
-// (uniform over the CTA; the error word is set).
-template <int BX, int BY, int NT, typename X, bool TMA, typename F>
+// (uniform over the CTA; the error word is set). MAP: the instance can read
+// ghost cells through the boundary rules (StageParams::map).
+template <int BX, int BY, int NT, typename X, bool TMA, bool MAP, typename F>
 __device__ __forceinline__ bool stage_region(const StageParams& P, int tx0, int ty0, double* raw,
                                              const CUtensorMap* tmap, F stage_cell)
 {
     constexpr int RW = BX + 12, RH = BY + 12, NU = RW * RH;
     const int tid = threadIdx.x;
+    const bool map = MAP && P.map;
+    const double bt = map ? boundary_time(P.gh) : 0.0;
+    auto mapped = [&](int idx, double (&v)[4]) {  // false: not a ghost cell, or one that is in memory
+        if constexpr (!MAP) return false;
+        const int ry = idx / RW, rx = idx - ry * RW;
+        const int gx = tx0 + rx, gy = ty0 + ry;
+        if (gx >= P.g.nx + 2 * kGhost || gy >= P.g.ny + 2 * kGhost) return false;
+        if (gx >= kGhost && gx < P.g.nx + kGhost && gy >= kGhost && gy < P.g.ny + kGhost) return false;
+        return ghost_value(P.g, P.q, P.gh.bc, gx, gy, P.gh.side, P.gh.dx, P.gh.dy, bt, v);
+    };
     if constexpr (TMA) {
         static_assert(BX % 2 == 0 && RW % 2 == 0, "TMA x offsets and rows must be 16-byte multiples");
         static_assert(RW <= 256 && RH <= 256, "TMA box too large");
@@ -1316,7 +1328,12 @@ __device__ __forceinline__ bool stage_region(const StageParams& P, int tx0, int 
             }
             for (int e = tid; e < X::N; e += NT) {
                 const int idx = X::cell(e);
-                stage_cell(idx, raw[idx], raw[NU + idx], raw[2 * NU + idx], raw[3 * NU + idx]);
+                double v[4];
+                if (!(map && mapped(idx, v))) {
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) v[m] = raw[m * NU + idx];
+                }
+                stage_cell(idx, v[0], v[1], v[2], v[3]);
             }
             return true;
         }
@@ -1330,9 +1347,28 @@ __device__ __forceinline__ bool stage_region(const StageParams& P, int tx0, int 
         const int gx = min(tx0 + rx, P.g.nx + 2 * kGhost - 1);
         const int gy = min(ty0 + ry, P.g.ny + 2 * kGhost - 1);
         const long long o = (long long)gy * pitch + gx;
-        stage_cell(idx, P.q[o], P.q[o + plane], P.q[o + 2 * plane], P.q[o + 3 * plane]);
+        double v[4];
+        if (!(map && mapped(idx, v))) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v[m] = P.q[o + m * plane];
+        }
+        stage_cell(idx, v[0], v[1], v[2], v[3]);
     }
     return true;
+}
+
+// The stage's step size for the whole block (in shared memory, after the next
+// barrier), and the scalars of a step that begins with this stage.
+template <bool MAP>
+__device__ __forceinline__ void stage_scalars(const StageParams& P, double* dt)
+{
+    if (threadIdx.x != 0) return;
+    if (MAP && P.map && P.gh.mode != 0) {
+        *dt = step_size(P.gh);
+        if (blockIdx.x == 0 && blockIdx.y == 0) begin_step(P.gh);
+    } else {
+        *dt = P.dt_ptr ? *P.dt_ptr : P.dt;
+    }
 }
 
 // The four components of face e: planes of n values in FP64, float4 in FP32.
@@ -1354,7 +1390,7 @@ __device__ __forceinline__ void load_face(const float* h, int, int e, float (&v)
 // [BY + 1][BX] in shared memory, written before the caller's barrier); ends
 // with all threads synchronised.
 template <typename T, int BX, int BY, int NT>
-__device__ __forceinline__ void finish_tile(const StageParams& P, const PhysT<T>& ph, T inv_dx, T inv_dy, int tx0, int ty0,
+__device__ __forceinline__ void finish_tile(const StageParams& P, double dt, const PhysT<T>& ph, T inv_dx, T inv_dy, int tx0, int ty0,
                                             const T* sHX, const T* sHY)
 {
     constexpr int NHX = (BX + 1) * BY, NHY = BX * (BY + 1);
@@ -1362,7 +1398,6 @@ __device__ __forceinline__ void finish_tile(const StageParams& P, const PhysT<T>
     const long long plane = P.g.plane;
     const int tid = threadIdx.x;
     // Phase 3: residual (Eq. deriv) and the FP64 stage update (Eq. rk).
-    const double dt = P.dt_ptr ? *P.dt_ptr : P.dt;
     const double cdt = P.cc * dt;
     constexpr bool kScaled = sizeof(T) == 8;
     const T sx = kScaled && P.qout ? T(cdt) * inv_dx : inv_dx, sy = kScaled && P.qout ? T(cdt) * inv_dy : inv_dy;
@@ -1471,6 +1506,8 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     ph.kq = P.ph.f32.kq;
     ph.lm = P.ph.riemann;
     const T inv_dx = P.ph.f32.inv_dx, inv_dy = P.ph.f32.inv_dy;
+    __shared__ double step_dt;
+    stage_scalars<false>(P, &step_dt);
 
     // Phase 0: stage the tile + halo as primitive variables (Eq. pressure).
     // Region cell (rx, ry) is padded cell (tx0 + rx, ty0 + ry).
@@ -1490,7 +1527,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     };
     static_assert(!TMA || L::template raw_offset<T>() + L::kRawBytes <= L::template raw_limit<T>(),
                   "TMA landing area overlaps live shared memory");
-    if (!stage_region<BX, BY, NT, X, TMA>(P, tx0, ty0, reinterpret_cast<double*>(smem_raw + L::template raw_offset<T>()), tmap,
+    if (!stage_region<BX, BY, NT, X, TMA, false>(P, tx0, ty0, reinterpret_cast<double*>(smem_raw + L::template raw_offset<T>()), tmap,
                                           stage_cell))
         return;
     if constexpr (LEARNED == 1) {
@@ -1702,7 +1739,7 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     }
     __syncthreads();
 
-    finish_tile<T, BX, BY, NT>(P, ph, inv_dx, inv_dy, tx0, ty0, sm + L::oHX, sm + L::oHY);
+    finish_tile<T, BX, BY, NT>(P, step_dt, ph, inv_dx, inv_dy, tx0, ty0, sm + L::oHX, sm + L::oHY);
 }
 
 // One CTA per tile; the tile + halo is staged by a tensor copy described by
