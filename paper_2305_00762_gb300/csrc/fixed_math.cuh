@@ -172,7 +172,7 @@ GBR_HD double to_double(const Pos& x)  // 1 <= e <= 2045
 // E) on the integer pipe, as split values (integer of at most kBits bits, not
 // necessarily normalised, and biased exponent): u = rho u / rho, v likewise, p
 // = (gamma - 1) (E - (rho u u + rho v v) / 2). An FP64 evaluation rounds every
-// step at 53 bits; here the steps keep 58 or more. A density that is not
+// step at 53 bits; here the steps keep 55 or more of their largest term. A density that is not
 // positive and normal, or a value that is not finite, gives exponents that every
 // later stencil refuses.
 struct Split {
@@ -227,18 +227,18 @@ GBR_HD void cell_of(double q0, double q1, double q2, double q3, const Pos& gm1, 
     const Split E = split(q3);
     const u64 y = rcp_mantissa((u64)c.r.m << (64 - kBits));  // half of 2^1023 / rho in units of 2^(-64 - e)
     const bool bad = c.r.m <= 0 || larger(larger(c.r.e, c.ru.e), larger(c.rv.e, E.e)) == 2047;
-    const int er = bad ? -4096 : 1024 - c.r.e;
-    c.u.m = mulhi(c.ru.m, y);
+    const int er = bad ? -4096 : 1023 - c.r.e;
+    c.u.m = mulhi(c.ru.m, y) << 1;  // (the products below keep what their factors' leading bits leave)
     c.u.e = c.ru.e + er;
-    c.v.m = mulhi(c.rv.m, y);
+    c.v.m = mulhi(c.rv.m, y) << 1;
     c.v.e = c.rv.e + er;
     c.ruu = product(c.ru, c.u);
     c.rvv = product(c.rv, c.v);
     Split t;  // E - (rho u u + rho v v) / 2
     t.e = larger(E.e, larger(c.ruu.e, c.rvv.e) - 1) + 1;
     t.m = aligned(E.m, E.e, t.e) - aligned(c.ruu.m, c.ruu.e - 1, t.e) - aligned(c.rvv.m, c.rvv.e - 1, t.e);
-    c.p.m = mulhi(t.m, gm1.m >> 1);
-    c.p.e = t.e + gm1.e - 1021;
+    c.p.m = mulhi(t.m, gm1.m >> 1) << 1;
+    c.p.e = t.e + gm1.e - 1022;
     if (bad) c.r.e = c.u.e = c.v.e = c.p.e = 2047;
     c.h = sum(E, c.p);
 }
