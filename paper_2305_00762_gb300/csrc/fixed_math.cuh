@@ -237,8 +237,8 @@ GBR_HD void cell_of(double q0, double q1, double q2, double q3, const Pos& gm1, 
     Split t;  // E - (rho u u + rho v v) / 2
     t.e = larger(E.e, larger(c.ruu.e, c.rvv.e) - 1) + 1;
     t.m = aligned(E.m, E.e, t.e) - aligned(c.ruu.m, c.ruu.e - 1, t.e) - aligned(c.rvv.m, c.rvv.e - 1, t.e);
-    c.p.m = mulhi(t.m, gm1.m >> 1) << 1;
-    c.p.e = t.e + gm1.e - 1022;
+    c.p.m = mulhi(t.m, gm1.m >> 1);
+    c.p.e = t.e + gm1.e - 1021;
     if (bad) c.r.e = c.u.e = c.v.e = c.p.e = 2047;
     c.h = sum(E, c.p);
 }
