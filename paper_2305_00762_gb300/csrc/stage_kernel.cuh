@@ -491,6 +491,8 @@ struct PhysT {
     int lm;                      // 1: shock-stable HLLC-LM dissipation
 };
 
+__device__ __forceinline__ bool no_value(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
+
 // HLLC in the form 1/2 (F_L + F_R) - 1/2 |A| (Q_R - Q_L), Eq. Riemann_revisit,
 // from the face states (rho, un, ut, p). The central part is Fs (flux
 // reconstruction) where `smooth`, else F(Q_L), F(Q_R) of the states
@@ -537,7 +539,10 @@ __device__ __forceinline__ void hllc_flux(const PhysT<double>& P, bool smooth, c
     const T SR = tmax(unR + cR, ut + ct);
     const T mL = rmul(rL, SL - unL), mR = rmul(rR, SR - unR);
     const T num = rfma(-mR, unR, rfma(mL, unL, pR - pL)), den = mL - mR;  // S* = num / den
-    const T Ss = rmul(num, trcp(den)), iL = trcp(SL - Ss), iR = trcp(SR - Ss);
+    // A state without a speed of sound (rho p <= 0, a NaN) has no flux: tmin and
+    // tmax may drop its NaN, so S* carries it into every component.
+    const bool none = no_value(cL) || no_value(cR);
+    const T Ss = none ? rmul(cL, cR) : rmul(num, trcp(den)), iL = trcp(SL - Ss), iR = trcp(SR - Ss);
     T aL = thalfabs(SL), aR = thalfabs(SR);
     const T aS = thalfabs(Ss);
     if (P.lm) {

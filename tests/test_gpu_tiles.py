@@ -70,3 +70,28 @@ def test_residual_does_not_depend_on_the_shape(env, form):
     ref = out[271]
     for R in out.values():
         assert np.array_equal(R, ref)
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("size", ["8x4", "16x8"])
+def test_no_flux_from_a_state_without_sound(env, size, form):
+    """A fast cell of negative pressure: the mean pressure with a neighbour is
+    negative too, so each of its faces falls back to the cells' own states; the
+    Roe average has a speed of sound (the velocities differ), the cell has none.
+    Such a face has no flux: NaN in every component, not the finite remainder of
+    a minimum that drops a NaN. The step reports the state."""
+    torch, O, gbr = env
+    nx, ny = SIZES[size]
+    c = make(form, nx, ny)
+    Q = c.Q.copy()
+    r, p = Q[0], 0.4 * (Q[3] - 0.5 * (Q[1] ** 2 + Q[2] ** 2) / Q[0])
+    u, v = Q[1, 10, 18] / r[10, 18] + 50.0, Q[2, 10, 18] / r[10, 18] + 50.0
+    Q[1:, 10, 18] = r[10, 18] * u, r[10, 18] * v, 0.5 * r[10, 18] * (u * u + v * v) - 5.0 * p[9:12, 17:20].max()
+    s = gbr.Solver.for_case(c, **FORMS[form])
+    s.set_state(Q)
+    s.step(1e-9)
+    assert s.sync(allow=(gbr.GBR_ERR_NONPHYSICAL,)) == gbr.GBR_ERR_NONPHYSICAL
+    out = s.get_state(allow=(gbr.GBR_ERR_NONPHYSICAL,))
+    for j, i in ((10, 18), (9, 18), (11, 18), (10, 17), (10, 19)):
+        assert np.isnan(out[:, j, i]).all(), (j, i)
+    s.close()
