@@ -398,16 +398,33 @@ struct FaceStates {
     bool ok;  // false: a stencil value too large, infinite or NaN
 };
 
+// Field 3 (shear) is ut itself. Returns whether its stencil is in range.
+template <int ORDER, typename F>
+GBR_HD bool shear_states(F load, double (&ut)[2])
+{
+    Stencil x;
+    load(2, x);
+    const int e = stencil_exponent(x);
+    Functionals R;
+    variable<ORDER>(x, e, R);
+    i64 l, r;
+    limited<ORDER>(R, l, r);
+    ut[0] = to_double(l, e);
+    ut[1] = to_double(r, e);
+    return e <= kExpMax;
+}
+
+// The other three, and the states (SHEAR: ut too).
 // load(m, x): the stencil of variable m (0 rho, 1 un, 2 ut, 3 p); of the face's
 // mean state, y = 1 / (2 rho c), rc2 = 2 rho c and ic2 = 1 / c^2. Fields: entropy
 // w2 = rho - p / c^2; w1, w4 = p -/+ rho c un; shear w3 = ut. Back: p =
 // (w1 + w4) / 2, un = (w4 - w1) y, rho = w2 + p / c^2.
-template <int ORDER, typename F>
+template <int ORDER, bool SHEAR = true, typename F>
 GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, FaceStates& o)
 {
     Functionals P;
     i64 sl, sr;
-    int ep, es, et, ew;
+    int ep, es, ew;
     {
         Stencil x;
         load(3, x);
@@ -453,18 +470,9 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         o.r[1] = to_double(aligned(sr, es, er) + mulhi(pr, fi), er);
         o.ok = er <= kExpMax && ev <= kExpMax;
     }
-    {  // field 3 (shear): ut
-        Stencil x;
-        load(2, x);
-        et = stencil_exponent(x);
-        Functionals R;
-        variable<ORDER>(x, et, R);
-        i64 tl, tr;
-        limited<ORDER>(R, tl, tr);
-        o.ut[0] = to_double(tl, et);
-        o.ut[1] = to_double(tr, et);
-    }
-    o.ok = o.ok && ew <= kExpMax && es <= kExpMax && et <= kExpMax;
+    bool in_range = true;
+    if constexpr (SHEAR) in_range = shear_states<ORDER>(load, o.ut);
+    o.ok = o.ok && ew <= kExpMax && es <= kExpMax && in_range;
 }
 
 // MEG7-cons: the reconstructed variables are rho, rho un, rho ut, E, projected

@@ -105,6 +105,9 @@ __device__ __forceinline__ void fixed_viscous(const FaceIn<double>& in, const do
     out[3] = rfma(-k.q, tn, rfma(-0.5, w, out[3]));
 }
 
+// Whether a CTA has a second thread for every face (whole warps of them).
+constexpr bool fixed_splits_faces(int faces, int threads) { return threads >= 2 * ((faces + 31) / 32 * 32); }
+
 template <int BX, int BY, int NT, bool VISC, int ORDER, bool TMA, bool CONS = false, bool MAP = false>
 __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, const int ty0, unsigned char* smem,
                                            const CUtensorMap* tmap = nullptr)
@@ -228,8 +231,20 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     }
     __syncthreads();
 
-    // Phase 2: every x face and y face of the tile, once (one thread per face).
-    for (int w = tid; w < L::NF; w += NT) {
+    // Phase 2: every x face and y face of the tile, once (one thread per face; in
+    // a tile with threads for it, a second one per face, a whole half of the CTA,
+    // evaluates what the states do not need, the shear field and the flux
+    // reconstruction: where one small tile is all an SM has, a face's chain of
+    // dependent instructions is the time, 64^2 step 50.0 -> 44.8 us).
+    constexpr int HALF = NT / 2;
+    constexpr bool SPLIT = fixed_splits_faces(L::NF, NT);
+    __shared__ double sT[SPLIT ? 6 * L::NF : 1];  // ut L, ut R, F of the face
+    auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };  // (reached from both halves' code)
+    for (int item = tid; item < (SPLIT ? NT : L::NF); item += NT) {
+        const bool second = SPLIT && item >= HALF;
+        const int wa = second ? item - HALF : item;
+        const bool live = !SPLIT || wa < L::NF;
+        const int w = live ? wa : L::NF - 1;
         const bool xf = w < L::NHX;
         const int w2 = xf ? w : w - L::NHX;
         const int fw = xf ? L::HXW : BX;
@@ -266,6 +281,48 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                 x.e[k] = sE[at + (k - 5) * su];
             }
         };
+        double Fs[4];
+        auto reconstruct = [&] {  // the central part where sigma = 1 (Sec. 2.4)
+            const int at = xf ? fr * L::FXW + fc + 4 : (fr + 4) * BX + fc, sf = xf ? 1 : BX;
+            const int nf = xf ? L::NFX : L::NFY;
+            const i64* fm = (xf ? sFX : sFY) + at;
+            const u16* fe = (xf ? sEX : sEY) + at;
+#pragma unroll 1
+            for (int m = 0; m < 4; ++m) {
+                const int pl = (m == 1 ? pn : m == 2 ? 3 - pn : m) * nf;
+                i64 q[10];
+                int e[10];
+#pragma unroll
+                for (int k = 0; k < 10; ++k) {
+                    q[k] = fm[pl + (k - 4) * sf];
+                    e[k] = fe[pl + (k - 4) * sf];
+                }
+                const double f = fx::recon_mean<ORDER>(q, e);
+                if (m == 0) Fs[0] = f;
+                if (m == 1) Fs[1] = f;
+                if (m == 2) Fs[2] = f;
+                if (m == 3) Fs[3] = f;
+            }
+        };
+        if constexpr (SPLIT) {
+            if (second) {
+                double ut[2] = {0.0, 0.0};
+                if constexpr (!CONS) {
+                    if (!fx::shear_states<ORDER>(load, ut)) ut[0] = __longlong_as_double(0x7ff8000000000000ll);  // refused
+                }
+                if (!trouble) reconstruct();
+                if (live) {
+                    sT[w] = ut[0];
+                    sT[L::NF + w] = ut[1];
+                    if (!trouble) {
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) sT[(2 + m) * L::NF + w] = Fs[m];
+                    }
+                }
+                meet();
+                break;
+            }
+        }
         // Characteristic projection at the arithmetic-mean state, every
         // factor from one reciprocal square root y = 1/sqrt(gamma p rho).
         // (Twice the means: X = (2 rho)(2 gamma p), y = 1/sqrt(X) = 1/(2 rho c),
@@ -281,7 +338,13 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         bool ok;
         if constexpr (!CONS) {
             fx::FaceStates s;
-            fx::face_states<ORDER>(load, y, xx * y, ic2, s);
+            fx::face_states<ORDER, !SPLIT>(load, y, xx * y, ic2, s);
+            if constexpr (SPLIT) {
+                meet();
+                s.ut[0] = sT[w];
+                s.ut[1] = sT[L::NF + w];
+                s.ok = s.ok && fx::exponent(s.ut[0]) != 2047;
+            }
             rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
             rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
             ok = s.ok;
@@ -307,6 +370,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                     return e;
                 },
                 C, s);
+            if constexpr (SPLIT) meet();
             ok = s.ok;
             // Back with the right eigenvectors, to primitives: rho un = u rho
             // + c d, rho ut = v rho + w3, so un = u + a, ut = v + b with a =
@@ -338,29 +402,13 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             utR = cell(2, su);
             pR = cell(3, su);
         }
-        // Flux reconstruction of the central part where sigma = 1 (Sec. 2.4).
-        double Fs[4];
-        if (!trouble) {
-            const int at = xf ? fr * L::FXW + fc + 4 : (fr + 4) * BX + fc, sf = xf ? 1 : BX;
-            const int nf = xf ? L::NFX : L::NFY;
-            const i64* fm = (xf ? sFX : sFY) + at;
-            const u16* fe = (xf ? sEX : sEY) + at;
-#pragma unroll 1
-            for (int m = 0; m < 4; ++m) {
-                const int pl = (m == 1 ? pn : m == 2 ? 3 - pn : m) * nf;
-                i64 q[10];
-                int e[10];
+        // Flux reconstruction (Sec. 2.4).
+        if constexpr (SPLIT) {
+            if (!live) break;
 #pragma unroll
-                for (int k = 0; k < 10; ++k) {
-                    q[k] = fm[pl + (k - 4) * sf];
-                    e[k] = fe[pl + (k - 4) * sf];
-                }
-                const double f = fx::recon_mean<ORDER>(q, e);
-                if (m == 0) Fs[0] = f;
-                if (m == 1) Fs[1] = f;
-                if (m == 2) Fs[2] = f;
-                if (m == 3) Fs[3] = f;
-            }
+            for (int m = 0; m < 4; ++m) Fs[m] = trouble ? 0.0 : sT[(2 + m) * L::NF + w];
+        } else if (!trouble) {
+            reconstruct();
         }
         double out[4];
         hllc_flux(ph, !trouble, Fs, rL, unL, utL, pL, rR, unR, utR, pR, out);
@@ -451,13 +499,13 @@ cudaError_t launch_fixed_tiles(const StageParams& p, cudaStream_t s)
 // (1024^2 step 1.94 ms; 16 x 16 with 288 threads 2.03, 20 x 12 1.97, 28 x 8
 // 2.05). A grid of few tiles is bound by the tiles the busiest SM gets, so a
 // smaller tile that divides the work further wins: 16 x 8 with its 280 faces in
-// one round, 8 x 4 where even that leaves SMs idle. A step's time is close to
-// 50 us + c k with k the tiles of the busiest SM and c = 63, 36.5 and 15.5 us
-// (measured at 32^2 .. 1024^2: 64^2 70 us with 8 x 4, 125 us with 16 x 15;
-// 200^2 167 us with 16 x 8, 181 / 182 us with the others; 256^2 181 us with
-// 16 x 15, 205 / 267 us with the others); the smallest c k is taken, k rounded
-// up while it is small and the last wave counts. The result does not depend on
-// the shape.
+// one round, 8 x 4 where even that leaves SMs idle. A step's time grows with c k,
+// k the tiles of the busiest SM and c = 63, 36.5 and 15.5; the smallest c k is
+// taken, k rounded up while it is small and the last wave counts (measured, us
+// with 16 x 15 / 16 x 8 / 8 x 4: 64^2 106 / 72 / 43, 96^2 106 / 72 / 51, 128^2
+// 106 / 72 / 93, 136^2 110 / 97 / 95, 176^2 107 / 107 / 169, 200^2 168 / 149 / 214;
+// nowhere in 48^2 .. 200^2 is the choice more than 7% off the best). The result
+// does not depend on the shape.
 inline cudaError_t fixed_tile_shape(const Grid& g, TileShape* t)
 {
     static PerDevice<int> sm_count;
@@ -484,7 +532,7 @@ cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
     TileShape t;
     const cudaError_t e = fixed_tile_shape(p.g, &t);
     if (e != cudaSuccess) return e;
-    if (t.bx == 8) return launch_fixed_tiles<8, 4, 96, VISC, ORDER, CONS>(p, s);
+    if (t.bx == 8) return launch_fixed_tiles<8, 4, 192, VISC, ORDER, CONS>(p, s);
     if (t.by == 8) return launch_fixed_tiles<16, 8, 288, VISC, ORDER, CONS>(p, s);
     return launch_fixed_tiles<16, 15, 256, VISC, ORDER, CONS>(p, s);
 }
