@@ -435,7 +435,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             in.tut = gt + (3 - pn) * nt;
             in.stq = xf ? 1 : L::GXW;
             in.tr0 = gt;
-            fixed_viscous<CONS>(in, u0, u1, ph.gm1, P.ph.visc[xf ? 0 : 1], out);
+            fixed_viscous<CONS>(in, u0, u1, ph.gm1, P.visc[xf ? 0 : 1], out);
         }
         if (xf) {
 #pragma unroll

@@ -203,6 +203,7 @@ StageParams stage_params(gbr_ctx* c, const double* q)
     memset(&p, 0, sizeof(p));
     p.g = c->g;
     p.ph = c->ph;
+    viscous_factors(p);
     p.q = q;
     p.qn = c->Qn;
     p.err = &c->ds->err;

@@ -103,13 +103,6 @@ struct Physics {
     // spends FP64 divisions on them: gamma - 1, 1/(gamma - 1), the heat
     // conduction coefficient mu / (Pr (gamma - 1)), 1/dx, 1/dy.
     double gm1, igm1, kq, inv_dx, inv_dy;
-    // Coefficients of the FP64 form's viscous flux, [0] x faces, [1] y faces:
-    // with hn, ht the cell sizes along and across the normal and gradients at 60
-    // times their value, 8/3 mu / hn, mu / (180 ht), 2 mu / hn, mu / (120 ht),
-    // 2 gamma kq / hn (see fixed_viscous).
-    struct {
-        double nn, ntt, nt, tn, q;
-    } visc[2];
     // The same rounded to FP32, for the FP32 form (a conversion issues on the
     // FP64 pipe, and every thread would do seven).
     struct {
@@ -125,14 +118,6 @@ inline void derive_physics(Physics& ph)
     ph.kq = ph.mu / (ph.Pr * (ph.gamma - 1.0));
     ph.inv_dx = 1.0 / ph.dx;
     ph.inv_dy = 1.0 / ph.dy;
-    for (int k = 0; k < 2; ++k) {
-        const double in = k ? ph.inv_dy : ph.inv_dx, it = k ? ph.inv_dx : ph.inv_dy;
-        ph.visc[k].nn = 8.0 / 3.0 * ph.mu * in;
-        ph.visc[k].ntt = ph.mu * it / 180.0;
-        ph.visc[k].nt = 2.0 * ph.mu * in;
-        ph.visc[k].tn = ph.mu * it / 120.0;
-        ph.visc[k].q = 2.0 * ph.gamma * ph.kq * in;
-    }
     ph.f32.gamma = (float)ph.gamma;
     ph.f32.gm1 = (float)ph.gm1;
     ph.f32.igm1 = (float)ph.igm1;
@@ -186,7 +171,27 @@ struct StageParams {
     // ghost fill came before.
     int map;
     GhostParams gh;
+    // Coefficients of the FP64 form's viscous flux, [0] x faces, [1] y faces:
+    // with hn, ht the cell sizes along and across the normal and gradients at 60
+    // times their value, 8/3 mu / hn, mu / (180 ht), 2 mu / hn, mu / (120 ht),
+    // 2 gamma kq / hn (see fixed_viscous). Not in Physics, which a batch's CTAs copy
+    // for every tile (ensemble of 16 grids, FP32 + sensor: 21.35 -> 20.14 ms without).
+    struct {
+        double nn, ntt, nt, tn, q;
+    } visc[2];
 };
+inline void viscous_factors(StageParams& p)
+{
+    const Physics& ph = p.ph;
+    for (int k = 0; k < 2; ++k) {
+        const double in = k ? ph.inv_dy : ph.inv_dx, it = k ? ph.inv_dx : ph.inv_dy;
+        p.visc[k].nn = 8.0 / 3.0 * ph.mu * in;
+        p.visc[k].ntt = ph.mu * it / 180.0;
+        p.visc[k].nt = 2.0 * ph.mu * in;
+        p.visc[k].tn = ph.mu * it / 120.0;
+        p.visc[k].q = 2.0 * ph.gamma * ph.kq * in;
+    }
+}
 
 // One grid of a batch, as the device sees it. tiles_x / tile_begin describe
 // the current tile shape: tile t of the batch belongs to the case with the

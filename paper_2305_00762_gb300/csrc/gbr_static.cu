@@ -132,6 +132,7 @@ extern "C" int gbr_step_static(const double* Q_in, double* Q_out, int nx, int ny
     memset(&sp, 0, sizeof(sp));
     sp.g = g;
     sp.ph = ph;
+    viscous_factors(sp);
     sp.qn = Qn;
     sp.err = &ds->err;
     sp.dt = dt;
