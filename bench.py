@@ -95,10 +95,10 @@ FP32_PEAK_NOMINAL = 80550.0   # 152 SMs x 128 FP32 lanes x 2 flop (FMA) x 2.07 G
 # (dram__bytes_read.sum + dram__bytes_write.sum) of
 # `bench.py --profile-only --n N --steps 2 --warmup 1 --state-cache ...`.
 # Re-measure when the kernel changes (None: not measured for this kernel).
-F64_STAGE_DRAM_BYTES = {1024: 59.58e6, 4096: 1405.94e6}
+F64_STAGE_DRAM_BYTES = {1024: 61.03e6, 4096: 1402.97e6}
 # FP64 thread instructions (DADD + DMUL + DFMA) per cell-update of the FP64 stage
-# kernel, from an ncu capture (profiles/fixed_kernel_f64.md).
-F64_STAGE_FP64_INST = 181.0
+# kernel, from an ncu capture (profiles/fixed_kernel_f64_riemann1024_dram.md).
+F64_STAGE_FP64_INST = 185.1
 
 
 def fma_peaks():
