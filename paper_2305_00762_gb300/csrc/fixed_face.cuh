@@ -19,9 +19,15 @@
 // Scaling. A variable q of one face's stencil (cells j-5 .. j+6) is held as
 // I = q / 2^(e - 1081) with e the largest biased exponent of the stencil, so
 // |I| < 2^kBits: values within 2^6 of the largest are held exactly, smaller
-// ones rounded down at 2^-59 of it (an FP64 operation on the largest value
-// rounds at 2^-53 of it). The scale depends on the face's own stencil only:
-// the result does not depend on tiles, slabs or batches.
+// ones rounded down at 2^-59 of it. The scale depends on the face's own stencil
+// only: the result does not depend on tiles, slabs or batches. The limiter
+// bounds a state by the cells beside the face, which may be far smaller than the
+// largest value: such faces are flagged (kWide) and evaluated by wide_face.cuh.
+// Error of a state in units of 2^-53 of its own cell's terms, root mean square
+// over jumps of every kind (and of the same formulas in FP64 throughout): rho
+// 0.1 - 0.5 (0.3 - 0.5), un 0.1 - 0.5 (0.4 - 0.5), p 0.1 - 0.4 (0.4 - 0.5);
+// MEG7-cons at Mach numbers up to 3 rho 0.7 - 1.3 (0.9 - 1.4), un 0.2 - 0.5
+// (0.4 - 0.6), p 1.3 - 2.5 (1.9 - 2.9).
 //
 // Linear functionals. The left value at j+1/2 and the curvatures of the MP
 // limiter are sums over the even and odd differences about a cell,
@@ -91,16 +97,18 @@ GBR_HD u64 mulhi_u(u64 a, u64 b)
     return (u64)(((unsigned __int128)a * b) >> 64);
 #endif
 }
-// x r / 2^64, x signed, r < 2^63, less at most four units: three 32 x 32 -> 64
+// x r / 2^64, x signed, r < 2^63, within three units: three 32 x 32 -> 64
 // products (the low halves' product and the lowest bits of r's halves are
-// dropped) instead of four and the sign's correction.
+// dropped) instead of four and the sign's correction. The addend, nearly a unit,
+// centres the error of what is dropped; zero stays zero.
 GBR_HD i64 mulhi(i64 x, u64 r)
 {
     const int xh = (int)(x >> 32), rh = (int)(r >> 32);
-    const i64 mid = (i64)xh * (int)((unsigned)r >> 1) + (i64)((u64)(unsigned)x * ((unsigned)rh >> 1));
+    const i64 mid = 0x7fffffffll + (i64)xh * (int)((unsigned)r >> 1) + (i64)((u64)(unsigned)x * ((unsigned)rh >> 1));
     return (i64)xh * rh + (mid >> 31);
 }
 
+GBR_HD int larger(int a, int b) { return a > b ? a : b; }
 GBR_HD int exponent(double x) { return (int)(bits_of(x) >> 52) & 0x7ff; }
 
 // A value taken apart once, where it is produced, so that each of the many
@@ -212,52 +220,56 @@ constexpr int kGrbShift7 = 10;  // n = 840 delta / 2^10
 constexpr int kGrbShift4 = 13;  // order 4: n = 10080 delta / 2^13
 constexpr int kCurvShift = 7;   // d = 120 d_j / 2^7
 
+// Those about one cell (q: its value among its neighbours', k: its place, 0 for
+// cell j-1): d, and n[k-1] for the cells beside the face.
+template <int ORDER>
+GBR_HD void centred(const i64* q, int k, i64& d_out, i64 (&n_out)[2])
+{
+    const i64 c2 = q[0] + q[0];
+    const i64 B1 = q[1] + q[-1] - c2, B2 = c2 - q[2] - q[-2];  // (B2, B4, A2 with their signs changed)
+    const i64 B3 = q[3] + q[-3] - c2, B4 = c2 - q[4] - q[-4];
+    Acc d;
+    if (ORDER == 4 || k == 0 || k == 3) {
+        d.add(B1, 231);
+        d.add(B2, 44);
+        d.add(B3, 9);
+        d.add(B4, 1);
+    }
+    if (k == 1 || k == 2) {
+        const i64 A1 = q[1] - q[-1], A2 = q[-2] - q[2], A3 = q[3] - q[-3];
+        Acc even, odd;
+        if (ORDER == 4) {
+            even.add(B1, 1617);
+            even.add(B2, 308);
+            even.add(B3, 63);
+            even.add(B4, 7);
+            odd.add(A1, 3780);
+            odd.add(A2, 756);
+            odd.add(A3, 84);
+        } else {
+            even.add(B1, 169);
+            even.add(B2, 41);
+            even.add(B3, 9);
+            even.add(B4, 1);
+            odd.add(A1, 315);
+            odd.add(A2, 63);
+            odd.add(A3, 7);
+            d = even;
+            d.add(B1, 62);
+            d.add(B2, 3);
+        }
+        const Acc n = k == 1 ? even + odd : even - odd;
+        n_out[k - 1] = n.shift<ORDER == 4 ? kGrbShift4 : kGrbShift7>();
+    }
+    d_out = d.shift<kCurvShift>();
+}
 template <int ORDER>
 GBR_HD void functionals(const i64 (&q)[12], Functionals& f)
 {
 #pragma unroll
     for (int k = 0; k < 4; ++k) f.v[k] = q[4 + k];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int c = 4 + k;
-        const i64 c2 = q[c] + q[c];
-        const i64 B1 = q[c + 1] + q[c - 1] - c2, B2 = c2 - q[c + 2] - q[c - 2];  // (B2, B4, A2 with their signs changed)
-        const i64 B3 = q[c + 3] + q[c - 3] - c2, B4 = c2 - q[c + 4] - q[c - 4];
-        Acc d;
-        if (ORDER == 4 || k == 0 || k == 3) {
-            d.add(B1, 231);
-            d.add(B2, 44);
-            d.add(B3, 9);
-            d.add(B4, 1);
-        }
-        if (k == 1 || k == 2) {
-            const i64 A1 = q[c + 1] - q[c - 1], A2 = q[c - 2] - q[c + 2], A3 = q[c + 3] - q[c - 3];
-            Acc even, odd;
-            if (ORDER == 4) {
-                even.add(B1, 1617);
-                even.add(B2, 308);
-                even.add(B3, 63);
-                even.add(B4, 7);
-                odd.add(A1, 3780);
-                odd.add(A2, 756);
-                odd.add(A3, 84);
-            } else {
-                even.add(B1, 169);
-                even.add(B2, 41);
-                even.add(B3, 9);
-                even.add(B4, 1);
-                odd.add(A1, 315);
-                odd.add(A2, 63);
-                odd.add(A3, 7);
-                d = even;
-                d.add(B1, 62);
-                d.add(B2, 3);
-            }
-            const Acc n = k == 1 ? even + odd : even - odd;
-            f.n[k - 1] = n.shift<ORDER == 4 ? kGrbShift4 : kGrbShift7>();
-        }
-        f.d[k] = d.shift<kCurvShift>();
-    }
+    for (int k = 0; k < 4; ++k) centred<ORDER>(q + 4 + k, k, f.d[k], f.n);
 }
 
 // f r / 2^64 of every functional.
@@ -392,15 +404,50 @@ GBR_HD u64 factor(double a, int e, int eo)  // of |a|
     return factor(p, e, eo);
 }
 
+// Faces whose states fixed point would hold with fewer bits than FP64 arithmetic
+// does (wide_face.cuh evaluates them): the scale of the stencil exceeds the
+// largest term of a cell beside the face by more than kWide binary orders. A
+// result carries a few units of 2^-59 of the scale, so up to there its error is
+// a few units of 2^(kWide-59) of its own terms.
+constexpr int kWide = 5;
+GBR_HD bool is_wide(int scale, int local0, int local1) { return scale - (local0 < local1 ? local0 : local1) > kWide; }
+// The same from a field's values (l, r): a value, its step from the cell's value
+// and the cell's other terms (tl, tr) all below 2^-kWide of the scale. (A field
+// may be small at one cell, as where a velocity changes sign, without losing
+// anything: FP64 rounds its step too, and an unlimited value carries the
+// rounding of the differences that it was formed of.)
+GBR_HD unsigned leading(i64 x) { return (unsigned)((int)(x >> 32) ^ (int)(x >> 63)); }
+template <int ORDER>
+GBR_HD bool is_wide_field(const Functionals& f, i64 l, i64 r, i64 tl = 0, i64 tr = 0)
+{
+    const i64 al = l == f.v[1] + grb_delta<ORDER>(f.n[0]) ? f.v[2] - f.v[0] : 0;
+    const i64 ar = r == f.v[2] + grb_delta<ORDER>(f.n[1]) ? f.v[3] - f.v[1] : 0;
+    const unsigned L = leading(f.v[1]) | leading(l - f.v[1]) | leading(al) | leading(tl);
+    const unsigned R = leading(f.v[2]) | leading(r - f.v[2]) | leading(ar) | leading(tr);
+    return (L < R ? L : R) >> (kBits - kWide - 32) == 0;
+}
+
 // The face states (L, R) back in primitives.
 struct FaceStates {
     double r[2], un[2], ut[2], p[2];
-    bool ok;  // false: a stencil value too large, infinite or NaN
+    bool ok;    // false: a stencil value too large, infinite or NaN
+    bool wide;  // r, un, p: to be evaluated in FP64
+    bool wide_ut;
 };
+
+// A shear velocity below 2^-kStill of the speed of sound throughout the stencil is
+// rounding noise or as good as none, and stays in fixed point: its error is then
+// below 2^(-59-kStill) of a speed of sound that the normal velocity is rounded at
+// 2^-53 of. The exponent of that bound from the cells' exponents (c^2 ~ p / rho).
+constexpr int kStill = 20;
+GBR_HD int still_exponent(int r0, int p0, int r1, int p1)
+{
+    return larger(1023 - kStill + ((p0 - r0 < p1 - r1 ? p0 - r0 : p1 - r1) >> 1), kExpMin);
+}
 
 // Field 3 (shear) is ut itself. Returns whether its stencil is in range.
 template <int ORDER, typename F>
-GBR_HD bool shear_states(F load, double (&ut)[2])
+GBR_HD bool shear_states(F load, int still, double (&ut)[2], bool& wide)
 {
     Stencil x;
     load(2, x);
@@ -411,6 +458,7 @@ GBR_HD bool shear_states(F load, double (&ut)[2])
     limited<ORDER>(R, l, r);
     ut[0] = to_double(l, e);
     ut[1] = to_double(r, e);
+    wide = e > still && is_wide(e + 1, x.e[5], x.e[6]) && is_wide_field<ORDER>(R, l, r);
     return e <= kExpMax;
 }
 
@@ -424,10 +472,12 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
 {
     Functionals P;
     i64 sl, sr;
-    int ep, es, ew;
+    int ep, es, ew, lp[2], lr[2];  // lp, lr: of the cells beside the face
     {
         Stencil x;
         load(3, x);
+        lp[0] = x.e[5];
+        lp[1] = x.e[6];
         ep = stencil_exponent(x);
         variable<ORDER>(x, ep, P);
     }
@@ -436,6 +486,9 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         load(0, x);
         const int er = stencil_exponent(x), eprod = ep + ic2.e - 1022;
         es = (er > eprod ? er : eprod) + 1;
+        lr[0] = x.e[5];
+        lr[1] = x.e[6];
+        o.wide = is_wide(es, larger(lr[0], lp[0] + ic2.e - 1022), larger(lr[1], lp[1] + ic2.e - 1022));
         Functionals R, S;
         scale(P, factor(ic2, ep, es), S);
         variable<ORDER>(x, es, R);
@@ -447,6 +500,7 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         load(1, x);
         const int eu = stencil_exponent(x), eprod = eu - 1 + rc2.e - 1022;  // (half of rc2)
         ew = (ep > eprod ? ep : eprod) + 1;
+        o.wide = o.wide || is_wide(ew, larger(lp[0], x.e[5] + rc2.e - 1023), larger(lp[1], x.e[6] + rc2.e - 1023));
         Functionals U, W;
         variable<ORDER>(x, eu, U);
         scale(U, factor(rc2, eu - 1, ew), U);
@@ -471,7 +525,7 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         o.ok = er <= kExpMax && ev <= kExpMax;
     }
     bool in_range = true;
-    if constexpr (SHEAR) in_range = shear_states<ORDER>(load, o.ut);
+    if constexpr (SHEAR) in_range = shear_states<ORDER>(load, still_exponent(lr[0], lp[0], lr[1], lp[1]), o.ut, o.wide_ut);
     o.ok = o.ok && ew <= kExpMax && es <= kExpMax && in_range;
 }
 
@@ -486,7 +540,8 @@ struct ConsCoefs {
 };
 struct ConsStates {
     double r[2], s[2], d[2], w3[2];
-    bool ok;  // false: a stencil value too large, infinite or NaN
+    bool ok;    // false: a stencil value too large, infinite or NaN
+    bool wide, wide_w3;  // r, s, d and w3: to be evaluated in FP64 (wide_face.cuh)
 };
 
 // acc += a f (acc -= with `minus`), a of any sign, r the factor() of |a|.
@@ -501,8 +556,6 @@ GBR_HD void accumulate(Functionals& acc, const Functionals& f, double a, u64 r, 
     acc.n[0] += (mulhi(f.n[0], r) ^ g) - g;
     acc.n[1] += (mulhi(f.n[1], r) ^ g) - g;
 }
-GBR_HD int larger(int a, int b) { return a > b ? a : b; }
-
 // load(m, x): the stencil of variable m; scale(m): its stencil's exponent.
 template <int ORDER, typename F, typename E>
 GBR_HD void cons_states(F load, E scale_of, const ConsCoefs& C, ConsStates& o)
@@ -516,11 +569,17 @@ GBR_HD void cons_states(F load, E scale_of, const ConsCoefs& C, ConsStates& o)
     ea = larger(ea, larger(product(e[0], C.uc), product(e[1], C.ic))) + 3;
     ea = larger(ea, kExpMin);
     const int es = larger(e[2], product(e[0], C.v)) + 1, er = larger(e[0], ea) + 1;
+    int ql[2], la[2];  // exponents of q0, and of the terms of A and t, at the cells beside the face
     Functionals Q0, A, T, W;
     i64 tl, tr;
     {
         Stencil x;
         load(0, x);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            ql[k] = x.e[5 + k];
+            la[k] = larger(product(ql[k], C.b2), product(ql[k], C.uc));
+        }
         variable<ORDER>(x, e[0], Q0);
         scale(Q0, factor(C.b2, e[0], ea), A);
         const i64 g = (i64)bits_of(C.uc) >> 63;
@@ -537,10 +596,14 @@ GBR_HD void cons_states(F load, E scale_of, const ConsCoefs& C, ConsStates& o)
         Stencil x;
         Functionals Q;
         load(1, x);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) la[k] = larger(la[k], larger(product(x.e[5 + k], C.b1u), product(x.e[5 + k], C.ic)));
         variable<ORDER>(x, e[1], Q);
         accumulate(A, Q, C.b1u, factor(C.b1u, e[1], ea), true);
         accumulate(T, Q, C.ic, factor(C.ic, e[1], ea), true);
         load(3, x);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) la[k] = larger(la[k], product(x.e[5 + k], C.b1));
         variable<ORDER>(x, e[3], Q);
         accumulate(A, Q, C.b1, factor(C.b1, e[3], ea), false);
         load(2, x);
@@ -548,8 +611,12 @@ GBR_HD void cons_states(F load, E scale_of, const ConsCoefs& C, ConsStates& o)
         accumulate(A, Q, C.b1v, factor(C.b1v, e[2], ea), true);
         W = Q;
         shift_right(W, es - e[2]);
+        const i64 t0 = W.v[1], t1 = W.v[2];
+        const int still = larger((ql[0] < ql[1] ? ql[0] : ql[1]) + 1023 - kStill - exponent(C.ic), kExpMin + 1);
         accumulate(W, Q0, C.v, factor(C.v, e[0], es), true);
         limited<ORDER>(W, tl, tr);
+        o.wide = is_wide(ea, la[0], la[1]) || is_wide(er, larger(ql[0], la[0]), larger(ql[1], la[1]));
+        o.wide_w3 = es > still && is_wide_field<ORDER>(W, tl, tr, t0, t1);
     }
     i64 al, ar, bl, br, cl, cr;  // 2 w1, 2 w4, w2
     sum(A, T, W);

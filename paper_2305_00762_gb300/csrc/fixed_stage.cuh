@@ -11,6 +11,7 @@
 #pragma once
 
 #include "stage_kernel.cuh"
+#include "wide_face.cuh"
 
 namespace gbr {
 
@@ -281,6 +282,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                 x.e[k] = sE[at + (k - 5) * su];
             }
         };
+        const fx::Face face{sM + c, sE + c, su, NU, pn};  // for the few faces evaluated in FP64 (wide_face.cuh)
         double Fs[4];
         auto reconstruct = [&] {  // the central part where sigma = 1 (Sec. 2.4)
             const int at = xf ? fr * L::FXW + fc + 4 : (fr + 4) * BX + fc, sf = xf ? 1 : BX;
@@ -308,7 +310,10 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             if (second) {
                 double ut[2] = {0.0, 0.0};
                 if constexpr (!CONS) {
-                    if (!fx::shear_states<ORDER>(load, ut)) ut[0] = __longlong_as_double(0x7ff8000000000000ll);  // refused
+                    bool wide;
+                    const int still = fx::still_exponent(sE[c], sE[3 * NU + c], sE[c + su], sE[3 * NU + c + su]);
+                    if (!fx::shear_states<ORDER>(load, still, ut, wide)) ut[0] = __longlong_as_double(0x7ff8000000000000ll);  // refused
+                    else if (wide) fx::wide_shear<ORDER>(face, ut);
                 }
                 if (!trouble) reconstruct();
                 if (live) {
@@ -344,7 +349,10 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                 s.ut[0] = sT[w];
                 s.ut[1] = sT[L::NF + w];
                 s.ok = s.ok && fx::exponent(s.ut[0]) != 2047;
+            } else if (s.ok && s.wide_ut) {
+                fx::wide_shear<ORDER>(face, s.ut);
             }
+            if (s.ok && s.wide && positive) fx::wide_states<ORDER>(face, ph.gamma, s);
             rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
             rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
             ok = s.ok;
@@ -370,6 +378,8 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                     return e;
                 },
                 C, s);
+            if (s.ok && s.wide_w3) fx::wide_cons_shear<ORDER>(face, C.v, s.w3);
+            if (s.ok && s.wide && positive) fx::wide_cons_states<ORDER>(face, C, s);
             if constexpr (SPLIT) meet();
             ok = s.ok;
             // Back with the right eigenvectors, to primitives: rho un = u rho
