@@ -475,6 +475,8 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
 // code for it costs registers that they need (1024^2 2.0% slower with it).
 constexpr bool fixed_maps_ghosts(int bx) { return bx == 8; }
 
+constexpr int kMaxTileRows = 65535;  // of a launch's y extent
+
 // One CTA per tile, two CTAs per SM (viscous MEG7-cons: one, by shared memory).
 template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS>
 __global__ void __launch_bounds__(NT, CONS && VISC ? 1 : 2)
@@ -482,7 +484,9 @@ __global__ void __launch_bounds__(NT, CONS && VISC ? 1 : 2)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     dependent_start();
-    fixed_tile<BX, BY, NT, VISC, ORDER, true, CONS, fixed_maps_ghosts(BX)>(P, blockIdx.x * BX, blockIdx.y * BY, smem_raw, &tmap);
+    const int ty = blockIdx.z * gridDim.y + blockIdx.y;  // (the rows of tiles in planes of at most kMaxTileRows)
+    if (ty * BY >= P.g.ny) return;
+    fixed_tile<BX, BY, NT, VISC, ORDER, true, CONS, fixed_maps_ghosts(BX)>(P, blockIdx.x * BX, ty * BY, smem_raw, &tmap);
 }
 
 template <int BX, int BY, int NT, bool VISC, int ORDER, bool CONS>
@@ -500,7 +504,8 @@ cudaError_t launch_fixed_tiles(const StageParams& p, cudaStream_t s)
     CUtensorMap map;
     e = encode_state_map(p.g, p.q, F::G::RW, F::G::RH, &map);
     if (e != cudaSuccess) return e;
-    dim3 grid((p.g.nx + BX - 1) / BX, (p.g.ny + BY - 1) / BY);
+    const int rows = (p.g.ny + BY - 1) / BY, planes = (rows + kMaxTileRows - 1) / kMaxTileRows;
+    dim3 grid((p.g.nx + BX - 1) / BX, planes == 1 ? rows : kMaxTileRows, planes);
     return launch_dependent(kern, grid, NT, F::bytes, s, p, map);
 }
 

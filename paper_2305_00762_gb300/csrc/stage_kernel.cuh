@@ -1370,7 +1370,7 @@ __device__ __forceinline__ void stage_scalars(const StageParams& P, double* dt)
     if (threadIdx.x != 0) return;
     if (MAP && P.map && P.gh.mode != 0) {
         *dt = step_size(P.gh);
-        if (blockIdx.x == 0 && blockIdx.y == 0) begin_step(P.gh);
+        if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) begin_step(P.gh);
     } else {
         *dt = P.dt_ptr ? *P.dt_ptr : P.dt;
     }
