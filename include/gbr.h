@@ -31,6 +31,12 @@
  * gbr_set_state. Calls with a NULL context or out-of-range arguments return
  * GBR_ERR_ARG and change nothing.
  *
+ * Range (precision 64). Face states are formed from densities, velocities and
+ * pressures (MEG7-cons: components) between 2^-895 (4e-270) and 2^877 (1e264):
+ * a face with a larger magnitude, an infinity or a NaN among its twelve cells
+ * takes the adjacent cells' states, and a variable below the range in all of
+ * them counts as zero. Wavespeeds are those of the whole FP64 range.
+ *
  * Streams. All work is issued on the context's stream (the legacy default
  * stream until gbr_set_stream). Host-buffer transfers synchronise that stream.
  */

@@ -115,9 +115,22 @@ __device__ __forceinline__ T tmax(T a, T b) { return a > b ? a : b; }
 // FP32: one min / max instruction (the same value for operands that are not NaN)
 __device__ __forceinline__ float tmin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ float tmax(float a, float b) { return fmaxf(a, b); }
-// FP64 roots and reciprocals come from the integer pipe (fixed_math.cuh).
-__device__ __forceinline__ double tsqrt(double x) { return __double_as_longlong(x) == 0 ? x : x * fx::rsqrt(x); }
+// FP64 roots and reciprocals come from the integer pipe (fixed_math.cuh), whose
+// results for subnormal operands, and reciprocals below the normal range, are not
+// the rounded ones: where a value may be any (the wavespeed of a cell), those
+// and the special values take the division and the root themselves, out of line.
+__device__ __noinline__ static double plain_root(double x) { return sqrt(x); }
+__device__ __noinline__ static double plain_reciprocal(double x) { return 1.0 / x; }
+__device__ __forceinline__ double tsqrt(double x)  // x normal and positive, or any other
+{
+    return (unsigned)(__double2hiint(x) - 0x00100000) < 0x7fe00000u ? x * fx::rsqrt(x) : plain_root(x);
+}
 __device__ __forceinline__ float tsqrt(float x) { return sqrtf(x); }
+__device__ __forceinline__ double tinverse(double x)  // normal, with a normal reciprocal, or any other
+{
+    return (unsigned)((__double2hiint(x) & 0x7fffffff) - 0x00100000) < 0x7fb00000u ? fx::rcp(x) : plain_reciprocal(x);
+}
+__device__ __forceinline__ float tinverse(float x) { return 1.f / x; }
 __device__ __forceinline__ double trsqrt(double x) { return fx::rsqrt(x); }
 __device__ __forceinline__ float trsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double trcp(double x) { return fx::rcp(x); }
@@ -219,7 +232,7 @@ template <typename T>
 __device__ __forceinline__ void prims_of(double q0, double q1, double q2, double q3, T gm1, T& r, T& u, T& v, T& p)
 {
     r = from_f64<T>(q0);
-    const T ir = trcp(r);
+    const T ir = tinverse(r);
     u = from_f64<T>(q1) * ir;
     v = from_f64<T>(q2) * ir;
     if constexpr (sizeof(T) == 8)  // (rho u^2 from the momentum: one product fewer, exact state)
@@ -238,7 +251,7 @@ __device__ __forceinline__ T cell_wavespeed_t(double q0, double q1, double q2, d
 {
     T r, u, v, p;
     prims_of(q0, q1, q2, q3, gm1, r, u, v, p);
-    const T ir = trcp(r);
+    const T ir = tinverse(r);
     const T cs = tsqrt(gamma * p * ir);
     T l = tmax((tabs(u) + cs) * inv_dx, (tabs(v) + cs) * inv_dy);
     if (mu > T(0)) {
