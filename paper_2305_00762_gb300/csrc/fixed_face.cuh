@@ -39,11 +39,13 @@
 // changed. They are formed once per variable and then projected (ten
 // functionals per variable instead of six values and six gradients).
 //
-// The MP test (Eq. mp5Condition) is not taken: where it passes, Phi^L lies
-// between Phi_j and Phi^MP, so inside both intervals of Eq. mp-procedure, and
-// the clamp to [Phi^min, Phi^max] returns it unchanged; on integers this
-// holds exactly. (The test's threshold 1e-40 moves the result by at most
-// 1e-20, below one unit of any FP64 value that such a face state enters.)
+// The MP test (Eq. mp5Condition, (Phi^L - Phi_j)(Phi^L - Phi^MP) <= 1e-40) is
+// not taken: where the product is not positive, Phi^L lies between Phi_j and
+// Phi^MP, so inside both intervals of Eq. mp-procedure, and the clamp to
+// [Phi^min, Phi^max] returns it unchanged; on integers this holds exactly. A
+// positive product up to 1e-40 moves the result by at most 1e-20. Faces where
+// that is more than rounding (fields below about 2^-12) are evaluated with the
+// test (kSmall).
 //
 // Overflow. With |I| < 2^59 = M after projection the largest intermediate is
 // the bound UL = Phi_j + 7 (Phi_j - Phi_{j-1}), at most 15 M < 2^63 (LC: 14.7 M).
@@ -53,8 +55,10 @@
 
 #ifdef __CUDACC__
 #define GBR_HD __host__ __device__ __forceinline__
+#define GBR_OUTLINE __host__ __device__ __noinline__
 #else
 #define GBR_HD inline
+#define GBR_OUTLINE __attribute__((noinline))
 #include <string.h>
 #endif
 
@@ -411,6 +415,10 @@ GBR_HD u64 factor(double a, int e, int eo)  // of |a|
 // a few units of 2^(kWide-59) of its own terms.
 constexpr int kWide = 5;
 GBR_HD bool is_wide(int scale, int local0, int local1) { return scale - (local0 < local1 ? local0 : local1) > kWide; }
+// Nor are faces where the MP test's threshold tells: 1e-20 (2^-66.4) times what a
+// field is carried at (2^k) is 2^-55 or more of the field's scale.
+constexpr int kSmall = kOne - 70;
+GBR_HD bool is_small(int scale, int k) { return scale - k <= kSmall; }
 // The same from a field's values (l, r): a value, its step from the cell's value
 // and the cell's other terms (tl, tr) all below 2^-kWide of the scale. (A field
 // may be small at one cell, as where a velocity changes sign, without losing
@@ -438,11 +446,14 @@ struct FaceStates {
 // A shear velocity below 2^-kStill of the speed of sound throughout the stencil is
 // rounding noise or as good as none, and stays in fixed point: its error is then
 // below 2^(-59-kStill) of a speed of sound that the normal velocity is rounded at
-// 2^-53 of. The exponent of that bound from the cells' exponents (c^2 ~ p / rho).
+// 2^-53 of. The exponent of that bound from the speed's (the cells': c^2 ~ p / rho).
+// Nor is the MP test's 1e-20 taken into account for a shear velocity unless it
+// exceeds what the speed of sound is rounded at; then nothing is still either.
 constexpr int kStill = 20;
+GBR_HD int still_exponent(int c) { return c <= kSmall + 5 ? kExpMin : larger(c - kStill, kExpMin); }
 GBR_HD int still_exponent(int r0, int p0, int r1, int p1)
 {
-    return larger(1023 - kStill + ((p0 - r0 < p1 - r1 ? p0 - r0 : p1 - r1) >> 1), kExpMin);
+    return still_exponent(1023 + ((p0 - r0 < p1 - r1 ? p0 - r0 : p1 - r1) >> 1));
 }
 
 // Field 3 (shear) is ut itself. Returns whether its stencil is in range.
@@ -458,7 +469,7 @@ GBR_HD bool shear_states(F load, int still, double (&ut)[2], bool& wide)
     limited<ORDER>(R, l, r);
     ut[0] = to_double(l, e);
     ut[1] = to_double(r, e);
-    wide = e > still && is_wide(e + 1, x.e[5], x.e[6]) && is_wide_field<ORDER>(R, l, r);
+    wide = e > still && ((still == kExpMin && is_small(e, 0)) || (is_wide(e + 1, x.e[5], x.e[6]) && is_wide_field<ORDER>(R, l, r)));
     return e <= kExpMax;
 }
 
@@ -488,7 +499,7 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         es = (er > eprod ? er : eprod) + 1;
         lr[0] = x.e[5];
         lr[1] = x.e[6];
-        o.wide = is_wide(es, larger(lr[0], lp[0] + ic2.e - 1022), larger(lr[1], lp[1] + ic2.e - 1022));
+        o.wide = is_small(es, 0) || is_wide(es, larger(lr[0], lp[0] + ic2.e - 1022), larger(lr[1], lp[1] + ic2.e - 1022));
         Functionals R, S;
         scale(P, factor(ic2, ep, es), S);
         variable<ORDER>(x, es, R);
@@ -500,7 +511,7 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         load(1, x);
         const int eu = stencil_exponent(x), eprod = eu - 1 + rc2.e - 1022;  // (half of rc2)
         ew = (ep > eprod ? ep : eprod) + 1;
-        o.wide = o.wide || is_wide(ew, larger(lp[0], x.e[5] + rc2.e - 1023), larger(lp[1], x.e[6] + rc2.e - 1023));
+        o.wide = o.wide || is_small(ew, 1024 - ic2.e) || is_wide(ew, larger(lp[0], x.e[5] + rc2.e - 1023), larger(lp[1], x.e[6] + rc2.e - 1023));
         Functionals U, W;
         variable<ORDER>(x, eu, U);
         scale(U, factor(rc2, eu - 1, ew), U);
@@ -612,11 +623,11 @@ GBR_HD void cons_states(F load, E scale_of, const ConsCoefs& C, ConsStates& o)
         W = Q;
         shift_right(W, es - e[2]);
         const i64 t0 = W.v[1], t1 = W.v[2];
-        const int still = larger((ql[0] < ql[1] ? ql[0] : ql[1]) + 1023 - kStill - exponent(C.ic), kExpMin + 1);
+        const int still = still_exponent((ql[0] < ql[1] ? ql[0] : ql[1]) + 1023 - exponent(C.ic));  // (momenta: rho c)
         accumulate(W, Q0, C.v, factor(C.v, e[0], es), true);
         limited<ORDER>(W, tl, tr);
-        o.wide = is_wide(ea, la[0], la[1]) || is_wide(er, larger(ql[0], la[0]), larger(ql[1], la[1]));
-        o.wide_w3 = es > still && is_wide_field<ORDER>(W, tl, tr, t0, t1);
+        o.wide = is_small(ea, 1) || is_wide(ea, la[0], la[1]) || is_wide(er, larger(ql[0], la[0]), larger(ql[1], la[1]));
+        o.wide_w3 = es > still + 1 && ((still == kExpMin && is_small(es, 0)) || is_wide_field<ORDER>(W, tl, tr, t0, t1));
     }
     i64 al, ar, bl, br, cl, cr;  // 2 w1, 2 w4, w2
     sum(A, T, W);

@@ -21,15 +21,16 @@
 // accuracy costs, us a pass without / with: 64^2 vortex 880 / 898, four-quadrant
 // 400^2 1451 / 1592, 1024^2 3986 / 4138, MEG7-cons 400^2 1921 / 2567, double Mach
 // 1024 x 256 (a shock of ratio 116 through four tiles a row) 1881 / 2221.
+//
+// The MP test's absolute threshold, which fixed point leaves out, is applied here,
+// and faces where it tells (kSmall: densities below 2^-12) are evaluated here too:
+// four-quadrant flow 1024^2 in units with densities of 1e-4 8.5 ms a pass.
 #pragma once
 
 #include "fixed_math.cuh"
 
-#ifdef __CUDACC__
-#define GBR_OUTLINE __host__ __device__ __noinline__
-#else
+#ifndef __CUDACC__
 #include <math.h>
-#define GBR_OUTLINE __attribute__((noinline))
 #endif
 
 namespace gbr {
