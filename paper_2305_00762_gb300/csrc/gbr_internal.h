@@ -267,7 +267,7 @@ cudaError_t launch_sensor_train(const void* X_bf16, const unsigned char* y, long
                                 float* v, float* loss, cudaStream_t s);
 cudaError_t launch_wavespeed(const Grid& g, const Physics& ph, const double* q, unsigned long long* lam,
                              int precision, cudaStream_t s);
-cudaError_t launch_stage_f64(const StageParams& p, cudaStream_t s);
+cudaError_t launch_stage_f64(const StageParams& p, cudaStream_t s);  // p.res or p.qout, not both
 // Whether the FP64 stage of this grid can read ghost cells through the boundary
 // rules (StageParams::map).
 cudaError_t stage_f64_maps_ghosts(const Grid& g, bool* maps);

@@ -14,6 +14,8 @@ cudaError_t stage_f64_maps_ghosts(const Grid& g, bool* maps)
 
 cudaError_t launch_stage_f64(const StageParams& p, cudaStream_t s)
 {
+    // (with a stage update the kernel holds -dt Res in the residual's place: finish_tile)
+    if (p.res && p.qout) return cudaErrorInvalidValue;
     if (p.ph.cons) return launch_stage_cons_f64(p, s);
     if (p.ph.order == 4) return launch_stage_order4_f64(p, s);
     if (p.ph.mu > 0.0) return launch_stage_viscous_f64(p, s);
