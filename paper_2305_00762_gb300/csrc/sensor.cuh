@@ -13,6 +13,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace gbr {
@@ -20,8 +21,6 @@ namespace gbr {
 constexpr int kSensorIn = 50;
 constexpr int kSensorK = 64;      // padded input width
 constexpr int kSensorH = 32;      // hidden width
-// Row pitches of the transposed weights in the device copy (the kernels
-// re-order them into the tensor cores' core-matrix layout in shared memory).
 // Position of element (n, k) of a K-major operand in 8 x 8 core matrices (8
 // rows of 16 bytes each) with kgroups of them along k: the tensor cores'
 // shared-memory layout without swizzle.
@@ -48,11 +47,13 @@ struct alignas(16) SensorDev {
     __nv_bfloat16 w2c[kSensorH * kSensorH];
     float b1[kSensorH], b2[kSensorH], w3[kSensorH], b3, pad[3];
 };
+static_assert(offsetof(SensorDev, w1c) == 0 && offsetof(SensorDev, w2c) == sizeof(__nv_bfloat16) * kSensorH * kSensorK,
+              "copy_weights takes both arrays as one run of 16-byte words");
 // The weights into shared memory (16-byte aligned), by the whole block.
 __device__ __forceinline__ void copy_weights(const SensorDev* w, __nv_bfloat16* w1c, __nv_bfloat16* w2c)
 {
     constexpr int n1 = kSensorH * kSensorK / 8, n2 = kSensorH * kSensorH / 8;
-    const uint4* a = reinterpret_cast<const uint4*>(w->w1c);  // w2c follows w1c
+    const uint4* a = reinterpret_cast<const uint4*>(w);
     for (int i = threadIdx.x; i < n1 + n2; i += blockDim.x)
         (i < n1 ? reinterpret_cast<uint4*>(w1c)[i] : reinterpret_cast<uint4*>(w2c)[i - n1]) = a[i];
 }
