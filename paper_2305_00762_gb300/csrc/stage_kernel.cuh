@@ -10,9 +10,8 @@
 //
 // T is the arithmetic type of the stencil, reconstruction and flux work: float
 // here (the FP32 form); the FP64 form runs the same phases on the integer pipe
-// (fixed_stage.cuh) and shares the staging, the Riemann solver's frame, the
-// viscous flux and the stage update. The state, the stage combination and the
-// positivity check are always FP64.
+// (fixed_stage.cuh) and shares the staging, the wavespeed and the stage update.
+// The state, the stage combination and the positivity check are always FP64.
 #pragma once
 
 #include <cuda.h>
@@ -177,23 +176,12 @@ template <typename T>
 __device__ __forceinline__ bool mp_accept(T x, T thr) { return x <= thr; }
 
 // The last step of Eq. mp-procedure from Phi_j, Phi_{j+1}, Phi^MD, Phi^UL,
-// Phi^LC and the GRB value pl. Phi^min = max(min(Phi_j, Phi_{j+1}, MD),
-// min(Phi_j, UL, LC)) is min(Phi_j, max(min(Phi_{j+1}, MD), min(UL, LC)))
-// (min distributes over max), and likewise Phi^max: four comparisons each
-// instead of five. Phi^min <= Phi_j <= Phi^max, so pl + minmod(Phi^min - pl,
-// Phi^max - pl) is the median of pl, Phi^min and Phi^max: pl clamped to
-// [Phi^min, Phi^max], taken without arithmetic (the formula's value up to
-// the rounding of (Phi^min - pl) + pl).
-template <typename T>
-__device__ __forceinline__ T mp_clamp(T p2, T p3, T md, T ul, T lc, T pl)
-{
-    const T pmin = tmin(p2, tmax(tmin(p3, md), tmin(ul, lc)));
-    const T pmax = tmax(p2, tmin(tmax(p3, md), tmax(ul, lc)));
-    return tmin(tmax(pl, pmin), pmax);
-}
-// FP32: the bounds as the paper writes them, each a maximum (minimum) of two
-// three-operand minima (maxima), the min / max instructions taking three
-// operands.
+// Phi^LC and the GRB value pl: Phi^min <= Phi_j <= Phi^max, so pl +
+// minmod(Phi^min - pl, Phi^max - pl) is the median of pl, Phi^min and Phi^max,
+// pl clamped to [Phi^min, Phi^max], taken without arithmetic (the formula's
+// value up to the rounding of (Phi^min - pl) + pl). The bounds as the paper
+// writes them, each a maximum (minimum) of two three-operand minima (maxima),
+// the min / max instructions taking three operands.
 __device__ __forceinline__ float fmin3(float a, float b, float c)
 {
     float r;
@@ -1655,9 +1643,8 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
     // face; x and y faces share the call, with pointers and strides chosen
     // per face).
     {
-        // Whole warps iterate together (the limiter packing in meg7_pair
-        // needs all 32 lanes); a lane past the last face repeats it and
-        // stores nothing.
+        // Whole warps iterate together; a lane past the last face repeats it
+        // and stores nothing.
         for (int w0 = tid & ~31; w0 < L::NF; w0 += NT) {
             const bool valid = w0 + (tid & 31) < L::NF;
             const int w = valid ? w0 + (tid & 31) : L::NF - 1;
@@ -1763,17 +1750,17 @@ __device__ __forceinline__ void stage_tile(const StageParams& P, const int tx0, 
 // One CTA per tile; the tile + halo is staged by a tensor copy described by
 // tmap (the stage's input state, see encode_state_map). Each instance is
 // held to the register budget of the CTAs per SM that its shared memory
-// allows (FP64: 2, 1 for MEG7-cons; FP32: 3, 2 viscous or MEG7-cons): small
-// source changes could otherwise push the allocation over the budget and cut
+// allows (3; 2 viscous, MEG7-cons or with the fused sensor): small source
+// changes could otherwise push the allocation over the budget and cut
 // the resident warps.
-template <typename T, bool VISC, bool CONS, int LEARNED = 0>
+template <bool VISC, bool CONS, int LEARNED = 0>
 constexpr int stage_min_blocks()
 {
-    return sizeof(T) == 8 ? (CONS ? 1 : 2) : ((VISC || CONS || LEARNED == 2) ? 2 : 3);
+    return (VISC || CONS || LEARNED == 2) ? 2 : 3;
 }
 
 template <typename T, int BX, int BY, int NT, bool VISC, int LEARNED, int ORDER, bool CONS>
-__global__ void __launch_bounds__(NT, stage_min_blocks<T, VISC, CONS, LEARNED>()) stage_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
+__global__ void __launch_bounds__(NT, stage_min_blocks<VISC, CONS, LEARNED>()) stage_kernel(const StageParams P, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     dependent_start();
