@@ -509,19 +509,8 @@ cudaError_t launch_fixed_tiles(const StageParams& p, cudaStream_t s)
     return launch_dependent(kern, grid, NT, F::bytes, s, p, map);
 }
 
-// Tile shapes. The faces of 16 x 15 (511) are two rounds of 256 threads without
-// spills at 128 registers, the fastest per cell where there are tiles enough
-// (1024^2 step 1.94 ms; 16 x 16 with 288 threads 2.03, 20 x 12 1.97, 28 x 8
-// 2.05). A grid of few tiles is bound by the tiles the busiest SM gets, so a
-// smaller tile that divides the work further wins: 16 x 8 with its 280 faces in
-// one round, 8 x 4 where even that leaves SMs idle. A step's time grows with c k,
-// k the tiles of the busiest SM and c = 63, 36.5 and 15.5; the smallest c k is
-// taken, k rounded up while it is small and the last wave counts (measured, us
-// with 16 x 15 / 16 x 8 / 8 x 4: 64^2 106 / 72 / 43, 96^2 106 / 72 / 51, 128^2
-// 106 / 72 / 93, 136^2 110 / 97 / 95, 176^2 107 / 107 / 169, 200^2 168 / 149 / 214;
-// nowhere in 48^2 .. 200^2 is the choice more than 7% off the best). The result
-// does not depend on the shape.
-inline cudaError_t fixed_tile_shape(const Grid& g, TileShape* t)
+// The shape of tile_rule.h on the current device.
+inline cudaError_t fixed_tile_shape(const Grid& g, bool cons, bool viscous, TileShape* t)
 {
     static PerDevice<int> sm_count;
     int sms = 0;
@@ -531,13 +520,7 @@ inline cudaError_t fixed_tile_shape(const Grid& g, TileShape* t)
         return r != cudaSuccess ? r : cudaDeviceGetAttribute(v, cudaDevAttrMultiProcessorCount, dev);
     });
     if (e != cudaSuccess) return e;
-    auto cost = [&](int bx, int by, double c) {
-        const double k = (double)((g.nx + bx - 1) / bx) * ((g.ny + by - 1) / by) / sms;
-        const double up = (double)(long long)k;
-        return c * (k <= 16.0 ? (k > up ? up + 1.0 : up) : k + 0.5);
-    };
-    const double big = cost(16, 15, 63.0), mid = cost(16, 8, 36.5), tiny = cost(8, 4, 15.5);
-    *t = tiny < mid && tiny < big ? TileShape{8, 4} : mid < big ? TileShape{16, 8} : TileShape{16, 15};
+    *t = fixed_tile_rule(g.nx, g.ny, sms, cons, viscous);
     return cudaSuccess;
 }
 
@@ -545,7 +528,7 @@ template <bool VISC, int ORDER, bool CONS = false>
 cudaError_t launch_fixed(const StageParams& p, cudaStream_t s)
 {
     TileShape t;
-    const cudaError_t e = fixed_tile_shape(p.g, &t);
+    const cudaError_t e = fixed_tile_shape(p.g, CONS, VISC, &t);
     if (e != cudaSuccess) return e;
     if (t.bx == 8) return launch_fixed_tiles<8, 4, 192, VISC, ORDER, CONS>(p, s);
     if (t.by == 8) return launch_fixed_tiles<16, 8, 288, VISC, ORDER, CONS>(p, s);

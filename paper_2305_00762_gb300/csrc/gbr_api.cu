@@ -190,7 +190,7 @@ int ghosts(gbr_ctx* c, double* q, int mode, double dt, double cfl, double dt_max
 int stage_ghosts(gbr_ctx* c, StageParams& p, double* q, int mode, double dt, double cfl, double dt_max, double c_stage)
 {
     bool maps = false;
-    if (c->precision == 64) GBR_TRY(stage_f64_maps_ghosts(c->g, &maps));
+    if (c->precision == 64) GBR_TRY(stage_f64_maps_ghosts(c->g, c->ph, &maps));
     if (!maps) return ghosts(c, q, mode, dt, cfl, dt_max, c_stage);
     p.map = 1;
     p.gh = ghost_params(c, q, mode, dt, cfl, dt_max, c_stage);

@@ -8,6 +8,8 @@
 
 #include <atomic>
 
+#include "tile_rule.h"
+
 namespace gbr {
 
 // Per-device launch set-up (kernel attributes and occupancy-derived grid
@@ -210,10 +212,6 @@ struct BatchCase {
     long long ghost_begin;  // first batch ghost cell of this case
 };
 
-struct TileShape {
-    int bx, by;
-};
-
 cudaError_t launch_ghosts(const GhostParams& p, cudaStream_t s);
 cudaError_t launch_set_time(DevScalars* d, int cur, double t, cudaStream_t s);
 // Ghost cells of buffer `buf` (0, 1, 2) of every case; with mode 2 the first
@@ -270,7 +268,7 @@ cudaError_t launch_wavespeed(const Grid& g, const Physics& ph, const double* q, 
 cudaError_t launch_stage_f64(const StageParams& p, cudaStream_t s);  // p.res or p.qout, not both
 // Whether the FP64 stage of this grid can read ghost cells through the boundary
 // rules (StageParams::map).
-cudaError_t stage_f64_maps_ghosts(const Grid& g, bool* maps);
+cudaError_t stage_f64_maps_ghosts(const Grid& g, const Physics& ph, bool* maps);
 cudaError_t launch_stage_f32(const StageParams& p, cudaStream_t s);
 cudaError_t launch_stage_viscous_f64(const StageParams& p, cudaStream_t s);
 cudaError_t launch_stage_order4_f64(const StageParams& p, cudaStream_t s);

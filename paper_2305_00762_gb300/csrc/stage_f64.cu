@@ -4,10 +4,10 @@
 
 namespace gbr {
 
-cudaError_t stage_f64_maps_ghosts(const Grid& g, bool* maps)
+cudaError_t stage_f64_maps_ghosts(const Grid& g, const Physics& ph, bool* maps)
 {
     TileShape t;
-    const cudaError_t e = fixed_tile_shape(g, &t);
+    const cudaError_t e = fixed_tile_shape(g, ph.cons != 0, ph.mu > 0.0, &t);
     if (e == cudaSuccess) *maps = fixed_maps_ghosts(t.bx);
     return e;
 }
