@@ -55,10 +55,8 @@
 
 #ifdef __CUDACC__
 #define GBR_HD __host__ __device__ __forceinline__
-#define GBR_OUTLINE __host__ __device__ __noinline__
 #else
 #define GBR_HD inline
-#define GBR_OUTLINE __attribute__((noinline))
 #include <string.h>
 #endif
 
@@ -224,56 +222,52 @@ constexpr int kGrbShift7 = 10;  // n = 840 delta / 2^10
 constexpr int kGrbShift4 = 13;  // order 4: n = 10080 delta / 2^13
 constexpr int kCurvShift = 7;   // d = 120 d_j / 2^7
 
-// Those about one cell (q: its value among its neighbours', k: its place, 0 for
-// cell j-1): d, and n[k-1] for the cells beside the face.
-template <int ORDER>
-GBR_HD void centred(const i64* q, int k, i64& d_out, i64 (&n_out)[2])
-{
-    const i64 c2 = q[0] + q[0];
-    const i64 B1 = q[1] + q[-1] - c2, B2 = c2 - q[2] - q[-2];  // (B2, B4, A2 with their signs changed)
-    const i64 B3 = q[3] + q[-3] - c2, B4 = c2 - q[4] - q[-4];
-    Acc d;
-    if (ORDER == 4 || k == 0 || k == 3) {
-        d.add(B1, 231);
-        d.add(B2, 44);
-        d.add(B3, 9);
-        d.add(B4, 1);
-    }
-    if (k == 1 || k == 2) {
-        const i64 A1 = q[1] - q[-1], A2 = q[-2] - q[2], A3 = q[3] - q[-3];
-        Acc even, odd;
-        if (ORDER == 4) {
-            even.add(B1, 1617);
-            even.add(B2, 308);
-            even.add(B3, 63);
-            even.add(B4, 7);
-            odd.add(A1, 3780);
-            odd.add(A2, 756);
-            odd.add(A3, 84);
-        } else {
-            even.add(B1, 169);
-            even.add(B2, 41);
-            even.add(B3, 9);
-            even.add(B4, 1);
-            odd.add(A1, 315);
-            odd.add(A2, 63);
-            odd.add(A3, 7);
-            d = even;
-            d.add(B1, 62);
-            d.add(B2, 3);
-        }
-        const Acc n = k == 1 ? even + odd : even - odd;
-        n_out[k - 1] = n.shift<ORDER == 4 ? kGrbShift4 : kGrbShift7>();
-    }
-    d_out = d.shift<kCurvShift>();
-}
 template <int ORDER>
 GBR_HD void functionals(const i64 (&q)[12], Functionals& f)
 {
 #pragma unroll
     for (int k = 0; k < 4; ++k) f.v[k] = q[4 + k];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) centred<ORDER>(q + 4 + k, k, f.d[k], f.n);
+    for (int k = 0; k < 4; ++k) {
+        const int c = 4 + k;
+        const i64 c2 = q[c] + q[c];
+        const i64 B1 = q[c + 1] + q[c - 1] - c2, B2 = c2 - q[c + 2] - q[c - 2];  // (B2, B4, A2 with their signs changed)
+        const i64 B3 = q[c + 3] + q[c - 3] - c2, B4 = c2 - q[c + 4] - q[c - 4];
+        Acc d;
+        if (ORDER == 4 || k == 0 || k == 3) {
+            d.add(B1, 231);
+            d.add(B2, 44);
+            d.add(B3, 9);
+            d.add(B4, 1);
+        }
+        if (k == 1 || k == 2) {
+            const i64 A1 = q[c + 1] - q[c - 1], A2 = q[c - 2] - q[c + 2], A3 = q[c + 3] - q[c - 3];
+            Acc even, odd;
+            if (ORDER == 4) {
+                even.add(B1, 1617);
+                even.add(B2, 308);
+                even.add(B3, 63);
+                even.add(B4, 7);
+                odd.add(A1, 3780);
+                odd.add(A2, 756);
+                odd.add(A3, 84);
+            } else {
+                even.add(B1, 169);
+                even.add(B2, 41);
+                even.add(B3, 9);
+                even.add(B4, 1);
+                odd.add(A1, 315);
+                odd.add(A2, 63);
+                odd.add(A3, 7);
+                d = even;
+                d.add(B1, 62);
+                d.add(B2, 3);
+            }
+            const Acc n = k == 1 ? even + odd : even - odd;
+            f.n[k - 1] = n.shift<ORDER == 4 ? kGrbShift4 : kGrbShift7>();
+        }
+        f.d[k] = d.shift<kCurvShift>();
+    }
 }
 
 // f r / 2^64 of every functional.

@@ -238,13 +238,15 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     // reconstruction: where one small tile is all an SM has, a face's chain of
     // dependent instructions is the time, 64^2 step 50.0 -> 44.8 us).
     constexpr int HALF = NT / 2;
+    static_assert(NT % 32 == 0, "whole warps");
     constexpr bool SPLIT = fixed_splits_faces(L::NF, NT);
     __shared__ double sT[SPLIT ? 6 * L::NF : 1];  // ut L, ut R, F of the face
     auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };  // (reached from both halves' code)
-    for (int item = tid; item < (SPLIT ? NT : L::NF); item += NT) {
+    // Whole warps: a lane past the last face repeats it and stores nothing.
+    for (int item = tid; item < (SPLIT ? NT : (L::NF + 31) / 32 * 32); item += NT) {
         const bool second = SPLIT && item >= HALF;
         const int wa = second ? item - HALF : item;
-        const bool live = !SPLIT || wa < L::NF;
+        const bool live = wa < L::NF;
         const int w = live ? wa : L::NF - 1;
         const bool xf = w < L::NHX;
         const int w2 = xf ? w : w - L::NHX;
@@ -282,7 +284,8 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                 x.e[k] = sE[at + (k - 5) * su];
             }
         };
-        const fx::Face face{sM + c, sE + c, su, NU, pn};  // for the few faces evaluated in FP64 (wide_face.cuh)
+        const fx::WideFace face{sM, sE, NU, RW, c, xf};  // for the few faces of wide_face.cuh
+        auto any = [](bool b) { return __any_sync(0xffffffffu, b); };
         double Fs[4];
         auto reconstruct = [&] {  // the central part where sigma = 1 (Sec. 2.4)
             const int at = xf ? fr * L::FXW + fc + 4 : (fr + 4) * BX + fc, sf = xf ? 1 : BX;
@@ -312,8 +315,10 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                 if constexpr (!CONS) {
                     bool wide;
                     const int still = fx::still_exponent(sE[c], sE[3 * NU + c], sE[c + su], sE[3 * NU + c + su]);
-                    if (!fx::shear_states<ORDER>(load, still, ut, wide)) ut[0] = __longlong_as_double(0x7ff8000000000000ll);  // refused
-                    else if (wide) fx::wide_shear<ORDER>(face, ut);
+                    const bool in_range = fx::shear_states<ORDER>(load, still, ut, wide);
+                    wide = wide && in_range;
+                    if (any(wide)) fx::wide_shear_warp<ORDER>(face, wide, ut);
+                    if (!in_range) ut[0] = __longlong_as_double(0x7ff8000000000000ll);  // refused
                 }
                 if (!trouble) reconstruct();
                 if (live) {
@@ -349,10 +354,12 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                 s.ut[0] = sT[w];
                 s.ut[1] = sT[L::NF + w];
                 s.ok = s.ok && fx::exponent(s.ut[0]) != 2047;
-            } else if (s.ok && s.wide_ut) {
-                fx::wide_shear<ORDER>(face, s.ut);
+            } else {
+                const bool wide = s.ok && s.wide_ut;
+                if (any(wide)) fx::wide_shear_warp<ORDER>(face, wide, s.ut);
             }
-            if (s.ok && s.wide && positive) fx::wide_states<ORDER>(face, ph.gamma, s);
+            const bool wide = s.ok && s.wide && positive;
+            if (any(wide)) fx::wide_states_warp<ORDER>(face, wide, ph.gamma, s);
             rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
             rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
             ok = s.ok;
@@ -378,8 +385,9 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                     return e;
                 },
                 C, s);
-            if (s.ok && s.wide_w3) fx::wide_cons_shear<ORDER>(face, C.v, s.w3);
-            if (s.ok && s.wide && positive) fx::wide_cons_states<ORDER>(face, C, s);
+            const bool wide_w3 = s.ok && s.wide_w3, wide = s.ok && s.wide && positive;
+            if (any(wide_w3)) fx::wide_cons_shear_warp<ORDER>(face, wide_w3, C.v, s.w3);
+            if (any(wide)) fx::wide_cons_states_warp<ORDER>(face, wide, C, s);
             if constexpr (SPLIT) meet();
             ok = s.ok;
             // Back with the right eigenvectors, to primitives: rho un = u rho
@@ -413,8 +421,8 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             pR = cell(3, su);
         }
         // Flux reconstruction (Sec. 2.4).
+        if (!live) break;  // (the last round)
         if constexpr (SPLIT) {
-            if (!live) break;
 #pragma unroll
             for (int m = 0; m < 4; ++m) Fs[m] = trouble ? 0.0 : sT[(2 + m) * L::NF + w];
         } else if (!trouble) {

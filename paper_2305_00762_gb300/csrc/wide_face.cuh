@@ -12,19 +12,24 @@
 // too, and the projection and the limiter in FP64.
 //
 // Such faces lie within six cells of a jump by a factor of 16 or more, or have a
-// shear velocity far below the stencil's. They are few (2% of the faces of a
-// developed four-quadrant flow), so the code is kept out of line: inlined, its
-// registers would be taken from every face. FP64 operations a face: 22 for the
-// shear field, 110 for the other three (with gradients and differences in FP64
-// as well 78 and 290: one instruction holds the FP64 pipe for 19 clocks however
-// few lanes are active, and a warp with one such face issues them all). What the
-// accuracy costs, us a pass without / with: 64^2 vortex 880 / 898, four-quadrant
-// 400^2 1451 / 1592, 1024^2 3986 / 4138, MEG7-cons 400^2 1921 / 2567, double Mach
-// 1024 x 256 (a shock of ratio 116 through four tiles a row) 1881 / 2221.
+// shear velocity far below the stencil's: 2% of the faces of a developed
+// four-quadrant flow, scattered over a sixth of its warps. What they cost is a
+// chain of dependent instructions that the rest of the CTA waits for, so a warp
+// takes its faces eight at a time, four lanes a face: a lane forms the functionals
+// about one of the cells j-1 .. j+2, and then the limited value of one side. The
+// code is kept out of line: inlined, its registers would be taken from every face.
+// (One face a lane, gradients and differences in FP64 as well: four-quadrant 1024^2
+// 4.18 ms a pass, double Mach 2.51; a lane a face with the functionals on integers
+// 4.17 and 2.22; four lanes 4.13 and 2.11.)
+//
+// What the accuracy costs, us a pass without / with flags and this code: 64^2 vortex
+// 880 / 897, four-quadrant 400^2 1450 / 1591, 1024^2 3983 / 4135, 4096^2 30770 /
+// 32250, viscous 1280 x 640 3752 / 3862, MEG7-cons 400^2 1918 / 2386, double Mach
+// 1024 x 256 (a shock of ratio 116 through four tiles a row) 1878 / 2115. The flags
+// are 2% everywhere; a tile with a line of such faces takes 1.25 times as long.
 //
 // The MP test's absolute threshold, which fixed point leaves out, is applied here,
-// and faces where it tells (kSmall: densities below 2^-12) are evaluated here too:
-// four-quadrant flow 1024^2 in units with densities of 1e-4 8.5 ms a pass.
+// and faces where it tells (kSmall: densities below 2^-12) are evaluated here too.
 #pragma once
 
 #include "fixed_math.cuh"
@@ -55,36 +60,103 @@ struct Face {
     GBR_HD int at(int v) const { return (v == 1 ? normal : v == 2 ? 3 - normal : v) * values; }  // variable rho, un, ut, p
 };
 
-// Functionals (fixed_face.cuh) as doubles.
-struct WideFunctionals {
-    double v[4], n[2], d[4];
+// The four lanes of a face. V is a value of each; each(f) is f(k) of lane k,
+// pick(x, k) lane k's value, own(x, k) the same where k is the lane itself.
+#ifdef __CUDACC__
+struct WideLanes {
+    typedef double V;
+    int base;  // the first one
+    template <typename F>
+    __device__ __forceinline__ V each(F f) const { return f((int)threadIdx.x & 3); }
+    __device__ __forceinline__ double pick(const V& x, int k) const { return __shfl_sync(0xffffffffu, x, base + k); }
+    __device__ __forceinline__ double own(const V& x, int) const { return x; }
+};
+#define GBR_LANES __device__ __forceinline__
+#define GBR_LANES_CALL __device__ __noinline__
+#else
+struct WideLanes {
+    struct V {
+        double x[4];
+    };
+    template <typename F>
+    V each(F f) const { return V{{f(0), f(1), f(2), f(3)}}; }
+    double pick(const V& a, int k) const { return a.x[k]; }
+    double own(const V& a, int k) const { return a.x[k]; }
+};
+#define GBR_LANES inline
+#define GBR_LANES_CALL inline
+#endif
+
+// A variable or field about the cells j-1 .. j+2 (lane k: cell j-1+k): its value,
+// the curvature functional d, and for k = 1, 2 the GRB functional n of the left
+// and the right value (fixed_face.cuh).
+struct WideField {
+    WideLanes::V v, d, n;
 };
 template <int ORDER>
-GBR_HD void wide_functionals(const Face& f, int variable, WideFunctionals& o)
+GBR_HD void wide_functionals(const Face& f, int variable, int k, double& v, double& d, double& n)
 {
-    const int at = f.at(variable);
-    i64 m[12];
-    int e[12];
+    const int at = f.at(variable) + (k - 1) * f.step;
+    i64 q[9];
+    int e[9], s = kExpMin;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        m[k] = f.m[at + (k - 5) * f.step];
-        e[k] = f.e[at + (k - 5) * f.step];
+    for (int c = 0; c < 9; ++c) {
+        q[c] = f.m[at + (c - 4) * f.step];
+        e[c] = f.e[at + (c - 4) * f.step];
+        s = larger(s, e[c]);
     }
+    v = unsplit(q[4], e[4]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        o.v[k] = unsplit(m[4 + k], e[4 + k]);
-        int s = kExpMin;
-#pragma unroll
-        for (int c = 0; c < 9; ++c) s = larger(s, e[k + c]);
-        i64 q[9];
-#pragma unroll
-        for (int c = 0; c < 9; ++c) q[c] = aligned(m[k + c], e[k + c], s);
-        i64 d, n[2];
-        centred<ORDER>(q + 4, k, d, n);
-        o.d[k] = to_double(d, s);
-        if (k == 1) o.n[0] = to_double(n[0], s);
-        if (k == 2) o.n[1] = to_double(n[1], s);
+    for (int c = 0; c < 9; ++c) q[c] = aligned(q[c], e[c], s);
+    const i64 c2 = q[4] + q[4];
+    const i64 B1 = q[5] + q[3] - c2, B2 = c2 - q[6] - q[2];  // (B2, B4, A2 with their signs changed)
+    const i64 B3 = q[7] + q[1] - c2, B4 = c2 - q[8] - q[0];
+    const i64 A1 = q[5] - q[3], A2 = q[2] - q[6], A3 = q[7] - q[1];
+    Acc curv, even, odd;
+    curv.add(B1, 231);
+    curv.add(B2, 44);
+    curv.add(B3, 9);
+    curv.add(B4, 1);
+    if (ORDER == 4) {
+        even.add(B1, 1617);
+        even.add(B2, 308);
+        even.add(B3, 63);
+        even.add(B4, 7);
+        odd.add(A1, 3780);
+        odd.add(A2, 756);
+        odd.add(A3, 84);
+    } else {
+        even.add(B1, 169);
+        even.add(B2, 41);
+        even.add(B3, 9);
+        even.add(B4, 1);
+        odd.add(A1, 315);
+        odd.add(A2, 63);
+        odd.add(A3, 7);
     }
+    const Acc sum = k == 2 ? even - odd : even + odd;
+    d = to_double(curv.shift<kCurvShift>(), s);
+    n = to_double(sum.shift<ORDER == 4 ? kGrbShift4 : kGrbShift7>(), s);
+}
+template <int ORDER>
+GBR_LANES WideField wide_variable(const WideLanes& L, const Face& f, int variable)
+{
+    WideField o;
+#ifdef __CUDACC__
+    wide_functionals<ORDER>(f, variable, (int)threadIdx.x & 3, o.v, o.d, o.n);
+#else
+    for (int k = 0; k < 4; ++k) wide_functionals<ORDER>(f, variable, k, o.v.x[k], o.d.x[k], o.n.x[k]);
+#endif
+    return o;
+}
+// x + a y
+GBR_LANES WideField combine(const WideLanes& L, const WideField& x, double a, const WideField& y)
+{
+    WideField o;
+    o.v = L.each([&](int k) { return fmadd(a, L.own(y.v, k), L.own(x.v, k)); });
+    o.d = L.each([&](int k) { return fmadd(a, L.own(y.d, k), L.own(x.d, k)); });
+    o.n = L.each([&](int k) { return fmadd(a, L.own(y.n, k), L.own(x.n, k)); });
+    return o;
 }
 
 // minmod and the clamp on the bits (values that are not NaN).
@@ -105,125 +177,184 @@ GBR_HD double mp_clamp(double p2, double p3, double md, double ul, double lc, do
     return of_bits((u64)(k ^ ((k >> 63) & 0x7fffffffffffffffll)));
 }
 
-// The MEG7 values (Eqs. grb, mp5Condition, mp-procedure) left and right of the
-// face of a field carried at `scale` times its value.
+// The MEG7 values (Eqs. grb, mp5Condition, mp-procedure) of a field carried at
+// `scale` times its value: the left one in lanes 0 and 2, the right one in 1 and 3.
 template <int ORDER>
-GBR_HD void wide_limited(const WideFunctionals& f, double scale, double& vl, double& vr)
+GBR_LANES WideLanes::V wide_limited(const WideLanes& L, const WideField& f, double scale)
 {
     constexpr double kN = ORDER == 4 ? 8192.0 / 10080.0 : 1024.0 / 840.0, kD = 128.0 / 120.0;  // n, d -> delta, d_j
     const double st = 1e-20 * scale, thr = st * st;
-    const double b = f.v[2] - f.v[1], a[2] = {f.v[0] - f.v[1], f.v[3] - f.v[2]};
-    const double md = 0.5 * fmadd(-kD, minmod(f.d[1], f.d[2]), f.v[1] + f.v[2]);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const double c = f.v[1 + k], delta = kN * f.n[k], m = minmod(k ? -b : b, -7.0 * a[k]);
-        double v = c + delta;
-        if (!(delta * (delta - m) <= thr)) {
-            const double mm = minmod(f.d[1 + k], f.d[k ? 3 : 0]);
-            v = mp_clamp(c, f.v[2 - k], md, fmadd(-7.0, a[k], c), fmadd(4.0 / 3.0 * kD, mm, fmadd(-0.5, a[k], c)), v);
-        }
-        (k ? vr : vl) = v;
-    }
-}
-// o = x + a y, every functional
-GBR_HD void combine(const WideFunctionals& x, double a, const WideFunctionals& y, WideFunctionals& o)
-{
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        o.v[k] = fmadd(a, y.v[k], x.v[k]);
-        o.d[k] = fmadd(a, y.d[k], x.d[k]);
-    }
-    o.n[0] = fmadd(a, y.n[0], x.n[0]);
-    o.n[1] = fmadd(a, y.n[1], x.n[1]);
+    return L.each([&](int k) {
+        const int s = k & 1;
+        const double c = L.pick(f.v, 1 + s), o = L.pick(f.v, 2 - s), a = L.pick(f.v, 3 * s) - c;  // own cell, across, behind
+        const double dc = L.pick(f.d, 1 + s), da = L.pick(f.d, 2 - s), db = L.pick(f.d, 3 * s);
+        const double delta = kN * L.pick(f.n, 1 + s), m = minmod(o - c, -7.0 * a), v = c + delta;
+        const double md = 0.5 * fmadd(-kD, minmod(dc, da), c + o), ul = fmadd(-7.0, a, c);
+        const double lc = fmadd(4.0 / 3.0 * kD, minmod(dc, db), fmadd(-0.5, a, c));
+        return delta * (delta - m) <= thr ? v : mp_clamp(c, o, md, ul, lc, v);
+    });
 }
 
+// ut; and rho, un and p, of fields as in face_states: p -/+ rho c un and rho -
+// p / c^2 (the sides in the lanes of wide_limited).
 template <int ORDER>
-GBR_OUTLINE void wide_shear(Face f, double (&ut)[2])
+GBR_LANES WideLanes::V wide_shear(const WideLanes& L, const Face& f)
 {
-    WideFunctionals x;
-    wide_functionals<ORDER>(f, 2, x);
-    wide_limited<ORDER>(x, 1.0, ut[0], ut[1]);
+    return wide_limited<ORDER>(L, wide_variable<ORDER>(L, f, 2), 1.0);
 }
-
-// rho, un and p of both sides. Fields as in face_states: p -/+ rho c un and
-// rho - p / c^2.
 template <int ORDER>
-GBR_OUTLINE void wide_states(Face f, double gamma, FaceStates& o)
+GBR_LANES void wide_states(const WideLanes& L, const Face& f, double gamma, WideLanes::V& ro, WideLanes::V& uo, WideLanes::V& po)
 {
-    WideFunctionals P, X, W;
-    wide_functionals<ORDER>(f, 3, P);
-    wide_functionals<ORDER>(f, 0, X);
-    const double r = 0.5 * (X.v[1] + X.v[2]), gp = gamma * (0.5 * (P.v[1] + P.v[2]));
+    const WideField P = wide_variable<ORDER>(L, f, 3), R = wide_variable<ORDER>(L, f, 0);
+    const double r = 0.5 * (L.pick(R.v, 1) + L.pick(R.v, 2)), gp = gamma * (0.5 * (L.pick(P.v, 1) + L.pick(P.v, 2)));
     const double y = rsqrt(gp * r), c = gp * y, rc = r * c, ic = r * y, ic2 = ic * ic;
-    double s[2], l[2], h[2];
-    combine(X, -ic2, P, W);
-    wide_limited<ORDER>(W, 1.0, s[0], s[1]);
-    wide_functionals<ORDER>(f, 1, X);
-#pragma unroll 1
-    for (int k = 0; k < 2; ++k) {  // (one copy of the limiter)
-        combine(P, k ? rc : -rc, X, W);
-        double a, b;
-        wide_limited<ORDER>(W, 2.0 * c * c, a, b);
-        if (k) l[1] = a, h[1] = b;
-        else l[0] = a, h[0] = b;
-    }
-    const double be = 0.5 * ic2, hrc = 0.5 * y, pl = l[0] + l[1], pr = h[0] + h[1];
-    o.r[0] = fmadd(be, pl, s[0]);
-    o.r[1] = fmadd(be, pr, s[1]);
-    o.un[0] = hrc * (l[1] - l[0]);
-    o.un[1] = hrc * (h[1] - h[0]);
-    o.p[0] = 0.5 * pl;
-    o.p[1] = 0.5 * pr;
+    const WideLanes::V s = wide_limited<ORDER>(L, combine(L, R, -ic2, P), 1.0);
+    const WideField U = wide_variable<ORDER>(L, f, 1);
+    const WideLanes::V a = wide_limited<ORDER>(L, combine(L, P, -rc, U), 2.0 * c * c);
+    const WideLanes::V b = wide_limited<ORDER>(L, combine(L, P, rc, U), 2.0 * c * c);
+    ro = L.each([&](int k) { return fmadd(0.5 * ic2, L.own(a, k) + L.own(b, k), L.own(s, k)); });
+    uo = L.each([&](int k) { return 0.5 * y * (L.own(b, k) - L.own(a, k)); });
+    po = L.each([&](int k) { return 0.5 * (L.own(a, k) + L.own(b, k)); });
 }
 
-// MEG7-cons: w3, and the others.
+// MEG7-cons: w3, and the others of ConsStates. (Four variables and four fields: a
+// call each, 400^2 pass 2465 -> 2402 us; for the primitive form's a call is slower
+// than the copies, 1024^2 4131 -> 4157.)
 template <int ORDER>
-GBR_OUTLINE void wide_cons_shear(Face f, double v, double (&w3)[2])
+GBR_LANES_CALL WideField wide_variable_call(WideLanes L, Face f, int variable)
 {
-    WideFunctionals Q, W;
-    wide_functionals<ORDER>(f, 0, Q);
-    wide_functionals<ORDER>(f, 2, W);
-    combine(W, -v, Q, W);
-    wide_limited<ORDER>(W, 1.0, w3[0], w3[1]);
+    return wide_variable<ORDER>(L, f, variable);
 }
 template <int ORDER>
-GBR_OUTLINE void wide_cons_states(Face f, ConsCoefs C, ConsStates& o)
+GBR_LANES_CALL WideLanes::V wide_limited_call(WideLanes L, WideField f, double scale)
 {
-    WideFunctionals Q, A, T, W;  // A and t as in cons_states
-    double l[2], h[2];
-    wide_functionals<ORDER>(f, 3, Q);
+    return wide_limited<ORDER>(L, f, scale);
+}
+template <int ORDER>
+GBR_LANES WideLanes::V wide_cons_shear(const WideLanes& L, const Face& f, double v)
+{
+    const WideField Q = wide_variable_call<ORDER>(L, f, 0), W = wide_variable_call<ORDER>(L, f, 2);
+    return wide_limited_call<ORDER>(L, combine(L, W, -v, Q), 1.0);
+}
+template <int ORDER>
+GBR_LANES void wide_cons_states(const WideLanes& L, const Face& f, const ConsCoefs& C, WideLanes::V& ro, WideLanes::V& so, WideLanes::V& uo)
+{
+    WideField zero, Q = wide_variable_call<ORDER>(L, f, 3);
+    zero.v = zero.d = zero.n = L.each([](int) { return 0.0; });
+    WideField A = combine(L, zero, C.b1, Q), T;  // A and t as in cons_states
+    Q = wide_variable_call<ORDER>(L, f, 1);
+    A = combine(L, A, -C.b1u, Q);
+    T = combine(L, zero, -C.ic, Q);
+    A = combine(L, A, -C.b1v, wide_variable_call<ORDER>(L, f, 2));
+    Q = wide_variable_call<ORDER>(L, f, 0);
+    A = combine(L, A, C.b2, Q);
+    T = combine(L, T, C.uc, Q);
+    const WideLanes::V a = wide_limited_call<ORDER>(L, combine(L, A, 1.0, T), 2.0);   // 2 w1
+    const WideLanes::V b = wide_limited_call<ORDER>(L, combine(L, A, -1.0, T), 2.0);  // 2 w4
+    const WideLanes::V c = wide_limited_call<ORDER>(L, combine(L, Q, -1.0, A), 1.0);  // w2
+    so = L.each([&](int k) { return 0.5 * (L.own(a, k) + L.own(b, k)); });
+    uo = L.each([&](int k) { return 0.5 * (L.own(b, k) - L.own(a, k)); });
+    ro = L.each([&](int k) { return L.own(so, k) + L.own(c, k); });
+}
+
+#ifdef __CUDACC__
+// The faces of a warp that are flagged, by the whole warp: work(L, src) with the
+// lanes L of a face and the lane src it belongs to (a group without one repeats
+// the first), then take(from) with the lane that holds the left values of this
+// lane's face (the next one holds the right ones), or -1.
+template <typename W, typename T>
+__device__ __forceinline__ void wide_faces(bool wide, W work, T take)
+{
+    const int lane = (int)threadIdx.x & 31;
+    unsigned todo = __ballot_sync(0xffffffffu, wide);
+    while (todo) {
+        unsigned rest = todo;
+        int src = __ffs((int)todo) - 1;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) A.v[k] = C.b1 * Q.v[k], A.d[k] = C.b1 * Q.d[k];
-    A.n[0] = C.b1 * Q.n[0], A.n[1] = C.b1 * Q.n[1];
-    wide_functionals<ORDER>(f, 1, Q);
-    combine(A, -C.b1u, Q, A);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) T.v[k] = -C.ic * Q.v[k], T.d[k] = -C.ic * Q.d[k];
-    T.n[0] = -C.ic * Q.n[0], T.n[1] = -C.ic * Q.n[1];
-    wide_functionals<ORDER>(f, 2, Q);
-    combine(A, -C.b1v, Q, A);
-    wide_functionals<ORDER>(f, 0, Q);
-    combine(A, C.b2, Q, A);
-    combine(T, C.uc, Q, T);
-    combine(Q, -1.0, A, Q);
-    double s[2];
-#pragma unroll 1
-    for (int k = 0; k < 3; ++k) {  // 2 w1, 2 w4, w2
-        double a, b;
-        if (k < 2) combine(A, k ? -1.0 : 1.0, T, W);
-        else W = Q;
-        wide_limited<ORDER>(W, k < 2 ? 2.0 : 1.0, a, b);
-        if (k == 0) l[0] = a, h[0] = b;
-        if (k == 1) l[1] = a, h[1] = b;
-        if (k == 2) s[0] = a, s[1] = b;
+        for (int g = 0; g < 8; ++g) {
+            if (g == lane >> 2 && rest) src = __ffs((int)rest) - 1;
+            rest &= rest - 1u;
+        }
+        work(WideLanes{lane & 28}, src);
+        const int rank = __popc(todo & ((1u << lane) - 1u));
+        take(((todo >> lane) & 1u) && rank < 8 ? 4 * rank : -1);
+        todo = rest;
     }
-    o.s[0] = 0.5 * (l[0] + l[1]);
-    o.s[1] = 0.5 * (h[0] + h[1]);
-    o.d[0] = 0.5 * (l[1] - l[0]);
-    o.d[1] = 0.5 * (h[1] - h[0]);
-    o.r[0] = o.s[0] + s[0];
-    o.r[1] = o.s[1] + s[1];
 }
+// Lane `from`'s x (the left value) and the next one's, where from >= 0.
+__device__ __forceinline__ void wide_take(double x, int from, double (&o)[2])
+{
+    const double l = __shfl_sync(0xffffffffu, x, from & 31), r = __shfl_sync(0xffffffffu, x, (from + 1) & 31);
+    if (from >= 0) {
+        o[0] = l;
+        o[1] = r;
+    }
+}
+// The planes and the face of each lane: the cell before it and its direction.
+struct WideFace {
+    const i64* m;
+    const unsigned short* e;
+    int values, row;  // values per plane; distance of rows
+    int cell;
+    bool x;
+    __device__ __forceinline__ Face of(int src) const
+    {
+        const int c = __shfl_sync(0xffffffffu, 2 * cell + (x ? 1 : 0), src);
+        return Face{m + (c >> 1), e + (c >> 1), c & 1 ? 1 : row, values, c & 1 ? 1 : 2};
+    }
+};
+template <int ORDER>
+__device__ __noinline__ void wide_shear_warp(WideFace f, bool wide, double (&ut)[2])
+{
+    double u;
+    wide_faces(
+        wide, [&](const WideLanes& L, int src) { u = wide_shear<ORDER>(L, f.of(src)); }, [&](int from) { wide_take(u, from, ut); });
+}
+template <int ORDER>
+__device__ __noinline__ void wide_states_warp(WideFace f, bool wide, double gamma, FaceStates& o)
+{
+    double r, u, p;
+    wide_faces(
+        wide, [&](const WideLanes& L, int src) { wide_states<ORDER>(L, f.of(src), gamma, r, u, p); },
+        [&](int from) {
+            wide_take(r, from, o.r);
+            wide_take(u, from, o.un);
+            wide_take(p, from, o.p);
+        });
+}
+template <int ORDER>
+__device__ __noinline__ void wide_cons_shear_warp(WideFace f, bool wide, double v, double (&w3)[2])
+{
+    double w;
+    wide_faces(
+        wide, [&](const WideLanes& L, int src) { w = wide_cons_shear<ORDER>(L, f.of(src), __shfl_sync(0xffffffffu, v, src)); },
+        [&](int from) { wide_take(w, from, w3); });
+}
+template <int ORDER>
+__device__ __noinline__ void wide_cons_states_warp(WideFace f, bool wide, ConsCoefs C, ConsStates& o)
+{
+    double r, s, d;
+    wide_faces(
+        wide,
+        [&](const WideLanes& L, int src) {
+            auto of = [&](double x) { return __shfl_sync(0xffffffffu, x, src); };
+            ConsCoefs S;
+            S.b1 = of(C.b1);
+            S.b1u = of(C.b1u);
+            S.b1v = of(C.b1v);
+            S.b2 = of(C.b2);
+            S.uc = of(C.uc);
+            S.ic = of(C.ic);
+            S.v = of(C.v);
+            wide_cons_states<ORDER>(L, f.of(src), S, r, s, d);
+        },
+        [&](int from) {
+            wide_take(r, from, o.r);
+            wide_take(s, from, o.s);
+            wide_take(d, from, o.d);
+        });
+}
+#endif
 
 }  // namespace fx
 }  // namespace gbr

@@ -49,6 +49,8 @@ static void sides(const R* q, int order, R& l, R& r)
     for (int k = 0; k < 5; ++k) a[k] = q[8 - k], b[k] = -e[8 - k];
     r = meg(a, b, order);
 }
+typedef fx::WideLanes::V Lanes;
+static const fx::WideLanes four{};
 // four variables of 12 cells as planes with a step, y-face order where `normal` is 2
 struct Data {
     double v[4][12];
@@ -100,8 +102,15 @@ static int prim(int lr)
         fx::FaceStates o;
         fx::face_states<ORDER>(D, fx::pos(0.5 * y), fx::pos(2 * rc), fx::pos(ic2), o);
         if (!o.ok) return std::printf("refused\n"), 1;
-        if (o.wide) fx::wide_states<ORDER>(D.face(), 1.4, o);
-        if (o.wide_ut) fx::wide_shear<ORDER>(D.face(), o.ut);
+        if (o.wide) {
+            Lanes r, u, p;
+            fx::wide_states<ORDER>(four, D.face(), 1.4, r, u, p);
+            for (int s = 0; s < 2; ++s) o.r[s] = r.x[s], o.un[s] = u.x[s], o.p[s] = p.x[s];
+        }
+        if (o.wide_ut) {
+            const Lanes t = fx::wide_shear<ORDER>(four, D.face());
+            for (int s = 0; s < 2; ++s) o.ut[s] = t.x[s];
+        }
         R w[4][2];
         for (int f = 0; f < 4; ++f) {
             R q[12];
@@ -150,8 +159,15 @@ static int cons(int lr)
         fx::ConsStates o;
         fx::cons_states<7>(D, [&](int m) { fx::Stencil x; D(m, x); return fx::stencil_exponent(x); }, C, o);
         if (!o.ok) return std::printf("refused\n"), 1;
-        if (o.wide_w3) fx::wide_cons_shear<7>(D.face(), C.v, o.w3);
-        if (o.wide) fx::wide_cons_states<7>(D.face(), C, o);
+        if (o.wide_w3) {
+            const Lanes t = fx::wide_cons_shear<7>(four, D.face(), C.v);
+            for (int s = 0; s < 2; ++s) o.w3[s] = t.x[s];
+        }
+        if (o.wide) {
+            Lanes r, t, d;
+            fx::wide_cons_states<7>(four, D.face(), C, r, t, d);
+            for (int s = 0; s < 2; ++s) o.r[s] = r.x[s], o.s[s] = t.x[s], o.d[s] = d.x[s];
+        }
         R w[4][2];
         for (int f = 0; f < 4; ++f) {
             R q[12];
