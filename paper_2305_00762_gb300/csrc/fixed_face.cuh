@@ -43,9 +43,9 @@
 // not taken: where the product is not positive, Phi^L lies between Phi_j and
 // Phi^MP, so inside both intervals of Eq. mp-procedure, and the clamp to
 // [Phi^min, Phi^max] returns it unchanged; on integers this holds exactly. A
-// positive product up to 1e-40 moves the result by at most 1e-20. Faces where
-// that is more than rounding (fields below about 2^-12) are evaluated with the
-// test (kSmall).
+// positive product up to 1e-40 moves the result by at most 1e-20. Where that is
+// more than rounding (fields below about 2^-12), faces with a limited value that
+// close to its unlimited one are evaluated with the test (is_small_field).
 //
 // Overflow. With |I| < 2^59 = M after projection the largest intermediate is
 // the bound UL = Phi_j + 7 (Phi_j - Phi_{j-1}), at most 15 M < 2^63 (LC: 14.7 M).
@@ -55,8 +55,10 @@
 
 #ifdef __CUDACC__
 #define GBR_HD __host__ __device__ __forceinline__
+#define GBR_CALL __host__ __device__ __noinline__
 #else
 #define GBR_HD inline
+#define GBR_CALL inline
 #include <string.h>
 #endif
 
@@ -409,10 +411,29 @@ GBR_HD u64 factor(double a, int e, int eo)  // of |a|
 // a few units of 2^(kWide-59) of its own terms.
 constexpr int kWide = 5;
 GBR_HD bool is_wide(int scale, int local0, int local1) { return scale - (local0 < local1 ? local0 : local1) > kWide; }
-// Nor are faces where the MP test's threshold tells: 1e-20 (2^-66.4) times what a
-// field is carried at (2^k) is 2^-55 or more of the field's scale.
+// Nor are faces where the MP test's threshold may tell: a value it leaves unlimited
+// lies within 1e-20 (2^-66.4) of the limiter's, times 2^k where the field is carried
+// at up to 2^k times its value. Asked where that is 2^-55 or more of the scale.
 constexpr int kSmall = kOne - 70;
 GBR_HD bool is_small(int scale, int k) { return scale - k <= kSmall; }
+GBR_HD bool within(i64 d, int bits)
+{
+    const i64 g = d >> 63;
+    return d != 0 && ((d ^ g) >> (bits < 62 ? bits : 62)) == 0;
+}
+// (a call, so that other faces branch past it)
+template <int ORDER>
+GBR_CALL bool small_tells(i64 cl, i64 nl, i64 l, i64 cr, i64 nr, i64 r, int bits)
+{
+    return within(cl + grb_delta<ORDER>(nl) - l, bits) || within(cr + grb_delta<ORDER>(nr) - r, bits);
+}
+template <int ORDER>
+GBR_HD bool is_small_field(const Functionals& f, i64 l, i64 r, int scale, int k)
+{
+    bool s = false;
+    if (is_small(scale, k)) s = small_tells<ORDER>(f.v[1], f.n[0], l, f.v[2], f.n[1], r, kOne - 66 - scale + k);
+    return s;
+}
 // The same from a field's values (l, r): a value, its step from the cell's value
 // and the cell's other terms (tl, tr) all below 2^-kWide of the scale. (A field
 // may be small at one cell, as where a velocity changes sign, without losing
@@ -463,7 +484,7 @@ GBR_HD bool shear_states(F load, int still, double (&ut)[2], bool& wide)
     limited<ORDER>(R, l, r);
     ut[0] = to_double(l, e);
     ut[1] = to_double(r, e);
-    wide = e > still && ((still == kExpMin && is_small(e, 0)) || (is_wide(e + 1, x.e[5], x.e[6]) && is_wide_field<ORDER>(R, l, r)));
+    wide = e > still && ((still == kExpMin && is_small_field<ORDER>(R, l, r, e, 0)) || (is_wide(e + 1, x.e[5], x.e[6]) && is_wide_field<ORDER>(R, l, r)));
     return e <= kExpMax;
 }
 
@@ -493,19 +514,20 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         es = (er > eprod ? er : eprod) + 1;
         lr[0] = x.e[5];
         lr[1] = x.e[6];
-        o.wide = is_small(es, 0) || is_wide(es, larger(lr[0], lp[0] + ic2.e - 1022), larger(lr[1], lp[1] + ic2.e - 1022));
+        o.wide = is_wide(es, larger(lr[0], lp[0] + ic2.e - 1022), larger(lr[1], lp[1] + ic2.e - 1022));
         Functionals R, S;
         scale(P, factor(ic2, ep, es), S);
         variable<ORDER>(x, es, R);
         difference(R, S, R);
         limited<ORDER>(R, sl, sr);
+        o.wide = o.wide || is_small_field<ORDER>(R, sl, sr, es, 0);
     }
     {  // fields 1 and 4 (u -/+ c), carried as p -/+ rho c un
         Stencil x;
         load(1, x);
         const int eu = stencil_exponent(x), eprod = eu - 1 + rc2.e - 1022;  // (half of rc2)
         ew = (ep > eprod ? ep : eprod) + 1;
-        o.wide = o.wide || is_small(ew, 1024 - ic2.e) || is_wide(ew, larger(lp[0], x.e[5] + rc2.e - 1023), larger(lp[1], x.e[6] + rc2.e - 1023));
+        o.wide = o.wide || is_wide(ew, larger(lp[0], x.e[5] + rc2.e - 1023), larger(lp[1], x.e[6] + rc2.e - 1023));
         Functionals U, W;
         variable<ORDER>(x, eu, U);
         scale(U, factor(rc2, eu - 1, ew), U);
@@ -513,8 +535,10 @@ GBR_HD void face_states(F load, const Pos& y, const Pos& rc2, const Pos& ic2, Fa
         i64 ml, mr, pl, pr;
         difference(P, U, W);
         limited<ORDER>(W, ml, mr);
+        o.wide = o.wide || is_small_field<ORDER>(W, ml, mr, ew, 1024 - ic2.e);  // (carried at 2 c^2 times the paper's)
         sum(P, U, W);
         limited<ORDER>(W, pl, pr);
+        o.wide = o.wide || is_small_field<ORDER>(W, pl, pr, ew, 1024 - ic2.e);
         const int ev = ew + y.e - 1021;  // (half the mantissa: a bit to spare)
         const bool some = ev >= kExpMin;  // smaller velocities count as zero
         o.un[0] = to_double(some ? mulhi(pl - ml, y.m >> 1) : 0, some ? ev : kExpMin);
@@ -620,18 +644,21 @@ GBR_HD void cons_states(F load, E scale_of, const ConsCoefs& C, ConsStates& o)
         const int still = still_exponent((ql[0] < ql[1] ? ql[0] : ql[1]) + 1023 - exponent(C.ic));  // (momenta: rho c)
         accumulate(W, Q0, C.v, factor(C.v, e[0], es), true);
         limited<ORDER>(W, tl, tr);
-        o.wide = is_small(ea, 1) || is_wide(ea, la[0], la[1]) || is_wide(er, larger(ql[0], la[0]), larger(ql[1], la[1]));
-        o.wide_w3 = es > still + 1 && ((still == kExpMin && is_small(es, 0)) || is_wide_field<ORDER>(W, tl, tr, t0, t1));
+        o.wide = is_wide(ea, la[0], la[1]) || is_wide(er, larger(ql[0], la[0]), larger(ql[1], la[1]));
+        o.wide_w3 = es > still + 1 && ((still == kExpMin && is_small_field<ORDER>(W, tl, tr, es, 0)) || is_wide_field<ORDER>(W, tl, tr, t0, t1));
     }
     i64 al, ar, bl, br, cl, cr;  // 2 w1, 2 w4, w2
     sum(A, T, W);
     limited<ORDER>(W, al, ar);
+    o.wide = o.wide || is_small_field<ORDER>(W, al, ar, ea, 1);
     difference(A, T, W);
     limited<ORDER>(W, bl, br);
+    o.wide = o.wide || is_small_field<ORDER>(W, bl, br, ea, 1);
     shift_right(Q0, er - e[0]);
     shift_right(A, er - ea);
     difference(Q0, A, W);
     limited<ORDER>(W, cl, cr);
+    o.wide = o.wide || is_small_field<ORDER>(W, cl, cr, er, 0);
     o.s[0] = to_double(al + bl, ea - 1);
     o.s[1] = to_double(ar + br, ea - 1);
     o.d[0] = to_double(bl - al, ea - 1);

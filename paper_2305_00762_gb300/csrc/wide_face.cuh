@@ -23,13 +23,15 @@
 // 4.17 and 2.22; four lanes 4.13 and 2.11.)
 //
 // What the accuracy costs, us a pass without / with flags and this code: 64^2 vortex
-// 880 / 897, four-quadrant 400^2 1450 / 1591, 1024^2 3983 / 4135, 4096^2 30770 /
-// 32250, viscous 1280 x 640 3752 / 3862, MEG7-cons 400^2 1918 / 2386, double Mach
-// 1024 x 256 (a shock of ratio 116 through four tiles a row) 1878 / 2115. The flags
-// are 2% everywhere; a tile with a line of such faces takes 1.25 times as long.
+// 880 / 902, four-quadrant 400^2 1450 / 1590, 1024^2 3983 / 4157, 4096^2 30770 /
+// 32640, viscous 1280 x 640 3752 / 3888, MEG7-cons 400^2 1918 / 2387, double Mach
+// 1024 x 256 (a shock of ratio 116 through four tiles a row) 1878 / 2124. The flags
+// are 2.5% everywhere; a tile with a line of such faces takes 1.25 times as long.
 //
 // The MP test's absolute threshold, which fixed point leaves out, is applied here,
-// and faces where it tells (kSmall: densities below 2^-12) are evaluated here too.
+// and faces where it may tell (is_small_field) are evaluated here too: none in
+// ordinary units; four-quadrant 1024^2 with densities of 1e-4 4.19 ms a pass, 1e-12
+// 4.30, 1e-20 5.28.
 #pragma once
 
 #include "fixed_math.cuh"
