@@ -106,6 +106,38 @@ __device__ __forceinline__ void fixed_viscous(const FaceIn<double>& in, const do
     out[3] = rfma(-k.q, tn, rfma(-0.5, w, out[3]));
 }
 
+// The flagged faces of a tile (list: ns whose states, then from L::NF nt whose shear
+// velocities are) shared out among all warps, eight a warp: rho, un and p to S,
+// ut to T (two planes each).
+template <typename L, int BX, int NT, int ORDER>
+__device__ __noinline__ void fixed_share(const long long* m, const unsigned short* e, const unsigned short* list, int ns, int nt,
+                                         double gamma, double* S, double* T)
+{
+    const int tid = threadIdx.x, js = (ns + 7) / 8, jobs = js + (nt + 7) / 8;
+    for (int job = tid >> 5; job < jobs; job += NT / 32) {
+        const bool states = job < js;
+        const int at = 8 * (states ? job : job - js) + ((tid & 31) >> 2), n = states ? ns : nt, k = tid & 3;
+        const int w = list[(states ? 0 : L::NF) + min(at, n - 1)];
+        const bool xf = w < L::NHX, keep = at < n && k < 2;
+        const int w2 = xf ? w : w - L::NHX, fw = xf ? L::HXW : BX, fr = w2 / fw, fc = w2 - fr * fw;
+        const int c = (fr + (xf ? 6 : 5)) * L::RW + fc + (xf ? 5 : 6);
+        const fx::Face f{m + c, e + c, xf ? 1 : L::RW, L::NU, xf ? 1 : 2};
+        const fx::WideLanes lanes{(tid & 31) & 28};
+        if (states) {
+            double r, u, p;
+            fx::wide_states<ORDER>(lanes, f, gamma, r, u, p);
+            if (keep) {
+                S[k * L::NF + w] = r;
+                S[(2 + k) * L::NF + w] = u;
+                S[(4 + k) * L::NF + w] = p;
+            }
+        } else {
+            const double u = fx::wide_shear<ORDER>(lanes, f);
+            if (keep) T[k * L::NF + w] = u;
+        }
+    }
+}
+
 // Whether a CTA has a second thread for every face (whole warps of them).
 constexpr bool fixed_splits_faces(int faces, int threads) { return threads >= 2 * ((faces + 31) / 32 * 32); }
 
@@ -193,6 +225,27 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     if (!staged) return;
     __syncthreads();
 
+    constexpr int HALF = NT / 2;
+    static_assert(NT % 32 == 0, "whole warps");
+    constexpr bool SPLIT = fixed_splits_faces(L::NF, NT);
+    __shared__ double sT[SPLIT ? 6 * L::NF : 1];  // ut L, ut R, F of the face
+    auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };  // (reached from both halves' code)
+    // There too the faces of wide_face.cuh are shared out among all warps, by lists
+    // of those whose states or shear velocities are flagged: one CTA an SM waits for
+    // the slowest of its warps (pass of four steps, each warp its own / shared: double
+    // Mach 60 x 24 468 / 335 us, viscous 100 x 50 502 / 393, four-quadrant 60 x 60 279
+    // / 248, 64^2 vortex, which has none, 45.1 / 45.4 a step; as part of the kernel
+    // instead of a call 51.6, the code of a short launch being fetched as it runs).
+    constexpr bool SHARE = SPLIT && !CONS;
+    __shared__ double sS[SHARE ? 6 * L::NF : 1];  // rho L, R, un L, R, p L, R of a flagged face
+    __shared__ u16 sList[SHARE ? 2 * L::NF : 1];
+    __shared__ int sCount[2];
+    auto share = [&] {  // after both halves have met; true: they meet again
+        const int ns = sCount[0], nt = sCount[1];
+        if (ns + nt > 0) fixed_share<L, BX, NT, ORDER>(sM, sE, sList, ns, nt, ph.gamma, sS, sT);
+        return ns + nt > 0;
+    };
+
     // Phase 1: detector flags, and the gradients the viscous flux takes.
     auto flag = [&](int c, int st) {
         return trouble_filtered(sR + c, st, [&] {
@@ -202,6 +255,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
             return trouble_cell(r + 2, 1);
         }) ? 1 : 0;
     };
+    if (SHARE && tid < 2) sCount[tid] = 0;
     for (int idx = tid; idx < L::NPX; idx += NT) {
         const int a = idx / L::PXW, b = idx - a * L::PXW;
         sPX[idx] = flag((a + 6) * RW + (b + 3), 1);
@@ -237,11 +291,6 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
     // evaluates what the states do not need, the shear field and the flux
     // reconstruction: where one small tile is all an SM has, a face's chain of
     // dependent instructions is the time, 64^2 step 50.0 -> 44.8 us).
-    constexpr int HALF = NT / 2;
-    static_assert(NT % 32 == 0, "whole warps");
-    constexpr bool SPLIT = fixed_splits_faces(L::NF, NT);
-    __shared__ double sT[SPLIT ? 6 * L::NF : 1];  // ut L, ut R, F of the face
-    auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };  // (reached from both halves' code)
     // Whole warps: a lane past the last face repeats it and stores nothing.
     for (int item = tid; item < (SPLIT ? NT : (L::NF + 31) / 32 * 32); item += NT) {
         const bool second = SPLIT && item >= HALF;
@@ -316,8 +365,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                     bool wide;
                     const int still = fx::still_exponent(sE[c], sE[3 * NU + c], sE[c + su], sE[3 * NU + c + su]);
                     const bool in_range = fx::shear_states<ORDER>(load, still, ut, wide);
-                    wide = wide && in_range;
-                    if (any(wide)) fx::wide_shear_warp<ORDER>(face, wide, ut);
+                    if (wide && in_range && live) sList[L::NF + atomicAdd(&sCount[1], 1)] = (u16)w;
                     if (!in_range) ut[0] = __longlong_as_double(0x7ff8000000000000ll);  // refused
                 }
                 if (!trouble) reconstruct();
@@ -330,6 +378,9 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
                     }
                 }
                 meet();
+                if constexpr (SHARE) {
+                    if (share()) meet();
+                }
                 break;
             }
         }
@@ -349,17 +400,27 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
         if constexpr (!CONS) {
             fx::FaceStates s;
             fx::face_states<ORDER, !SPLIT>(load, y, xx * y, ic2, s);
+            const bool wide = s.ok && s.wide && positive;
             if constexpr (SPLIT) {
+                if (wide && live) sList[atomicAdd(&sCount[0], 1)] = (u16)w;
                 meet();
+                if (share()) meet();
                 s.ut[0] = sT[w];
                 s.ut[1] = sT[L::NF + w];
                 s.ok = s.ok && fx::exponent(s.ut[0]) != 2047;
+                if (wide) {
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        s.r[k] = sS[k * L::NF + w];
+                        s.un[k] = sS[(2 + k) * L::NF + w];
+                        s.p[k] = sS[(4 + k) * L::NF + w];
+                    }
+                }
             } else {
-                const bool wide = s.ok && s.wide_ut;
-                if (any(wide)) fx::wide_shear_warp<ORDER>(face, wide, s.ut);
+                const bool wide_ut = s.ok && s.wide_ut;
+                if (any(wide_ut)) fx::wide_shear_warp<ORDER>(face, wide_ut, s.ut);
+                if (any(wide)) fx::wide_states_warp<ORDER>(face, wide, ph.gamma, s);
             }
-            const bool wide = s.ok && s.wide && positive;
-            if (any(wide)) fx::wide_states_warp<ORDER>(face, wide, ph.gamma, s);
             rL = s.r[0], unL = s.un[0], utL = s.ut[0], pL = s.p[0];
             rR = s.r[1], unR = s.un[1], utR = s.ut[1], pR = s.p[1];
             ok = s.ok;
