@@ -95,10 +95,14 @@ FP32_PEAK_NOMINAL = 80550.0   # 152 SMs x 128 FP32 lanes x 2 flop (FMA) x 2.07 G
 # (dram__bytes_read.sum + dram__bytes_write.sum) of
 # `bench.py --profile-only --n N --steps 2 --warmup 1 --state-cache ...`.
 # Re-measure when the kernel changes (None: not measured for this kernel).
-F64_STAGE_DRAM_BYTES = {1024: 61.03e6, 4096: 1402.97e6}
+F64_STAGE_DRAM_BYTES = {1024: 62.49e6, 4096: 1405.71e6}
 # FP64 thread instructions (DADD + DMUL + DFMA) per cell-update of the FP64 stage
-# kernel, from an ncu capture (profiles/fixed_kernel_f64_riemann1024_dram.md).
-F64_STAGE_FP64_INST = 185.1
+# kernel, from an ncu capture (profiles/fixed_kernel_f64_riemann1024_dram.md). The
+# count is of the 1024^2 window state's mean stage; it depends on the flow (the
+# faces on each side of the detector, those beside strong jumps) by a few per cent
+# (its stages: 178 to 196), and is applied to every state.
+F64_STAGE_FP64_INST = 185.6
+F64_STAGE_FP64_INST_STATE = "1024x1024 window state, mean of three stages (ncu)"
 
 
 def fma_peaks():
@@ -612,7 +616,8 @@ def roofline(costs, cells, r64, fma, hbm_peak, n):
                             else "nominal: 152 SMs x 2 FP64 FMA/clk x 2.07 GHz (probe unavailable)"),
             "peak_nominal": FP64_PEAK_NOMINAL / 2.0, "frac_of_nominal": achieved / (FP64_PEAK_NOMINAL / 2.0),
             "kernel": "fixed_kernel (fused residual + RK stage, linear work on the integer pipe)",
-            "fp64_inst_per_cell_update": F64_STAGE_FP64_INST, "flop_per_cell_update": flop_cell,
+            "fp64_inst_per_cell_update": F64_STAGE_FP64_INST, "fp64_inst_counted_on": F64_STAGE_FP64_INST_STATE,
+            "flop_per_cell_update": flop_cell,
             "algorithmic_gflops": alg, "algorithmic_over_fp64_fma_peak": alg / fma_peak,
             "stage_ms_avg": stage_s * 1e3,
             "hbm_achieved_gbs": hbm, "hbm_peak_gbs": hbm_peak, "hbm_frac": hbm / hbm_peak}

@@ -12,9 +12,10 @@
 // pipe saturated) 1024^2 6.57 ms, 400^2 1.28 ms, viscous 1280 x 640 6.06 ms;
 // with the face states here 3.66 / 0.73 / 3.93 ms; with the roots and
 // reciprocals, the primitives, the cell fluxes and their reconstruction on
-// integers too (fixed_math.cuh, fixed_stage.cuh) 1.94 / 0.37 / 2.13 ms. The
-// stage is then bound by the integer pipe and FP64 about alike (54% and 58% of
-// what each can issue), at 16 warps an SM.
+// integers too (fixed_math.cuh, fixed_stage.cuh) 1.99 / 0.36 / 1.88 ms, and
+// 2.08 / 0.40 / 1.94 ms with the faces beside strong jumps at the accuracy of their
+// own cells (wide_face.cuh). The stage is then bound by the integer pipe and FP64
+// about alike (57% and 61% of what each can issue), at 16 warps an SM.
 //
 // Scaling. A variable q of one face's stencil (cells j-5 .. j+6) is held as
 // I = q / 2^(e - 1081) with e the largest biased exponent of the stencil, so

@@ -4,10 +4,10 @@
 // face's stencils are aligned to their own scale by a shift each; face states
 // (fixed_face.cuh), flux reconstruction and the viscous gradients are integer
 // sums, and so are the primitives and the cell fluxes (fixed_math.cuh). FP64
-// arithmetic remains for the Riemann solver, the viscous flux and the stage
-// update. With CONS (MEG7-cons)
-// the planes taken apart are the conservative variables, and the primitives of
-// the cells beside faces are kept as they are.
+// arithmetic remains for the Riemann solver, the viscous flux, the stage update
+// and the limiter of the few faces beside strong jumps (wide_face.cuh). With CONS
+// (MEG7-cons) the planes taken apart are the conservative variables, and the
+// primitives of the cells beside faces are kept as they are.
 #pragma once
 
 #include "stage_kernel.cuh"
@@ -540,7 +540,7 @@ __device__ __forceinline__ void fixed_tile(const StageParams& P, const int tx0, 
 
 // The instances of the smallest tile read ghost cells through the boundary
 // rules: on the grids that take it a ghost fill before every stage is a
-// quarter of the step (64^2: 57 -> 49 us without), where in the larger tiles the
+// quarter of the step (64^2: 57 -> 50 us without), where in the larger tiles the
 // code for it costs registers that they need (1024^2 2.0% slower with it).
 constexpr bool fixed_maps_ghosts(int bx) { return bx == 8; }
 

@@ -23,9 +23,9 @@
 // 4.17 and 2.22; four lanes 4.13 and 2.11.)
 //
 // What the accuracy costs, us a pass without / with flags and this code: 64^2 vortex
-// 880 / 902, four-quadrant 400^2 1450 / 1590, 1024^2 3983 / 4157, 4096^2 30770 /
-// 32640, viscous 1280 x 640 3752 / 3888, MEG7-cons 400^2 1918 / 2387, double Mach
-// 1024 x 256 (a shock of ratio 116 through four tiles a row) 1878 / 2124. The flags
+// 880 / 908, four-quadrant 400^2 1450 / 1597, 1024^2 3983 / 4147, 4096^2 30770 /
+// 32640, viscous 1280 x 640 3752 / 3877, MEG7-cons 400^2 1918 / 2389, double Mach
+// 1024 x 256 (a shock of ratio 116 through four tiles a row) 1878 / 2114. The flags
 // are 2.5% everywhere; a tile with a line of such faces takes 1.25 times as long.
 //
 // The MP test's absolute threshold, which fixed point leaves out, is applied here,
